@@ -1,6 +1,8 @@
-"""ctypes binding of libuniql.so: argument marshalling only.
+"""Python binding of libuniql.so: argument marshalling only.
 
-Function names follow the C ABI (include/uniql.h).  Tensors are torch CUDA tensors used
+The calls of the hot path are entry points of a C extension (csrc/pybind.cpp: marshalling them through ctypes cost
+5 - 8 us of host time a call, more than the launch); the rest goes through ctypes, which also stays open to callers of
+the C ABI through lib().  Function names follow the C ABI (include/uniql.h).  Tensors are torch CUDA tensors used
 as device buffers; the current torch stream is passed unless one is given.  There is no
 fallback: if the CUDA library is missing or fails to load, importing this module raises.
 """
@@ -8,7 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
-from typing import List, Optional, Sequence, Tuple
+from typing import Optional, Sequence, Tuple
 
 import torch
 
@@ -47,6 +49,7 @@ if not os.path.exists(LIB_PATH):
     raise ImportError("libuniql.so is not built (run `python -m paper_2512_03383_b200.build`); "
                       "there is no fallback path")
 _lib = ctypes.CDLL(LIB_PATH)
+from . import _calls  # noqa: E402  (links against the library loaded above and torch's)
 
 _vp, _i, _i64, _sz, _d = ctypes.c_void_p, ctypes.c_int, ctypes.c_int64, ctypes.c_size_t, ctypes.c_double
 _lib.uniql_version.restype = _i
@@ -191,18 +194,6 @@ def workspace_status(ws: Optional[torch.Tensor] = None) -> int:
     return int(out.value)
 
 
-def qlinear(x, packed_w, scales, zeros, M, K, N, k_in, k_out, y, stream=None) -> None:
-    _check(_lib.uniql_qlinear(_ptr(x), _ptr(packed_w), _ptr(scales), _ptr(zeros), M, K, N, k_in, k_out, _ptr(y),
-                              _stream(stream)), "uniql_qlinear")
-
-
-def qlinear_noalloc(x, packed_w, scales, zeros, M, K, N, k_in, k_out, y, stream=None) -> None:
-    """uniql_qlinear for callers that must not allocate device memory: the kernel's scratch is a fixed
-    array inside the library (decode sizes only, M <= 16)."""
-    _check(_lib.uniql_qlinear_noalloc(_ptr(x), _ptr(packed_w), _ptr(scales), _ptr(zeros), M, K, N, k_in, k_out,
-                                      _ptr(y), _stream(stream)), "uniql_qlinear_noalloc")
-
-
 def noalloc_status() -> int:
     """Status word of the uniql_qlinear_noalloc calls made so far (synchronises the device; allocates nothing)."""
     v = ctypes.c_int(0)
@@ -210,90 +201,20 @@ def noalloc_status() -> int:
     return int(v.value)
 
 
-def qlinear_ex(x, ldx, packed_w, scales, zeros, bias, M, K, N, in_map, k_in, out_map, k_out, y, ldy,
-               workspace=None, stream=None) -> None:
-    im, om = chanmap(in_map), chanmap(out_map)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(_lib.uniql_qlinear_ex(_ptr(x), ldx, _dt(x), _ptr(packed_w), _ptr(scales), _ptr(zeros), _ptr(bias), M, K,
-                                 N, _mapref(im), k_in, _mapref(om), k_out, _ptr(y), ldy, _ptr(workspace), ws_bytes,
-                                 _stream(stream)), "uniql_qlinear_ex")
-
-
-def qlinear_multi(x, ldx, M, K, in_map, k_in, jobs: List[dict], workspace=None, stream=None) -> None:
-    """jobs: dicts with packed_w, scales, zeros, bias(None), N, k_out, out_map(None), y, ldy."""
-    arr = (_Job * len(jobs))()
-    keep = []
-    for i, j in enumerate(jobs):
-        om = chanmap(j.get("out_map"))
-        keep.append(om)
-        arr[i].packed_w = j["packed_w"].data_ptr()
-        arr[i].scales = j["scales"].data_ptr()
-        arr[i].zeros = j["zeros"].data_ptr()
-        arr[i].bias = None if j.get("bias") is None else j["bias"].data_ptr()
-        arr[i].N = j["N"]
-        arr[i].k_out = j.get("k_out", 0)
-        arr[i].out_map = ctypes.pointer(om) if om is not None else None
-        arr[i].y = j["y"].data_ptr()
-        arr[i].ldy = j["ldy"]
-    im = chanmap(in_map)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(_lib.uniql_qlinear_multi(_ptr(x), ldx, _dt(x), M, K, _mapref(im), k_in, len(jobs), arr, _ptr(workspace),
-                                    ws_bytes, _stream(stream)), "uniql_qlinear_multi")
-
-
-def qk_rope_proj(x, ldx, wq, sq, zq, wk, sk, zk, bq, bk, M, K, n_q_heads, n_kv_heads, head_dim, head_keep,
-                 retained_idx, pos, theta, inv_freq, q_out, ldq, k_out, ldk, workspace=None, stream=None) -> None:
-    f = None
-    if inv_freq is not None:
-        f = (ctypes.c_double * len(inv_freq))(*[float(v) for v in inv_freq])
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(_lib.uniql_qk_rope_proj(_ptr(x), ldx, _dt(x), _ptr(wq), _ptr(sq), _ptr(zq), _ptr(wk), _ptr(sk), _ptr(zk),
-                                   _ptr(bq), _ptr(bk), M, K, n_q_heads, n_kv_heads, head_dim, head_keep,
-                                   _ptr(retained_idx), _ptr(pos), float(theta), f, _ptr(q_out), ldq, _ptr(k_out),
-                                   ldk, _ptr(workspace), ws_bytes, _stream(stream)), "uniql_qk_rope_proj")
-
-
 def mlp_workspace_bytes(M: int, hidden: int, inter: int) -> int:
     return int(_lib.uniql_mlp_workspace_bytes(M, hidden, inter))
 
 
-def mlp_swiglu_decode(x, ldx, wg, sg, zg, wu, su, zu, wd, sd, zd, M, hidden, inter, k_int, h, ldh, y, ldy,
-                      fuse=-1, workspace=None, stream=None) -> None:
-    if x.dtype != torch.float16 or h.dtype != torch.float16 or y.dtype != torch.float16:
-        raise TypeError("uniql_mlp_swiglu_decode computes in fp16")
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(_lib.uniql_mlp_swiglu_decode(_ptr(x), ldx, _ptr(wg), _ptr(sg), _ptr(zg), _ptr(wu), _ptr(su), _ptr(zu),
-                                        _ptr(wd), _ptr(sd), _ptr(zd), M, hidden, inter, k_int, _ptr(h), ldh,
-                                        _ptr(y), ldy, int(fuse), _ptr(workspace), ws_bytes, _stream(stream)),
-           "uniql_mlp_swiglu_decode")
-
-
-def mlp_swiglu(x, ldx, wg, sg, zg, wu, su, zu, wd, sd, zd, M, hidden, inter, k_int, h, ldh, y, ldy,
-               workspace=None, stream=None) -> None:
-    """uniql_mlp_swiglu: the SwiGLU MLP block for fp16 or bf16 activations and any M (x, h, y of one type)."""
-    if h.dtype != x.dtype or y.dtype != x.dtype:
-        raise TypeError("x, h and y must have the same type")
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(_lib.uniql_mlp_swiglu(_ptr(x), ldx, _dt(x), _ptr(wg), _ptr(sg), _ptr(zg), _ptr(wu), _ptr(su), _ptr(zu),
-                                 _ptr(wd), _ptr(sd), _ptr(zd), M, hidden, inter, k_int, _ptr(h), ldh, _ptr(y), ldy,
-                                 _ptr(workspace), ws_bytes, _stream(stream)), "uniql_mlp_swiglu")
-
-
-def qkv_rope_proj(x, ldx, wq, sq, zq, wk, sk, zk, wv, sv, zv, bq, bk, bv, M, K, n_q_heads, n_kv_heads, head_dim,
-                  head_keep, v_keep, retained_idx, pos, theta, inv_freq, q_out, ldq, k_out, ldk, v_out, ldv,
-                  workspace=None, stream=None) -> None:
-    f = None
-    if inv_freq is not None:
-        f = (ctypes.c_double * len(inv_freq))(*[float(v) for v in inv_freq])
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(_lib.uniql_qkv_rope_proj(_ptr(x), ldx, _dt(x), _ptr(wq), _ptr(sq), _ptr(zq), _ptr(wk), _ptr(sk), _ptr(zk),
-                                    _ptr(wv), _ptr(sv), _ptr(zv), _ptr(bq), _ptr(bk), _ptr(bv), M, K, n_q_heads,
-                                    n_kv_heads, head_dim, head_keep, v_keep, _ptr(retained_idx), _ptr(pos),
-                                    float(theta), f, _ptr(q_out), ldq, _ptr(k_out), ldk, _ptr(v_out), ldv,
-                                    _ptr(workspace), ws_bytes, _stream(stream)), "uniql_qkv_rope_proj")
-
-
-def embed_rows(packed, scales, zeros, ids, out, bad_id=None, stream=None) -> None:
-    V, K = packed.shape[0], packed.shape[1] * 2
-    _check(_lib.uniql_embed_rows(_ptr(packed), _ptr(scales), _ptr(zeros), V, K, _ptr(ids), ids.numel(), _dt(out),
-                                 _ptr(out), out.stride(0), _ptr(bad_id), _stream(stream)), "uniql_embed_rows")
+# The hot entry points, arguments as in the C ABI with tensors for pointers (None: NULL), channel maps as sequences of
+# (start, period, keep, count), `workspace` a tensor or None (the library's own), `stream` last and optional:
+#   qlinear, qlinear_noalloc(x, packed_w, scales, zeros, M, K, N, k_in, k_out, y, stream)
+#   qlinear_ex(x, ldx, packed_w, scales, zeros, bias, M, K, N, in_map, k_in, out_map, k_out, y, ldy, workspace, stream)
+#   qlinear_multi(x, ldx, M, K, in_map, k_in, jobs, workspace, stream)
+#       jobs: dicts with packed_w, scales, zeros, bias(None), N, k_out, out_map(None), y, ldy
+#   qk_rope_proj, qkv_rope_proj, mlp_swiglu, mlp_swiglu_decode (fp16, with fuse=-1 before workspace)
+#   embed_rows(packed, scales, zeros, ids, out, bad_id, stream)
+_calls.set_error(UniqlError)
+qlinear, qlinear_noalloc, qlinear_ex, qlinear_multi = (
+    _calls.qlinear, _calls.qlinear_noalloc, _calls.qlinear_ex, _calls.qlinear_multi)
+qk_rope_proj, qkv_rope_proj = _calls.qk_rope_proj, _calls.qkv_rope_proj
+mlp_swiglu_decode, mlp_swiglu, embed_rows = _calls.mlp_swiglu_decode, _calls.mlp_swiglu, _calls.embed_rows

@@ -353,6 +353,24 @@ extern "C" int uniql_qlinear(const void* x, const uint8_t* packed_w, const void*
 
 namespace {
 
+// Rotation frequencies as fractions of a turn.  A model calls with the same head_dim and theta (or table) for every
+// layer and token, and 64 powers and extended-precision fractions cost 7 us of host time, three times the launch: each
+// thread keeps the table it made last, next to the arguments it was made from.
+void rope_turns(int head_dim, double theta, const double* inv_freq, unsigned long long* turn) {
+  struct Table { int head_dim = 0; bool given = false; double theta = 0, freq[kMaxHalfDim]; unsigned long long turn[kMaxHalfDim]; };
+  static thread_local Table t;
+  const int half = head_dim / 2;
+  const bool same = t.head_dim == head_dim && t.given == (inv_freq != nullptr) &&
+                    (inv_freq ? memcmp(t.freq, inv_freq, (size_t)half * sizeof(double)) == 0 : t.theta == theta);
+  if (!same) {
+    t.head_dim = head_dim; t.given = inv_freq != nullptr; t.theta = theta;
+    if (inv_freq) memcpy(t.freq, inv_freq, (size_t)half * sizeof(double));
+    for (int i = 0; i < half; ++i)
+      t.turn[i] = rope_turn_of(inv_freq ? inv_freq[i] : pow(theta, -2.0 * (double)i / (double)head_dim));
+  }
+  memcpy(turn, t.turn, (size_t)half * sizeof(turn[0]));
+}
+
 // Q and K projections with the rotary epilogue and, when wv is given, the V projection (plain rows, the
 // leading v_keep of every key-value head) as a third job of the same launch.
 int qkv_rope_impl(const void* x, int ldx, int dt, const uint8_t* wq, const void* sq, const void* zq,
@@ -393,8 +411,7 @@ int qkv_rope_impl(const void* x, int ldx, int dt, const uint8_t* wq, const void*
   p.x = x; p.ldx = ldx; p.dt = dt; p.M = M; p.K = K; p.k_in = K;
   p.n_jobs = wv ? 3 : 2;
   p.idx = retained_idx; p.pos = pos;
-  for (int i = 0; i < head_dim / 2; ++i)
-    p.rope_turn[i] = rope_turn_of(inv_freq ? inv_freq[i] : pow(theta, -2.0 * (double)i / (double)head_dim));
+  rope_turns(head_dim, theta, inv_freq, p.rope_turn);
   for (int j = 0; j < 2; ++j) {
     JobDev& d = p.job[j];
     int nh = j == 0 ? n_q_heads : n_kv_heads;
