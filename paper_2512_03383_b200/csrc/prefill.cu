@@ -284,6 +284,12 @@ __device__ inline void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
+// one lane of a converged warp (always the same one)
+__device__ inline bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r != 0;
+}
 // arrives on `bar` when all MMAs issued so far by this thread have completed
 __device__ inline void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -427,7 +433,7 @@ template <typename T, bool CONV, bool HEADS>
 __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__ Params p,
                                                          const __grid_constant__ PrefillCfg c) {
   extern __shared__ unsigned char psmem_raw[];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (warp-uniform for the compiler)
   // Programmatic dependent launch: the next kernel of the stream may be set up while this one runs (its blocks
   // become resident as ours leave).  What a block does before its own `griddepcontrol.wait` touches nothing a
   // predecessor may still write or read: barriers, tensor memory, and the weights, which no kernel writes (the
@@ -787,7 +793,9 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     }
   } else if (warp == 1) {
     // ===================================================================== MMA issue
-    if (lane == 0) {
+    // (the whole warp walks the loop, so that stage indexes, parities and descriptors are warp-uniform; one elected
+    //  lane issues)
+    {
       int s = 0; uint32_t par = 0; int tcount = 0;         // weight stage and its parity
       int sb = 0; uint32_t parb = 0;                       // activation box slot and its parity
       SegIter si; si.init(c, blockIdx.x, gridDim.x);
@@ -809,30 +817,39 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)((acc0 + h) * MAXBN);
             const uint64_t bdesc = smem_desc_sw128(sbase + B_RING + sb * B_BYTES);
+            if (elect_one()) {
 #pragma unroll
-            for (int k16 = 0; k16 < BK / 16; ++k16)     // 32 bytes along K per MMA: +2 in the address field
-              umma_f16(d_tmem, adesc + 2 * k16, bdesc + 2 * k16, c.idesc, (kb > sg.kb0 || k16 > 0) ? 1u : 0u);
-            umma_commit(empty_b + 8 * sb);              // the box is free once these MMAs have read it
+              for (int k16 = 0; k16 < BK / 16; ++k16)     // 32 bytes along K per MMA: +2 in the address field
+                umma_f16(d_tmem, adesc + 2 * k16, bdesc + 2 * k16, c.idesc, (kb > sg.kb0 || k16 > 0) ? 1u : 0u);
+              umma_commit(empty_b + 8 * sb);              // the box is free once these MMAs have read it
+              if (h == h_hi - 1) umma_commit(empty_a + 8 * s);   // ... and the weight stage after the last of them
+            }
+            __syncwarp();
             if (++sb == BSLOTS) { sb = 0; parb ^= 1; }
           }
           if (failed) break;
-          umma_commit(empty_a + 8 * s);                 // ... and the weight stage after the last of them
           if (++s == PSTAGES) { s = 0; par ^= 1; }
         }
         if (failed) break;
-        for (int h = h_lo; h < h_hi; ++h) umma_commit(acc_full + 8 * (acc0 + h));
         // (the de-quantiser warps that help with the last segment's epilogue cannot follow the phases of the
         //  accumulator barriers -- a parity wait cannot tell "not yet" from "two phases ago" -- so the last
         //  segment completes a barrier of its own, which has this one phase)
         SegIter peek = si;
         Seg nxt;
-        if (!peek.next(nxt)) umma_commit(last_full);
+        const bool last = !peek.next(nxt);
+        if (elect_one()) {
+          for (int h = h_lo; h < h_hi; ++h) umma_commit(acc_full + 8 * (acc0 + h));
+          if (last) umma_commit(last_full);
+        }
+        __syncwarp();
       }
       if (c.pair_split && crank == 0 && !failed) {
         // the first block of a pair: once its own MMAs are complete nothing reads its rings any more
         if (pmbar_wait(last_full, 0, abort_flag)) {
-          asm volatile("fence.acq_rel.cluster;" ::: "memory");
-          pmbar_arrive_peer(ppeer_addr(px_ready, 1u));
+          if (lane == 0) {
+            asm volatile("fence.acq_rel.cluster;" ::: "memory");
+            pmbar_arrive_peer(ppeer_addr(px_ready, 1u));
+          }
         } else {
           failed = true;
         }
