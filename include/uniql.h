@@ -21,7 +21,7 @@
  *    host before anything is launched; nothing aborts or throws.
  *  - There is no CPU fallback: without a usable CUDA device calls return
  *    UNIQL_ERR_CUDA.
- *  - Decode launches (M <= 16) and the launches of the tensor-core kernel (M > 16, bf16) carry the
+ *  - Decode launches (M <= 16) and the launches of the tensor-core kernel (M > 16) carry the
  *    programmatic-stream-serialization attribute: back-to-back calls on one stream overlap their launch
  *    set-up and first weight stages with the tail of the preceding one (1.6 us per decode launch, 2 - 4 us
  *    per tensor-core launch), while everything that can depend on the preceding kernel (activations,
@@ -76,15 +76,15 @@ typedef enum {
 
 typedef enum { UNIQL_F16 = 0, UNIQL_BF16 = 1 } uniql_dtype;
 
-/* Kernel selection, for A/B tests.  AUTO: fp16 batches of M <= 16 take the persistent decode kernel
- * (UNIQL_PATH_DECODE); where the input map lies on 4- but not on 8-channel boundaries (head dims 108 and 84 on the
+/* Kernel selection, for A/B tests.  AUTO: batches of M <= 16 take the persistent decode kernel
+ * (UNIQL_PATH_DECODE; bf16 wherever its 16-byte loads apply: input blocks on 8-channel boundaries, or re-laid on them); where the input map lies on 4- but not on 8-channel boundaries (head dims 108 and 84 on the
  * input side of o_proj, 1740 of 2048 leading channels) a small kernel in front re-lays the activations on
  * 8-channel boundaries in the workspace, and batches of M <= 4 for which that is not possible (no room in the
  * workspace, blocks that do not start on 8-channel boundaries) take the streaming kernel (UNIQL_PATH_GEMV:
  * every warp copies its own share of the codes through a private shared-memory ring) when its rules hold (one
  * input family, every start / keep / period a multiple of 4, K a multiple of 512, x 8-byte aligned with ldx a
  * multiple of 4, scale and zero-point arrays 8-byte aligned); everything
- * else (M > 16, bf16) the tensor-core (prefill) kernel when its alignment rules hold (activations 16-byte
+ * else the tensor-core (prefill) kernel when its alignment rules hold (activations 16-byte
  * aligned with a row pitch that is a multiple of 8, input map a leading block or one family of per-head
  * blocks on 64-channel boundaries with keep % 8 == 0), otherwise the generic kernel. */
 typedef enum { UNIQL_PATH_AUTO = 0, UNIQL_PATH_GENERIC = 1, UNIQL_PATH_DECODE = 2,
@@ -313,9 +313,9 @@ int uniql_qkv_rope_proj(const void* x, int ldx, int dt, const uint8_t* wq, const
  * uniql_workspace_init; after a UNIQL_ERR_TIMEOUT status it must be zeroed again before reuse. */
 size_t uniql_mlp_workspace_bytes(int M, int hidden, int inter);
 /* The same block for either activation type and any M: dt = UNIQL_F16 with M <= 16 is
- * uniql_mlp_swiglu_decode(fuse = -1); everything else (M > 16, and bf16 at any M) takes the two launches of
- * the tensor-core kernel described above, x, h and y all of type dt (bf16: the tensor cores run on an fp16
- * copy of x and of h, as for uniql_qlinear; h is rounded to bf16 once).  Same argument meaning and errors. */
+ * uniql_mlp_swiglu_decode(fuse = -1), and bf16 at M <= 16 the same two launches in bf16 where their limits hold (else
+ * as larger batches); M > 16 takes the two launches of the tensor-core kernel described above, x, h and y all of type
+ * dt (bf16: the tensor cores run on an fp16 copy of x and of h, as for uniql_qlinear; h is rounded to bf16 once).  Same argument meaning and errors. */
 int uniql_mlp_swiglu(const void* x, int ldx, int dt, const uint8_t* wg, const void* sg, const void* zg,
                      const uint8_t* wu, const void* su, const void* zu, const uint8_t* wd, const void* sd,
                      const void* zd, int M, int hidden, int inter, int k_int, void* h, int ldh, void* y,

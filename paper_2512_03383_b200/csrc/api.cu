@@ -135,13 +135,11 @@ int relay_candidate(const Params& p, Params* q) {
   return keep8;
 }
 
-int dispatch(const Params& p_in, void* workspace, size_t ws_bytes, void* stream) {
-  if (cudaPeekAtLastError() != cudaSuccess) return UNIQL_ERR_CUDA;
+int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, void* stream) {
   LaunchCfg cfg{workspace, ws_bytes, (cudaStream_t)stream};
-  int path = g_path.load();
   Params p = p_in;
   bool dec_ok = p.M <= 16 && decode_supported(p);
-  // every batch the decode kernel does not take (more than 16 rows, bf16) goes to the tensor cores when the maps
+  // every batch the decode kernel does not take (more than 16 rows) goes to the tensor cores when the maps
   // allow it: at 17..63 rows the generic kernel measured 13 to 26 times slower (930 us against 71 us for the
   // Llama-3-8B gate|up at M = 17)
   bool pre_ok = prefill_supported(p);
@@ -154,12 +152,16 @@ int dispatch(const Params& p_in, void* workspace, size_t ws_bytes, void* stream)
   bool relaid = false;
   // Everything else that misses a fast kernel only because of where its activations lie (blocks of 108 or 84
   // channels, an odd row pitch) gets them re-laid in the workspace by a small kernel in front: 5..16 rows then run
-  // on the integer path of the decode kernel, larger batches and bf16 on the tensor cores.
+  // on the integer path of the decode kernel, larger batches on the tensor cores.
   if (!gv && path != UNIQL_PATH_GENERIC) {
-    const bool decode_size = p.M <= 16 && p.dt == UNIQL_F16 && path != UNIQL_PATH_PREFILL;
-    const bool slow = decode_size ? !(dec_ok && decode_integer_path(p)) : !pre_ok;
+    bool decode_size = p.M <= 16 && path != UNIQL_PATH_PREFILL;
     Params q;
     int keep8 = 0;
+    // (bf16 at decode sizes that the integer path cannot take even re-laid: the tensor cores, as larger batches)
+    if (decode_size && p.dt != UNIQL_F16 && path == UNIQL_PATH_AUTO && !dec_ok &&
+        !(relay_candidate(p, &q) != 0 && decode_supported(q)))
+      decode_size = false;
+    const bool slow = decode_size ? !(dec_ok && decode_integer_path(p)) : !pre_ok;
     if (slow && path != (decode_size ? UNIQL_PATH_PREFILL : UNIQL_PATH_DECODE) && (keep8 = relay_candidate(p, &q)) != 0 &&
         (decode_size ? (decode_supported(q) && decode_integer_path(q)) : prefill_supported(q))) {
       if (!cfg.workspace) {
@@ -234,6 +236,17 @@ int dispatch(const Params& p_in, void* workspace, size_t ws_bytes, void* stream)
     return launch_prefill(p, cfg);
   }
   return launch_generic(p, cfg);
+}
+
+// bf16 at decode sizes ran on the tensor-core kernel until the decode kernel took that type (Qwen2.5-7B layer at two
+// rows: 146 us), and it still does where the caller's workspace holds that kernel's scratch but not the decode kernel's.
+int dispatch(const Params& p, void* workspace, size_t ws_bytes, void* stream) {
+  if (cudaPeekAtLastError() != cudaSuccess) return UNIQL_ERR_CUDA;
+  const int path = g_path.load();
+  const int rc = dispatch_as(p, path, workspace, ws_bytes, stream);
+  if (rc == UNIQL_ERR_WORKSPACE && path == UNIQL_PATH_AUTO && p.dt != UNIQL_F16 && p.M <= 16)
+    return dispatch_as(p, UNIQL_PATH_PREFILL, workspace, ws_bytes, stream);
+  return rc;
 }
 
 }  // namespace
@@ -524,11 +537,13 @@ extern "C" size_t uniql_mlp_workspace_bytes(int M, int hidden, int inter) {
   return a > b ? (a > c ? a : c) : (b > c ? b : c);
 }
 
-extern "C" int uniql_mlp_swiglu_decode(const void* x, int ldx, const uint8_t* wg, const void* sg, const void* zg,
-                                       const uint8_t* wu, const void* su, const void* zu, const uint8_t* wd,
-                                       const void* sd, const void* zd, int M, int hidden, int inter, int k_int,
-                                       void* h, int ldh, void* y, int ldy, int fuse, void* workspace,
-                                       size_t ws_bytes, void* stream) {
+namespace {
+
+// The SwiGLU block for either activation type: decode sizes on the decode kernel, the rest on the tensor cores.
+int mlp_block(const void* x, int ldx, int dt, const uint8_t* wg, const void* sg, const void* zg, const uint8_t* wu,
+              const void* su, const void* zu, const uint8_t* wd, const void* sd, const void* zd, int M, int hidden,
+              int inter, int k_int, void* h, int ldh, void* y, int ldy, int fuse, void* workspace, size_t ws_bytes,
+              void* stream) {
   if (!x || !h || !y) return UNIQL_ERR_NULL;
   if (M < 1 || hidden < kGroup || inter < kGroup || k_int < 1 || k_int > inter) return UNIQL_ERR_SHAPE;
   if (ldx < hidden || ldh < k_int || ldy < hidden) return UNIQL_ERR_SHAPE;
@@ -545,17 +560,24 @@ extern "C" int uniql_mlp_swiglu_decode(const void* x, int ldx, const uint8_t* wg
     rc = lib_workspace(&cfg.workspace, &cfg.ws_bytes, cfg.stream);
     if (rc != UNIQL_OK) return rc;
   }
-  if (M > 16) {
-    if (fuse == 1) return UNIQL_ERR_UNSUPPORTED;
-    return mlp_tensor_core(x, ldx, UNIQL_F16, wg, sg, zg, wu, su, zu, wd, sd, zd, M, hidden, inter, k_int, h, ldh, y, ldy, cfg);
-  }
+  auto tensor_core = [&]() -> int {
+    return mlp_tensor_core(x, ldx, dt, wg, sg, zg, wu, su, zu, wd, sd, zd, M, hidden, inter, k_int, h, ldh, y, ldy, cfg);
+  };
+  if (M > 16) return fuse == 1 ? UNIQL_ERR_UNSUPPORTED : tensor_core();
   MlpDecode d;
   memset(&d, 0, sizeof(d));
+  d.dt = dt;
   d.x = x; d.ldx = ldx; d.M = M; d.hidden = hidden; d.inter = inter; d.k_int = k_int;
   d.wg = wg; d.wu = wu; d.wd = wd;
   d.sg = (const __half*)sg; d.zg = (const __half*)zg; d.su = (const __half*)su; d.zu = (const __half*)zu;
   d.sd = (const __half*)sd; d.zd = (const __half*)zd;
   d.h = h; d.ldh = ldh; d.y = y; d.ldy = ldy;
+  if (dt != UNIQL_F16) {
+    // bf16: the decode kernel where its rules and the workspace allow it, else the tensor cores as for larger batches
+    const bool too_small = workspace && ws_bytes < mlp_decode_workspace_bytes(M, hidden, inter);
+    if ((g_path.load() != UNIQL_PATH_AUTO && g_path.load() != UNIQL_PATH_DECODE) || too_small || !mlp_decode_supported(d))
+      return tensor_core();
+  }
   // one to four rows: two launches of the streaming kernel (unless one launch or the persistent kernel is asked for)
   if (fuse != 1 && gemv_mlp_supported(d) &&
       (g_path.load() == UNIQL_PATH_GEMV ||
@@ -585,28 +607,22 @@ extern "C" int uniql_mlp_swiglu_decode(const void* x, int ldx, const uint8_t* wg
   return run(d);
 }
 
+}  // namespace
+
+extern "C" int uniql_mlp_swiglu_decode(const void* x, int ldx, const uint8_t* wg, const void* sg, const void* zg,
+                                       const uint8_t* wu, const void* su, const void* zu, const uint8_t* wd,
+                                       const void* sd, const void* zd, int M, int hidden, int inter, int k_int,
+                                       void* h, int ldh, void* y, int ldy, int fuse, void* workspace,
+                                       size_t ws_bytes, void* stream) {
+  return mlp_block(x, ldx, UNIQL_F16, wg, sg, zg, wu, su, zu, wd, sd, zd, M, hidden, inter, k_int, h, ldh, y, ldy, fuse,
+                   workspace, ws_bytes, stream);
+}
+
 extern "C" int uniql_mlp_swiglu(const void* x, int ldx, int dt, const uint8_t* wg, const void* sg, const void* zg,
                                 const uint8_t* wu, const void* su, const void* zu, const uint8_t* wd, const void* sd,
                                 const void* zd, int M, int hidden, int inter, int k_int, void* h, int ldh, void* y,
                                 int ldy, void* workspace, size_t ws_bytes, void* stream) {
   if (dt != UNIQL_F16 && dt != UNIQL_BF16) return UNIQL_ERR_DTYPE;
-  if (dt == UNIQL_F16 && M <= 16)
-    return uniql_mlp_swiglu_decode(x, ldx, wg, sg, zg, wu, su, zu, wd, sd, zd, M, hidden, inter, k_int, h, ldh, y, ldy,
-                                   -1, workspace, ws_bytes, stream);
-  if (!x || !h || !y) return UNIQL_ERR_NULL;
-  if (M < 1 || hidden < kGroup || inter < kGroup || k_int < 1 || k_int > inter) return UNIQL_ERR_SHAPE;
-  if (ldx < hidden || ldh < k_int || ldy < hidden) return UNIQL_ERR_SHAPE;
-  int rc = check_weight(wg, sg, zg, inter);
-  if (!rc) rc = check_weight(wu, su, zu, inter);
-  if (!rc) rc = check_weight(wd, sd, zd, hidden);
-  if (rc) return rc;
-  if ((((uintptr_t)x) | ((uintptr_t)h) | ((uintptr_t)y)) & 1) return UNIQL_ERR_ALIGN;
-  if (workspace && (((uintptr_t)workspace) & 255)) return UNIQL_ERR_ALIGN;
-  if (cudaPeekAtLastError() != cudaSuccess) return UNIQL_ERR_CUDA;
-  LaunchCfg cfg{workspace, ws_bytes, (cudaStream_t)stream};
-  if (!cfg.workspace) {
-    rc = lib_workspace(&cfg.workspace, &cfg.ws_bytes, cfg.stream);
-    if (rc != UNIQL_OK) return rc;
-  }
-  return mlp_tensor_core(x, ldx, dt, wg, sg, zg, wu, su, zu, wd, sd, zd, M, hidden, inter, k_int, h, ldh, y, ldy, cfg);
+  return mlp_block(x, ldx, dt, wg, sg, zg, wu, su, zu, wd, sd, zd, M, hidden, inter, k_int, h, ldh, y, ldy, -1, workspace,
+                   ws_bytes, stream);
 }

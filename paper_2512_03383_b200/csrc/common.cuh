@@ -168,12 +168,13 @@ size_t decode_workspace_header_bytes();   // counters + status word: the part th
 // SwiGLU MLP at decode (Section 3.2, MLP paragraph: y = (silu(x Wg^T) * (x Wu^T)) Wd^T with the trailing `inter - k_int`
 // sorted intermediate channels pruned): leading k_int rows of Wg, Wu and leading k_int columns of Wd.
 struct MlpDecode {
-  const void* x; int ldx;      // [M][hidden] fp16
+  const void* x; int ldx;      // [M][hidden] of type dt (as h and y)
+  int dt;
   int M, hidden, inter, k_int;
   const uint8_t *wg, *wu, *wd; // packed [inter][hidden/2], [inter][hidden/2], [hidden][inter/2]
   const __half *sg, *zg, *su, *zu, *sd, *zd;
-  void* h; int ldh;            // [M][k_int] fp16: the gated activations (written, then read)
-  void* y; int ldy;            // [M][hidden] fp16
+  void* h; int ldh;            // [M][k_int]: the gated activations (written, then read)
+  void* y; int ldy;            // [M][hidden]
 };
 // fuse != 0: both products in one launch (UNIQL_ERR_UNSUPPORTED when the shapes do not allow it);
 // fuse == 0: two launches.

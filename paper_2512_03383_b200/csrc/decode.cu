@@ -1,4 +1,4 @@
-// Decode kernel (M = 1..16) of the pruned 4-bit linear layer, sm_100a.
+// Decode kernel (M = 1..16; fp16, and bf16 on the integer path) of the pruned 4-bit linear layer, sm_100a.
 //
 // The decode step streams every retained weight exactly once, so the kernel is built around keeping
 // HBM busy: one persistent block per SM whose producer warp keeps a ring of shared-memory stages
@@ -316,13 +316,14 @@ __device__ inline int compact_channel(const Phase& P, int ch) {
 
 // Quantises the activations of one launch once (streamed mode): half-warp (batch row m, visited group lv).
 // Rows m >= M of the vr / 2 row slots are written as zeros.
+template <typename T>
 __global__ void __launch_bounds__(256) xquant_kernel(const Phase P, int M, int vr, int g_total, unsigned char* xq,
                                                      float2* xg, int xg_stride) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");            // x may come from the preceding kernel
   const int rows = vr >> 1;
   const int n_units = g_total * rows * 16;
-  const __half* x = reinterpret_cast<const __half*>(P.x);
+  const T* x = reinterpret_cast<const T*>(P.x);
   for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < ((n_units + 31) & ~31); u += gridDim.x * blockDim.x) {
     const int u16 = u & 15, pair = u < n_units ? u >> 4 : 0;
     const int lv = pair / rows, m = pair - lv * rows;
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(256) xquant_kernel(const Phase P, int M, int v
     uint2 hi2, lo2;
     int isum;
     float inv_scale;
-    quantise16(in, hi2, lo2, isum, inv_scale);
+    quantise16<T>(in, hi2, lo2, isum, inv_scale);
     if (u < n_units) {
       const int off = (u16 >> 2) * 32 + (u16 & 3) * 8;
       *reinterpret_cast<uint2*>(xq + ((size_t)lv * vr + 2 * m) * 128 + off) = hi2;
@@ -524,11 +525,13 @@ struct UnitIter {
 // tiles of the int8 MMA, each holding the high and the low byte of four batch rows.
 // NPH: phases (2: the fused SwiGLU MLP, integer path only).  XS: activations streamed through the ring.
 // XC: blocks are launched as clusters of two that share the staging of the activations.
-template <int MT, bool ONECOL, int NT, int NPH, bool XS, bool XC>
+// T: activation and output type (bf16: integer path only).  A template parameter although a model never mixes the two:
+// as a flag of the launch it cost the instance for nine to sixteen rows more spills in its loop (Llama-3-8B layer at
+// sixteen rows 79 -> 85 us).
+template <int MT, bool ONECOL, int NT, int NPH, bool XS, bool XC, typename T>
 __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ Params p,
                                                         const __grid_constant__ DecodeCfg c) {
   extern __shared__ unsigned char smem_raw[];
-  using T = __half;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // the stage ring starts on a 1024-byte boundary (the swizzle pattern repeats every 1024 bytes)
   const uint32_t raw = (uint32_t)__cvta_generic_to_shared(smem_raw);
@@ -890,7 +893,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
       for (int i = ctid; i < Gk * 8 * MT; i += CTH) xg[i] = make_float2(0.f, 0.f);
       if (!consumer_sync()) return false;
     }
-    if (NT > 0) {
+    if constexpr (NT > 0) {
       // Integer path.  Per (batch row, group) the activations become 16-bit fixed point, x_i = rint(x * 2^e)
       // with 2^e the largest power of two that keeps the group's maximum at or below 32639 (so that the high
       // byte of x_i + 128 stays a signed byte; exact for every element within a factor 8..16 of the maximum,
@@ -934,7 +937,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
           uint2 hi2, lo2;
           int isum;
           float inv_scale;
-          quantise16(in[q4], hi2, lo2, isum, inv_scale);
+          quantise16<T>(in[q4], hi2, lo2, isum, inv_scale);
           if (in_range) {
             // word j of lane quarter c' (u16 = c'*4 + j): 8 bytes at c'*32 + j*8 of the group's 128 bytes
             const int off = lv * 128 + (u16 >> 2) * 32 + (u16 & 3) * 8;
@@ -968,7 +971,8 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
         if (!ok) { *abort_flag = 1; give_up(); return false; }
         return true;
       }
-    } else if (c.x_vec) {
+    } else {
+    if (c.x_vec) {
       const int n_units = Gn * p.M * 16;
       constexpr int UN = 4;                                        // loads in flight per thread
       for (int u0 = ctid; u0 < ((n_units + 31) & ~31); u0 += CTH * UN) {   // whole warps stay in the shuffles
@@ -1031,6 +1035,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
         }
         if (lane == 0) xg[lv * 8 * MT + m] = make_float2(-(se + so), -(1024.f * se + 64.f * so));
       }
+    }
     }
     if (!consumer_sync()) return false;
     return true;
@@ -1520,9 +1525,9 @@ void fill_split(const DecodeCfg& c, Phase* P) {
   P->by_bt0 = fast_div((unsigned)P->bt0, ut * (unsigned long long)c.n_rp);
 }
 
-template <int MT, bool ONECOL, int NT, int NPH, bool XS = false, bool XC = false>
-int launch_t(const Params& p, const DecodeCfg& c, size_t smem, cudaStream_t stream) {
-  auto kern = decode_kernel<MT, ONECOL, NT, NPH, XS, XC>;
+template <int MT, bool ONECOL, int NT, int NPH, bool XS, bool XC, typename T>
+int launch_as(const Params& p, const DecodeCfg& c, size_t smem, cudaStream_t stream) {
+  auto kern = decode_kernel<MT, ONECOL, NT, NPH, XS, XC, T>;
   {
     // the shared-memory limit of this instance is raised once per device (the call costs about a microsecond)
     static std::mutex mu;
@@ -1572,6 +1577,15 @@ int launch_t(const Params& p, const DecodeCfg& c, size_t smem, cudaStream_t stre
   if (cudaLaunchKernelEx(&lc, kern, p, cc) == cudaSuccess) return UNIQL_OK;
   cudaGetLastError();
   return as_clusters ? UNIQL_ERR_UNSUPPORTED : UNIQL_ERR_CUDA;
+}
+
+template <int MT, bool ONECOL, int NT, int NPH, bool XS = false, bool XC = false>
+int launch_t(const Params& p, const DecodeCfg& c, size_t smem, cudaStream_t stream) {
+  if constexpr (NT > 0 && NPH == 1) {
+    if (p.dt == UNIQL_BF16) return launch_as<MT, ONECOL, NT, NPH, XS, XC, __nv_bfloat16>(p, c, smem, stream);
+  }
+  if (p.dt != UNIQL_F16) return UNIQL_ERR_UNSUPPORTED;
+  return launch_as<MT, ONECOL, NT, NPH, XS, XC, __half>(p, c, smem, stream);
 }
 
 // Visited groups of the input map: from the first to the last 128-channel group that holds a retained
@@ -1672,7 +1686,7 @@ size_t stream_need(const DecodeCfg& c, int M, int g_total, size_t need, StreamWs
   return o->xg_off + (size_t)o->g_pad * 8 * o->slots;
 }
 // The tensor map over the quantised copy, and the small kernel in front that writes it (once per launch).
-int stream_setup(DecodeCfg& c, const Phase& P, int M, int g_total, unsigned char* ws, const StreamWs& o,
+int stream_setup(DecodeCfg& c, const Phase& P, int dt, int M, int g_total, unsigned char* ws, const StreamWs& o,
                  cudaStream_t stream) {
   EncodeTiledFn enc = encoder();
   if (!enc) return UNIQL_ERR_CUDA;
@@ -1695,7 +1709,7 @@ int stream_setup(DecodeCfg& c, const Phase& P, int M, int g_total, unsigned char
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = attr;
   lc.numAttrs = opt(kOptPdl) ? 1 : 0;
-  if (cudaLaunchKernelEx(&lc, xquant_kernel, P, M, c.vr, g_total, ws + o.xq_off,
+  if (cudaLaunchKernelEx(&lc, dt == UNIQL_BF16 ? xquant_kernel<__nv_bfloat16> : xquant_kernel<__half>, P, M, c.vr, g_total, ws + o.xq_off,
                          reinterpret_cast<float2*>(ws + o.xg_off), o.slots) != cudaSuccess) {
     cudaGetLastError();
     return UNIQL_ERR_CUDA;
@@ -1714,7 +1728,8 @@ int decode_streams_batch(const Params& p) {
 
 int decode_supported(const Params& p) {
   if (p.M < 1 || p.M > 16) return 0;
-  if (p.dt != UNIQL_F16) return 0;
+  // (bf16 activations: the integer path only, whose staging takes either type to the same 16-bit fixed point)
+  if (p.dt != UNIQL_F16 && (opt(kOptDecodeI8) == 0 || !decode_integer_path(p))) return 0;
   if ((p.K % (2 * kGroup)) != 0) return 0;
   if (count_tile_fams(p) > kMaxTF) return 0;
   const int gran = copy_granule(p.K / kGroup);
@@ -1902,7 +1917,7 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
     }
   }
   if (c.x_stream) {
-    const int rc = stream_setup(c, c.ph[0], p.M, g_total, ws, sw, cfg.stream);
+    const int rc = stream_setup(c, c.ph[0], p.dt, p.M, g_total, ws, sw, cfg.stream);
     if (rc != UNIQL_OK) return rc;
   }
   if (i8 && p.M > 4 && p.M <= 8) {
@@ -1933,6 +1948,7 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
 // ---------------------------------------------------------------------------------------- SwiGLU MLP
 int mlp_decode_supported(const MlpDecode& d) {
   if (d.M < 1 || d.M > 16) return 0;
+  if (d.dt != UNIQL_F16 && opt(kOptDecodeI8) == 0) return 0;
   if (d.hidden < 2 * kGroup || d.inter < 2 * kGroup) return 0;
   if ((d.hidden % (2 * kGroup)) != 0 || (d.inter % (2 * kGroup)) != 0) return 0;
   if (d.k_int < 8 || d.k_int > d.inter || (d.k_int % 8) != 0) return 0;
@@ -1958,7 +1974,7 @@ int launch_mlp_phases(const MlpDecode& d, int first, int count, const LaunchCfg&
   memset(&p, 0, sizeof(p));
   p.x = first == 0 ? d.x : d.h;
   p.ldx = first == 0 ? d.ldx : d.ldh;
-  p.dt = UNIQL_F16;
+  p.dt = d.dt;
   p.M = d.M;
   p.K = first == 0 ? d.hidden : d.inter;
   p.k_in = first == 0 ? d.hidden : d.k_int;
@@ -2057,7 +2073,7 @@ int launch_mlp_phases(const MlpDecode& d, int first, int count, const LaunchCfg&
     c.grid_wait_limit = shift > 0 ? (shift >= 21 ? 1 : kGridWaitLimit >> shift) : kGridWaitLimit;
   }
   if (c.x_stream) {
-    const int rc = stream_setup(c, c.ph[0], d.M, c.ph[0].g_total, ws, sw, cfg.stream);
+    const int rc = stream_setup(c, c.ph[0], d.dt, d.M, c.ph[0].g_total, ws, sw, cfg.stream);
     if (rc != UNIQL_OK) return rc;
     return launch_t<2, false, 4, 1, true>(p, c, smem, cfg.stream);
   }
@@ -2092,7 +2108,7 @@ int launch_mlp_decode(const MlpDecode& d, int fuse, const LaunchCfg& cfg) {
   // the narrow tiles, the streamed or shared staging of the plain path as they apply
   Params p;
   memset(&p, 0, sizeof(p));
-  p.x = d.h; p.ldx = d.ldh; p.dt = UNIQL_F16; p.M = d.M; p.K = d.inter; p.k_in = d.k_int;
+  p.x = d.h; p.ldx = d.ldh; p.dt = d.dt; p.M = d.M; p.K = d.inter; p.k_in = d.k_int;
   p.imap.n_fam = 1; p.imap.total = d.k_int; p.imap.fam[0] = Fam{0, d.k_int, d.k_int, 1}; p.imap.base[0] = 0;
   p.n_jobs = 1;
   JobDev& jd = p.job[0];

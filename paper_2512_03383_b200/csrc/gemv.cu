@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(GTH, 1) gemv_kernel(const __grid_constant__ Gv
         uint2 hi2, lo2;
         int isum;
         float inv_scale;
-        quantise16(in[k], hi2, lo2, isum, inv_scale);
+        quantise16<__half>(in[k], hi2, lo2, isum, inv_scale);
         const int u16 = u & 15;
         const int off = lvv[k] * 128 + (u16 >> 2) * 32 + (u16 & 3) * 8;
         *reinterpret_cast<uint2*>(xb + (size_t)(2 * mm[k]) * xrow + off) = hi2;
@@ -617,7 +617,7 @@ int launch_gemv(const Params& p, const LaunchCfg& cfg) {
 // SwiGLU MLP (Section 3.2, MLP paragraph) as two launches of the streaming kernel: gate and up rows of the same
 // channel in one lane with silu(g) * u as the epilogue, then the down projection over the leading k_int channels of h.
 int gemv_mlp_supported(const MlpDecode& d) {
-  if (d.M < 1 || d.M > 4) return 0;
+  if (d.M < 1 || d.M > 4 || d.dt != UNIQL_F16) return 0;
   if ((d.hidden % (GCH * kGroup)) != 0 || (d.inter % (GCH * kGroup)) != 0) return 0;
   if (d.k_int < 4 || d.k_int > d.inter || (d.k_int % 4) != 0) return 0;
   if ((d.ldx % 4) != 0 || (d.ldh % 4) != 0 || d.ldx < d.hidden || d.ldh < d.k_int || d.ldy < d.hidden) return 0;

@@ -1,9 +1,8 @@
-// Activation quantisation shared by the decode kernels (sm_100a): fp16 activations become 16-bit fixed point
+// Activation quantisation shared by the decode kernels (sm_100a): fp16 or bf16 activations become 16-bit fixed point
 // per (batch row, 128-channel group), split in two signed bytes, so that the 4-bit codes can go to the int8
 // tensor-core MMA as they lie in memory.
 #pragma once
-#include <cuda_fp16.h>
-#include <stdint.h>
+#include "common.cuh"
 
 namespace uniql {
 
@@ -11,15 +10,19 @@ namespace uniql {
 // point against the group's maximum, x_i = rint(x * 2^e) = 256 * hi + lo with both bytes signed.  Returns this
 // lane's bytes in the order the nibbles leave a weight word (even codes first), the group's integer sum and
 // 2^-e (NaN when the group holds a non-finite activation).  Every lane of the warp must call it (shuffles over the sixteen lanes).
+// T = bf16: 8 significand bits, exact for every element within a factor 2^7 of its group's maximum.  The exponent e is
+// capped at 120 so that 2^e and 2^-e stay normal fp32 numbers: groups whose maximum is under 2^-106 lose bits below 2^-120.
+template <typename T>
 __device__ inline void quantise16(const uint4& in, uint2& hi2, uint2& lo2, int& isum_out, float& inv_scale_out) {
-  const __half2* h2 = reinterpret_cast<const __half2*>(&in);
+  using T2 = typename DT<T>::T2;
+  const T2* h2 = reinterpret_cast<const T2*>(&in);
   float f[8];
   // the group's maximum is taken on the magnitude bits as integers: Inf and NaN compare above every finite value,
   // where a floating-point maximum would drop a NaN
   uint32_t amax_bits = 0u;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const float2 v = __half22float2(h2[i]);
+    const float2 v = DT<T>::to_f2(h2[i]);
     f[2 * i] = v.x; f[2 * i + 1] = v.y;
     amax_bits = max(amax_bits, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu));
   }
@@ -29,7 +32,7 @@ __device__ inline void quantise16(const uint4& in, uint2& hi2, uint2& lo2, int& 
   const bool finite = amax_bits < 0x7f800000u;
   int e = 0;
   if (amax_bits != 0u && finite) {
-    e = 14 - ((int)(amax_bits >> 23) - 127);
+    e = min(14 - ((int)(amax_bits >> 23) - 127), 120);
     if (amax * __uint_as_float((uint32_t)(127 + e) << 23) > 32639.f) --e;     // keep the high byte of x_i + 128 signed
   }
   // a group that holds an Inf or a NaN gets a NaN factor: every output that uses the group becomes NaN
