@@ -187,6 +187,14 @@ int gemv_supported(const Params& p);
 size_t gemv_workspace_bytes(int M, int K, int N_total);
 int launch_gemv_mlp(const MlpDecode& d, const LaunchCfg& cfg);
 int gemv_mlp_supported(const MlpDecode& d);
+// tensor-core kernel for up to 128 rows (csrc/batch.cu), taken by launch_prefill where its rules hold
+int launch_batch(const Params& p, const LaunchCfg& cfg);
+int batch_supported(const Params& p);
+// fp16 copy of bf16 activations [M][k_in], row pitch ldo (a multiple of 8; the columns from k_in on are zeros)
+int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo, cudaStream_t stream);
+// tensor map over activations [M][k_in] for boxes of 64 channels x `rows` tokens, 128-byte swizzle
+int encode_x_map(void* map, const void* x, int k_in, int M, int ldx, int rows, bool bf16);
+int device_sms();             // SMs of the current device
 int launch_prefill(const Params& p, const LaunchCfg& cfg);
 int prefill_supported(const Params& p);
 size_t prefill_workspace_bytes(int M, int K);

@@ -48,13 +48,11 @@
 #include <mutex>
 #include <type_traits>
 
-#include "common.cuh"
+#include "tc.cuh"
 
 namespace uniql {
 namespace {
 
-constexpr int BMW = 128;            // weight rows per tile (MMA M)
-constexpr int BK = 64;              // k per stage: 128 bytes of fp16 / bf16, one swizzle row
 constexpr int MAXBN = 256;          // tokens per tile (MMA N), at most
 constexpr int PSTAGES = 4;                   // ring of de-quantised weight stages (one k-block each)
 constexpr int BSLOTS = 4;                    // ring of activation boxes (one k-block of MAXBN tokens each)
@@ -68,7 +66,6 @@ constexpr int PTH = NWARPS * 32;
 constexpr int DQ_WARP0 = 8, DQ_WARPS = 8;      // warps 8 .. 8 + 2 * DQ_WARPS - 1: the de-quantisers and epilogue helpers
 constexpr int DQ_TEAM_WARPS = 6;               // twelve of them convert: two teams of six warps on alternate stages
 constexpr int EPI_WARP0 = 4;
-constexpr int kPWait = 1 << 20;
 constexpr int kMaxPJobs = kMaxJobs;
 
 struct PrefillCfg {
@@ -185,214 +182,6 @@ struct SegIter {
 // block whose range [U*b/B, U*(b+1)/B) of the left-over units holds unit u (exact in fp64 for these magnitudes)
 __device__ inline int sk_owner(long u, long B, long U) {
   return (int)floor(((double)(u + 1) * (double)B - 1.0) / (double)U);
-}
-
-// ---------------------------------------------------------------------------------------- PTX
-__device__ inline void pmbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ inline void pmbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ inline void pmbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ inline bool pmbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-// `relaxed`: sleep between polls (roles that run several stages ahead and must not steal issue slots)
-__device__ inline bool pmbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, bool relaxed = false) {
-  for (int i = 0; i < kPWait; ++i) {
-    if (pmbar_try(bar, parity)) return true;
-    if (relaxed) __nanosleep(200);
-    if ((i & 63) == 63 && *abort_flag) return false;
-  }
-  *abort_flag = 1;
-  return false;
-}
-// ---- clusters of two (a tile's contraction split over a pair of blocks)
-__device__ inline uint32_t pcluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// address of `addr` (shared memory of this block) in block `rank` of the cluster
-__device__ inline uint32_t ppeer_addr(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-// generic address of `ptr` (shared memory of this block) in block `rank` of the cluster
-__device__ inline float* ppeer_generic(void* ptr, uint32_t rank) {
-  unsigned long long r;
-  asm volatile("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"(reinterpret_cast<unsigned long long>(ptr)), "r"(rank));
-  return reinterpret_cast<float*>(r);
-}
-template <int STRIDE, int K = 0>
-__device__ inline void pld_add_f32x16(uint32_t base, const uint32_t (&v)[16], float (&val)[16]) {
-  if constexpr (K < 16) {
-    float o;
-    asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(o) : "r"(base), "n"(K * STRIDE) : "memory");
-    val[K] = __uint_as_float(v[K]) + o;
-    pld_add_f32x16<STRIDE, K + 1>(base, v, val);
-  }
-}
-__device__ inline void pmbar_arrive_peer(uint32_t addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
-}
-__device__ inline bool pmbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  for (int i = 0; i < kPWait; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    if (ok) return true;
-    __nanosleep(100);
-    if ((i & 63) == 63 && *abort_flag) return false;
-  }
-  *abort_flag = 1;
-  return false;
-}
-__device__ inline void tma_box2(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(bar) : "memory");
-}
-__device__ inline void tmem_alloc(uint32_t smem_dst, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols) : "memory");
-}
-__device__ inline void tmem_relinquish() {
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ inline void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-__device__ inline void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ inline void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// D[tmem] (+)= A[smem desc] * B[smem desc]; accumulate == 0 overwrites D
-__device__ inline void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// one lane of a converged warp (always the same one)
-__device__ inline bool elect_one() {
-  uint32_t r;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
-  return r != 0;
-}
-// arrives on `bar` when all MMAs issued so far by this thread have completed
-__device__ inline void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-// 32 consecutive fp32 columns of this thread's TMEM lane
-__device__ inline void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr) : "memory");
-}
-__device__ inline void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr) : "memory");
-}
-__device__ inline void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ inline void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// Shared-memory matrix descriptor of a K-major tile whose rows are 128 bytes (64 fp16/bf16), 128-byte
-// swizzle: 8-row groups 1024 bytes apart (stride byte offset), leading byte offset unused (1),
-// descriptor version 1 (sm_100), layout type 2 (SWIZZLE_128B).
-__device__ inline uint64_t smem_desc_sw128(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFF) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-__device__ inline uint32_t pand_or(uint32_t a, uint32_t mask, uint32_t magic) {
-  uint32_t d;
-  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(a), "r"(mask), "r"(magic));
-  return d;
-}
-
-// ---------------------------------------------------------------------------------------- tile rows
-// Row r (0..127) of local weight tile `tl` of a job: stored weight row, or -1 when the row is empty.
-// Rope jobs: rows 2i and 2i + 1 are the two members of rotation pair i (first-half member, then its partner),
-// so that the two sit in neighbouring lanes of the epilogue warp that rotates them.  SwiGLU pairs (pair == 1)
-// likewise: rows 2i and 2i + 1 are retained row i of the gate matrix and of the up matrix.
-struct RowInfo { int stored; int out_col; int pair_c; int head; };
-__device__ inline RowInfo tile_row(const JobDev& jb, int tl, int r) {
-  RowInfo o;
-  o.stored = -1; o.out_col = -1; o.pair_c = 0; o.head = 0;
-  if (jb.rope.enabled) {
-    const int half = jb.rope.head_keep >> 1;
-    const int P = tl * (BMW / 2) + (r >> 1);
-    if (P >= jb.rope.n_heads * half) return o;
-    const int h = P / half, cc = P - h * half, hi = r & 1;
-    o.stored = h * jb.rope.head_dim + hi * (jb.rope.head_dim >> 1) + cc;
-    o.out_col = h * jb.rope.head_keep + hi * half + cc;
-    o.pair_c = cc; o.head = h;
-  } else if (jb.pair == 1) {
-    const int j = tl * (BMW / 2) + (r >> 1);
-    if (j >= jb.k_out) return o;
-    o.stored = (jb.omap.n_fam == 1 && jb.omap.fam[0].count == 1) ? jb.omap.fam[0].start + j
-                                                                  : map_compact_to_stored(jb.omap, j);
-    o.out_col = j;
-    o.pair_c = r & 1;          // 0: row of the gate matrix, 1: row of the up matrix
-  } else {
-    const int j = tl * BMW + r;
-    if (j >= jb.k_out) return o;
-    o.stored = (jb.omap.n_fam == 1 && jb.omap.fam[0].count == 1) ? jb.omap.fam[0].start + j
-                                                                  : map_compact_to_stored(jb.omap, j);
-    o.out_col = j;
-  }
-  return o;
-}
-
-// Two bf16 values of a word as two fp16 values (exact for magnitudes in fp16's normal range, which
-// holds LLM activations; larger magnitudes saturate at +-65504 instead of becoming infinite).
-__device__ inline uint32_t bf16x2_to_f16x2(uint32_t w) {
-  uint32_t d;
-  asm("cvt.rn.satfinite.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(__uint_as_float(w & 0xffff0000u)), "f"(__uint_as_float(w << 16)));
-  return d;
-}
-
-// Eight codes of one 32-bit word, in input-channel order, as eight fp16 values packed in a uint4:
-// byte b -> (1024 + c_even, 64 + c_odd) as an fp16 pair (one PRMT, one LOP3), minus (1032, 72) = the
-// exact (c-8) pair, then one fp16 FMA per pair: (c-8)*s + cz with cz = fp16(s*(8-z)).  s is the stored
-// fp16 scale itself, (c-8)*s + cz is rounded once; the only other error is the rounding of cz (2^-12
-// of at most 8 s, shared by the 128 weights of a group).
-__device__ inline uint4 dequant_word(uint32_t w, __half2 s2, __half2 cz2) {
-  uint32_t o[4];
-  const __half2 off = __halves2half2(__ushort_as_half(0x6408), __ushort_as_half(0x5480));
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const uint32_t t = __byte_perm(w, 0u, 0x4040u + 0x0101u * b);
-    const uint32_t v = pand_or(t, 0x00f0000fu, 0x54006400u);
-    const __half2 r = __hfma2(__hsub2(*reinterpret_cast<const __half2*>(&v), off), s2, cz2);
-    o[b] = *reinterpret_cast<const uint32_t*>(&r);
-  }
-  return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
 // bf16 activations -> fp16 copy in the workspace, once per call (every weight tile re-reads the tile of
@@ -520,117 +309,10 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
       const int t = sg.tile;
       const int wt = t / c.n_ttiles, tt = t - wt * c.n_ttiles;
       const int jn = job_of_wt(wt);
-      const JobDev& jb = p.job[jn];
       const int tl = wt - c.wtile_begin[jn];
-      T* y = reinterpret_cast<T*>(jb.y);
-      const T* bias = reinterpret_cast<const T*>(jb.bias);
-      const bool rope = jb.rope.enabled != 0;
       // this thread owns tile row etid (= its TMEM lane); a rope pair sits in lanes 2i, 2i + 1
-      const RowInfo ri = tile_row(jb, tl, etid);
-      float b_own = 0.f;
-      unsigned long long turn = 0;
-      const bool swiglu = jb.pair == 1;
-      if (ri.stored >= 0) {
-        const T* bias_own = (swiglu && (etid & 1)) ? reinterpret_cast<const T*>(p.job[jn + 1].bias) : bias;
-        if (bias_own) b_own = DT<T>::to_f(bias_own[ri.stored]);
-        if (rope) {
-          const int half = jb.rope.head_keep >> 1;
-          int pidx = p.idx[(ri.head / jb.rope.rep) * half + ri.pair_c];
-          pidx = min(max(pidx, 0), (jb.rope.head_dim >> 1) - 1);
-          turn = p.rope_turn[pidx];
-        }
-      }
-      // bias, rotary embedding, rounding and store of 32 tokens of this row (all lanes of the warp call it)
-      auto store_chunk = [&](int tok0, const auto& val) {
-        constexpr int NV = (int)(sizeof(val) / sizeof(float));
-        const int m0 = tt * ntok + tok0;
-        if (rope) {
-          // the even lane of a pair rotates the even tokens, the odd lane the odd ones: one exchange hands
-          // each the other member's value of its token, and it stores both rotated members
-          const bool second = (lane & 1) != 0;
-          const int half = jb.rope.head_keep >> 1;
-          const float b_other = __shfl_xor_sync(0xffffffffu, b_own, 1);
-          const float b_lo = second ? b_other : b_own, b_hi = second ? b_own : b_other;
-          const bool live = ri.stored >= 0;
-          const int left = p.M - m0, odd = second ? 1 : 0;
-          T* yp = y + (live ? ri.out_col - (second ? half : 0) : 0) + (size_t)(m0 + odd) * jb.ldy;   // this lane's first token
-          const size_t step = 2 * (size_t)jb.ldy;
-          const int32_t* pp = p.pos + m0 + odd;
-          if (left >= NV) {                       // a whole chunk of tokens: no test per token
-#pragma unroll
-            for (int k = 0; k < NV; k += 2) {
-              const float got = __shfl_xor_sync(0xffffffffu, second ? val[k] : val[k + 1], 1);
-              const float lo = (second ? got : val[k]) + b_lo, hi = (second ? val[k + 1] : got) + b_hi;
-              float cs, sn;
-              rope_cos_sin(__ldg(pp + k), turn, cs, sn);
-              if (live) {
-                yp[0] = DT<T>::from_f(fmaf(-hi, sn, lo * cs));
-                yp[half] = DT<T>::from_f(fmaf(lo, sn, hi * cs));
-              }
-              yp += step;
-            }
-          } else {
-#pragma unroll
-            for (int k = 0; k < NV; k += 2) {
-              if (k >= left) break;
-              const float got = __shfl_xor_sync(0xffffffffu, second ? val[k] : val[k + 1], 1);
-              const float lo = (second ? got : val[k]) + b_lo, hi = (second ? val[k + 1] : got) + b_hi;
-              if (live && k + odd < left) {
-                float cs, sn;
-                rope_cos_sin(__ldg(pp + k), turn, cs, sn);
-                yp[0] = DT<T>::from_f(fmaf(-hi, sn, lo * cs));
-                yp[half] = DT<T>::from_f(fmaf(lo, sn, hi * cs));
-              }
-              yp += step;
-            }
-          }
-        } else if (swiglu) {
-          // as for a rotation pair: the even lane (gate row) takes the even tokens, the odd lane (up row) the odd
-          // ones, one exchange gives each the other matrix's sum of its token; h = silu(g) * u, one rounding
-          // (the approximate division: two instructions instead of ten in warps that share the issue slots
-          //  with the de-quantisers; exp(-g) beyond fp32 gives a quotient of zero, the limit of silu)
-          const bool second = (lane & 1) != 0;
-          const float b_other = __shfl_xor_sync(0xffffffffu, b_own, 1);
-          const float b_g = second ? b_other : b_own, b_u = second ? b_own : b_other;
-          const bool live = ri.stored >= 0;
-          const int left = p.M - m0, odd = second ? 1 : 0;
-          T* yp = y + (live ? ri.out_col : 0) + (size_t)(m0 + odd) * jb.ldy;          // this lane's first token
-          const size_t step = 2 * (size_t)jb.ldy;
-          if (left >= NV) {                       // a whole chunk of tokens: no test per token
-#pragma unroll
-            for (int k = 0; k < NV; k += 2) {
-              const float got = __shfl_xor_sync(0xffffffffu, second ? val[k] : val[k + 1], 1);
-              const float g = (second ? got : val[k]) + b_g, u = (second ? val[k + 1] : got) + b_u;
-              if (live) *yp = DT<T>::from_f(__fdividef(g, 1.f + __expf(-g)) * u);
-              yp += step;
-            }
-          } else {
-#pragma unroll
-            for (int k = 0; k < NV; k += 2) {
-              if (k >= left) break;
-              const float got = __shfl_xor_sync(0xffffffffu, second ? val[k] : val[k + 1], 1);
-              const float g = (second ? got : val[k]) + b_g, u = (second ? val[k + 1] : got) + b_u;
-              if (live && k + odd < left) *yp = DT<T>::from_f(__fdividef(g, 1.f + __expf(-g)) * u);
-              yp += step;
-            }
-          }
-        } else {
-          if (ri.stored < 0) return;
-          T* yr = y + ri.out_col + (size_t)m0 * jb.ldy;
-          const int left = p.M - m0;
-          if (left >= NV) {                       // a whole chunk of tokens: no test per token
-#pragma unroll
-            for (int k = 0; k < NV; ++k) { *yr = DT<T>::from_f(val[k] + b_own); yr += jb.ldy; }
-          } else {
-#pragma unroll
-            for (int k = 0; k < NV; ++k) {
-              if (k >= left) break;
-              *yr = DT<T>::from_f(val[k] + b_own);
-              yr += jb.ldy;
-            }
-          }
-        }
-      };
+      const RowStore<T> rs(p, jn, tl, etid);
+      auto store_chunk = [&](int tok0, const auto& val) { rs.store(p, tt * ntok + tok0, val); };
       for (int h = h_lo; h < h_hi && !failed && !acc_known_full; ++h)
         if (!pmbar_wait(acc_full + 8 * (acc0 + h), au & 1, abort_flag)) failed = true;
       if (failed) return;
@@ -808,12 +490,12 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
         const int au = c.nh == 2 ? tcount : (tcount >> 1);   // earlier tiles that used this tile's accumulator(s)
         const int h_lo = sg.half < 0 ? 0 : sg.half, h_hi = sg.half < 0 ? c.nh : sg.half + 1;   // (a half tile is a block's last)
         for (int kb = sg.kb0; kb < sg.kb1 && !failed; ++kb) {
-          if (!pmbar_wait(full_a + 8 * s, par, abort_flag)) { failed = true; break; }
+          if (!pmbar_wait_warp(full_a + 8 * s, par, abort_flag)) { failed = true; break; }
           const uint64_t adesc = smem_desc_sw128(sbase + s * A_BYTES);
           for (int h = h_lo; h < h_hi; ++h) {
-            if (kb == sg.kb0 && au >= 1 && !pmbar_wait(acc_empty + 8 * (acc0 + h), (au - 1) & 1, abort_flag)) { failed = true; break; }
+            if (kb == sg.kb0 && au >= 1 && !pmbar_wait_warp(acc_empty + 8 * (acc0 + h), (au - 1) & 1, abort_flag)) { failed = true; break; }
             // (bf16: the de-quantisers waited for the activation box themselves and converted it)
-            if (!CONV && !pmbar_wait(full_b + 8 * sb, parb, abort_flag)) { failed = true; break; }
+            if (!CONV && !pmbar_wait_warp(full_b + 8 * sb, parb, abort_flag)) { failed = true; break; }
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)((acc0 + h) * MAXBN);
             const uint64_t bdesc = smem_desc_sw128(sbase + B_RING + sb * B_BYTES);
@@ -845,7 +527,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
       }
       if (c.pair_split && crank == 0 && !failed) {
         // the first block of a pair: once its own MMAs are complete nothing reads its rings any more
-        if (pmbar_wait(last_full, 0, abort_flag)) {
+        if (pmbar_wait_warp(last_full, 0, abort_flag)) {
           if (lane == 0) {
             asm volatile("fence.acq_rel.cluster;" ::: "memory");
             pmbar_arrive_peer(ppeer_addr(px_ready, 1u));
@@ -1040,14 +722,6 @@ PEncodeFn p_encoder() {
   return fn;
 }
 
-int p_sm_count() {
-  int dev = 0, v = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess &&
-      cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-    return v;
-  return 148;
-}
-
 int host_job_tiles(const JobDev& j) {
   if (j.pair == 2) return 0;                                       // its rows ride in the tiles of the job before
   if (j.pair == 1) return (j.k_out + BMW / 2 - 1) / (BMW / 2);
@@ -1098,6 +772,50 @@ int launch_pt(const Params& p, const PrefillCfg& c, int grid, cudaStream_t strea
 
 }  // namespace
 
+int device_sms() {
+  static std::atomic<int> n[64] = {};
+  int dev = 0, v = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+  if ((v = n[dev].load(std::memory_order_relaxed)) > 0) return v;
+  if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) return 148;
+  n[dev].store(v);
+  return v;
+}
+
+int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo, cudaStream_t stream) {
+  const long units = (long)M * (ldo / 8), most = (long)device_sms() * 8;
+  const long blocks = (units + 255) / 256;
+  cudaLaunchConfig_t lc;
+  memset(&lc, 0, sizeof(lc));
+  lc.gridDim = dim3((unsigned)(blocks < most ? blocks : most));
+  lc.blockDim = dim3(256);
+  lc.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = attr;
+  lc.numAttrs = opt(kOptPdl) ? 1 : 0;
+  if (cudaLaunchKernelEx(&lc, x_to_f16_kernel, reinterpret_cast<const __nv_bfloat16*>(x), ldx, M, k_in, reinterpret_cast<__half*>(out), ldo) !=
+      cudaSuccess) {
+    cudaGetLastError();
+    return UNIQL_ERR_CUDA;
+  }
+  return UNIQL_OK;
+}
+
+int encode_x_map(void* map, const void* x, int k_in, int M, int ldx, int rows, bool bf16) {
+  PEncodeFn enc = p_encoder();
+  if (!enc) return UNIQL_ERR_CUDA;
+  const cuuint64_t dims[2] = {(cuuint64_t)k_in, (cuuint64_t)M};
+  const cuuint64_t strides[1] = {(cuuint64_t)ldx * 2};
+  const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)rows};
+  const cuuint32_t es[2] = {1, 1};
+  const CUresult r = enc(reinterpret_cast<CUtensorMap*>(map), bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
+                         const_cast<void*>(x), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                         CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? UNIQL_OK : UNIQL_ERR_CUDA;
+}
+
 // The tensor-core path takes: the leading k_in input channels (the hidden dimension D_h is never pruned,
 // D_int is pruned as a leading block: Section 3.4) or one family of per-head kept blocks (the input side of
 // o_proj / out_proj: heads on 64-channel boundaries, keep a multiple of 8), any output map, both activation types.
@@ -1119,9 +837,12 @@ int prefill_supported(const Params& p) {
 }
 
 int launch_prefill(const Params& p, const LaunchCfg& cfg) {
-  PEncodeFn enc = p_encoder();
-  if (!enc) return UNIQL_ERR_CUDA;
   if (!cfg.workspace || cfg.ws_bytes < decode_workspace_header_bytes()) return UNIQL_ERR_WORKSPACE;   // status word
+  // up to 128 rows: the batch kernel (bf16: where the workspace has room for the fp16 copy)
+  if (batch_supported(p) &&
+      (p.dt != UNIQL_BF16 || (opt(kOptPrefillConvert) != 1 && cfg.ws_bytes >= ((decode_workspace_header_bytes() + 255) & ~(size_t)255) +
+                                                                               (size_t)p.M * ((p.k_in + 63) / 64 * 64) * 2 + 256)))
+    return launch_batch(p, cfg);
   const int env_grid = opt(kOptPrefillGrid), env_streamk = opt(kOptPrefillStreamk);
   PrefillCfg c;
   memset(&c, 0, sizeof(c));
@@ -1142,7 +863,7 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
   // instruction descriptor: fp32 accumulate, A and B of the activation type, both K-major, N = bn, M = 128
   c.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(c.bn >> 3) << 17) | ((uint32_t)(BMW >> 4) << 24);
   c.status = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(cfg.workspace) + decode_status_offset());
-  const int sms = p_sm_count();
+  const int sms = device_sms();
   // workspace: [header: counters, status][fp16 copy of bf16 activations][stream-K partial tiles]
   size_t ws_used = (decode_workspace_header_bytes() + 255) & ~(size_t)255;
   c.counters = reinterpret_cast<int*>(cfg.workspace);
@@ -1286,37 +1007,12 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
       if (pl.atomic && cudaMemsetAsync(c.partials, 0, pl.sums, cfg.stream) != cudaSuccess) return UNIQL_ERR_CUDA;
     }
     if (x16) {
-      const long units = (long)p.M * (x16_ld / 8);
-      long blocks = (units + 255) / 256;
-      if (blocks > (long)sms * 8) blocks = (long)sms * 8;
-      cudaLaunchConfig_t lc;
-      memset(&lc, 0, sizeof(lc));
-      lc.gridDim = dim3((unsigned)blocks);
-      lc.blockDim = dim3(256);
-      lc.stream = cfg.stream;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[0].val.programmaticStreamSerializationAllowed = 1;
-      lc.attrs = attr;
-      lc.numAttrs = opt(kOptPdl) ? 1 : 0;
-      if (cudaLaunchKernelEx(&lc, x_to_f16_kernel, reinterpret_cast<const __nv_bfloat16*>(p.x), p.ldx, p.M, p.k_in, x16, x16_ld) != cudaSuccess) {
-        cudaGetLastError();
-        return UNIQL_ERR_CUDA;
-      }
+      const int rc = launch_x_to_f16(p.x, p.ldx, p.M, p.k_in, x16, x16_ld, cfg.stream);
+      if (rc != UNIQL_OK) return rc;
     }
   }
-  {
-    const cuuint64_t dims[2] = {(cuuint64_t)p.k_in, (cuuint64_t)p.M};
-    const cuuint64_t strides[1] = {(cuuint64_t)ldxs * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)c.bn};
-    const cuuint32_t es[2] = {1, 1};
-    const CUresult r = enc(&c.xmap, conv_in_kernel ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
-                           2, const_cast<void*>(xsrc), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return UNIQL_ERR_CUDA;
-  }
-  int rc;
+  int rc = encode_x_map(&c.xmap, xsrc, p.k_in, p.M, ldxs, c.bn, conv_in_kernel);
+  if (rc != UNIQL_OK) return rc;
   if (p.dt == UNIQL_BF16)
     rc = conv_in_kernel ? launch_pt<__nv_bfloat16, true>(p, c, grid, cfg.stream)
                         : launch_pt<__nv_bfloat16, false>(p, c, grid, cfg.stream);
@@ -1334,7 +1030,7 @@ size_t prefill_workspace_bytes(int M, int K) {
   // status word and counters (shared header) + room for the fp16 copy of bf16 activations + the slots of tiles
   // split along K: fewer than two per SM, of 256 tokens, or of 512 where tiles take both accumulators
   return ((decode_workspace_header_bytes() + 255) & ~(size_t)255) + (size_t)M * ((K + 63) / 64 * 64) * 2 + 256 +
-         (size_t)2 * p_sm_count() * (M > MAXBN ? 2 * MAXBN : MAXBN) * BMW * 4;
+         (size_t)2 * device_sms() * (M > MAXBN ? 2 * MAXBN : MAXBN) * BMW * 4;
 }
 
 }  // namespace uniql

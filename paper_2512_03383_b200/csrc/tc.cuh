@@ -1,0 +1,352 @@
+// What the tensor-core kernels share: PTX wrappers (barriers, TMA, tcgen05), the rows of a weight tile, nibbles to fp16,
+// and the epilogue of a thread that owns one weight row of a tile.
+#pragma once
+#include <stdint.h>
+
+#include "common.cuh"
+
+namespace uniql {
+
+constexpr int BMW = 128;            // weight rows per tile (MMA M)
+constexpr int BK = 64;              // input channels per k-block: 128 bytes of fp16 / bf16, one swizzle row
+constexpr int kPWait = 1 << 20;     // polls of a bounded wait
+
+// ---------------------------------------------------------------------------------------- PTX
+__device__ inline void pmbar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ inline void pmbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ inline void pmbar_expect_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ inline bool pmbar_try(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
+// `relaxed`: sleep between polls (roles that run several stages ahead and must not steal issue slots)
+__device__ inline bool pmbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, bool relaxed = false) {
+  for (int i = 0; i < kPWait; ++i) {
+    if (pmbar_try(bar, parity)) return true;
+    if (relaxed) __nanosleep(200);
+    if ((i & 63) == 63 && *abort_flag) return false;
+  }
+  *abort_flag = 1;
+  return false;
+}
+// The same for a whole warp: one answer for all lanes (a warp whose lanes disagreed about an expired wait would part, and
+// its next warp-wide instruction would wait for the missing lanes).
+__device__ inline bool pmbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, bool relaxed = false) {
+  return __all_sync(0xffffffffu, pmbar_wait(bar, parity, abort_flag, relaxed));
+}
+// ---- clusters of two (a tile's contraction split over a pair of blocks)
+__device__ inline uint32_t pcluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// address of `addr` (shared memory of this block) in block `rank` of the cluster
+__device__ inline uint32_t ppeer_addr(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// generic address of `ptr` (shared memory of this block) in block `rank` of the cluster
+__device__ inline float* ppeer_generic(void* ptr, uint32_t rank) {
+  unsigned long long r;
+  asm volatile("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"(reinterpret_cast<unsigned long long>(ptr)), "r"(rank));
+  return reinterpret_cast<float*>(r);
+}
+template <int STRIDE, int K = 0>
+__device__ inline void pld_add_f32x16(uint32_t base, const uint32_t (&v)[16], float (&val)[16]) {
+  if constexpr (K < 16) {
+    float o;
+    asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(o) : "r"(base), "n"(K * STRIDE) : "memory");
+    val[K] = __uint_as_float(v[K]) + o;
+    pld_add_f32x16<STRIDE, K + 1>(base, v, val);
+  }
+}
+__device__ inline void pmbar_arrive_peer(uint32_t addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+__device__ inline bool pmbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  for (int i = 0; i < kPWait; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    if (ok) return true;
+    __nanosleep(100);
+    if ((i & 63) == 63 && *abort_flag) return false;
+  }
+  *abort_flag = 1;
+  return false;
+}
+__device__ inline void tma_box2(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+      ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+__device__ inline void tmem_alloc(uint32_t smem_dst, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols) : "memory");
+}
+__device__ inline void tmem_relinquish() {
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ inline void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+__device__ inline void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ inline void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+// D[tmem] (+)= A[smem desc] * B[smem desc]; accumulate == 0 overwrites D
+__device__ inline void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// one lane of a converged warp (always the same one)
+__device__ inline bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r != 0;
+}
+// arrives on `bar` when all MMAs issued so far by this thread have completed
+__device__ inline void umma_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+// 32 consecutive fp32 columns of this thread's TMEM lane
+__device__ inline void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr) : "memory");
+}
+__device__ inline void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr) : "memory");
+}
+__device__ inline void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ inline void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// Shared-memory matrix descriptor of a K-major tile whose rows are 128 bytes (64 fp16/bf16), 128-byte
+// swizzle: 8-row groups 1024 bytes apart (stride byte offset), leading byte offset unused (1),
+// descriptor version 1 (sm_100), layout type 2 (SWIZZLE_128B).
+__device__ inline uint64_t smem_desc_sw128(uint32_t addr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((addr & 0x3FFFF) >> 4);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+__device__ inline uint32_t pand_or(uint32_t a, uint32_t mask, uint32_t magic) {
+  uint32_t d;
+  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(a), "r"(mask), "r"(magic));
+  return d;
+}
+
+// ---------------------------------------------------------------------------------------- tile rows
+// Row r (0..127) of local weight tile `tl` of a job: stored weight row, or -1 when the row is empty.
+// Rope jobs: rows 2i and 2i + 1 are the two members of rotation pair i (first-half member, then its partner),
+// so that the two sit in neighbouring lanes of the epilogue warp that rotates them.  SwiGLU pairs (pair == 1)
+// likewise: rows 2i and 2i + 1 are retained row i of the gate matrix and of the up matrix.
+struct RowInfo { int stored; int out_col; int pair_c; int head; };
+__device__ inline RowInfo tile_row(const JobDev& jb, int tl, int r) {
+  RowInfo o;
+  o.stored = -1; o.out_col = -1; o.pair_c = 0; o.head = 0;
+  if (jb.rope.enabled) {
+    const int half = jb.rope.head_keep >> 1;
+    const int P = tl * (BMW / 2) + (r >> 1);
+    if (P >= jb.rope.n_heads * half) return o;
+    const int h = P / half, cc = P - h * half, hi = r & 1;
+    o.stored = h * jb.rope.head_dim + hi * (jb.rope.head_dim >> 1) + cc;
+    o.out_col = h * jb.rope.head_keep + hi * half + cc;
+    o.pair_c = cc; o.head = h;
+  } else if (jb.pair == 1) {
+    const int j = tl * (BMW / 2) + (r >> 1);
+    if (j >= jb.k_out) return o;
+    o.stored = (jb.omap.n_fam == 1 && jb.omap.fam[0].count == 1) ? jb.omap.fam[0].start + j
+                                                                  : map_compact_to_stored(jb.omap, j);
+    o.out_col = j;
+    o.pair_c = r & 1;          // 0: row of the gate matrix, 1: row of the up matrix
+  } else {
+    const int j = tl * BMW + r;
+    if (j >= jb.k_out) return o;
+    o.stored = (jb.omap.n_fam == 1 && jb.omap.fam[0].count == 1) ? jb.omap.fam[0].start + j
+                                                                  : map_compact_to_stored(jb.omap, j);
+    o.out_col = j;
+  }
+  return o;
+}
+
+// Two bf16 values of a word as two fp16 values (exact for magnitudes in fp16's normal range, which
+// holds LLM activations; larger magnitudes saturate at +-65504 instead of becoming infinite).
+__device__ inline uint32_t bf16x2_to_f16x2(uint32_t w) {
+  uint32_t d;
+  asm("cvt.rn.satfinite.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(__uint_as_float(w & 0xffff0000u)), "f"(__uint_as_float(w << 16)));
+  return d;
+}
+
+// Eight codes of one 32-bit word, in input-channel order, as eight fp16 values packed in a uint4:
+// byte b -> (1024 + c_even, 64 + c_odd) as an fp16 pair (one PRMT, one LOP3), minus (1032, 72) = the
+// exact (c-8) pair, then one fp16 FMA per pair: (c-8)*s + cz with cz = fp16(s*(8-z)).  s is the stored
+// fp16 scale itself, (c-8)*s + cz is rounded once; the only other error is the rounding of cz (2^-12
+// of at most 8 s, shared by the 128 weights of a group).
+__device__ inline uint4 dequant_word(uint32_t w, __half2 s2, __half2 cz2) {
+  uint32_t o[4];
+  const __half2 off = __halves2half2(__ushort_as_half(0x6408), __ushort_as_half(0x5480));
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const uint32_t t = __byte_perm(w, 0u, 0x4040u + 0x0101u * b);
+    const uint32_t v = pand_or(t, 0x00f0000fu, 0x54006400u);
+    const __half2 r = __hfma2(__hsub2(*reinterpret_cast<const __half2*>(&v), off), s2, cz2);
+    o[b] = *reinterpret_cast<const uint32_t*>(&r);
+  }
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+
+// ---------------------------------------------------------------------------------------- epilogue of a row
+// Bias, rotary embedding (Section 3.2, fused RoPE) or gated product, one rounding and the stores of a thread that owns
+// row `r` of local tile `tl` of job `jn` (its TMEM lane); the two members of a pair sit in lanes 2i and 2i + 1.
+template <typename T>
+struct RowStore {
+  RowInfo ri;
+  T* y;
+  int ldy, half;
+  bool rope, swiglu;
+  float b_own;
+  unsigned long long turn;
+
+  __device__ inline RowStore(const Params& p, int jn, int tl, int r) {
+    const JobDev& jb = p.job[jn];
+    y = reinterpret_cast<T*>(jb.y);
+    ldy = jb.ldy;
+    rope = jb.rope.enabled != 0;
+    swiglu = jb.pair == 1;
+    half = jb.rope.head_keep >> 1;
+    ri = tile_row(jb, tl, r);
+    b_own = 0.f;
+    turn = 0;
+    if (ri.stored >= 0) {
+      const T* bias = reinterpret_cast<const T*>((swiglu && (r & 1)) ? p.job[jn + 1].bias : jb.bias);
+      if (bias) b_own = DT<T>::to_f(bias[ri.stored]);
+      if (rope) {
+        int pidx = p.idx[(ri.head / jb.rope.rep) * half + ri.pair_c];
+        pidx = min(max(pidx, 0), (jb.rope.head_dim >> 1) - 1);
+        turn = p.rope_turn[pidx];
+      }
+    }
+  }
+  // tokens m0 .. m0 + NV - 1 of the row (all lanes of the warp call it)
+  template <int NV>
+  __device__ inline void store(const Params& p, int m0, const float (&val)[NV]) const {
+    const int lane = threadIdx.x & 31;
+    if (rope) {
+      // the even lane of a pair rotates the even tokens, the odd lane the odd ones: one exchange hands
+      // each the other member's value of its token, and it stores both rotated members
+      const bool second = (lane & 1) != 0;
+      const float b_other = __shfl_xor_sync(0xffffffffu, b_own, 1);
+      const float b_lo = second ? b_other : b_own, b_hi = second ? b_own : b_other;
+      const bool live = ri.stored >= 0;
+      const int left = p.M - m0, odd = second ? 1 : 0;
+      T* yp = y + (live ? ri.out_col - (second ? half : 0) : 0) + (size_t)(m0 + odd) * ldy;   // this lane's first token
+      const size_t step = 2 * (size_t)ldy;
+      const int32_t* pp = p.pos + m0 + odd;
+      if (left >= NV) {                       // a whole chunk of tokens: no test per token
+#pragma unroll
+        for (int k = 0; k < NV; k += 2) {
+          const float got = __shfl_xor_sync(0xffffffffu, second ? val[k] : val[k + 1], 1);
+          const float lo = (second ? got : val[k]) + b_lo, hi = (second ? val[k + 1] : got) + b_hi;
+          float cs, sn;
+          rope_cos_sin(__ldg(pp + k), turn, cs, sn);
+          if (live) {
+            yp[0] = DT<T>::from_f(fmaf(-hi, sn, lo * cs));
+            yp[half] = DT<T>::from_f(fmaf(lo, sn, hi * cs));
+          }
+          yp += step;
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < NV; k += 2) {
+          if (k >= left) break;
+          const float got = __shfl_xor_sync(0xffffffffu, second ? val[k] : val[k + 1], 1);
+          const float lo = (second ? got : val[k]) + b_lo, hi = (second ? val[k + 1] : got) + b_hi;
+          if (live && k + odd < left) {
+            float cs, sn;
+            rope_cos_sin(__ldg(pp + k), turn, cs, sn);
+            yp[0] = DT<T>::from_f(fmaf(-hi, sn, lo * cs));
+            yp[half] = DT<T>::from_f(fmaf(lo, sn, hi * cs));
+          }
+          yp += step;
+        }
+      }
+    } else if (swiglu) {
+      // as for a rotation pair: the even lane (gate row) takes the even tokens, the odd lane (up row) the odd
+      // ones, one exchange gives each the other matrix's sum of its token; h = silu(g) * u, one rounding
+      // (the approximate division: two instructions instead of ten in warps that share the issue slots
+      //  with the de-quantisers; exp(-g) beyond fp32 gives a quotient of zero, the limit of silu)
+      const bool second = (lane & 1) != 0;
+      const float b_other = __shfl_xor_sync(0xffffffffu, b_own, 1);
+      const float b_g = second ? b_other : b_own, b_u = second ? b_own : b_other;
+      const bool live = ri.stored >= 0;
+      const int left = p.M - m0, odd = second ? 1 : 0;
+      T* yp = y + (live ? ri.out_col : 0) + (size_t)(m0 + odd) * ldy;          // this lane's first token
+      const size_t step = 2 * (size_t)ldy;
+      if (left >= NV) {                       // a whole chunk of tokens: no test per token
+#pragma unroll
+        for (int k = 0; k < NV; k += 2) {
+          const float got = __shfl_xor_sync(0xffffffffu, second ? val[k] : val[k + 1], 1);
+          const float g = (second ? got : val[k]) + b_g, u = (second ? val[k + 1] : got) + b_u;
+          if (live) *yp = DT<T>::from_f(__fdividef(g, 1.f + __expf(-g)) * u);
+          yp += step;
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < NV; k += 2) {
+          if (k >= left) break;
+          const float got = __shfl_xor_sync(0xffffffffu, second ? val[k] : val[k + 1], 1);
+          const float g = (second ? got : val[k]) + b_g, u = (second ? val[k + 1] : got) + b_u;
+          if (live && k + odd < left) *yp = DT<T>::from_f(__fdividef(g, 1.f + __expf(-g)) * u);
+          yp += step;
+        }
+      }
+    } else {
+      if (ri.stored < 0) return;
+      T* yr = y + ri.out_col + (size_t)m0 * ldy;
+      const int left = p.M - m0;
+      if (left >= NV) {                       // a whole chunk of tokens: no test per token
+#pragma unroll
+        for (int k = 0; k < NV; ++k) { *yr = DT<T>::from_f(val[k] + b_own); yr += ldy; }
+      } else {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+          if (k >= left) break;
+          *yr = DT<T>::from_f(val[k] + b_own);
+          yr += ldy;
+        }
+      }
+    }
+  }
+};
+
+}  // namespace uniql
