@@ -5,8 +5,8 @@
 // of HBM and at most 1 us of tensor time, but every code has to become an fp16 value on the way.  The prefill kernel
 // writes those values to shared memory, one 64-channel k-block (4 KB of codes) per hand-shake, and took 0.45 us per
 // k-block and SM whatever the batch: 1.3 TB/s.  Here
-//  - a stage is 256 channels of 128 weight rows (16 KB of codes), fetched by cp.async up to seven stages ahead, so that
-//    100 KB per SM are in flight and the hand-shakes are a quarter as many per byte;
+//  - a stage is 256 channels of 128 weight rows (16 KB of codes), one TMA box or a few, fetched up to eight stages ahead,
+//    so that 100 KB per SM are in flight and the hand-shakes are a quarter as many per byte;
 //  - a de-quantiser thread owns a weight row (= a lane of tensor memory) and 64 channels of the stage: two 16-byte
 //    shared loads, 64 values in 32 registers, ONE tcgen05.st: nothing goes back through shared memory, where 16 KB
 //    written and 16 KB read per 8192 weights alone would take 256 cycles against the 195 that HBM needs for their codes;
@@ -17,16 +17,20 @@
 // Roles (one persistent block per SM, 24 warps):
 //   warp 0       activations by TMA: four boxes [64 k x N tokens] per stage, 128-byte swizzle
 //   warp 1       tensor-memory allocation, MMA issue (16 per stage)
-//   warps 2, 3   loaders: codes and scales of a stage by cp.async, 64 rows each
+//   warps 2, 3   loaders: codes by TMA (warp 2), scales and zero-points by cp.async (64 rows each)
 //   warps 4..7   epilogue (bias, rotation or gated product, store; RowStore)
 //   warps 8..23  de-quantisers: warp w rows 32 (w % 4) .. + 31, channels 64 ((w - 8) / 4) .. + 63 of every stage; they
 //                share the epilogue of the block's last segment
 // Tensor memory: two accumulators of N columns, then two or three A stages of 128 columns.
 //
-// Work split: every block runs the same number of whole tiles; the stages of the tiles left over are cut into equal
-// ranges (stream-K), run FIRST, so that their hand-over overlaps the whole tiles.  A part goes to a slot in the workspace
-// ([token][row] fp32); the last block of a tile to arrive adds the slots in block order (deterministic).
-// Pruning (Section 3.4): the rows of a tile are compact output channels mapped to stored rows per lane; the input side is
+// Work split: clusters of p blocks share a tile, every block a p-th of its stages; the cluster takes tiles round-robin.
+// Each block then owns every p-th chunk of 16 tokens: it leaves its fp32 sums of the other chunks in a slot of its own
+// ([token][row], L2), tells the peers (remote arrivals on a barrier in their shared memory), and adds up and finishes its
+// own chunks, always in rank order (deterministic).  No block is the last one that reads everybody's parts: with
+// tiles cut into ranges for single blocks, the last block to arrive finished 6 - 9 us after its last MMA, and the next
+// launch's activations waited for it.
+// Pruning (Section 3.4): a family of kept row blocks is a 3-D tensor (byte in row, row in block, block) as in the decode
+// kernel; a tile is up to 128 rows of one block, or several whole blocks of a box each; the input side is
 // the leading k_in channels (the tensor map of x ends there) or the kept channels of heads whose k-blocks are all
 // visited (pruned words of a partly kept k-block become zero weights).
 // Every wait is bounded; on expiry the block raises a flag, all roles leave, the status word is set.
@@ -46,25 +50,38 @@ constexpr int NW = 24, NTHB = NW * 32;
 constexpr int WST_BYTES = BMW * 128;           // codes of a stage: 128 bytes per row, 16-byte pieces XOR-swizzled by row
 constexpr int SZ_BYTES = BMW * 8;              // two scales and two zero-points per row: [row] half2 s, [row] half2 z
 constexpr int WSTAGE = WST_BYTES + SZ_BYTES;
+constexpr int kMaxBF = 8;                      // row families of a launch
 constexpr int MAX_WST = 8, MAX_BST = 4, MAX_AST = 3;
 constexpr int LOADERS = 2, LD_WARP0 = 2, EPI0 = 4, DQ0 = 8, DQN = 16;
 constexpr int kSmemBatch = 227 * 1024;
 constexpr int kTokChunk = 16;                  // tokens per epilogue pass
 
+// One family of kept row blocks {start, period, keep, count} of a job.  Plain: a block of up to 128 rows is one box and
+// `per_tile` blocks share a tile; a longer block takes `tpb` tiles of its own.  Rotation pairs and SwiGLU pairs: rows are
+// pairs, a tile holds half as many, and each block has two boxes (first and second half of a head; gate and up).
+struct BFam {
+  int tile_begin, job, mode;
+  int keep, count, start, period, out_base;
+  int box_rows, per_tile, tpb;
+};
+enum { kBPlain = 0, kBRope = 1, kBSwiglu = 2 };
+
 struct BatchCfg {
+  CUtensorMap wmap[kMaxBF];  // packed weights of each family
+  CUtensorMap wmap_up;       // SwiGLU: the up matrix (wmap[] holds the gate matrix)
   CUtensorMap xmap;          // activations: (k, token), box 64 x n
   int n;                     // tokens of an MMA: M rounded up to 16
   int n_ast, acc_stride, a_base;               // tensor memory: A stages, columns between the accumulators, first A column
   int wst, bst, off_w, off_bar;                // ring depths and shared-memory offsets (the activation ring is first)
-  int wtile_begin[kMaxJobs + 1];
+  BFam fam[kMaxBF];
+  int n_fam;
   int n_tiles, n_kb, spt;    // weight tiles of 128 rows, k-blocks, stages per tile
   int kb_first;              // first stored k-block
   int head_kb, head_keep;    // per-head maps: k-blocks and kept channels per head (0: leading block)
   uint32_t idesc;
-  int base, left, sharers;   // whole tiles per block; tiles left over; blocks that share the stages of those
+  int p;                     // blocks per tile (cluster size)
   int* status;
-  int* counters;
-  float* partials;           // one slot [n tokens][128 rows] per (left-over tile, block) piece
+  float* partials;           // two slots [n tokens][128 rows] fp32 per block (p > 1)
 };
 
 __device__ inline void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
@@ -85,9 +102,6 @@ __device__ inline void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
         "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]) : "memory");
 }
 __device__ inline void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ inline void bcp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
 // (through L1: eight consecutive stages use the same 32-byte sector of a row's scales)
 __device__ inline void bcp_async4(uint32_t dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
@@ -96,35 +110,63 @@ __device__ inline void bcp_async_arrive(uint32_t bar) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// A block's work as segments (tile, stages [s0, s1)): its range of the left-over tiles first, then its whole tiles.
+// Row r (a lane of tensor memory) of a tile: what it is, and where its codes lie in a stage.
+struct BRow { RowInfo info; int smem_row; };
+__device__ inline BRow batch_row(const BatchCfg& c, const Params& p, const BFam& f, int tile, int r) {
+  BRow o;
+  o.info.stored = -1; o.info.out_col = -1; o.info.pair_c = 0; o.info.head = 0;
+  const int tl = tile - f.tile_begin, m = r & 1;
+  const bool pairs = f.mode != kBPlain;
+  const int i = pairs ? r >> 1 : r;                   // row or pair within the tile
+  int h, row, b = 0;
+  if (f.per_tile == 0) {                              // a long block: this is one of its tiles
+    h = tl / f.tpb;
+    row = (tl - h * f.tpb) * (pairs ? BMW / 2 : BMW) + i;
+    o.smem_row = pairs ? m * (BMW / 2) + i : i;
+  } else {
+    b = i / f.box_rows;
+    row = i - b * f.box_rows;
+    h = tl * f.per_tile + b;
+    o.smem_row = (pairs ? (2 * b + m) * f.box_rows + row : i) & (BMW - 1);
+    if (b >= f.per_tile) row = f.keep;                // (rows behind the tile's last box)
+  }
+  if (row >= f.keep || h >= f.count) return o;
+  const JobDev& jb = p.job[f.job];
+  if (f.mode == kBRope) {
+    o.info.stored = h * jb.rope.head_dim + m * (jb.rope.head_dim >> 1) + row;
+    o.info.out_col = h * jb.rope.head_keep + m * f.keep + row;
+    o.info.pair_c = row; o.info.head = h;
+  } else {
+    o.info.stored = f.start + h * f.period + row;
+    o.info.out_col = f.out_base + h * f.keep + row;
+    o.info.pair_c = m;
+  }
+  return o;
+}
+__device__ inline const BFam& fam_of_tile(const BatchCfg& c, int t) {
+  int k = 0;
+  while (k + 1 < c.n_fam && t >= c.fam[k + 1].tile_begin) ++k;
+  return c.fam[k];
+}
+
+// A block's work: of every tile of its cluster the stages [s0, s1).  Which rank gets the longer shares rotates from tile
+// to tile.
 struct BSeg { int tile, s0, s1; };
 struct BSegIter {
-  int u, ue, t, t_end, spt, tail0;
-  __device__ inline void init(const BatchCfg& c, int b, int grid) {
-    spt = c.spt;
-    tail0 = c.base * grid;
-    t = b * c.base; t_end = t + c.base;
-    u = ue = 0;
-    if (b < c.sharers) {
-      const unsigned long long U = (unsigned long long)c.left * c.spt;
-      u = (int)(U * b / c.sharers); ue = (int)(U * (b + 1) / c.sharers);
-    }
+  int t, step, n, spt, p, r;
+  __device__ inline void init(const BatchCfg& c, int rank) {
+    p = c.p; spt = c.spt; n = c.n_tiles; r = rank;
+    t = (int)blockIdx.x / p; step = (int)gridDim.x / p;
   }
   __device__ inline bool next(BSeg& g) {
-    if (u < ue) {
-      const int tt = u / spt;
-      g.tile = tail0 + tt; g.s0 = u - tt * spt;
-      const int len = min(spt - g.s0, ue - u);
-      g.s1 = g.s0 + len;
-      u += len;
-      return true;
-    }
-    if (t < t_end) { g.tile = t++; g.s0 = 0; g.s1 = spt; return true; }
-    return false;
+    if (t >= n) return false;
+    g.tile = t;
+    g.s0 = spt * r / p; g.s1 = spt * (r + 1) / p;
+    t += step;
+    if (++r == p) r = 0;
+    return true;
   }
 };
-// the block whose range of the left-over stages holds stage u
-__device__ inline int bowner(int u, int B, int U) { return (int)((((unsigned long long)u + 1) * B - 1) / U); }
 
 template <typename T, bool HEADS>
 __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ Params p, const __grid_constant__ BatchCfg c) {
@@ -137,21 +179,19 @@ __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ 
   const uint32_t bars = sbase + (uint32_t)c.off_bar;
   const uint32_t w_full = bars, w_empty = w_full + 8 * MAX_WST, b_full = w_empty + 8 * MAX_WST, b_empty = b_full + 8 * MAX_BST;
   const uint32_t a_full = b_empty + 8 * MAX_BST, a_empty = a_full + 8 * MAX_AST;
-  const uint32_t acc_full = a_empty + 8 * MAX_AST, acc_empty = acc_full + 16, epi_bar = acc_empty + 16, help_bar = epi_bar + 8;
-  const uint32_t last_full = help_bar + 8;
-  unsigned char* misc = smem + c.off_bar + 8 * (2 * MAX_WST + 2 * MAX_BST + 2 * MAX_AST + 4 + 3);
+  const uint32_t acc_full = a_empty + 8 * MAX_AST, acc_empty = acc_full + 16, last_full = acc_empty + 16, xbar = last_full + 8, xlast = xbar + 64;   // exchange: two per quadrant; last tile
+  unsigned char* misc = smem + c.off_bar + 8 * (2 * MAX_WST + 2 * MAX_BST + 2 * MAX_AST + 4 + 1 + 12);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
-  volatile int* last_flag = reinterpret_cast<volatile int*>(misc + 8);
 
   if (tid == 0) {
-    for (int s = 0; s < MAX_WST; ++s) { pmbar_init(w_full + 8 * s, LOADERS * 32); pmbar_init(w_empty + 8 * s, DQN); }
+    for (int s = 0; s < MAX_WST; ++s) { pmbar_init(w_full + 8 * s, LOADERS * 32 + 1); pmbar_init(w_empty + 8 * s, DQN); }
     for (int s = 0; s < MAX_BST; ++s) { pmbar_init(b_full + 8 * s, 1); pmbar_init(b_empty + 8 * s, 1); }
     for (int s = 0; s < MAX_AST; ++s) { pmbar_init(a_full + 8 * s, DQN); pmbar_init(a_empty + 8 * s, 1); }
     for (int s = 0; s < 2; ++s) { pmbar_init(acc_full + 8 * s, 1); pmbar_init(acc_empty + 8 * s, 4); }
-    pmbar_init(epi_bar, 4);
-    pmbar_init(help_bar, 4 + DQN);
     pmbar_init(last_full, 1);
+    for (int q = 0; q < 8; ++q) pmbar_init(xbar + 8 * q, max(1, c.p - 1));
+    for (int q = 0; q < 4; ++q) pmbar_init(xlast + 8 * q, max(1, 5 * (c.p - 1)));
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -163,89 +203,81 @@ __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int grid = (int)gridDim.x;
+  const int rank = c.p > 1 ? (int)pcluster_rank() : 0;
+  if (c.p > 1) {                        // the peers' barriers exist before anything arrives at them
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
   bool failed = false;
-  auto job_of_tile = [&](int t) { int j = 0; while (j + 1 < p.n_jobs && t >= c.wtile_begin[j + 1]) ++j; return j; };
 
-  // ---- epilogue of one segment for the warp that calls it: token chunks ch0, ch0 + chs, ... (chs == 1: the epilogue warp
-  //      on its own, which also hands the accumulator back)
-  uint32_t epar = 0;
-  auto group_sync = [&](uint32_t bar) -> bool {
-    __syncwarp();
-    if (lane == 0) pmbar_arrive(bar);
-    const bool ok = pmbar_wait_warp(bar, epar, abort_flag);
-    epar ^= 1;
-    return ok;
+  // ---- epilogue of one tile for the warp that calls it: token chunks ch0, ch0 + chs, ... (chs == 1: the epilogue warp on
+  //      its own, which also hands the accumulator back; chs == 5: the last tile, shared with the de-quantiser warps)
+  auto row_store = [&](int tile) {                 // (made before the wait for the accumulator: several dependent loads)
+    const BFam& f = fam_of_tile(c, tile);
+    const int r = 32 * (warp & 3) + lane;
+    return RowStore<T>(p, f.job, batch_row(c, p, f, tile, r).info, (r & 1) != 0);
   };
-  auto epilogue_segment = [&](const BSeg& sg, int count, int ch0, int chs) {
+  auto epilogue_tile = [&](const RowStore<T>& rs, int count, int ch0, int chs) {
     const int q = warp & 3, acc = count & 1;
-    const int jn = job_of_tile(sg.tile);
-    const RowStore<T> rs(p, jn, sg.tile - c.wtile_begin[jn], 32 * q + lane);
     const uint32_t t_acc = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * c.acc_stride);
-    const uint32_t bar = chs == 1 ? epi_bar : help_bar;
+    const int n_ch = c.n / kTokChunk;
     tc_fence_after();
-    auto release = [&]() {                                     // (chs == 1) the accumulator's values are in registers
+    const size_t slot_f = (size_t)c.n * BMW;
+    float* slots = c.partials + (size_t)(count & 1) * slot_f + 32 * q + lane;      // + block * 2 slots + token * BMW
+    const int block0 = (int)blockIdx.x - rank;
+    if (c.p > 1) {
+      // the sums of the chunks that other blocks finish
+      float* mine = slots + (size_t)blockIdx.x * 2 * slot_f;
+      for (int ch = ch0; ch < n_ch; ch += chs) {
+        if (ch % c.p == rank) continue;
+        uint32_t v[16];
+        tmem_ld16(t_acc + (uint32_t)(ch * kTokChunk), v);
+        tmem_ld_wait();
+#pragma unroll
+        for (int k = 0; k < 16; ++k) __stcg(mine + (size_t)(ch * kTokChunk + k) * BMW, __uint_as_float(v[k]));
+      }
+      __syncwarp();
+      // (barriers alternate from tile to tile: a peer may be a tile ahead before another peer's arrival has come in)
+      const uint32_t xb = chs == 1 ? xbar + 32 * (count & 1) + 8 * q : xlast + 8 * q;
+      if (lane < c.p && lane != rank) {
+        asm volatile("fence.acq_rel.cluster;" ::: "memory");
+        pmbar_arrive_peer(ppeer_addr(xb, (uint32_t)lane));
+      }
+      const bool ok = __all_sync(0xffffffffu, pmbar_wait_cluster(xb, chs == 1 ? (count >> 1) & 1 : 0, abort_flag));
+      if (!ok) { failed = true; return; }
+    }
+    for (int ch = ch0; ch < n_ch; ch += chs) {
+      if (c.p > 1 && ch % c.p != rank) continue;
+      uint32_t v[16];
+      tmem_ld16(t_acc + (uint32_t)(ch * kTokChunk), v);
+      float val[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) val[k] = 0.f;
+      for (int r = 0; r < c.p; ++r) {
+        if (r == rank) {
+          tmem_ld_wait();
+#pragma unroll
+          for (int k = 0; k < 16; ++k) val[k] += __uint_as_float(v[k]);
+        } else {
+          const float* src = slots + (size_t)(block0 + r) * 2 * slot_f + (size_t)(ch * kTokChunk) * BMW;
+          float a[16];
+#pragma unroll
+          for (int k = 0; k < 16; ++k) a[k] = __ldcg(src + (size_t)k * BMW);
+#pragma unroll
+          for (int k = 0; k < 16; ++k) val[k] += a[k];
+        }
+      }
+      rs.store(p, ch * kTokChunk, val);
+    }
+    if (chs == 1) {                                            // the accumulator is free for the tile after the next
       tc_fence_before();
       __syncwarp();
       if (lane == 0) pmbar_arrive(acc_empty + 8 * acc);
-    };
-    const bool whole = sg.s0 == 0 && sg.s1 == c.spt;
-    const int tail0 = c.base * grid, lt = sg.tile - tail0;
-    const size_t slot_f = (size_t)c.n * BMW;
-    float* mine = whole ? nullptr : c.partials + ((size_t)lt + blockIdx.x) * slot_f + 32 * q + lane;
-    for (int tk = kTokChunk * ch0; tk < c.n; tk += kTokChunk * chs) {
-      uint32_t v[16];
-      tmem_ld16(t_acc + (uint32_t)tk, v);
-      tmem_ld_wait();
-      if (chs == 1 && tk + kTokChunk >= c.n) release();
-      if (whole) {
-        float val[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) val[k] = __uint_as_float(v[k]);
-        rs.store(p, tk, val);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 16; ++k) __stcg(mine + (size_t)(tk + k) * BMW, __uint_as_float(v[k]));
-      }
-    }
-    if (whole) return;
-    __threadfence();                                           // this thread's part is in place before ...
-    if (!group_sync(bar)) { failed = true; return; }
-    const int U = c.left * c.spt;
-    const int first = bowner(lt * c.spt, c.sharers, U), last = bowner(lt * c.spt + c.spt - 1, c.sharers, U);
-    const bool main_lane = warp == EPI0 && lane == 0;
-    if (main_lane) {
-      *last_flag = atomicAdd(&c.counters[sg.tile], 1) == last - first;      // ... the block's arrival shows
-      __threadfence();
-    }
-    if (!group_sync(bar)) { failed = true; return; }
-    if (*last_flag) {
-      const float* src0 = c.partials + ((size_t)lt + first) * slot_f + 32 * q + lane;
-      const int parts = last - first + 1;
-      for (int tk = kTokChunk * ch0; tk < c.n; tk += kTokChunk * chs) {
-        const float* src = src0 + (size_t)tk * BMW;
-        float val[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) val[k] = __ldcg(src + (size_t)k * BMW);
-        for (int s = 1; s < parts; s += 2) {                   // the loads of two slots in flight
-          const bool two = s + 1 < parts;
-          const float* sp = src + (size_t)s * slot_f;
-          float a[16], b[16];
-#pragma unroll
-          for (int k = 0; k < 16; ++k) a[k] = __ldcg(sp + (size_t)k * BMW);
-#pragma unroll
-          for (int k = 0; k < 16; ++k) b[k] = two ? __ldcg(sp + slot_f + (size_t)k * BMW) : 0.f;
-#pragma unroll
-          for (int k = 0; k < 16; ++k) val[k] = (val[k] + a[k]) + b[k];
-        }
-        rs.store(p, tk, val);
-      }
-      if (main_lane) c.counters[sg.tile] = 0;                  // ready for the next call
     }
   };
 
   BSegIter si;
-  si.init(c, (int)blockIdx.x, grid);
+  si.init(c, rank);
   BSeg sg;
   if (warp == 0) {
     // ===================================================================== activations
@@ -287,11 +319,15 @@ __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ 
         const uint32_t a0 = tmem + (uint32_t)(c.a_base + 128 * as);
         const uint32_t b0 = sbase + (uint32_t)(bs * KS * c.n) * 128u;
         if (elect_one()) {
-          for (int i = 0; i < nv; ++i) {
-            const uint64_t bd = smem_desc_sw128(b0 + (uint32_t)(i * c.n) * 128u);
+          uint64_t bd = smem_desc_sw128(b0);
+          const uint64_t step = (uint64_t)(c.n * 8);           // a box of n * 128 bytes, in the descriptor's 16-byte units
+#pragma unroll
+          for (int i = 0; i < KS; ++i) {
+            if (i >= nv) break;
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k)
               umma_ts(d, a0 + 32 * i + 8 * k, bd + 2 * k, c.idesc, (st > sg.s0 || i > 0 || k > 0) ? 1u : 0u);
+            bd += step;
           }
           umma_commit(a_empty + 8 * as);
           umma_commit(b_empty + 8 * bs);
@@ -311,101 +347,134 @@ __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ 
       __syncwarp();
     }
   } else if (warp < EPI0) {
-    // ===================================================================== loaders: 64 rows each
-    // A piece is 16 bytes: eight lanes fetch the 128 bytes of a row (four rows, four cache lines per instruction).
+    // ===================================================================== loaders
+    // Codes by TMA, issued by warp 2 (a box per lane).  (The first version copied them with cp.async, sixteen 16-byte
+    // pieces per lane and stage: 1100 cycles of issue per stage and loader warp, which set the pace.)  Scales and
+    // zero-points are two fp16 per row and stage at any row pitch: cp.async of 4 bytes, 64 rows per warp.
     const int r0 = (warp - LD_WARP0) * 64;
     const int G = p.K / kGroup;
     int s = 0, it = 0; uint32_t par = 1;
     while (!failed && si.next(sg)) {
-      const int jn = job_of_tile(sg.tile);
-      const JobDev& jb = p.job[jn];
-      const int tl = sg.tile - c.wtile_begin[jn];
-      const bool pair = jb.pair == 1;
-      // stored rows r0 + lane and r0 + 32 + lane (-1: empty, its sums are never stored)
-      const int row0 = tile_row(jb, tl, r0 + lane).stored, row1 = tile_row(jb, tl, r0 + 32 + lane).stored;
-      // odd rows of a SwiGLU pair come from the up matrix
-      const JobDev& jw = (pair && ((lane >> 3) & 1)) ? p.job[jn + 1] : jb;      // of the rows this lane fetches codes for
-      const JobDev& js = (pair && (lane & 1)) ? p.job[jn + 1] : jb;             // of the rows it fetches scales for
-      const uint8_t* wbase = jw.w + (size_t)c.kb_first * 32 + (lane & 7) * 16;
-      const __half* sb = js.scales + c.kb_first / 2;
-      const __half* zb = js.zeros + c.kb_first / 2;
-      const size_t kbytes = (size_t)p.K / 2;
+      const BFam& f = fam_of_tile(c, sg.tile);
+      const JobDev& js = p.job[f.job + ((f.mode == kBSwiglu && (lane & 1)) ? 1 : 0)];   // odd rows of a SwiGLU pair: the up matrix
+      const int row0 = batch_row(c, p, f, sg.tile, r0 + lane).info.stored, row1 = batch_row(c, p, f, sg.tile, r0 + 32 + lane).info.stored;
+      const __half* s0 = js.scales + c.kb_first / 2 + (size_t)max(row0, 0) * G;
+      const __half* z0 = js.zeros + c.kb_first / 2 + (size_t)max(row0, 0) * G;
+      const __half* s1 = js.scales + c.kb_first / 2 + (size_t)max(row1, 0) * G;
+      const __half* z1 = js.zeros + c.kb_first / 2 + (size_t)max(row1, 0) * G;
+      // this lane's box (warp 2): blocks beyond the family's last are left out
+      const int tl = sg.tile - f.tile_begin;
+      const CUtensorMap* tm = &c.wmap[&f - c.fam];
+      int boxes, by = 0, bz = 0;
+      if (f.per_tile == 0) {
+        const int h = tl / f.tpb;
+        by = (tl - h * f.tpb) * (f.mode == kBPlain ? BMW : BMW / 2);
+        boxes = f.mode == kBPlain ? 1 : 2;
+        bz = f.mode == kBRope ? 2 * h + lane : h;
+        if (f.mode == kBSwiglu && lane == 1) tm = &c.wmap_up;
+      } else {
+        const int h0 = tl * f.per_tile, nb = min(f.per_tile, f.count - h0);
+        boxes = f.mode == kBRope ? 2 * nb : nb;
+        bz = (f.mode == kBRope ? 2 * h0 : h0) + lane;
+      }
       for (int st = sg.s0; st < sg.s1; ++st, ++it) {
         if (it >= c.wst && !pmbar_wait_warp(w_empty + 8 * s, par, abort_flag)) { failed = true; break; }
-        const int nv = min(KS, c.n_kb - st * KS);
         const uint32_t dst = sbase + (uint32_t)(c.off_w + s * WSTAGE);
-        const bool piece = ((lane & 7) >> 1) < nv;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int rl = i * 4 + (lane >> 3);                                   // row within the 64
-          const int row = __shfl_sync(0xffffffffu, i < 8 ? row0 : row1, rl & 31);
-          if (row >= 0 && piece)
-            bcp_async16(dst + (uint32_t)((r0 + rl) * 128 + (((lane & 7) ^ (rl & 7)) * 16)), wbase + (size_t)row * kbytes + (size_t)st * (KS * 32));
+        if (warp == LD_WARP0) {
+          if (lane == 0) pmbar_expect_tx(w_full + 8 * s, (uint32_t)(boxes * f.box_rows) * 128u);
+          __syncwarp();
+          if (lane < boxes) tma_box_3d(dst + (uint32_t)(lane * f.box_rows) * 128u, tm, c.kb_first * 32 + st * 128, by, bz, w_full + 8 * s);
         }
         const uint32_t sd = dst + WST_BYTES + (uint32_t)((r0 + lane) * 4);
         if (row0 >= 0) {
-          bcp_async4(sd, sb + (size_t)row0 * G + st * 2);
-          bcp_async4(sd + BMW * 4, zb + (size_t)row0 * G + st * 2);
+          bcp_async4(sd, s0 + st * 2);
+          bcp_async4(sd + BMW * 4, z0 + st * 2);
         }
         if (row1 >= 0) {
-          bcp_async4(sd + 128, sb + (size_t)row1 * G + st * 2);
-          bcp_async4(sd + BMW * 4 + 128, zb + (size_t)row1 * G + st * 2);
+          bcp_async4(sd + 128, s1 + st * 2);
+          bcp_async4(sd + BMW * 4 + 128, z1 + st * 2);
         }
         bcp_async_arrive(w_full + 8 * s);
         if (++s == c.wst) { s = 0; par ^= 1; }
       }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
+    if (failed) {                           // let the copies still armed land before the block goes away
+      for (int j = it > c.wst ? it - c.wst : 0; j < it; ++j)
+        for (int i = 0; i < kPWait && !pmbar_try(w_full + 8 * (j % c.wst), (j / c.wst) & 1); ++i) {}
+    }
   } else if (warp >= DQ0) {
     // ===================================================================== de-quantisers
+    // Software-pipelined: the codes of the next stage are in registers before the current one is converted, and the
+    // tcgen05.st of a stage completes while the first half of the next is converted.
     const int q = warp & 3, kq = (warp - DQ0) >> 2;
     const int r = 32 * q + lane;
-    const uint32_t w_off = (uint32_t)(r * 128), x0 = (uint32_t)(((2 * kq) ^ (r & 7)) * 16), x1 = (uint32_t)(((2 * kq + 1) ^ (r & 7)) * 16);
     const uint32_t s_off = (uint32_t)(WST_BYTES + r * 4 + (kq >> 1) * 2);
     const uint32_t a_lane = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(c.a_base + 32 * kq);
     int ws = 0, as = 0, it = 0; uint32_t wpar = 0, apar = 1;
     int n_seg = 0;
     BSeg last_sg = {0, 0, 0};
+    int stored_as = -1;                          // A stage whose tcgen05.st is still to be announced
+    auto announce = [&]() {
+      if (stored_as < 0) return;
+      tmem_st_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) pmbar_arrive(a_full + 8 * stored_as);
+      stored_as = -1;
+    };
     while (!failed && si.next(sg)) {
       last_sg = sg;
       ++n_seg;
-      for (int st = sg.s0; st < sg.s1; ++st, ++it) {
-        if (!pmbar_wait_warp(w_full + 8 * ws, wpar, abort_flag)) { failed = true; break; }
+      const int sr = batch_row(c, p, fam_of_tile(c, sg.tile), sg.tile, r).smem_row;
+      const uint32_t x0 = (uint32_t)(sr * 128 + ((2 * kq) ^ (sr & 7)) * 16), x1 = (uint32_t)(sr * 128 + ((2 * kq + 1) ^ (sr & 7)) * 16);
+      uint32_t w[8];
+      __half sc, zp;
+      auto fetch = [&]() -> bool {               // codes, scale and zero-point of the next stage of the ring; the slot is free again
+        if (!pmbar_wait_warp(w_full + 8 * ws, wpar, abort_flag)) return false;
         const uint32_t src = sbase + (uint32_t)(c.off_w + ws * WSTAGE);
-        uint32_t w[8];
-        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(src + w_off + x0));
-        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]) : "r"(src + w_off + x1));
+        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(src + x0) : "memory");
+        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]) : "r"(src + x1) : "memory");
         unsigned short sh, zh;
-        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(sh) : "r"(src + s_off));
-        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(zh) : "r"(src + s_off + BMW * 4));
-        const __half sc = __ushort_as_half(sh);
+        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(sh) : "r"(src + s_off) : "memory");
+        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(zh) : "r"(src + s_off + BMW * 4) : "memory");
+        sc = __ushort_as_half(sh); zp = __ushort_as_half(zh);
+        __syncwarp();
+        if (lane == 0) pmbar_arrive(w_empty + 8 * ws);
+        if (++ws == c.wst) { ws = 0; wpar ^= 1; }
+        return true;
+      };
+      if (!fetch()) { failed = true; break; }
+      for (int st = sg.s0; st < sg.s1; ++st, ++it) {
         const __half2 s2 = __half2half2(sc);
-        const __half2 cz2 = __float2half2_rn((8.f - __half2float(__ushort_as_half(zh))) * __half2float(sc));
+        const __half2 cz2 = __float2half2_rn((8.f - __half2float(zp)) * __half2float(sc));
         uint32_t o[32];
         int valid = BK;
         if (HEADS) valid = min(BK, c.head_keep - ((st * KS + kq) % c.head_kb) * BK);
+        auto convert = [&](int j0) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const uint4 d = (!HEADS || j * 8 < valid) ? dequant_word(w[j], s2, cz2) : make_uint4(0, 0, 0, 0);
-          o[4 * j] = d.x; o[4 * j + 1] = d.y; o[4 * j + 2] = d.z; o[4 * j + 3] = d.w;
-        }
-        __syncwarp();
-        if (lane == 0) pmbar_arrive(w_empty + 8 * ws);
+          for (int j = j0; j < j0 + 4; ++j) {
+            const uint4 d = (!HEADS || j * 8 < valid) ? dequant_word(w[j], s2, cz2) : make_uint4(0, 0, 0, 0);
+            o[4 * j] = d.x; o[4 * j + 1] = d.y; o[4 * j + 2] = d.z; o[4 * j + 3] = d.w;
+          }
+        };
+        convert(0);
+        announce();
+        convert(4);
+        if (st + 1 < sg.s1 && !fetch()) { failed = true; break; }
         if (it >= c.n_ast && !pmbar_wait_warp(a_empty + 8 * as, apar, abort_flag)) { failed = true; break; }
         tc_fence_after();
         tmem_st32(a_lane + (uint32_t)(128 * as), o);
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) pmbar_arrive(a_full + 8 * as);
-        if (++ws == c.wst) { ws = 0; wpar ^= 1; }
+        stored_as = as;
         if (++as == c.n_ast) { as = 0; apar ^= 1; }
       }
+      if (!failed) announce();
     }
     if (!failed && n_seg > 0) {
       asm volatile("griddepcontrol.wait;" ::: "memory");
+      const RowStore<T> rs = row_store(last_sg.tile);
       if (!pmbar_wait_warp(last_full, 0, abort_flag)) failed = true;
-      if (!failed) epilogue_segment(last_sg, n_seg - 1, 1 + kq, 5);
+      if (!failed) epilogue_tile(rs, n_seg - 1, 1 + kq, 5);
     }
   } else {
     // ===================================================================== epilogue
@@ -415,10 +484,9 @@ __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ 
       BSegIter peek = si;
       BSeg nxt;
       const bool last = !peek.next(nxt);
+      const RowStore<T> rs = row_store(sg.tile);
       if (!pmbar_wait_warp(acc_full + 8 * (count & 1), (count >> 1) & 1, abort_flag)) { failed = true; break; }
-      // (the phase of help_bar starts at zero with the last segment; epi_bar's own is not used after it)
-      if (last) epar = 0;
-      epilogue_segment(sg, count, 0, last ? 5 : 1);
+      epilogue_tile(rs, count, 0, last ? 5 : 1);
     }
   }
   if (failed && lane == 0) atomicExch(c.status, UNIQL_ERR_TIMEOUT);
@@ -426,42 +494,108 @@ __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   if (warp == 1) tmem_dealloc(tmem, 512);
+  if (c.p > 1) {                        // no block leaves while a peer may still arrive at its barriers
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
 }
 
 // -------------------------------------------------------------------------------- host side
-int batch_tiles(const JobDev& j) {
-  if (j.pair == 2) return 0;                                       // its rows ride in the tiles of the job before
-  if (j.pair == 1) return (j.k_out + BMW / 2 - 1) / (BMW / 2);
-  if (j.rope.enabled) return (j.rope.n_heads * (j.rope.head_keep / 2) + BMW / 2 - 1) / (BMW / 2);
-  return (j.k_out + BMW - 1) / BMW;
-}
-
-template <typename T, bool HEADS>
-int launch_b(const Params& p, const BatchCfg& c, int grid, size_t smem, cudaStream_t stream) {
-  auto kern = batch_kernel<T, HEADS>;
-  {
-    static std::mutex mu;                    // (the shared-memory limit is raised once per device)
-    static bool done[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return UNIQL_ERR_CUDA;
-    std::lock_guard<std::mutex> lock(mu);
-    if (dev < 0 || dev >= 64 || !done[dev]) {
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBatch) != cudaSuccess) return UNIQL_ERR_CUDA;
-      if (dev >= 0 && dev < 64) done[dev] = true;
+// Row families of the launch, or 0 when there are more than it holds.
+int batch_families(const Params& p, BatchCfg* c) {
+  int n = 0, tiles = 0;
+  for (int j = 0; j < p.n_jobs; ++j) {
+    const JobDev& jb = p.job[j];
+    if (jb.pair == 2) continue;                                      // its rows ride in the tiles of the job before
+    const int nf = jb.rope.enabled ? 1 : jb.omap.n_fam;
+    for (int k = 0; k < nf; ++k) {
+      if (n == kMaxBF) return 0;
+      BFam f;
+      memset(&f, 0, sizeof(f));
+      f.tile_begin = tiles; f.job = j;
+      int rows;                                                      // rows (pairs) that a tile has room for
+      if (jb.rope.enabled) {
+        f.mode = kBRope; rows = BMW / 2;
+        f.keep = jb.rope.head_keep / 2; f.count = jb.rope.n_heads; f.start = 0; f.period = jb.rope.head_dim;
+      } else {
+        const Fam& a = jb.omap.fam[k];
+        f.mode = jb.pair == 1 ? kBSwiglu : kBPlain; rows = jb.pair == 1 ? BMW / 2 : BMW;
+        if (jb.pair == 1 && (nf != 1 || a.count != 1)) return 0;
+        f.keep = a.keep; f.count = a.count; f.start = a.start; f.period = a.count > 1 ? a.period : a.keep; f.out_base = jb.omap.base[k];
+      }
+      if (f.keep > rows || f.count == 1) {
+        f.box_rows = rows; f.per_tile = 0; f.tpb = (f.keep + rows - 1) / rows;
+        tiles += f.tpb * f.count;
+      } else {
+        f.box_rows = (f.keep + 7) / 8 * 8;                           // (the swizzle pattern repeats every 8 rows)
+        f.per_tile = rows / f.box_rows; f.tpb = 1;
+        if (f.per_tile < 1) f.per_tile = 1;
+        tiles += (f.count + f.per_tile - 1) / f.per_tile;
+      }
+      if (c) c->fam[n] = f;
+      ++n;
     }
   }
+  if (c) { c->n_fam = n; c->n_tiles = tiles; }
+  return n;
+}
+
+typedef void (*BatchKernel)(Params, BatchCfg);
+BatchKernel batch_instance(bool bf16, bool heads) {
+  if (bf16) return heads ? batch_kernel<__nv_bfloat16, true> : batch_kernel<__nv_bfloat16, false>;
+  return heads ? batch_kernel<__half, true> : batch_kernel<__half, false>;
+}
+
+struct BLaunch {
   cudaLaunchConfig_t lc;
-  memset(&lc, 0, sizeof(lc));
-  lc.gridDim = dim3(grid);
-  lc.blockDim = dim3(NTHB);
-  lc.dynamicSmemBytes = smem;
-  lc.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = attr;
-  lc.numAttrs = opt(kOptPdl) ? 1 : 0;
-  if (cudaLaunchKernelEx(&lc, kern, p, c) != cudaSuccess) { cudaGetLastError(); return UNIQL_ERR_CUDA; }
+  cudaLaunchAttribute attr[2];
+  BLaunch(int grid, int p, size_t smem, cudaStream_t stream) {
+    memset(this, 0, sizeof(*this));
+    lc.gridDim = dim3(grid);
+    lc.blockDim = dim3(NTHB);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = stream;
+    lc.attrs = attr;
+    if (p > 1) {
+      attr[lc.numAttrs].id = cudaLaunchAttributeClusterDimension;
+      attr[lc.numAttrs].val.clusterDim.x = p;
+      attr[lc.numAttrs].val.clusterDim.y = attr[lc.numAttrs].val.clusterDim.z = 1;
+      ++lc.numAttrs;
+    }
+    if (opt(kOptPdl)) {
+      attr[lc.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[lc.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+      ++lc.numAttrs;
+    }
+  }
+};
+
+constexpr int kMaxP = 8;
+// Clusters of p blocks that the device holds at once (one block per SM), asked once per device: resident[p].
+struct Residency { bool known = false; int clusters[kMaxP + 1]; };
+int residency(Residency* out) {
+  static std::mutex mu;
+  static Residency dev_res[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return UNIQL_ERR_CUDA;
+  std::lock_guard<std::mutex> lock(mu);
+  Residency& r = dev_res[dev];
+  if (!r.known) {
+    for (int k = 0; k < 4; ++k)
+      if (cudaFuncSetAttribute(batch_instance(k & 1, k & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBatch) != cudaSuccess)
+        return UNIQL_ERR_CUDA;
+    const int sms = device_sms();
+    r.clusters[0] = 0;
+    r.clusters[1] = sms;
+    for (int p = 2; p <= kMaxP; ++p) {
+      BLaunch l(sms / p * p, p, kSmemBatch, nullptr);
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, batch_instance(false, false), &l.lc) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      r.clusters[p] = n < sms / p ? n : sms / p;
+    }
+    r.known = true;
+  }
+  *out = r;
   return UNIQL_OK;
 }
 
@@ -480,15 +614,13 @@ int batch_supported(const Params& p) {
   if ((p.ldx % 8) != 0 || (((uintptr_t)p.x) & 15) != 0) return 0;
   for (int j = 0; j < p.n_jobs; ++j)
     if ((((uintptr_t)p.job[j].scales) | ((uintptr_t)p.job[j].zeros)) & 3) return 0;
-  return 1;
+  return batch_families(p, nullptr) > 0;
 }
 
 int launch_batch(const Params& p, const LaunchCfg& cfg) {
   BatchCfg c;
   memset(&c, 0, sizeof(c));
-  for (int j = 0; j < p.n_jobs; ++j) { c.wtile_begin[j] = c.n_tiles; c.n_tiles += batch_tiles(p.job[j]); }
-  for (int j = p.n_jobs; j <= kMaxJobs; ++j) c.wtile_begin[j] = c.n_tiles;
-  if (c.n_tiles < 1) return UNIQL_ERR_SHAPE;
+  if (batch_families(p, &c) < 1 || c.n_tiles < 1) return UNIQL_ERR_SHAPE;
   c.n = (p.M + 15) / 16 * 16;
   const Fam& a = p.imap.fam[0];
   const int kbh = (a.keep + BK - 1) / BK;
@@ -510,7 +642,6 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   c.off_bar = c.off_w + c.wst * WSTAGE;
   const size_t smem = 1024 + (size_t)c.off_bar + 512;
   c.status = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(cfg.workspace) + decode_status_offset());
-  c.counters = reinterpret_cast<int*>(cfg.workspace);
   size_t used = (decode_workspace_header_bytes() + 255) & ~(size_t)255;
   const void* x = p.x;
   int ldx = p.ldx;
@@ -519,37 +650,49 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
     x = reinterpret_cast<unsigned char*>(cfg.workspace) + used;
     used = (used + (size_t)p.M * ldx * 2 + 255) & ~(size_t)255;
   }
-  const int sms = device_sms();
-  int g = sms;
+  // The split: p blocks per tile where that shortens the longest block's work.  In stages of about half a microsecond: the
+  // rounds of the clusters that fit, a p-th of a tile's stages each, and about four stages for the exchange at the end.
+  Residency res;
+  int rc = residency(&res);
+  if (rc != UNIQL_OK) return rc;
   const int env_grid = opt(kOptPrefillGrid), env_split = opt(kOptPrefillStreamk);
-  if (env_grid >= 1 && env_grid <= sms) g = env_grid;
-  // The split: a stage takes about half a microsecond, a hand-over at a block's end (no whole tiles behind it) about
-  // seven stages more, in front of whole tiles about one.
-  c.base = c.n_tiles / g;
-  c.left = c.n_tiles - c.base * g;
-  c.sharers = 0;
-  int grid = g;
-  if (c.left > 0) {
-    const long U = (long)c.left * c.spt;
-    const long B = U < g ? U : g;
-    const double split = (double)U / B + (c.base == 0 ? 7.0 : 1.0);
-    const size_t slots = (size_t)(c.left + g) * c.n * BMW * 4;
-    const bool want = env_split >= 0 ? env_split >= 1 : split < c.spt;
-    if (want && c.n_tiles <= (1 << 16) && cfg.ws_bytes >= used + slots) c.sharers = (int)B;
-    else c.sharers = c.left;                    // one left-over tile each, whole
-    c.partials = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(cfg.workspace) + used);
-    if (c.base == 0) grid = c.sharers;
+  int best = 1, best_clusters = 1;
+  double best_cost = 1e30;
+  for (int k = 1; k <= kMaxP; ++k) {
+    int fit = res.clusters[k];
+    if (env_grid >= 1 && env_grid / k < fit) fit = env_grid / k;              // tests: several tiles per block on small problems
+    if (fit < 1 || k > c.spt) continue;
+    if (k > 1 && (env_split == 0 || cfg.ws_bytes < used + (size_t)fit * k * 2 * c.n * BMW * 4)) continue;
+    const int rounds = (c.n_tiles + fit - 1) / fit;
+    double cost = (double)rounds * c.spt / k + (k > 1 ? 4.0 : 0.0) + 0.3 * rounds;
+    if (env_split >= 1 && k > 1) cost *= 1e-3;                               // tests: split wherever it is possible
+    if (cost < best_cost) { best_cost = cost; best = k; best_clusters = c.n_tiles < fit ? c.n_tiles : fit; }
   }
+  c.p = best;
+  c.partials = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(cfg.workspace) + used);
   if (p.dt == UNIQL_BF16) {
-    const int rc = launch_x_to_f16(p.x, p.ldx, p.M, p.k_in, const_cast<void*>(x), ldx, cfg.stream);
+    rc = launch_x_to_f16(p.x, p.ldx, p.M, p.k_in, const_cast<void*>(x), ldx, cfg.stream);
     if (rc != UNIQL_OK) return rc;
   }
-  const int rc = encode_x_map(&c.xmap, x, p.k_in, p.M, ldx, c.n, false);
+  const int x_extent = (c.kb_first + c.n_kb) * (BK / 2);     // bytes of a row up to the last visited k-block
+  for (int k = 0; k < c.n_fam; ++k) {
+    const BFam& f = c.fam[k];
+    const JobDev& jb = p.job[f.job];
+    const bool rope = f.mode == kBRope;
+    rc = encode_w_map(&c.wmap[k], jb.w + (size_t)f.start * (p.K / 2), p.K, x_extent, f.keep, rope ? 2 * f.count : f.count,
+                      rope ? f.period / 2 : f.period, f.box_rows);
+    if (rc == UNIQL_OK && f.mode == kBSwiglu)
+      rc = encode_w_map(&c.wmap_up, p.job[f.job + 1].w + (size_t)f.start * (p.K / 2), p.K, x_extent, f.keep, 1, f.keep, f.box_rows);
+    if (rc != UNIQL_OK) return rc;
+  }
+  rc = encode_x_map(&c.xmap, x, p.k_in, p.M, ldx, c.n, false);
   if (rc != UNIQL_OK) return rc;
-  const bool heads = c.head_kb != 0;
-  if (p.dt == UNIQL_BF16)
-    return heads ? launch_b<__nv_bfloat16, true>(p, c, grid, smem, cfg.stream) : launch_b<__nv_bfloat16, false>(p, c, grid, smem, cfg.stream);
-  return heads ? launch_b<__half, true>(p, c, grid, smem, cfg.stream) : launch_b<__half, false>(p, c, grid, smem, cfg.stream);
+  BLaunch l(best_clusters * c.p, c.p, smem, cfg.stream);
+  if (cudaLaunchKernelEx(&l.lc, batch_instance(p.dt == UNIQL_BF16, c.head_kb != 0), p, c) != cudaSuccess) {
+    cudaGetLastError();
+    return UNIQL_ERR_CUDA;
+  }
+  return UNIQL_OK;
 }
 
 }  // namespace uniql

@@ -194,6 +194,8 @@ int batch_supported(const Params& p);
 int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo, cudaStream_t stream);
 // tensor map over activations [M][k_in] for boxes of 64 channels x `rows` tokens, 128-byte swizzle
 int encode_x_map(void* map, const void* x, int k_in, int M, int ldx, int rows, bool bf16);
+// tensor map over a family of kept row blocks of packed weights: (byte in row, row in block, block), 128-byte columns
+int encode_w_map(void* map, const uint8_t* base, int K, int x_extent, int keep, int count, int row_stride_rows, int box_rows);
 int device_sms();             // SMs of the current device
 int launch_prefill(const Params& p, const LaunchCfg& cfg);
 int prefill_supported(const Params& p);

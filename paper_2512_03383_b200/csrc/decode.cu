@@ -1451,20 +1451,23 @@ EncodeTiledFn encoder() {
   return fn;
 }
 
+}  // namespace
+
 // Packed rows of one family as a 3-D byte tensor (byte in row, row in block, block), 128-byte swizzled boxes.
-int encode_family(CUtensorMap* tm, const uint8_t* base, int K, int x_extent, int keep, int count, int row_stride_rows,
-                  int box_rows) {
+int encode_w_map(void* tm, const uint8_t* base, int K, int x_extent, int keep, int count, int row_stride_rows, int box_rows) {
   EncodeTiledFn enc = encoder();
   if (!enc) return UNIQL_ERR_CUDA;
   const cuuint64_t dims[3] = {(cuuint64_t)x_extent, (cuuint64_t)keep, (cuuint64_t)count};
   const cuuint64_t strides[2] = {(cuuint64_t)(K / 2), (cuuint64_t)row_stride_rows * (cuuint64_t)(K / 2)};
   const cuuint32_t box[3] = {128, (cuuint32_t)box_rows, 1};
   const cuuint32_t es[3] = {1, 1, 1};
-  const CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t*>(base), dims, strides, box, es,
+  const CUresult r = enc(reinterpret_cast<CUtensorMap*>(tm), CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t*>(base), dims, strides, box, es,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? UNIQL_OK : UNIQL_ERR_CUDA;
 }
+
+namespace {
 
 // Shared-memory plan for a given split; returns the total size in bytes (with the alignment slack).
 size_t plan_smem(DecodeCfg* c, int M, int MT, int gp, int stages, int part_bufs, bool i8) {
@@ -1850,7 +1853,7 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
       TileFam& f = c.tf[n_tf];
       f.tile_begin = tiles; f.tpb = (half + RB / 2 - 1) / (RB / 2); f.keep = half; f.count = jb.rope.n_heads;
       f.job = j; f.start = 0; f.period = jb.rope.head_dim; f.out_base = 0; f.mode = kRope; f.job2 = j;
-      const int rc = encode_family(&c.wmap[n_tf], jb.w, p.K, x_extent, half, 2 * jb.rope.n_heads,
+      const int rc = encode_w_map(&c.wmap[n_tf], jb.w, p.K, x_extent, half, 2 * jb.rope.n_heads,
                                    jb.rope.head_dim / 2, RB / 2);
       if (rc) return rc;
       tiles += f.tpb * f.count;
@@ -1863,7 +1866,7 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
         f.tile_begin = tiles; f.tpb = (a.keep + rows - 1) / rows; f.keep = a.keep; f.count = a.count;
         f.job = j; f.start = a.start; f.period = a.period; f.out_base = jb.omap.base[k];
         f.mode = narrow ? kNarrow : kPlain; f.job2 = j;
-        const int rc = encode_family(&c.wmap[n_tf], jb.w + (size_t)a.start * (p.K / 2), p.K, x_extent, a.keep,
+        const int rc = encode_w_map(&c.wmap[n_tf], jb.w + (size_t)a.start * (p.K / 2), p.K, x_extent, a.keep,
                                      a.count, a.count > 1 ? a.period : a.keep, rows);
         if (rc) return rc;
         tiles += f.tpb * f.count;
@@ -2033,8 +2036,8 @@ int launch_mlp_phases(const MlpDecode& d, int first, int count, const LaunchCfg&
       P.period = d.hidden; P.count = 1;
       f.mode = kSwiglu; f.job = 0; f.job2 = 1; f.keep = d.k_int; f.period = d.inter;
       f.tpb = (d.k_int + RB / 2 - 1) / (RB / 2);
-      rc = encode_family(&c.wmap[n_tf], d.wg, d.hidden, d.hidden / 2, d.k_int, 1, d.k_int, RB / 2);
-      if (!rc) rc = encode_family(&c.wmap_up, d.wu, d.hidden, d.hidden / 2, d.k_int, 1, d.k_int, RB / 2);
+      rc = encode_w_map(&c.wmap[n_tf], d.wg, d.hidden, d.hidden / 2, d.k_int, 1, d.k_int, RB / 2);
+      if (!rc) rc = encode_w_map(&c.wmap_up, d.wu, d.hidden, d.hidden / 2, d.k_int, 1, d.k_int, RB / 2);
     } else {
       P.x = d.h; P.ldx = d.ldh; P.K = d.inter; P.start = 0; P.keep = d.k_int; P.period = d.inter; P.count = 1;
       P.g_total = (d.k_int + kGroup - 1) / kGroup;
@@ -2042,7 +2045,7 @@ int launch_mlp_phases(const MlpDecode& d, int first, int count, const LaunchCfg&
       f.mode = narrow ? kNarrow : kPlain; f.job = 2; f.job2 = 2; f.keep = d.hidden; f.period = d.hidden;
       f.tpb = (d.hidden + rows - 1) / rows;
       const int x_extent = P.g_total * 64 < d.inter / 2 ? P.g_total * 64 : d.inter / 2;
-      rc = encode_family(&c.wmap[n_tf], d.wd, d.inter, x_extent, d.hidden, 1, d.hidden, rows);
+      rc = encode_w_map(&c.wmap[n_tf], d.wd, d.inter, x_extent, d.hidden, 1, d.hidden, rows);
     }
     if (rc) return rc;
     P.tiles = f.tpb;

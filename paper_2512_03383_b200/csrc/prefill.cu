@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
       const int jn = job_of_wt(wt);
       const int tl = wt - c.wtile_begin[jn];
       // this thread owns tile row etid (= its TMEM lane); a rope pair sits in lanes 2i, 2i + 1
-      const RowStore<T> rs(p, jn, tl, etid);
+      const RowStore<T> rs(p, jn, tile_row(p.job[jn], tl, etid), (etid & 1) != 0);
       auto store_chunk = [&](int tok0, const auto& val) { rs.store(p, tt * ntok + tok0, val); };
       for (int h = h_lo; h < h_hi && !failed && !acc_known_full; ++h)
         if (!pmbar_wait(acc_full + 8 * (acc0 + h), au & 1, abort_flag)) failed = true;

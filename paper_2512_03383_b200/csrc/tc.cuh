@@ -84,7 +84,7 @@ __device__ inline bool pmbar_wait_cluster(uint32_t bar, uint32_t parity, volatil
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     if (ok) return true;
-    __nanosleep(100);
+    __nanosleep(20);
     if ((i & 63) == 63 && *abort_flag) return false;
   }
   *abort_flag = 1;
@@ -94,6 +94,11 @@ __device__ inline void tma_box2(uint32_t dst, const CUtensorMap* tm, int x, int 
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
       ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+__device__ inline void tma_box_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+      ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
 }
 __device__ inline void tmem_alloc(uint32_t smem_dst, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols) : "memory");
@@ -227,7 +232,8 @@ __device__ inline uint4 dequant_word(uint32_t w, __half2 s2, __half2 cz2) {
 
 // ---------------------------------------------------------------------------------------- epilogue of a row
 // Bias, rotary embedding (Section 3.2, fused RoPE) or gated product, one rounding and the stores of a thread that owns
-// row `r` of local tile `tl` of job `jn` (its TMEM lane); the two members of a pair sit in lanes 2i and 2i + 1.
+// one row of a tile of job `jn` (`info`: which; odd: the up row of a SwiGLU pair); the two members of a pair sit in lanes
+// 2i and 2i + 1.
 template <typename T>
 struct RowStore {
   RowInfo ri;
@@ -237,18 +243,18 @@ struct RowStore {
   float b_own;
   unsigned long long turn;
 
-  __device__ inline RowStore(const Params& p, int jn, int tl, int r) {
+  __device__ inline RowStore(const Params& p, int jn, const RowInfo& info, bool odd) {
     const JobDev& jb = p.job[jn];
     y = reinterpret_cast<T*>(jb.y);
     ldy = jb.ldy;
     rope = jb.rope.enabled != 0;
     swiglu = jb.pair == 1;
     half = jb.rope.head_keep >> 1;
-    ri = tile_row(jb, tl, r);
+    ri = info;
     b_own = 0.f;
     turn = 0;
     if (ri.stored >= 0) {
-      const T* bias = reinterpret_cast<const T*>((swiglu && (r & 1)) ? p.job[jn + 1].bias : jb.bias);
+      const T* bias = reinterpret_cast<const T*>((swiglu && odd) ? p.job[jn + 1].bias : jb.bias);
       if (bias) b_own = DT<T>::to_f(bias[ri.stored]);
       if (rope) {
         int pidx = p.idx[(ri.head / jb.rope.rep) * half + ri.pair_c];
