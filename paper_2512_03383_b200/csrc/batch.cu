@@ -7,21 +7,24 @@
 // k-block and SM whatever the batch: 1.3 TB/s.  Here
 //  - a stage is 256 channels of 128 weight rows (16 KB of codes), one TMA box or a few, fetched up to eight stages ahead,
 //    so that 100 KB per SM are in flight and the hand-shakes are a quarter as many per byte;
-//  - a de-quantiser thread owns a weight row (= a lane of tensor memory) and 64 channels of the stage: two 16-byte
-//    shared loads, 64 values in 32 registers, ONE tcgen05.st: nothing goes back through shared memory, where 16 KB
-//    written and 16 KB read per 8192 weights alone would take 256 cycles against the 195 that HBM needs for their codes;
+//  - a de-quantiser thread owns a weight row (= a lane of tensor memory) and 128 channels of the stage: four 16-byte
+//    shared loads, two times 64 values in 32 registers and a tcgen05.st: nothing goes back through shared memory, where
+//    16 KB written and 16 KB read per 8192 weights alone would take 256 cycles against the 195 that HBM needs for their
+//    codes;
 //  - the MMAs take A from tensor memory (measured: 24 / 42 / 67 cycles per 128 x N x 16 at N = 16 / 64 / 128, against
-//    90 - 96 with A in shared memory), N is the batch rounded up to 16.
+//    90 - 96 with A in shared memory), N is the batch rounded up to 16;
+//  - two blocks share an SM (half of its shared memory, tensor memory and registers each).  A launch is 5 - 20 us of
+//    which a block spends 4 on its way to the first stage and 3 on the exchange at its end; with one block per SM
+//    nothing covered those, and blocks that entered late (their SM's predecessor had left late) left late again.
 // Measured figures stand at launch_batch().
 //
-// Roles (one persistent block per SM, 24 warps):
-//   warp 0       activations by TMA: four boxes [64 k x N tokens] per stage, 128-byte swizzle
-//   warp 1       tensor-memory allocation, MMA issue (16 per stage)
+// Roles (12 warps, two blocks per SM):
+//   warp 0       activations by TMA: two boxes [64 k x N tokens] per half stage, 128-byte swizzle
+//   warp 1       tensor-memory allocation, MMA issue (8 per half stage of 128 channels)
 //   warps 2, 3   loaders: codes by TMA (warp 2), scales and zero-points by cp.async (64 rows each)
-//   warps 4..7   epilogue (bias, rotation or gated product, store; RowStore)
-//   warps 8..23  de-quantisers: warp w rows 32 (w % 4) .. + 31, channels 64 ((w - 8) / 4) .. + 63 of every stage; they
-//                share the epilogue of the block's last segment
-// Tensor memory: two accumulators of N columns, then two or three A stages of 128 columns.
+//   warps 4..11  de-quantisers: warp w rows 32 (w % 4) .. + 31, channels 128 ((w - 4) / 4) .. + 127 of every stage, and
+//                then the tile's epilogue (bias, rotation or gated product, store; RowStore)
+// Tensor memory (256 columns): an accumulator of N columns, two or three half-stage A operands of 64 columns.
 //
 // Work split: clusters of p blocks share a tile, every block a p-th of its stages; the cluster takes tiles round-robin.
 // Each block then owns every p-th chunk of 16 tokens: it leaves its fp32 sums of the other chunks in a slot of its own
@@ -46,15 +49,16 @@ namespace uniql {
 namespace {
 
 constexpr int KS = 4;                          // k-blocks per stage
-constexpr int NW = 24, NTHB = NW * 32;
+constexpr int NTHB = 384;
 constexpr int WST_BYTES = BMW * 128;           // codes of a stage: 128 bytes per row, 16-byte pieces XOR-swizzled by row
 constexpr int SZ_BYTES = BMW * 8;              // two scales and two zero-points per row: [row] half2 s, [row] half2 z
 constexpr int WSTAGE = WST_BYTES + SZ_BYTES;
 constexpr int kMaxBF = 8;                      // row families of a launch
-constexpr int MAX_WST = 8, MAX_BST = 4, MAX_AST = 3;
-constexpr int LOADERS = 2, LD_WARP0 = 2, EPI0 = 4, DQ0 = 8, DQN = 16;
-constexpr int kSmemBatch = 227 * 1024;
-constexpr int kTokChunk = 16;                  // tokens per epilogue pass
+constexpr int MAX_WST = 6, MAX_BST = 4, MAX_AST = 3;
+constexpr int LOADERS = 2, LD_WARP0 = 2, DQ0 = 4, DQN = 8;
+constexpr int kSmemBatch = 113 * 1024;         // two blocks per SM
+constexpr int kTmemCols = 256;
+constexpr int kTokChunk = 8;                   // tokens per epilogue pass; chunk i is finished by block i % p of the cluster
 
 // One family of kept row blocks {start, period, keep, count} of a job.  Plain: a block of up to 128 rows is one box and
 // `per_tile` blocks share a tile; a longer block takes `tpb` tiles of its own.  Rotation pairs and SwiGLU pairs: rows are
@@ -71,7 +75,7 @@ struct BatchCfg {
   CUtensorMap wmap_up;       // SwiGLU: the up matrix (wmap[] holds the gate matrix)
   CUtensorMap xmap;          // activations: (k, token), box 64 x n
   int n;                     // tokens of an MMA: M rounded up to 16
-  int n_ast, acc_stride, a_base;               // tensor memory: A stages, columns between the accumulators, first A column
+  int n_ast, a_base;         // tensor memory: half-stage A operands, their first column
   int wst, bst, off_w, off_bar;                // ring depths and shared-memory offsets (the activation ring is first)
   BFam fam[kMaxBF];
   int n_fam;
@@ -89,6 +93,10 @@ __device__ inline void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
       ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ inline void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
 }
 // 32 columns of this thread's lane
 __device__ inline void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
@@ -169,34 +177,33 @@ struct BSegIter {
 };
 
 template <typename T, bool HEADS>
-__global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ Params p, const __grid_constant__ BatchCfg c) {
+__global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ Params p, const __grid_constant__ BatchCfg c) {
   extern __shared__ unsigned char bsm_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const uint32_t raw = (uint32_t)__cvta_generic_to_shared(bsm_raw);
   const uint32_t sbase = (raw + 1023u) & ~1023u;
   unsigned char* smem = bsm_raw + (sbase - raw);
   const uint32_t bars = sbase + (uint32_t)c.off_bar;
   const uint32_t w_full = bars, w_empty = w_full + 8 * MAX_WST, b_full = w_empty + 8 * MAX_WST, b_empty = b_full + 8 * MAX_BST;
   const uint32_t a_full = b_empty + 8 * MAX_BST, a_empty = a_full + 8 * MAX_AST;
-  const uint32_t acc_full = a_empty + 8 * MAX_AST, acc_empty = acc_full + 16, last_full = acc_empty + 16, xbar = last_full + 8, xlast = xbar + 64;   // exchange: two per quadrant; last tile
-  unsigned char* misc = smem + c.off_bar + 8 * (2 * MAX_WST + 2 * MAX_BST + 2 * MAX_AST + 4 + 1 + 12);
+  const uint32_t acc_full = a_empty + 8 * MAX_AST, acc_empty = acc_full + 8;
+  const uint32_t xbar = acc_empty + 8;             // exchange between the blocks of a cluster: two per quadrant
+  unsigned char* misc = smem + c.off_bar + 8 * (2 * MAX_WST + 2 * MAX_BST + 2 * MAX_AST + 2 + 8);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
 
   if (tid == 0) {
     for (int s = 0; s < MAX_WST; ++s) { pmbar_init(w_full + 8 * s, LOADERS * 32 + 1); pmbar_init(w_empty + 8 * s, DQN); }
     for (int s = 0; s < MAX_BST; ++s) { pmbar_init(b_full + 8 * s, 1); pmbar_init(b_empty + 8 * s, 1); }
-    for (int s = 0; s < MAX_AST; ++s) { pmbar_init(a_full + 8 * s, DQN); pmbar_init(a_empty + 8 * s, 1); }
-    for (int s = 0; s < 2; ++s) { pmbar_init(acc_full + 8 * s, 1); pmbar_init(acc_empty + 8 * s, 4); }
-    pmbar_init(last_full, 1);
-    for (int q = 0; q < 8; ++q) pmbar_init(xbar + 8 * q, max(1, c.p - 1));
-    for (int q = 0; q < 4; ++q) pmbar_init(xlast + 8 * q, max(1, 5 * (c.p - 1)));
+    for (int s = 0; s < MAX_AST; ++s) { pmbar_init(a_full + 8 * s, DQN / 2); pmbar_init(a_empty + 8 * s, 1); }
+    pmbar_init(acc_full, 1);
+    pmbar_init(acc_empty, DQN);
+    for (int q = 0; q < 8; ++q) pmbar_init(xbar + 8 * q, max(1, 2 * (c.p - 1)));
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    tmem_alloc((uint32_t)__cvta_generic_to_shared(const_cast<uint32_t*>(tmem_slot)), 512);
+    tmem_alloc((uint32_t)__cvta_generic_to_shared(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -210,70 +217,68 @@ __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ 
   }
   bool failed = false;
 
-  // ---- epilogue of one tile for the warp that calls it: token chunks ch0, ch0 + chs, ... (chs == 1: the epilogue warp on
-  //      its own, which also hands the accumulator back; chs == 5: the last tile, shared with the de-quantiser warps)
-  auto row_store = [&](int tile) {                 // (made before the wait for the accumulator: several dependent loads)
-    const BFam& f = fam_of_tile(c, tile);
-    const int r = 32 * (warp & 3) + lane;
-    return RowStore<T>(p, f.job, batch_row(c, p, f, tile, r).info, (r & 1) != 0);
-  };
-  auto epilogue_tile = [&](const RowStore<T>& rs, int count, int ch0, int chs) {
-    const int q = warp & 3, acc = count & 1;
-    const uint32_t t_acc = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * c.acc_stride);
+  // ---- epilogue of the block's tile number `count` for the de-quantiser warp that calls it; the two warps of a quadrant
+  //      (`half`) share the chunks
+  auto epilogue_tile = [&](const RowStore<T>& rs, int count, int half) {
+    const int q = warp & 3;
+    const uint32_t t_acc = tmem + ((uint32_t)(32 * q) << 16);
     const int n_ch = c.n / kTokChunk;
     tc_fence_after();
     const size_t slot_f = (size_t)c.n * BMW;
     float* slots = c.partials + (size_t)(count & 1) * slot_f + 32 * q + lane;      // + block * 2 slots + token * BMW
-    const int block0 = (int)blockIdx.x - rank;
+    const float* block0 = slots + (size_t)((int)blockIdx.x - rank) * 2 * slot_f;
     if (c.p > 1) {
       // the sums of the chunks that other blocks finish
       float* mine = slots + (size_t)blockIdx.x * 2 * slot_f;
-      for (int ch = ch0; ch < n_ch; ch += chs) {
+      for (int ch = half; ch < n_ch; ch += 2) {
         if (ch % c.p == rank) continue;
-        uint32_t v[16];
-        tmem_ld16(t_acc + (uint32_t)(ch * kTokChunk), v);
+        uint32_t v[8];
+        tmem_ld8(t_acc + (uint32_t)(ch * kTokChunk), v);
         tmem_ld_wait();
 #pragma unroll
-        for (int k = 0; k < 16; ++k) __stcg(mine + (size_t)(ch * kTokChunk + k) * BMW, __uint_as_float(v[k]));
+        for (int k = 0; k < 8; ++k) __stcg(mine + (size_t)(ch * kTokChunk + k) * BMW, __uint_as_float(v[k]));
       }
       __syncwarp();
       // (barriers alternate from tile to tile: a peer may be a tile ahead before another peer's arrival has come in)
-      const uint32_t xb = chs == 1 ? xbar + 32 * (count & 1) + 8 * q : xlast + 8 * q;
+      const uint32_t xb = xbar + 32 * (count & 1) + 8 * q;
       if (lane < c.p && lane != rank) {
         asm volatile("fence.acq_rel.cluster;" ::: "memory");
         pmbar_arrive_peer(ppeer_addr(xb, (uint32_t)lane));
       }
-      const bool ok = __all_sync(0xffffffffu, pmbar_wait_cluster(xb, chs == 1 ? (count >> 1) & 1 : 0, abort_flag));
+      const bool ok = __all_sync(0xffffffffu, pmbar_wait_cluster(xb, (count >> 1) & 1, abort_flag));
       if (!ok) { failed = true; return; }
     }
-    for (int ch = ch0; ch < n_ch; ch += chs) {
-      if (c.p > 1 && ch % c.p != rank) continue;
-      uint32_t v[16];
-      tmem_ld16(t_acc + (uint32_t)(ch * kTokChunk), v);
-      float val[16];
+    for (int own = half; rank + own * c.p < n_ch; own += 2) {
+      const int ch = rank + own * c.p;
+      uint32_t v[8];
+      tmem_ld8(t_acc + (uint32_t)(ch * kTokChunk), v);
+      float val[8];
 #pragma unroll
-      for (int k = 0; k < 16; ++k) val[k] = 0.f;
-      for (int r = 0; r < c.p; ++r) {
-        if (r == rank) {
-          tmem_ld_wait();
+      for (int k = 0; k < 8; ++k) val[k] = 0.f;
+      const float* src = block0 + (size_t)(ch * kTokChunk) * BMW;
+      for (int r0 = 0; r0 < c.p; r0 += 4) {                    // four blocks' sums in flight, added in rank order
+        float a[4][8];
 #pragma unroll
-          for (int k = 0; k < 16; ++k) val[k] += __uint_as_float(v[k]);
-        } else {
-          const float* src = slots + (size_t)(block0 + r) * 2 * slot_f + (size_t)(ch * kTokChunk) * BMW;
-          float a[16];
+        for (int r = 0; r < 4; ++r)
 #pragma unroll
-          for (int k = 0; k < 16; ++k) a[k] = __ldcg(src + (size_t)k * BMW);
+          for (int k = 0; k < 8; ++k)
+            a[r][k] = (r0 + r < c.p && r0 + r != rank) ? __ldcg(src + (size_t)(r0 + r) * 2 * slot_f + (size_t)k * BMW) : 0.f;
+        tmem_ld_wait();
 #pragma unroll
-          for (int k = 0; k < 16; ++k) val[k] += a[k];
-        }
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int k = 0; k < 8; ++k) val[k] += r0 + r == rank ? __uint_as_float(v[k]) : a[r][k];
       }
       rs.store(p, ch * kTokChunk, val);
     }
-    if (chs == 1) {                                            // the accumulator is free for the tile after the next
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) pmbar_arrive(acc_empty + 8 * acc);
-    }
+    tc_fence_before();                                         // the accumulator is free for the next tile
+    __syncwarp();
+    if (lane == 0) pmbar_arrive(acc_empty);
+  };
+  auto row_store = [&](int tile) {
+    const BFam& f = fam_of_tile(c, tile);
+    const int r = 32 * (warp & 3) + lane;
+    return RowStore<T>(p, f.job, batch_row(c, p, f, tile, r).info, (r & 1) != 0);
   };
 
   BSegIter si;
@@ -282,19 +287,22 @@ __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ 
   if (warp == 0) {
     // ===================================================================== activations
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    // Only now may the next launch's blocks come in: as two launches fit an SM, triggering at entry let the launch after
+    // the next one in as well, whose blocks then sat in slots that this launch's blocks needed.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     int s = 0, it = 0; uint32_t par = 1;
     const uint32_t box = (uint32_t)c.n * 128u;
     while (!failed && si.next(sg)) {
-      for (int st = sg.s0; st < sg.s1; ++st, ++it) {
-        if (it >= c.bst && !pmbar_wait_warp(b_empty + 8 * s, par, abort_flag, true)) { failed = true; break; }
-        const int v0 = st * KS, nv = min(KS, c.n_kb - v0);
+      for (int v0 = sg.s0 * KS; v0 < min(sg.s1 * KS, c.n_kb); v0 += KS / 2, ++it) {
+        if (it >= c.bst && !pmbar_wait_warp(b_empty + 8 * s, par, abort_flag)) { failed = true; break; }
+        const int nv = min(KS / 2, c.n_kb - v0);
         const uint32_t fb = b_full + 8 * s;
         if (elect_one()) {
           pmbar_expect_tx(fb, (uint32_t)nv * box);
           for (int i = 0; i < nv; ++i) {
             const int v = v0 + i;
             const int x = HEADS ? (v / c.head_kb) * c.head_keep + (v % c.head_kb) * BK : v * BK;
-            tma_box2(sbase + (uint32_t)(s * KS + i) * box, &c.xmap, x, 0, fb);
+            tma_box2(sbase + (uint32_t)(s * (KS / 2) + i) * box, &c.xmap, x, 0, fb);
           }
         }
         __syncwarp();
@@ -308,45 +316,38 @@ __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ 
   } else if (warp == 1) {
     // ===================================================================== MMA issue
     int as = 0, bs = 0, count = 0; uint32_t apar = 0, bpar = 0;
+    const uint64_t box_step = (uint64_t)(c.n * 8);             // a box of n * 128 bytes, in the descriptor's 16-byte units
     for (; !failed && si.next(sg); ++count) {
-      const int acc = count & 1, use = count >> 1;
-      const uint32_t d = tmem + (uint32_t)(acc * c.acc_stride);
-      if (use >= 1 && !pmbar_wait_warp(acc_empty + 8 * acc, (use - 1) & 1, abort_flag)) { failed = true; break; }
-      for (int st = sg.s0; st < sg.s1; ++st) {
-        if (!pmbar_wait_warp(b_full + 8 * bs, bpar, abort_flag) || !pmbar_wait_warp(a_full + 8 * as, apar, abort_flag)) { failed = true; break; }
+      if (count >= 1 && !pmbar_wait_warp(acc_empty, (count - 1) & 1, abort_flag)) { failed = true; break; }
+      for (int v0 = sg.s0 * KS; v0 < sg.s1 * KS; v0 += KS / 2) {
+        const int nv = c.n_kb - v0;                            // k-blocks of this half stage (none behind the last: only handed back)
+        if ((nv > 0 && !pmbar_wait_warp(b_full + 8 * bs, bpar, abort_flag)) || !pmbar_wait_warp(a_full + 8 * as, apar, abort_flag)) {
+          failed = true;
+          break;
+        }
         tc_fence_after();
-        const int nv = min(KS, c.n_kb - st * KS);
-        const uint32_t a0 = tmem + (uint32_t)(c.a_base + 128 * as);
-        const uint32_t b0 = sbase + (uint32_t)(bs * KS * c.n) * 128u;
+        const uint32_t a0 = tmem + (uint32_t)(c.a_base + 64 * as);
+        const uint64_t bd = smem_desc_sw128(sbase + (uint32_t)(bs * (KS / 2) * c.n) * 128u);
         if (elect_one()) {
-          uint64_t bd = smem_desc_sw128(b0);
-          const uint64_t step = (uint64_t)(c.n * 8);           // a box of n * 128 bytes, in the descriptor's 16-byte units
 #pragma unroll
-          for (int i = 0; i < KS; ++i) {
+          for (int i = 0; i < KS / 2; ++i) {
             if (i >= nv) break;
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k)
-              umma_ts(d, a0 + 32 * i + 8 * k, bd + 2 * k, c.idesc, (st > sg.s0 || i > 0 || k > 0) ? 1u : 0u);
-            bd += step;
+              umma_ts(tmem, a0 + 32 * i + 8 * k, bd + i * box_step + 2 * k, c.idesc, (v0 > sg.s0 * KS || i > 0 || k > 0) ? 1u : 0u);
           }
           umma_commit(a_empty + 8 * as);
-          umma_commit(b_empty + 8 * bs);
+          if (nv > 0) umma_commit(b_empty + 8 * bs);
         }
         __syncwarp();
         if (++as == c.n_ast) { as = 0; apar ^= 1; }
-        if (++bs == c.bst) { bs = 0; bpar ^= 1; }
+        if (nv > 0 && ++bs == c.bst) { bs = 0; bpar ^= 1; }
       }
       if (failed) break;
-      BSegIter peek = si;
-      BSeg nxt;
-      const bool last = !peek.next(nxt);
-      if (elect_one()) {
-        umma_commit(acc_full + 8 * acc);
-        if (last) umma_commit(last_full);      // (the helpers' own barrier: one phase, no parity to lose)
-      }
+      if (elect_one()) umma_commit(acc_full);
       __syncwarp();
     }
-  } else if (warp < EPI0) {
+  } else if (warp < DQ0) {
     // ===================================================================== loaders
     // Codes by TMA, issued by warp 2 (a box per lane).  (The first version copied them with cp.async, sixteen 16-byte
     // pieces per lane and stage: 1100 cycles of issue per stage and loader warp, which set the pace.)  Scales and
@@ -403,18 +404,17 @@ __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ 
       for (int j = it > c.wst ? it - c.wst : 0; j < it; ++j)
         for (int i = 0; i < kPWait && !pmbar_try(w_full + 8 * (j % c.wst), (j / c.wst) & 1); ++i) {}
     }
-  } else if (warp >= DQ0) {
-    // ===================================================================== de-quantisers
-    // Software-pipelined: the codes of the next stage are in registers before the current one is converted, and the
-    // tcgen05.st of a stage completes while the first half of the next is converted.
-    const int q = warp & 3, kq = (warp - DQ0) >> 2;
+  } else {
+    // ===================================================================== de-quantisers, then the tile's epilogue
+    // The tcgen05.st of a half stage completes while the first part of the next is converted, and the codes of the next
+    // stage are in registers before this one's last values are stored.
+    const int q = warp & 3, half = (warp - DQ0) >> 2;
     const int r = 32 * q + lane;
-    const uint32_t s_off = (uint32_t)(WST_BYTES + r * 4 + (kq >> 1) * 2);
-    const uint32_t a_lane = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(c.a_base + 32 * kq);
-    int ws = 0, as = 0, it = 0; uint32_t wpar = 0, apar = 1;
-    int n_seg = 0;
-    BSeg last_sg = {0, 0, 0};
-    int stored_as = -1;                          // A stage whose tcgen05.st is still to be announced
+    const uint32_t s_off = (uint32_t)(WST_BYTES + r * 4 + half * 2);
+    const uint32_t a_lane = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c.a_base;
+    int ws = 0; uint32_t wpar = 0;
+    int as = half, use = 0;                      // this warp's next A slot, the slot's earlier uses (n_ast >= 2)
+    int stored_as = -1;                          // A slot whose tcgen05.st is still to be announced
     auto announce = [&]() {
       if (stored_as < 0) return;
       tmem_st_wait();
@@ -423,18 +423,18 @@ __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ 
       if (lane == 0) pmbar_arrive(a_full + 8 * stored_as);
       stored_as = -1;
     };
-    while (!failed && si.next(sg)) {
-      last_sg = sg;
-      ++n_seg;
+    for (int count = 0; !failed && si.next(sg); ++count) {
       const int sr = batch_row(c, p, fam_of_tile(c, sg.tile), sg.tile, r).smem_row;
-      const uint32_t x0 = (uint32_t)(sr * 128 + ((2 * kq) ^ (sr & 7)) * 16), x1 = (uint32_t)(sr * 128 + ((2 * kq + 1) ^ (sr & 7)) * 16);
-      uint32_t w[8];
+      const uint32_t x_row = (uint32_t)(sr * 128), x_sw = (uint32_t)((half * 4) ^ (sr & 7)) * 16;   // piece i: x_sw ^ (16 i)
+      uint32_t w[16];
       __half sc, zp;
       auto fetch = [&]() -> bool {               // codes, scale and zero-point of the next stage of the ring; the slot is free again
         if (!pmbar_wait_warp(w_full + 8 * ws, wpar, abort_flag)) return false;
         const uint32_t src = sbase + (uint32_t)(c.off_w + ws * WSTAGE);
-        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(src + x0) : "memory");
-        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]) : "r"(src + x1) : "memory");
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[4 * i]), "=r"(w[4 * i + 1]), "=r"(w[4 * i + 2]), "=r"(w[4 * i + 3])
+                       : "r"(src + x_row + (x_sw ^ (16 * i))) : "memory");
         unsigned short sh, zh;
         asm volatile("ld.shared.u16 %0, [%1];" : "=h"(sh) : "r"(src + s_off) : "memory");
         asm volatile("ld.shared.u16 %0, [%1];" : "=h"(zh) : "r"(src + s_off + BMW * 4) : "memory");
@@ -445,55 +445,53 @@ __global__ void __launch_bounds__(NTHB, 1) batch_kernel(const __grid_constant__ 
         return true;
       };
       if (!fetch()) { failed = true; break; }
-      for (int st = sg.s0; st < sg.s1; ++st, ++it) {
+      for (int st = sg.s0; st < sg.s1; ++st) {
         const __half2 s2 = __half2half2(sc);
         const __half2 cz2 = __float2half2_rn((8.f - __half2float(zp)) * __half2float(sc));
         uint32_t o[32];
-        int valid = BK;
-        if (HEADS) valid = min(BK, c.head_keep - ((st * KS + kq) % c.head_kb) * BK);
-        auto convert = [&](int j0) {
+        int valid = 2 * BK;                      // kept channels of the half stage's k-blocks, one bit field each
+        if (HEADS) {
+          const int v = st * KS + 2 * half;
+          valid = min(BK, c.head_keep - (v % c.head_kb) * BK) | (min(BK, c.head_keep - ((v + 1) % c.head_kb) * BK) << 8);
+        }
+        auto convert = [&](int j0) {             // words j0 .. j0 + 3 of the sixteen
 #pragma unroll
-          for (int j = j0; j < j0 + 4; ++j) {
-            const uint4 d = (!HEADS || j * 8 < valid) ? dequant_word(w[j], s2, cz2) : make_uint4(0, 0, 0, 0);
-            o[4 * j] = d.x; o[4 * j + 1] = d.y; o[4 * j + 2] = d.z; o[4 * j + 3] = d.w;
+          for (int i = j0; i < j0 + 4; ++i) {
+            const int k = i & 7;
+            const bool kept = !HEADS || k * 8 < (i < 8 ? (valid & 255) : (valid >> 8));
+            const uint4 d = kept ? dequant_word(w[i], s2, cz2) : make_uint4(0, 0, 0, 0);
+            o[4 * k] = d.x; o[4 * k + 1] = d.y; o[4 * k + 2] = d.z; o[4 * k + 3] = d.w;
           }
         };
         convert(0);
         announce();
         convert(4);
-        if (st + 1 < sg.s1 && !fetch()) { failed = true; break; }
-        if (it >= c.n_ast && !pmbar_wait_warp(a_empty + 8 * as, apar, abort_flag)) { failed = true; break; }
+        // (the slot's previous user: the half stage n_ast earlier.  This warp wrote the half stage two earlier after a wait
+        //  that implies every half stage up to 2 + n_ast earlier is done, so the parity cannot be two phases old.)
+        if (use > 0 && !pmbar_wait_warp(a_empty + 8 * as, (use - 1) & 1, abort_flag)) { failed = true; break; }
         tc_fence_after();
-        tmem_st32(a_lane + (uint32_t)(128 * as), o);
+        tmem_st32(a_lane + (uint32_t)(64 * as), o);
+        convert(8);
+        convert(12);
+        if (st + 1 < sg.s1 && !fetch()) { failed = true; break; }
+        tmem_st32(a_lane + (uint32_t)(64 * as + 32), o);
         stored_as = as;
-        if (++as == c.n_ast) { as = 0; apar ^= 1; }
+        as += 2;
+        if (as >= c.n_ast) { as -= c.n_ast; ++use; }
       }
-      if (!failed) announce();
-    }
-    if (!failed && n_seg > 0) {
-      asm volatile("griddepcontrol.wait;" ::: "memory");
-      const RowStore<T> rs = row_store(last_sg.tile);
-      if (!pmbar_wait_warp(last_full, 0, abort_flag)) failed = true;
-      if (!failed) epilogue_tile(rs, n_seg - 1, 1 + kq, 5);
-    }
-  } else {
-    // ===================================================================== epilogue
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    int count = 0;
-    for (; !failed && si.next(sg); ++count) {
-      BSegIter peek = si;
-      BSeg nxt;
-      const bool last = !peek.next(nxt);
-      const RowStore<T> rs = row_store(sg.tile);
-      if (!pmbar_wait_warp(acc_full + 8 * (count & 1), (count >> 1) & 1, abort_flag)) { failed = true; break; }
-      epilogue_tile(rs, count, 0, last ? 5 : 1);
+      if (failed) break;
+      announce();
+      asm volatile("griddepcontrol.wait;" ::: "memory");       // outputs, positions and workspace: after the preceding kernel
+      const RowStore<T> rs = row_store(sg.tile);               // (several dependent loads, while the last MMAs run)
+      if (!pmbar_wait_warp(acc_full, count & 1, abort_flag)) { failed = true; break; }
+      epilogue_tile(rs, count, half);
     }
   }
   if (failed && lane == 0) atomicExch(c.status, UNIQL_ERR_TIMEOUT);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem, 512);
+  if (warp == 1) tmem_dealloc(tmem, kTmemCols);
   if (c.p > 1) {                        // no block leaves while a peer may still arrive at its barriers
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -571,7 +569,7 @@ struct BLaunch {
 };
 
 constexpr int kMaxP = 8;
-// Clusters of p blocks that the device holds at once (one block per SM), asked once per device: resident[p].
+// Clusters of p blocks that the device holds at once (two blocks per SM), asked once per device.
 struct Residency { bool known = false; int clusters[kMaxP + 1]; };
 int residency(Residency* out) {
   static std::mutex mu;
@@ -586,12 +584,12 @@ int residency(Residency* out) {
         return UNIQL_ERR_CUDA;
     const int sms = device_sms();
     r.clusters[0] = 0;
-    r.clusters[1] = sms;
+    r.clusters[1] = 2 * sms;
     for (int p = 2; p <= kMaxP; ++p) {
-      BLaunch l(sms / p * p, p, kSmemBatch, nullptr);
+      BLaunch l(2 * sms / p * p, p, kSmemBatch, nullptr);
       int n = 0;
       if (cudaOccupancyMaxActiveClusters(&n, batch_instance(false, false), &l.lc) != cudaSuccess) { cudaGetLastError(); n = 0; }
-      r.clusters[p] = n < sms / p ? n : sms / p;
+      r.clusters[p] = n < 2 * sms / p ? n : 2 * sms / p;
     }
     r.known = true;
   }
@@ -631,12 +629,11 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   c.head_keep = a.keep;
   // fp32 accumulate, A and B fp16, both K-major, N tokens, 128 rows
   c.idesc = (1u << 4) | ((uint32_t)(c.n >> 3) << 17) | ((uint32_t)(BMW >> 4) << 24);
-  c.acc_stride = c.n <= 64 ? 64 : 128;
   c.n_ast = c.n <= 64 ? 3 : 2;
-  c.a_base = 2 * c.acc_stride;
-  // shared memory: two to four stages of activations, the rest for the codes (deep: HBM's latency is theirs to cover)
-  c.bst = c.n > 80 ? 2 : (c.n > 32 ? 3 : 4);
-  c.off_w = c.bst * KS * c.n * 128;
+  c.a_base = c.n <= 64 ? 64 : 128;
+  // shared memory: two to four half stages of activations, the rest for the codes (HBM's latency is theirs to cover)
+  c.bst = c.n > 64 ? 2 : (c.n > 32 ? 3 : 4);
+  c.off_w = c.bst * (KS / 2) * c.n * 128;
   const int room = kSmemBatch - 1024 - 512 - c.off_w;
   c.wst = room / WSTAGE < MAX_WST ? room / WSTAGE : MAX_WST;
   c.off_bar = c.off_w + c.wst * WSTAGE;
@@ -650,8 +647,8 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
     x = reinterpret_cast<unsigned char*>(cfg.workspace) + used;
     used = (used + (size_t)p.M * ldx * 2 + 255) & ~(size_t)255;
   }
-  // The split: p blocks per tile where that shortens the longest block's work.  In stages of about half a microsecond: the
-  // rounds of the clusters that fit, a p-th of a tile's stages each, and about four stages for the exchange at the end.
+  // The split: p blocks per tile where that shortens the longest block's work.  In microseconds: the rounds of the clusters
+  // that fit, a p-th of a tile's stages each at 0.65 (one block per SM) or 1.05 (two), and 3 for the exchange.
   Residency res;
   int rc = residency(&res);
   if (rc != UNIQL_OK) return rc;
@@ -663,10 +660,12 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
     if (env_grid >= 1 && env_grid / k < fit) fit = env_grid / k;              // tests: several tiles per block on small problems
     if (fit < 1 || k > c.spt) continue;
     if (k > 1 && (env_split == 0 || cfg.ws_bytes < used + (size_t)fit * k * 2 * c.n * BMW * 4)) continue;
+    const int clusters = c.n_tiles < fit ? c.n_tiles : fit;
     const int rounds = (c.n_tiles + fit - 1) / fit;
-    double cost = (double)rounds * c.spt / k + (k > 1 ? 4.0 : 0.0) + 0.3 * rounds;
-    if (env_split >= 1 && k > 1) cost *= 1e-3;                               // tests: split wherever it is possible
-    if (cost < best_cost) { best_cost = cost; best = k; best_clusters = c.n_tiles < fit ? c.n_tiles : fit; }
+    double cost = rounds * ((double)c.spt / k * (clusters * k > device_sms() ? 1.05 : 0.65) + (k > 1 ? 3.0 : 1.0));
+    if (env_split >= 1 && env_split <= 3 && k > 1) cost *= 1e-3;              // tests: split wherever it is possible
+    if (env_split == 10 + k) cost = 0.0;                                     // ... over k blocks
+    if (cost < best_cost) { best_cost = cost; best = k; best_clusters = clusters; }
   }
   c.p = best;
   c.partials = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(cfg.workspace) + used);

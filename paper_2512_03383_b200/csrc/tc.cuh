@@ -42,8 +42,8 @@ __device__ inline bool pmbar_wait(uint32_t bar, uint32_t parity, volatile int* a
 }
 // The same for a whole warp: one answer for all lanes (a warp whose lanes disagreed about an expired wait would part, and
 // its next warp-wide instruction would wait for the missing lanes).
-__device__ inline bool pmbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, bool relaxed = false) {
-  return __all_sync(0xffffffffu, pmbar_wait(bar, parity, abort_flag, relaxed));
+__device__ inline bool pmbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, pmbar_wait(bar, parity, abort_flag));
 }
 // ---- clusters of two (a tile's contraction split over a pair of blocks)
 __device__ inline uint32_t pcluster_rank() {
