@@ -40,10 +40,27 @@ __device__ inline bool pmbar_wait(uint32_t bar, uint32_t parity, volatile int* a
   *abort_flag = 1;
   return false;
 }
+// As pmbar_try, but the hardware may suspend the thread for up to a microsecond until the phase completes.
+__device__ inline bool pmbar_try_suspend(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(bar), "r"(parity), "r"(1000u) : "memory");
+  return ok != 0;
+}
 // The same for a whole warp: one answer for all lanes (a warp whose lanes disagreed about an expired wait would part, and
 // its next warp-wide instruction would wait for the missing lanes).
 __device__ inline bool pmbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  return __all_sync(0xffffffffu, pmbar_wait(bar, parity, abort_flag));
+  if (__all_sync(0xffffffffu, pmbar_try(bar, parity))) return true;
+  bool ok = false;
+  for (int i = 0; i < kPWait && !ok; ++i) {
+    ok = pmbar_try_suspend(bar, parity);                // (polling without a suspend time costs issue slots: 3 % of a launch)
+    if (!ok && (i & 63) == 63 && *abort_flag) break;
+  }
+  if (!ok) *abort_flag = 1;
+  return __all_sync(0xffffffffu, ok);
 }
 // ---- clusters of two (a tile's contraction split over a pair of blocks)
 __device__ inline uint32_t pcluster_rank() {
