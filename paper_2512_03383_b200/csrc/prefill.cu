@@ -56,6 +56,7 @@ namespace {
 constexpr int MAXBN = 256;          // tokens per tile (MMA N), at most
 constexpr int PSTAGES = 4;                   // ring of de-quantised weight stages (one k-block each)
 constexpr int BSLOTS = 4;                    // ring of activation boxes (one k-block of MAXBN tokens each)
+constexpr int BSLOTS2 = 8;                   // ... of half boxes (block pairs: each block holds half of the tokens)
 constexpr int A_BYTES = BMW * BK * 2;        // 16 KB
 constexpr int B_BYTES = MAXBN * BK * 2;      // 32 KB
 constexpr int RING_BYTES = PSTAGES * A_BYTES + BSLOTS * B_BYTES;
@@ -218,7 +219,11 @@ __global__ void x_to_f16_kernel(const __nv_bfloat16* __restrict__ x, int ldx, in
 // T: activation / output type.  CONV: the activation tiles arrive as bf16 and are converted to fp16 in
 // shared memory by the de-quantisers (used when the workspace cannot hold a converted copy).
 // HEADS: the input map is a family of per-head blocks (else a leading block).
-template <typename T, bool CONV, bool HEADS>
+// PAIR: clusters of two blocks work on tiles of 256 weight rows with cta_group::2 MMAs.  Each block de-quantises 128 rows
+// into its own shared memory and fetches half of the tokens' boxes; the first block's MMA warp issues for both.  A block's
+// shared memory then takes in 16 instead of 32 KB of activations per 256 tokens and k-block, which with one block per tile
+// was what L2 could not deliver and the shared-memory port could not take beside the operand reads.
+template <typename T, bool CONV, bool HEADS, bool PAIR>
 __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__ Params p,
                                                          const __grid_constant__ PrefillCfg c) {
   extern __shared__ unsigned char psmem_raw[];
@@ -231,28 +236,31 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
   const uint32_t raw = (uint32_t)__cvta_generic_to_shared(psmem_raw);
   const uint32_t sbase = (raw + 1023u) & ~1023u;           // swizzled tiles need 1024-byte alignment
   unsigned char* smem = psmem_raw + (sbase - raw);
+  constexpr int NB = PAIR ? BSLOTS2 : BSLOTS;               // slots of the activation ring and their size
+  constexpr int NB_BYTES = PAIR ? B_BYTES / 2 : B_BYTES;
+  const int bid = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x, nblk = PAIR ? (int)gridDim.x >> 1 : (int)gridDim.x;
   const uint32_t bars = sbase + RING_BYTES;
   const uint32_t full_a = bars, empty_a = bars + 8 * PSTAGES;
-  const uint32_t full_b = bars + 16 * PSTAGES, empty_b = full_b + 8 * BSLOTS;
-  const uint32_t acc_full = full_b + 16 * BSLOTS, acc_empty = acc_full + 16, epi_bar = acc_full + 32;
+  const uint32_t full_b = bars + 16 * PSTAGES, empty_b = full_b + 8 * NB;
+  const uint32_t acc_full = full_b + 16 * NB, acc_empty = acc_full + 16, epi_bar = acc_full + 32;
   const uint32_t help_bar = acc_full + 40;         // the epilogue warps and the de-quantiser warps that help them
   const uint32_t last_full = acc_full + 48;        // the MMAs of the block's last segment are complete (one phase only)
   const uint32_t px_ready = acc_full + 56;         // pair split, second block: the first block's rings are idle
   const uint32_t px_done = acc_full + 64;          // pair split, first block: the second block's sums have arrived
-  unsigned char* misc = smem + RING_BYTES + 16 * PSTAGES + 16 * BSLOTS + 72;
+  unsigned char* misc = smem + RING_BYTES + 16 * PSTAGES + 16 * NB + 72;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
 
   if (tid == 0) {
     for (int s = 0; s < PSTAGES; ++s) {
-      pmbar_init(full_a + 8 * s, DQ_TEAM_WARPS);
+      pmbar_init(full_a + 8 * s, PAIR ? 2 * DQ_TEAM_WARPS : DQ_TEAM_WARPS);
       pmbar_init(empty_a + 8 * s, 1);
     }
-    for (int s = 0; s < BSLOTS; ++s) {
+    for (int s = 0; s < NB; ++s) {
       pmbar_init(full_b + 8 * s, 1);
       pmbar_init(empty_b + 8 * s, 1);
     }
-    for (int b = 0; b < 2; ++b) { pmbar_init(acc_full + 8 * b, 1); pmbar_init(acc_empty + 8 * b, 4); }
+    for (int b = 0; b < 2; ++b) { pmbar_init(acc_full + 8 * b, 1); pmbar_init(acc_empty + 8 * b, PAIR ? 8 : 4); }
     pmbar_init(epi_bar, 4);
     pmbar_init(help_bar, 4 + 2 * DQ_WARPS);
     pmbar_init(last_full, 1);
@@ -262,19 +270,26 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {                      // the whole tensor memory of the SM: two accumulators of 256 columns
-    tmem_alloc((uint32_t)__cvta_generic_to_shared(const_cast<uint32_t*>(tmem_slot)), 512);
-    tmem_relinquish();
+    const uint32_t slot = (uint32_t)__cvta_generic_to_shared(const_cast<uint32_t*>(tmem_slot));
+    if (PAIR) {
+      tmem_alloc_pair(slot, 512);
+    } else {
+      tmem_alloc(slot, 512);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const uint32_t crank = c.pair_split ? pcluster_rank() : 0u;
-  if (c.pair_split) {                   // the other block's barriers exist before anything is sent to it
+  const uint32_t crank = (PAIR || c.pair_split) ? pcluster_rank() : 0u;
+  if (PAIR || c.pair_split) {                   // the other block's barriers exist before anything is sent to it
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
 
+  // 128-row tile of its job that this block holds (PAIR: tiles are counted in pairs)
+  auto local_tile = [&](int wt, int jn) { return PAIR ? 2 * (wt - c.wtile_begin[jn]) + (int)crank : wt - c.wtile_begin[jn]; };
   auto job_of_wt = [&](int wt) { int j = 0; while (j + 1 < p.n_jobs && wt >= c.wtile_begin[j + 1]) ++j; return j; };
   bool failed = false;
 
@@ -309,7 +324,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
       const int t = sg.tile;
       const int wt = t / c.n_ttiles, tt = t - wt * c.n_ttiles;
       const int jn = job_of_wt(wt);
-      const int tl = wt - c.wtile_begin[jn];
+      const int tl = local_tile(wt, jn);
       // this thread owns tile row etid (= its TMEM lane); a rope pair sits in lanes 2i, 2i + 1
       const RowStore<T> rs(p, jn, tile_row(p.job[jn], tl, etid), (etid & 1) != 0);
       auto store_chunk = [&](int tok0, const auto& val) { rs.store(p, tt * ntok + tok0, val); };
@@ -325,7 +340,10 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
         if (((ch + 1) * EPI_TOK) % c.bn != 0) return;
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) pmbar_arrive(acc_empty + 8 * (acc0 + (ch * EPI_TOK) / c.bn));
+        if (lane == 0) {
+          const uint32_t eb = acc_empty + 8 * (acc0 + (ch * EPI_TOK) / c.bn);
+          if (PAIR) pmbar_signal_peer(ppeer_addr(eb, 0u)); else pmbar_arrive(eb);
+        }
       };
       if (sg.kb0 == 0 && sg.kb1 == c.n_kb) {
         // ---- the whole contraction of this tile ran here (this warp takes every chs-th chunk of 32 tokens;
@@ -378,8 +396,11 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
         }
         const bool main_lane = warp == EPI_WARP0 && lane == 0;
         const size_t slot_f = (size_t)ntok * BMW;
-        const int T0 = (c.n_tiles / (int)gridDim.x) * (int)gridDim.x;          // first left-over tile
-        float* mine = c.partials + ((size_t)(t - T0) + (c.sk_atomic ? 0 : blockIdx.x)) * slot_f;
+        const int T0 = (c.n_tiles / nblk) * nblk;              // first left-over tile
+        // (PAIR: two slots side by side, a block's own 128 rows in each)
+        auto slot_of = [&](int n) { return c.partials + (PAIR ? 2 * (size_t)n + crank : (size_t)n) * slot_f; };
+        float* mine = slot_of((t - T0) + (c.sk_atomic ? 0 : bid));
+        int* arrivals = &c.counters[PAIR ? 2 * t + (int)crank : t];
         if (pair_send) {
           // (the second block of a pair: its "slot" is the first block's rings, once they are idle)
           if (!pmbar_wait_cluster(px_ready, 0, abort_flag)) { failed = true; return; }
@@ -412,17 +433,18 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
         }
         __threadfence();                                       // this thread's part is in place before ...
         if (!(chs == 1 ? epi_sync() : help_sync())) { failed = true; return; }
-        const long U = (long)(c.n_tiles - T0) * c.n_kb, Bn = (long)gridDim.x < U ? (long)gridDim.x : U;
+        const long U = (long)(c.n_tiles - T0) * c.n_kb, Bn = (long)nblk < U ? (long)nblk : U;
         const long tu = (long)(t - T0) * c.n_kb;                               // the tile's first left-over unit
         const int first = sk_owner(tu, Bn, U), last = sk_owner(tu + c.n_kb - 1, Bn, U);
         if (main_lane) {
-          const int arrived = atomicAdd(&c.counters[t], 1);    // ... the block's arrival shows
+          const int arrived = atomicAdd(arrivals, 1);          // ... the block's arrival shows
           *last_flag = arrived == last - first;
           __threadfence();
         }
         if (!(chs == 1 ? epi_sync() : help_sync())) { failed = true; return; }
         if (*last_flag) {
-          const float* base = c.partials + ((size_t)(t - T0) + (c.sk_atomic ? 0 : first)) * slot_f;
+          const float* base = slot_of((t - T0) + (c.sk_atomic ? 0 : first));
+          const size_t part_f = PAIR ? 2 * slot_f : slot_f;    // from one block's part to the next one's
           const int parts = c.sk_atomic ? 1 : last - first + 1;
           // 16 tokens at a time, the loads of two slots in flight together (what the registers of a thread hold)
           for (int tk = 16 * ch0; tk < ntok; tk += 16 * chs) {
@@ -434,15 +456,15 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
               const bool two = s2 + 1 < parts;
               float a[16], b[16];
 #pragma unroll
-              for (int k = 0; k < 16; ++k) a[k] = __ldcg(src + (size_t)s2 * slot_f + (size_t)k * BMW);
+              for (int k = 0; k < 16; ++k) a[k] = __ldcg(src + (size_t)s2 * part_f + (size_t)k * BMW);
 #pragma unroll
-              for (int k = 0; k < 16; ++k) b[k] = two ? __ldcg(src + (size_t)(s2 + 1) * slot_f + (size_t)k * BMW) : 0.f;
+              for (int k = 0; k < 16; ++k) b[k] = two ? __ldcg(src + (size_t)(s2 + 1) * part_f + (size_t)k * BMW) : 0.f;
 #pragma unroll
               for (int k = 0; k < 16; ++k) val[k] = (val[k] + a[k]) + b[k];
             }
             store_chunk(tk, val);
           }
-          if (main_lane) c.counters[t] = 0;              // ready for the next call
+          if (main_lane) *arrivals = 0;                  // ready for the next call
         }
       }
   };
@@ -452,7 +474,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     if (lane == 0) {
       asm volatile("griddepcontrol.wait;" ::: "memory");   // the activations may come from the preceding kernel
       int s = 0; uint32_t par = 1; int jb = 0;             // box slot, parity of its previous use, boxes so far
-      SegIter si; si.init(c, blockIdx.x, gridDim.x);
+      SegIter si; si.init(c, bid, nblk);
       Seg sg;
       while (!failed && si.next(sg)) {
         const int tt = sg.tile % c.n_ttiles;
@@ -463,24 +485,33 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
           if (HEADS) kw.step(c, 1);
           const int h_lo = sg.half < 0 ? 0 : sg.half, h_hi = sg.half < 0 ? c.nh : sg.half + 1;
           for (int h = h_lo; h < h_hi; ++h, ++jb) {
-            if (jb >= BSLOTS && !pmbar_wait(empty_b + 8 * s, par, abort_flag, true)) { failed = true; break; }
+            if (jb >= NB && !pmbar_wait(empty_b + 8 * s, par, abort_flag, !PAIR)) { failed = true; break; }
             const uint32_t fb = full_b + 8 * s;
-            pmbar_expect_tx(fb, (uint32_t)(c.bn * BK * 2));
             // (a box that starts at or beyond the last token is all zeros: the tensor map ends at M)
-            tma_box2(sbase + B_RING + s * B_BYTES, &c.xmap, xcol, (tt * c.nh + h) * c.bn, fb);
-            if (++s == BSLOTS) { s = 0; par ^= 1; }
+            if (PAIR) {
+              // (both blocks' halves count on the first block's barrier, which it arms with the bytes of both)
+              if (crank == 0) pmbar_expect_tx(fb, (uint32_t)(c.bn * BK * 2));
+              tma_box2_pair(sbase + B_RING + s * NB_BYTES, &c.xmap, xcol, (tt * c.nh + h) * c.bn + (int)crank * (c.bn / 2), ppeer_addr(fb, 0u));
+            } else {
+              pmbar_expect_tx(fb, (uint32_t)(c.bn * BK * 2));
+              tma_box2(sbase + B_RING + s * NB_BYTES, &c.xmap, xcol, (tt * c.nh + h) * c.bn, fb);
+            }
+            if (++s == NB) { s = 0; par ^= 1; }
           }
         }
       }
+      if (failed)                           // copies may still be on their way into this block's shared memory: they land well
+        for (int i = 0; i < 1000; ++i) __nanosleep(200);        // within this time
     }
   } else if (warp == 1) {
     // ===================================================================== MMA issue
     // (the whole warp walks the loop, so that stage indexes, parities and descriptors are warp-uniform; one elected
     //  lane issues)
-    {
+    if (!PAIR || crank == 0) {
+      auto commit = [](uint32_t bar) { if (PAIR) umma_commit_pair(bar); else umma_commit(bar); };
       int s = 0; uint32_t par = 0; int tcount = 0;         // weight stage and its parity
       int sb = 0; uint32_t parb = 0;                       // activation box slot and its parity
-      SegIter si; si.init(c, blockIdx.x, gridDim.x);
+      SegIter si; si.init(c, bid, nblk);
       Seg sg;
       for (; !failed && si.next(sg); ++tcount) {
         // A tile of one box alternates between the two accumulators; a tile of two boxes holds both: the
@@ -498,16 +529,19 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
             if (!CONV && !pmbar_wait_warp(full_b + 8 * sb, parb, abort_flag)) { failed = true; break; }
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)((acc0 + h) * MAXBN);
-            const uint64_t bdesc = smem_desc_sw128(sbase + B_RING + sb * B_BYTES);
+            const uint64_t bdesc = smem_desc_sw128(sbase + B_RING + sb * NB_BYTES);
             if (elect_one()) {
 #pragma unroll
-              for (int k16 = 0; k16 < BK / 16; ++k16)     // 32 bytes along K per MMA: +2 in the address field
-                umma_f16(d_tmem, adesc + 2 * k16, bdesc + 2 * k16, c.idesc, (kb > sg.kb0 || k16 > 0) ? 1u : 0u);
-              umma_commit(empty_b + 8 * sb);              // the box is free once these MMAs have read it
-              if (h == h_hi - 1) umma_commit(empty_a + 8 * s);   // ... and the weight stage after the last of them
+              for (int k16 = 0; k16 < BK / 16; ++k16) {   // 32 bytes along K per MMA: +2 in the address field
+                const uint32_t more = (kb > sg.kb0 || k16 > 0) ? 1u : 0u;
+                if (PAIR) umma_f16_pair(d_tmem, adesc + 2 * k16, bdesc + 2 * k16, c.idesc, more);
+                else umma_f16(d_tmem, adesc + 2 * k16, bdesc + 2 * k16, c.idesc, more);
+              }
+              commit(empty_b + 8 * sb);                   // the box is free once these MMAs have read it
+              if (h == h_hi - 1) commit(empty_a + 8 * s); // ... and the weight stage after the last of them
             }
             __syncwarp();
-            if (++sb == BSLOTS) { sb = 0; parb ^= 1; }
+            if (++sb == NB) { sb = 0; parb ^= 1; }
           }
           if (failed) break;
           if (++s == PSTAGES) { s = 0; par ^= 1; }
@@ -520,8 +554,8 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
         Seg nxt;
         const bool last = !peek.next(nxt);
         if (elect_one()) {
-          for (int h = h_lo; h < h_hi; ++h) umma_commit(acc_full + 8 * (acc0 + h));
-          if (last) umma_commit(last_full);
+          for (int h = h_lo; h < h_hi; ++h) commit(acc_full + 8 * (acc0 + h));
+          if (last) commit(last_full);
         }
         __syncwarp();
       }
@@ -557,7 +591,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     const int G = p.K / kGroup;
     int done = 0;                      // stage iterations before this segment
     constexpr bool heads = HEADS;
-    SegIter si; si.init(c, blockIdx.x, gridDim.x);
+    SegIter si; si.init(c, bid, nblk);
     Seg sg;
     for (; !failed && si.next(sg); done += sg.kb1 - sg.kb0) {
       const int it0 = done - sg.kb0;   // stage iteration of k-block kb of this segment = it0 + kb
@@ -574,7 +608,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
       for (int m = 0; m < 2; ++m) {
         const int item = dt + m * TEAM_TH;
         const int r = (item >> 1) & (BMW - 1), hf = item & 1;
-        const RowInfo ri = tile_row(jb, wt - c.wtile_begin[jn], r);
+        const RowInfo ri = tile_row(jb, local_tile(wt, jn), r);
         live[m] = m < n_items && ri.stored >= 0;
         const JobDev& src = (jb.pair == 1 && (r & 1)) ? p.job[jn + 1] : jb;    // odd rows of a SwiGLU pair: the up matrix
         wrow[m] = src.w + (size_t)(live[m] ? ri.stored : 0) * (p.K / 2) + hf * 16;
@@ -654,7 +688,9 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
         }
         fence_async_smem();            // generic-proxy writes must be visible to the tensor core (async proxy)
         __syncwarp();
-        if (lane == 0) pmbar_arrive(full_a + 8 * s);
+        if (lane == 0) {
+          if (PAIR && crank != 0) pmbar_signal_peer(ppeer_addr(full_a + 8 * s, 0u)); else pmbar_arrive(full_a + 8 * s);
+        }
 #pragma unroll
         for (int m = 0; m < 2; ++m) { q0[m] = q1[m]; s0[m] = s1[m]; z0[m] = z1[m]; }
       }
@@ -664,7 +700,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     Seg last_sg = {0, 0, 0, -1};
     int n_seg = 0;
     {
-      SegIter sj; sj.init(c, blockIdx.x, gridDim.x);
+      SegIter sj; sj.init(c, bid, nblk);
       Seg sgj;
       while (sj.next(sgj)) { last_sg = sgj; ++n_seg; }
     }
@@ -679,7 +715,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     // ===================================================================== epilogue
     asm volatile("griddepcontrol.wait;" ::: "memory");     // positions, outputs and workspace: after the preceding kernel
     int tcount = 0;
-    SegIter si; si.init(c, blockIdx.x, gridDim.x);
+    SegIter si; si.init(c, bid, nblk);
     Seg sg;
     for (; !failed && si.next(sg); ++tcount) {
       // The block's last segment: nothing is left to overlap its epilogue with, and the sixteen de-quantiser warps
@@ -695,8 +731,14 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem_base, 512);
-  if (c.pair_split) {                   // neither block of a pair leaves while the other may still send to it
+  if (PAIR) {                           // (tensor memory of both blocks is given back together, after the last MMA)
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (warp == 1) tmem_dealloc_pair(tmem_base, 512);
+  } else if (warp == 1) {
+    tmem_dealloc(tmem_base, 512);
+  }
+  if (PAIR || c.pair_split) {                   // neither block of a pair leaves while the other may still send to it
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
@@ -729,10 +771,10 @@ int host_job_tiles(const JobDev& j) {
   return (j.k_out + BMW - 1) / BMW;
 }
 
-template <typename T, bool CONV, bool HEADS>
+template <typename T, bool CONV, bool HEADS, bool PAIR>
 int launch_pth(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stream) {
   const size_t smem = 1024 + (size_t)RING_BYTES + 512;
-  auto kern = prefill_kernel<T, CONV, HEADS>;
+  auto kern = prefill_kernel<T, CONV, HEADS, PAIR>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return UNIQL_ERR_CUDA;
   cudaLaunchConfig_t lc;
@@ -746,7 +788,7 @@ int launch_pth(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stre
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = attr;
   lc.numAttrs = opt(kOptPdl) ? 1 : 0;
-  if (c.pair_split) {
+  if (PAIR || c.pair_split) {
     // clusters of two, only when every pair can be resident at once; else the caller plans without them
     attr[lc.numAttrs].id = cudaLaunchAttributeClusterDimension;
     attr[lc.numAttrs].val.clusterDim.x = 2;
@@ -762,12 +804,43 @@ int launch_pth(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stre
     }
     if (n_clusters * 2 < grid) return UNIQL_ERR_UNSUPPORTED;
   }
-  if (cudaLaunchKernelEx(&lc, kern, p, c) != cudaSuccess) { cudaGetLastError(); return c.pair_split ? UNIQL_ERR_UNSUPPORTED : UNIQL_ERR_CUDA; }
+  if (cudaLaunchKernelEx(&lc, kern, p, c) != cudaSuccess) { cudaGetLastError(); return PAIR || c.pair_split ? UNIQL_ERR_UNSUPPORTED : UNIQL_ERR_CUDA; }
   return UNIQL_OK;
 }
-template <typename T, bool CONV>
+template <typename T, bool CONV, bool PAIR>
 int launch_pt(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stream) {
-  return c.km_period != 0 ? launch_pth<T, CONV, true>(p, c, grid, stream) : launch_pth<T, CONV, false>(p, c, grid, stream);
+  return c.km_period != 0 ? launch_pth<T, CONV, true, PAIR>(p, c, grid, stream) : launch_pth<T, CONV, false, PAIR>(p, c, grid, stream);
+}
+
+// Clusters of two blocks of the pair kernel that the device holds at once (asked once per device; the instances need the
+// same resources).
+int pair_capacity() {
+  static std::atomic<int> n[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int v = n[dev].load(std::memory_order_relaxed);
+  if (v != 0) return v - 1;
+  auto kern = prefill_kernel<__half, false, false, true>;
+  const size_t smem = 1024 + (size_t)RING_BYTES + 512;
+  cudaLaunchConfig_t lc;
+  memset(&lc, 0, sizeof(lc));
+  lc.gridDim = dim3((unsigned)(device_sms() / 2 * 2));
+  lc.blockDim = dim3(PTH);
+  lc.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  lc.attrs = attr;
+  lc.numAttrs = 1;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&v, kern, &lc) != cudaSuccess) {
+    cudaGetLastError();
+    v = 0;
+  }
+  if (v > device_sms() / 2) v = device_sms() / 2;
+  n[dev].store(v + 1);
+  return v;
 }
 
 }  // namespace
@@ -901,21 +974,34 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
   // Both tile widths are costed with these figures and the cheaper one runs: wide tiles win where they still fill
   // the SMs (Qwen2.5-7B gate at M = 512..4096: 17-22 % faster), narrow ones where wide tiles would leave most SMs
   // without a tile (q / o projections at M = 512) or push a few left-over tiles into a round of their own.
-  int g2 = sms;
-  if (env_grid >= 1 && env_grid <= sms) g2 = env_grid;            // tests: odd splits on small problems
+  int g1 = sms;
+  if (env_grid >= 1 && env_grid <= sms) g1 = env_grid;            // tests: odd splits on small problems
   bool any_rope = false;
   for (int j = 0; j < p.n_jobs; ++j) any_rope = any_rope || p.job[j].rope.enabled != 0;
-  struct Plan { int nh, ttiles, tiles, left; bool streamk, atomic, halves, pair; size_t sums; double us; };
+  // Block pairs (cta_group::2): tiles of 256 rows, a cluster of two blocks where the other plans have one block.
+  const int opt_pair = opt(kOptPrefillPair);
+  int wt2 = 0, gp = 0;
+  // (options that steer the one-block plans, forced by tests, keep the pairs out unless they are forced too)
+  const bool pair_auto = opt_pair < 0 && env_grid == 0 && env_streamk <= 0 && opt(kOptPrefillDual) <= 0;
+  if (c.bn == MAXBN && !conv_in_kernel && (pair_auto || opt_pair >= 1)) {
+    for (int j = 0; j < p.n_jobs; ++j) wt2 += (host_job_tiles(p.job[j]) + 1) / 2;
+    gp = pair_capacity();
+    if (env_grid >= 1 && env_grid < gp) gp = env_grid;
+  }
+  struct Plan { int nh, ttiles, tiles, left, g; bool streamk, atomic, halves, pair, cg2; size_t sums; double us; };
   static std::atomic<bool> pair_refused{false};       // a cluster launch was refused once: planned without from then on
-  auto plan_for = [&](int nh) {
+  auto plan_for = [&](int nh, bool cg2) {
     Plan q;
     q.nh = nh;
+    q.cg2 = cg2;
+    const int g2 = cg2 ? gp : g1;
+    q.g = g2;
     const int ntok = c.bn * nh;
     q.ttiles = (p.M + ntok - 1) / ntok;
-    const long tiles = (long)wt * q.ttiles;
+    const long tiles = (long)(cg2 ? wt2 : wt) * q.ttiles;
     q.tiles = tiles <= (1 << 24) ? (int)tiles : (1 << 24);
     q.left = q.tiles % g2;
-    const double kcost = nh == 2 ? 1.07 : 0.65;
+    const double kcost = cg2 ? (nh == 2 ? 0.62 : 0.36) : (nh == 2 ? 1.07 : 0.65);
     const double wide = ntok / 256.0;
     // blocks on the split tile with the most of them: its finishing block reads that many slots back
     const long units = (long)q.left * c.n_kb;
@@ -924,7 +1010,7 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     double hand_over;
     q.atomic = false;
     // a k-block of a one-box tile by the number of busy SMs (0.45 us with 28 of them, 0.61 us with all)
-    auto kb1 = [&](int busy) { return 0.42 + 0.19 * (busy < g2 ? busy : g2) / g2; };
+    auto kb1 = [&](int busy) { return cg2 ? 0.34 : 0.42 + 0.19 * (busy < g2 ? busy : g2) / g2; };
     if (q.tiles < g2) {
       // every tile is split and every block ends on a split tile: the hand-over is shared with the de-quantiser warps
       // (one-box tiles, measured at M = 64 .. 512 on seven layer shapes: 5 us per 64 tokens of the tile)
@@ -952,26 +1038,29 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     const int rounds = (q.tiles + g2 - 1) / g2;
     double us_whole = (double)rounds * c.n_kb * kcost;
     if (nh == 1 && q.tiles <= g2) us_whole = c.n_kb * kb1(q.tiles);
-    if (nh == 2)
+    if (nh == 2 && cg2)
+      us_whole = (double)rounds * (c.n_kb * 0.62 + 10.0);
+    else if (nh == 2)
       us_whole = (double)(q.tiles / g2) * c.n_kb * 0.96 + (q.left ? c.n_kb * (0.90 + 0.06 * q.left / g2) : 0.0) + 10.0 * (rounds - 1);
     // one fp32 slot per (left-over tile, block) piece, or one sum per left-over tile
-    q.sums = (size_t)(q.atomic ? q.left : q.left + g2) * ntok * BMW * 4;
+    q.sums = (size_t)(q.atomic ? q.left : q.left + g2) * ntok * BMW * 4 * (cg2 ? 2 : 1);
     const bool want = env_streamk >= 0 ? (env_streamk >= 1) : (q.left != 0 && us_split < us_whole);
-    q.streamk = want && q.left != 0 && cfg.ws_bytes >= ws_used + q.sums && q.tiles <= (1 << 16);
+    q.streamk = want && q.left != 0 && cfg.ws_bytes >= ws_used + q.sums && q.tiles <= (1 << 15);
     q.us = q.streamk ? us_split : us_whole;
     // Tiles of two boxes left over after the whole rounds, when they are few: each runs as two half tiles (one box,
     // 256 tokens) on two blocks, a block's last segment -- no hand-over, and the round takes a one-box tile's time
     // (0.45 - 0.6 us per k-block by the number of busy SMs) instead of a two-box tile's on a few SMs.
     q.halves = false;
     if (nh == 2 && q.left != 0 && 2 * q.left <= g2 && q.tiles > g2 && !conv_in_kernel && env_streamk < 1 && opt(kOptPrefillDual) != 2) {
-      const double us_halves = (double)(q.tiles / g2) * (c.n_kb * 0.96 + 10.0) + c.n_kb * (0.45 + 0.15 * 2 * q.left / g2);
+      const double us_halves = cg2 ? (double)(q.tiles / g2) * (c.n_kb * 0.62 + 10.0) + c.n_kb * 0.34
+                                   : (double)(q.tiles / g2) * (c.n_kb * 0.96 + 10.0) + c.n_kb * (0.45 + 0.15 * 2 * q.left / g2);
       if (us_halves < q.us || opt(kOptPrefillDual) == 3) { q.halves = true; q.streamk = false; q.us = us_halves; }
     }
     // Few tiles of one box (at most one for every two SMs): a cluster of two blocks per tile, half of the
     // contraction each, the second block's sums handed over through the first one's shared memory (about 5 us
     // against the 11 - 28 us of a hand-over through the workspace; a k-block takes the same 0.5 - 0.65 us).
     q.pair = false;
-    if (nh == 1 && 2 * q.tiles <= sms && c.n_kb >= 4 && env_grid == 0 && !pair_refused.load() && (env_streamk < 0 || env_streamk == 3)) {
+    if (nh == 1 && !cg2 && 2 * q.tiles <= sms && c.n_kb >= 4 && env_grid == 0 && !pair_refused.load() && (env_streamk < 0 || env_streamk == 3)) {
       const double us_pair = (double)(c.n_kb - c.n_kb / 2) * kb1(2 * q.tiles) + 1.0 + 4.5 * wide + (any_rope ? 3.0 : 0.0);
       // (against a split over all SMs it has to be 10 % ahead: with long contractions the two come out level and
       //  the split measured ahead, Qwen2.5-7B down projection at M = 512)
@@ -979,13 +1068,21 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     }
     return q;
   };
-  Plan pl = plan_for(1);
+  Plan pl = plan_for(1, false);
   {
     // -1: by cost, 0: never, 1: wherever M > 256; tests: 2 the same without half tiles, 3 with them wherever they fit
     const int dual = opt(kOptPrefillDual);
     if (p.M > MAXBN && dual != 0) {
-      const Plan p2 = plan_for(2);
+      const Plan p2 = plan_for(2, false);
       if (dual >= 1 || p2.us < pl.us) pl = p2;
+    }
+    if (gp >= 1 && env_streamk != 3) {
+      // (tests: 1 / 2 force pairs with one or two boxes per tile)
+      for (int nh = 1; nh <= 2; ++nh) {
+        if ((nh == 2 && (p.M <= MAXBN || dual == 0)) || (nh == 1 && p.M > MAXBN && dual >= 1)) continue;
+        const Plan q = plan_for(nh, true);
+        if (opt_pair == nh || (opt_pair < 0 && (q.us < pl.us))) pl = q;
+      }
     }
   }
   c.helpers = opt(kOptPrefillHelpers) != 0;
@@ -994,15 +1091,21 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
   c.pair_split = pl.pair ? 1 : 0;
   c.n_ttiles = pl.ttiles;
   c.n_tiles = pl.tiles;
+  if (pl.cg2) {
+    int w = 0;
+    for (int j = 0; j < p.n_jobs; ++j) { c.wtile_begin[j] = w; w += (host_job_tiles(p.job[j]) + 1) / 2; }
+    for (int j = p.n_jobs; j <= kMaxPJobs; ++j) c.wtile_begin[j] = w;
+    c.idesc = (c.idesc & ~(0x1fu << 24)) | ((uint32_t)((2 * BMW) >> 4) << 24);       // 256 rows
+  }
   if ((long)wt * pl.ttiles > (1 << 24)) return UNIQL_ERR_SHAPE;
-  int grid = c.n_tiles < g2 ? c.n_tiles : g2;
+  int grid = c.n_tiles < pl.g ? c.n_tiles : pl.g;
   if (pl.pair) grid = 2 * c.n_tiles;
   {
     if (pl.streamk) {
       c.streamk = 1;
       c.sk_atomic = pl.atomic ? 1 : 0;
       c.partials = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(cfg.workspace) + ws_used);
-      grid = g2;
+      grid = pl.g;
       // (slots are written before they are read; sums start at zero)
       if (pl.atomic && cudaMemsetAsync(c.partials, 0, pl.sums, cfg.stream) != cudaSuccess) return UNIQL_ERR_CUDA;
     }
@@ -1011,13 +1114,16 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
       if (rc != UNIQL_OK) return rc;
     }
   }
-  int rc = encode_x_map(&c.xmap, xsrc, p.k_in, p.M, ldxs, c.bn, conv_in_kernel);
+  if (pl.cg2) grid *= 2;
+  int rc = encode_x_map(&c.xmap, xsrc, p.k_in, p.M, ldxs, pl.cg2 ? c.bn / 2 : c.bn, conv_in_kernel);
   if (rc != UNIQL_OK) return rc;
-  if (p.dt == UNIQL_BF16)
-    rc = conv_in_kernel ? launch_pt<__nv_bfloat16, true>(p, c, grid, cfg.stream)
-                        : launch_pt<__nv_bfloat16, false>(p, c, grid, cfg.stream);
+  if (pl.cg2)
+    rc = p.dt == UNIQL_BF16 ? launch_pt<__nv_bfloat16, false, true>(p, c, grid, cfg.stream) : launch_pt<__half, false, true>(p, c, grid, cfg.stream);
+  else if (p.dt == UNIQL_BF16)
+    rc = conv_in_kernel ? launch_pt<__nv_bfloat16, true, false>(p, c, grid, cfg.stream)
+                        : launch_pt<__nv_bfloat16, false, false>(p, c, grid, cfg.stream);
   else
-    rc = launch_pt<__half, false>(p, c, grid, cfg.stream);
+    rc = launch_pt<__half, false, false>(p, c, grid, cfg.stream);
   if (rc == UNIQL_ERR_UNSUPPORTED && c.pair_split) {
     // the pairs cannot all be resident (or clusters cannot be launched here): planned again without them
     pair_refused.store(true);
