@@ -56,11 +56,11 @@ namespace {
 constexpr int MAXBN = 256;          // tokens per tile (MMA N), at most
 constexpr int PSTAGES = 4;                   // ring of de-quantised weight stages (one k-block each)
 constexpr int BSLOTS = 4;                    // ring of activation boxes (one k-block of MAXBN tokens each)
-constexpr int BSLOTS2 = 8;                   // ... of half boxes (block pairs: each block holds half of the tokens)
+constexpr int PSTAGES2 = 4, BSLOTS2 = 8;     // block pairs: weight stages, and half boxes (each block holds half of the tokens)
 constexpr int A_BYTES = BMW * BK * 2;        // 16 KB
 constexpr int B_BYTES = MAXBN * BK * 2;      // 32 KB
 constexpr int RING_BYTES = PSTAGES * A_BYTES + BSLOTS * B_BYTES;
-constexpr int B_RING = PSTAGES * A_BYTES;    // the activation boxes follow the weight stages
+constexpr int RING2_BYTES = PSTAGES2 * A_BYTES + BSLOTS2 * B_BYTES / 2;
 constexpr int EPI_TOK = 32;                  // tokens per epilogue pass
 constexpr int NWARPS = 24;
 constexpr int PTH = NWARPS * 32;
@@ -222,8 +222,9 @@ __global__ void x_to_f16_kernel(const __nv_bfloat16* __restrict__ x, int ldx, in
 // PAIR: clusters of two blocks work on tiles of 256 weight rows with cta_group::2 MMAs.  Each block de-quantises 128 rows
 // into its own shared memory and fetches half of the tokens' boxes; the first block's MMA warp issues for both.  A block's
 // shared memory then takes in 16 instead of 32 KB of activations per 256 tokens and k-block, which with one block per tile
-// was what L2 could not deliver and the shared-memory port could not take beside the operand reads.
-template <typename T, bool CONV, bool HEADS, bool PAIR>
+// was what L2 could not deliver and the shared-memory port could not take beside the operand reads.  PAIR = 1 / 2: one or
+// two boxes of 256 tokens per tile.
+template <typename T, bool CONV, bool HEADS, int PAIR>
 __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__ Params p,
                                                          const __grid_constant__ PrefillCfg c) {
   extern __shared__ unsigned char psmem_raw[];
@@ -239,21 +240,25 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
   constexpr int NB = PAIR ? BSLOTS2 : BSLOTS;               // slots of the activation ring and their size
   constexpr int NB_BYTES = PAIR ? B_BYTES / 2 : B_BYTES;
   const int bid = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x, nblk = PAIR ? (int)gridDim.x >> 1 : (int)gridDim.x;
-  const uint32_t bars = sbase + RING_BYTES;
-  const uint32_t full_a = bars, empty_a = bars + 8 * PSTAGES;
-  const uint32_t full_b = bars + 16 * PSTAGES, empty_b = full_b + 8 * NB;
+  constexpr int NA = PAIR ? PSTAGES2 : PSTAGES;             // weight stages
+  constexpr int RING = PAIR ? RING2_BYTES : RING_BYTES;
+  constexpr int B_RING = NA * A_BYTES;                      // the activation boxes follow the weight stages
+  constexpr int TEAM_WARPS = PAIR == 1 ? DQ_WARPS : DQ_TEAM_WARPS;
+  const uint32_t bars = sbase + RING;
+  const uint32_t full_a = bars, empty_a = bars + 8 * NA;
+  const uint32_t full_b = bars + 16 * NA, empty_b = full_b + 8 * NB;
   const uint32_t acc_full = full_b + 16 * NB, acc_empty = acc_full + 16, epi_bar = acc_full + 32;
   const uint32_t help_bar = acc_full + 40;         // the epilogue warps and the de-quantiser warps that help them
   const uint32_t last_full = acc_full + 48;        // the MMAs of the block's last segment are complete (one phase only)
   const uint32_t px_ready = acc_full + 56;         // pair split, second block: the first block's rings are idle
   const uint32_t px_done = acc_full + 64;          // pair split, first block: the second block's sums have arrived
-  unsigned char* misc = smem + RING_BYTES + 16 * PSTAGES + 16 * NB + 72;
+  unsigned char* misc = smem + RING + 16 * NA + 16 * NB + 72;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
 
   if (tid == 0) {
-    for (int s = 0; s < PSTAGES; ++s) {
-      pmbar_init(full_a + 8 * s, PAIR ? 2 * DQ_TEAM_WARPS : DQ_TEAM_WARPS);
+    for (int s = 0; s < NA; ++s) {
+      pmbar_init(full_a + 8 * s, PAIR ? 2 * TEAM_WARPS : TEAM_WARPS);
       pmbar_init(empty_a + 8 * s, 1);
     }
     for (int s = 0; s < NB; ++s) {
@@ -544,7 +549,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
             if (++sb == NB) { sb = 0; parb ^= 1; }
           }
           if (failed) break;
-          if (++s == PSTAGES) { s = 0; par ^= 1; }
+          if (++s == NA) { s = 0; par ^= 1; }
         }
         if (failed) break;
         // (the de-quantiser warps that help with the last segment's epilogue cannot follow the phases of the
@@ -582,12 +587,15 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     // gate at M = 2048 296 -> 266 us with tiles of 256 tokens, 251 -> 232 us with 512).  The four warps 9, 13, 17,
     // 21 only help with the block's last epilogue (below).
     const int sc = warp & 3;
-    if (sc != 1) {
-    const int pos = ((warp - DQ_WARP0) >> 2) * 3 + (sc == 0 ? 0 : sc - 1);      // 0..11 among the twelve
-    const int team = pos / DQ_TEAM_WARPS;
-    const int dt = (pos - team * DQ_TEAM_WARPS) * 32 + lane;                    // 0..191
-    constexpr int TEAM_TH = DQ_TEAM_WARPS * 32;
-    const int n_items = dt + TEAM_TH < 2 * BMW ? 2 : 1;                         // items dt and dt + 192 of 256
+    // Pairs with one box per tile: all sixteen warps, two teams of eight with one item per thread.  (The MMA lane of a pair
+    // has half as much to issue per k-block, and a k-block half the time: with twelve warps a team's two rounds of items,
+    // 1130 cycles, set the pace.  With two boxes per tile the twelve are 4 % faster there too.)
+    if (TEAM_WARPS == DQ_WARPS || sc != 1) {
+    const int pos = TEAM_WARPS == DQ_WARPS ? warp - DQ_WARP0 : ((warp - DQ_WARP0) >> 2) * 3 + (sc == 0 ? 0 : sc - 1);   // among the sixteen or twelve
+    const int team = pos >= TEAM_WARPS ? 1 : 0;
+    const int dt = (pos - team * TEAM_WARPS) * 32 + lane;                       // 0..191 or 0..255
+    constexpr int TEAM_TH = TEAM_WARPS * 32;
+    const int n_items = PAIR == 1 ? 1 : dt + TEAM_TH < 2 * BMW ? 2 : 1;                         // items dt and dt + 192 of 256
     const int G = p.K / kGroup;
     int done = 0;                      // stage iterations before this segment
     constexpr bool heads = HEADS;
@@ -606,6 +614,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
       int hf_of[2], r7[2];
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
+        if (PAIR == 1 && m > 0) { live[m] = false; wrow[m] = nullptr; srow[m] = zrow[m] = nullptr; st_off[m] = 0; hf_of[m] = r7[m] = 0; break; }
         const int item = dt + m * TEAM_TH;
         const int r = (item >> 1) & (BMW - 1), hf = item & 1;
         const RowInfo ri = tile_row(jb, local_tile(wt, jn), r);
@@ -641,8 +650,8 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
       }
       for (int kb = kb0; kb < sg.kb1; kb += 2) {
         const int it = it0 + kb;
-        const int s = it & (PSTAGES - 1);
-        const uint32_t use = (uint32_t)(it / PSTAGES);
+        const int s = it % NA;
+        const uint32_t use = (uint32_t)(it / NA);
         uint4 q1[2];
         __half s1[2], z1[2];
         const bool more = kb + 2 < sg.kb1;
@@ -654,7 +663,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
           q1[m] = make_uint4(0, 0, 0, 0); s1[m] = s0[m]; z1[m] = z0[m];
           if (live[m] && more) fetch(m, st1, q1[m], s1[m], z1[m]);
         }
-        if (it >= PSTAGES && !pmbar_wait(empty_a + 8 * s, (use - 1) & 1, abort_flag)) { failed = true; break; }
+        if (it >= NA && !pmbar_wait(empty_a + 8 * s, (use - 1) & 1, abort_flag)) { failed = true; break; }
 #pragma unroll
         for (int m = 0; m < 2; ++m) {
           if (m >= n_items) break;
@@ -771,9 +780,9 @@ int host_job_tiles(const JobDev& j) {
   return (j.k_out + BMW - 1) / BMW;
 }
 
-template <typename T, bool CONV, bool HEADS, bool PAIR>
+template <typename T, bool CONV, bool HEADS, int PAIR>
 int launch_pth(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stream) {
-  const size_t smem = 1024 + (size_t)RING_BYTES + 512;
+  const size_t smem = 1024 + (size_t)(PAIR ? RING2_BYTES : RING_BYTES) + 512;
   auto kern = prefill_kernel<T, CONV, HEADS, PAIR>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return UNIQL_ERR_CUDA;
@@ -807,7 +816,7 @@ int launch_pth(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stre
   if (cudaLaunchKernelEx(&lc, kern, p, c) != cudaSuccess) { cudaGetLastError(); return PAIR || c.pair_split ? UNIQL_ERR_UNSUPPORTED : UNIQL_ERR_CUDA; }
   return UNIQL_OK;
 }
-template <typename T, bool CONV, bool PAIR>
+template <typename T, bool CONV, int PAIR>
 int launch_pt(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stream) {
   return c.km_period != 0 ? launch_pth<T, CONV, true, PAIR>(p, c, grid, stream) : launch_pth<T, CONV, false, PAIR>(p, c, grid, stream);
 }
@@ -820,8 +829,8 @@ int pair_capacity() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   int v = n[dev].load(std::memory_order_relaxed);
   if (v != 0) return v - 1;
-  auto kern = prefill_kernel<__half, false, false, true>;
-  const size_t smem = 1024 + (size_t)RING_BYTES + 512;
+  auto kern = prefill_kernel<__half, false, false, 1>;
+  const size_t smem = 1024 + (size_t)RING2_BYTES + 512;
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
   lc.gridDim = dim3((unsigned)(device_sms() / 2 * 2));
@@ -1117,13 +1126,15 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
   if (pl.cg2) grid *= 2;
   int rc = encode_x_map(&c.xmap, xsrc, p.k_in, p.M, ldxs, pl.cg2 ? c.bn / 2 : c.bn, conv_in_kernel);
   if (rc != UNIQL_OK) return rc;
-  if (pl.cg2)
-    rc = p.dt == UNIQL_BF16 ? launch_pt<__nv_bfloat16, false, true>(p, c, grid, cfg.stream) : launch_pt<__half, false, true>(p, c, grid, cfg.stream);
-  else if (p.dt == UNIQL_BF16)
-    rc = conv_in_kernel ? launch_pt<__nv_bfloat16, true, false>(p, c, grid, cfg.stream)
-                        : launch_pt<__nv_bfloat16, false, false>(p, c, grid, cfg.stream);
+  if (p.dt == UNIQL_BF16)
+    rc = conv_in_kernel ? launch_pt<__nv_bfloat16, true, 0>(p, c, grid, cfg.stream)
+         : !pl.cg2      ? launch_pt<__nv_bfloat16, false, 0>(p, c, grid, cfg.stream)
+         : c.nh == 1    ? launch_pt<__nv_bfloat16, false, 1>(p, c, grid, cfg.stream)
+                        : launch_pt<__nv_bfloat16, false, 2>(p, c, grid, cfg.stream);
   else
-    rc = launch_pt<__half, false, false>(p, c, grid, cfg.stream);
+    rc = !pl.cg2     ? launch_pt<__half, false, 0>(p, c, grid, cfg.stream)
+         : c.nh == 1 ? launch_pt<__half, false, 1>(p, c, grid, cfg.stream)
+                     : launch_pt<__half, false, 2>(p, c, grid, cfg.stream);
   if (rc == UNIQL_ERR_UNSUPPORTED && c.pair_split) {
     // the pairs cannot all be resident (or clusters cannot be launched here): planned again without them
     pair_refused.store(true);
