@@ -57,10 +57,12 @@ constexpr int MAXBN = 256;          // tokens per tile (MMA N), at most
 constexpr int PSTAGES = 4;                   // ring of de-quantised weight stages (one k-block each)
 constexpr int BSLOTS = 4;                    // ring of activation boxes (one k-block of MAXBN tokens each)
 constexpr int PSTAGES2 = 4, BSLOTS2 = 8;     // block pairs: weight stages, and half boxes (each block holds half of the tokens)
+constexpr int PSTAGES1 = 6;                  // ... with one box per tile: stages of weights and a half box, one pair of barriers
 constexpr int A_BYTES = BMW * BK * 2;        // 16 KB
 constexpr int B_BYTES = MAXBN * BK * 2;      // 32 KB
 constexpr int RING_BYTES = PSTAGES * A_BYTES + BSLOTS * B_BYTES;
 constexpr int RING2_BYTES = PSTAGES2 * A_BYTES + BSLOTS2 * B_BYTES / 2;
+static_assert(PSTAGES1 * (A_BYTES + B_BYTES / 2) == RING2_BYTES, "the pair instances use the same shared memory");
 constexpr int EPI_TOK = 32;                  // tokens per epilogue pass
 constexpr int NWARPS = 24;
 constexpr int PTH = NWARPS * 32;
@@ -237,17 +239,19 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
   const uint32_t raw = (uint32_t)__cvta_generic_to_shared(psmem_raw);
   const uint32_t sbase = (raw + 1023u) & ~1023u;           // swizzled tiles need 1024-byte alignment
   unsigned char* smem = psmem_raw + (sbase - raw);
-  constexpr int NB = PAIR ? BSLOTS2 : BSLOTS;               // slots of the activation ring and their size
+  constexpr int NB = PAIR == 1 ? PSTAGES1 : PAIR ? BSLOTS2 : BSLOTS;               // slots of the activation ring and their size
   constexpr int NB_BYTES = PAIR ? B_BYTES / 2 : B_BYTES;
   const int bid = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x, nblk = PAIR ? (int)gridDim.x >> 1 : (int)gridDim.x;
-  constexpr int NA = PAIR ? PSTAGES2 : PSTAGES;             // weight stages
+  constexpr int NA = PAIR == 1 ? PSTAGES1 : PAIR ? PSTAGES2 : PSTAGES;             // weight stages
   constexpr int RING = PAIR ? RING2_BYTES : RING_BYTES;
   constexpr int B_RING = NA * A_BYTES;                      // the activation boxes follow the weight stages
   constexpr int TEAM_WARPS = PAIR == 1 ? DQ_WARPS : DQ_TEAM_WARPS;
   const uint32_t bars = sbase + RING;
   const uint32_t full_a = bars, empty_a = bars + 8 * NA;
-  const uint32_t full_b = bars + 16 * NA, empty_b = full_b + 8 * NB;
-  const uint32_t acc_full = full_b + 16 * NB, acc_empty = acc_full + 16, epi_bar = acc_full + 32;
+  // (PAIR == 1: a stage's weights and its half box share one pair of barriers -- the MMA warp's loop is one chain of
+  //  dependent instructions, 890 cycles per k-block with two waits and two commits where the MMAs take 512)
+  const uint32_t full_b = PAIR == 1 ? full_a : bars + 16 * NA, empty_b = PAIR == 1 ? empty_a : full_b + 8 * NB;
+  const uint32_t acc_full = bars + 16 * NA + 16 * NB, acc_empty = acc_full + 16, epi_bar = acc_full + 32;
   const uint32_t help_bar = acc_full + 40;         // the epilogue warps and the de-quantiser warps that help them
   const uint32_t last_full = acc_full + 48;        // the MMAs of the block's last segment are complete (one phase only)
   const uint32_t px_ready = acc_full + 56;         // pair split, second block: the first block's rings are idle
@@ -258,10 +262,10 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
 
   if (tid == 0) {
     for (int s = 0; s < NA; ++s) {
-      pmbar_init(full_a + 8 * s, PAIR ? 2 * TEAM_WARPS : TEAM_WARPS);
+      pmbar_init(full_a + 8 * s, PAIR ? 2 * TEAM_WARPS + (PAIR == 1 ? 1 : 0) : TEAM_WARPS);
       pmbar_init(empty_a + 8 * s, 1);
     }
-    for (int s = 0; s < NB; ++s) {
+    for (int s = 0; s < NB && PAIR != 1; ++s) {
       pmbar_init(full_b + 8 * s, 1);
       pmbar_init(empty_b + 8 * s, 1);
     }
@@ -531,19 +535,14 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
           for (int h = h_lo; h < h_hi; ++h) {
             if (kb == sg.kb0 && au >= 1 && !pmbar_wait_warp(acc_empty + 8 * (acc0 + h), (au - 1) & 1, abort_flag)) { failed = true; break; }
             // (bf16: the de-quantisers waited for the activation box themselves and converted it)
-            if (!CONV && !pmbar_wait_warp(full_b + 8 * sb, parb, abort_flag)) { failed = true; break; }
+            if (!CONV && PAIR != 1 && !pmbar_wait_warp(full_b + 8 * sb, parb, abort_flag)) { failed = true; break; }
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)((acc0 + h) * MAXBN);
             const uint64_t bdesc = smem_desc_sw128(sbase + B_RING + sb * NB_BYTES);
             if (elect_one()) {
-#pragma unroll
-              for (int k16 = 0; k16 < BK / 16; ++k16) {   // 32 bytes along K per MMA: +2 in the address field
-                const uint32_t more = (kb > sg.kb0 || k16 > 0) ? 1u : 0u;
-                if (PAIR) umma_f16_pair(d_tmem, adesc + 2 * k16, bdesc + 2 * k16, c.idesc, more);
-                else umma_f16(d_tmem, adesc + 2 * k16, bdesc + 2 * k16, c.idesc, more);
-              }
-              commit(empty_b + 8 * sb);                   // the box is free once these MMAs have read it
-              if (h == h_hi - 1) commit(empty_a + 8 * s); // ... and the weight stage after the last of them
+              umma_kblock<PAIR != 0>(d_tmem, adesc, bdesc, c.idesc, kb > sg.kb0 ? 1u : 0u);
+              if (PAIR != 1) commit(empty_b + 8 * sb);    // the box is free once these MMAs have read it
+              if (PAIR == 1 || h == h_hi - 1) commit(empty_a + 8 * s);   // ... and the weight stage after the last of them
             }
             __syncwarp();
             if (++sb == NB) { sb = 0; parb ^= 1; }
