@@ -56,12 +56,12 @@ namespace {
 constexpr int MAXBN = 256;          // tokens per tile (MMA N), at most
 constexpr int PSTAGES = 4;                   // ring of de-quantised weight stages (one k-block each)
 constexpr int BSLOTS = 4;                    // ring of activation boxes (one k-block of MAXBN tokens each)
-constexpr int PSTAGES2 = 4, BSLOTS2 = 8;     // block pairs: weight stages, and half boxes (each block holds half of the tokens)
-constexpr int PSTAGES1 = 6;                  // ... with one box per tile: stages of weights and a half box, one pair of barriers
+// block pairs: stages of weights and the k-block's half boxes (each block holds half of the tokens), one or two of them
+constexpr int PSTAGES1 = 6, PSTAGES2 = 4;
 constexpr int A_BYTES = BMW * BK * 2;        // 16 KB
 constexpr int B_BYTES = MAXBN * BK * 2;      // 32 KB
 constexpr int RING_BYTES = PSTAGES * A_BYTES + BSLOTS * B_BYTES;
-constexpr int RING2_BYTES = PSTAGES2 * A_BYTES + BSLOTS2 * B_BYTES / 2;
+constexpr int RING2_BYTES = PSTAGES2 * (A_BYTES + B_BYTES);
 static_assert(PSTAGES1 * (A_BYTES + B_BYTES / 2) == RING2_BYTES, "the pair instances use the same shared memory");
 constexpr int EPI_TOK = 32;                  // tokens per epilogue pass
 constexpr int NWARPS = 24;
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
   const uint32_t raw = (uint32_t)__cvta_generic_to_shared(psmem_raw);
   const uint32_t sbase = (raw + 1023u) & ~1023u;           // swizzled tiles need 1024-byte alignment
   unsigned char* smem = psmem_raw + (sbase - raw);
-  constexpr int NB = PAIR == 1 ? PSTAGES1 : PAIR ? BSLOTS2 : BSLOTS;               // slots of the activation ring and their size
+  constexpr int NB = PAIR == 1 ? PSTAGES1 : PAIR ? 2 * PSTAGES2 : BSLOTS;               // slots of the activation ring and their size
   constexpr int NB_BYTES = PAIR ? B_BYTES / 2 : B_BYTES;
   const int bid = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x, nblk = PAIR ? (int)gridDim.x >> 1 : (int)gridDim.x;
   constexpr int NA = PAIR == 1 ? PSTAGES1 : PAIR ? PSTAGES2 : PSTAGES;             // weight stages
@@ -248,9 +248,9 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
   constexpr int TEAM_WARPS = PAIR == 1 ? DQ_WARPS : DQ_TEAM_WARPS;
   const uint32_t bars = sbase + RING;
   const uint32_t full_a = bars, empty_a = bars + 8 * NA;
-  // (PAIR == 1: a stage's weights and its half box share one pair of barriers -- the MMA warp's loop is one chain of
-  //  dependent instructions, 890 cycles per k-block with two waits and two commits where the MMAs take 512)
-  const uint32_t full_b = PAIR == 1 ? full_a : bars + 16 * NA, empty_b = PAIR == 1 ? empty_a : full_b + 8 * NB;
+  // (PAIR: a stage's weights and its half boxes share one pair of barriers -- the MMA warp's loop is one chain of
+  //  dependent instructions, 890 cycles per k-block of one box with two waits and two commits where the MMAs take 512)
+  const uint32_t full_b = PAIR ? full_a : bars + 16 * NA, empty_b = PAIR ? empty_a : full_b + 8 * NB;
   const uint32_t acc_full = bars + 16 * NA + 16 * NB, acc_empty = acc_full + 16, epi_bar = acc_full + 32;
   const uint32_t help_bar = acc_full + 40;         // the epilogue warps and the de-quantiser warps that help them
   const uint32_t last_full = acc_full + 48;        // the MMAs of the block's last segment are complete (one phase only)
@@ -262,10 +262,10 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
 
   if (tid == 0) {
     for (int s = 0; s < NA; ++s) {
-      pmbar_init(full_a + 8 * s, PAIR ? 2 * TEAM_WARPS + (PAIR == 1 ? 1 : 0) : TEAM_WARPS);
+      pmbar_init(full_a + 8 * s, PAIR ? 2 * TEAM_WARPS + 1 : TEAM_WARPS);
       pmbar_init(empty_a + 8 * s, 1);
     }
-    for (int s = 0; s < NB && PAIR != 1; ++s) {
+    for (int s = 0; s < NB && !PAIR; ++s) {
       pmbar_init(full_b + 8 * s, 1);
       pmbar_init(empty_b + 8 * s, 1);
     }
@@ -480,7 +480,36 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
 
   if (warp == 0) {
     // ===================================================================== activations by TMA
-    if (lane == 0) {
+    if (PAIR) {
+      // (warp-uniform, as the MMA warp: one lane walking this loop took longer per k-block than the MMAs do)
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      constexpr int NH = PAIR == 1 ? 1 : 2;
+      const uint32_t rfull = ppeer_addr(full_a, 0u);       // both blocks' half boxes count on the first block's barriers
+      int s = 0, it = 0; uint32_t par = 1;
+      SegIter si; si.init(c, bid, nblk);
+      Seg sg;
+      while (!failed && si.next(sg)) {
+        const int n_box = NH == 1 || sg.half >= 0 ? 1 : 2;
+        const int y0 = ((sg.tile % c.n_ttiles) * NH + (NH == 2 && sg.half > 0 ? 1 : 0)) * MAXBN + (int)crank * (MAXBN / 2);
+        KWalk kw;
+        if (HEADS) kw.start(c, sg.kb0);
+        for (int kb = sg.kb0; kb < sg.kb1; ++kb, ++it) {
+          const int x = HEADS ? kw.xcol(c) : kb * BK;
+          if (HEADS) kw.step(c, 1);
+          if (it >= NA && !pmbar_wait_warp(empty_a + 8 * s, par, abort_flag)) { failed = true; break; }
+          if (elect_one()) {
+            if (crank == 0) pmbar_expect_tx(full_a + 8 * s, (uint32_t)(n_box * MAXBN * BK * 2));
+            const uint32_t dst = sbase + B_RING + s * NH * NB_BYTES;
+            tma_box2_pair(dst, &c.xmap, x, y0, rfull + 8 * s);
+            if (n_box == 2) tma_box2_pair(dst + NB_BYTES, &c.xmap, x, y0 + MAXBN, rfull + 8 * s);
+          }
+          __syncwarp();
+          if (++s == NA) { s = 0; par ^= 1; }
+        }
+      }
+      if (failed)                           // copies may still be on their way into this block's shared memory: they land well
+        for (int i = 0; i < 1000; ++i) __nanosleep(200);        // within this time
+    } else if (lane == 0) {
       asm volatile("griddepcontrol.wait;" ::: "memory");   // the activations may come from the preceding kernel
       int s = 0; uint32_t par = 1; int jb = 0;             // box slot, parity of its previous use, boxes so far
       SegIter si; si.init(c, bid, nblk);
@@ -494,17 +523,11 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
           if (HEADS) kw.step(c, 1);
           const int h_lo = sg.half < 0 ? 0 : sg.half, h_hi = sg.half < 0 ? c.nh : sg.half + 1;
           for (int h = h_lo; h < h_hi; ++h, ++jb) {
-            if (jb >= NB && !pmbar_wait(empty_b + 8 * s, par, abort_flag, !PAIR)) { failed = true; break; }
+            if (jb >= NB && !pmbar_wait(empty_b + 8 * s, par, abort_flag, true)) { failed = true; break; }
             const uint32_t fb = full_b + 8 * s;
             // (a box that starts at or beyond the last token is all zeros: the tensor map ends at M)
-            if (PAIR) {
-              // (both blocks' halves count on the first block's barrier, which it arms with the bytes of both)
-              if (crank == 0) pmbar_expect_tx(fb, (uint32_t)(c.bn * BK * 2));
-              tma_box2_pair(sbase + B_RING + s * NB_BYTES, &c.xmap, xcol, (tt * c.nh + h) * c.bn + (int)crank * (c.bn / 2), ppeer_addr(fb, 0u));
-            } else {
-              pmbar_expect_tx(fb, (uint32_t)(c.bn * BK * 2));
-              tma_box2(sbase + B_RING + s * NB_BYTES, &c.xmap, xcol, (tt * c.nh + h) * c.bn, fb);
-            }
+            pmbar_expect_tx(fb, (uint32_t)(c.bn * BK * 2));
+            tma_box2(sbase + B_RING + s * NB_BYTES, &c.xmap, xcol, (tt * c.nh + h) * c.bn, fb);
             if (++s == NB) { s = 0; par ^= 1; }
           }
         }
@@ -532,6 +555,33 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
         for (int kb = sg.kb0; kb < sg.kb1 && !failed; ++kb) {
           if (!pmbar_wait_warp(full_a + 8 * s, par, abort_flag)) { failed = true; break; }
           const uint64_t adesc = smem_desc_sw128(sbase + s * A_BYTES);
+          if (PAIR == 2) {
+            // (one wait and one commit per k-block; the same shape for one box measured 20 % slower than the loop below)
+            constexpr int NH = 2;
+            const uint64_t bdesc = smem_desc_sw128(sbase + B_RING + s * NH * NB_BYTES);
+            const uint32_t more = kb > sg.kb0 ? 1u : 0u;
+            const int n_box = h_hi - h_lo;
+            if (kb == sg.kb0 && au >= 1) {                // (the accumulators are still being drained: one after the other)
+              for (int h = 0; h < n_box; ++h) {
+                if (!pmbar_wait_warp(acc_empty + 8 * (acc0 + h_lo + h), (au - 1) & 1, abort_flag)) { failed = true; break; }
+                tc_fence_after();
+                if (elect_one()) umma_kblock<true>(tmem_base + (uint32_t)((acc0 + h_lo + h) * MAXBN), adesc, bdesc + h * (NB_BYTES >> 4), c.idesc, 0u);
+                __syncwarp();
+              }
+              if (failed) break;
+              if (elect_one()) umma_commit_pair(empty_a + 8 * s);
+            } else {
+              tc_fence_after();
+              if (elect_one()) {
+                umma_kblock<true>(tmem_base + (uint32_t)((acc0 + h_lo) * MAXBN), adesc, bdesc, c.idesc, more);
+                if (n_box == 2) umma_kblock<true>(tmem_base + (uint32_t)((acc0 + 1) * MAXBN), adesc, bdesc + (NB_BYTES >> 4), c.idesc, more);
+                umma_commit_pair(empty_a + 8 * s);        // the stage is free once these MMAs have read it
+              }
+            }
+            __syncwarp();
+            if (++s == NA) { s = 0; par ^= 1; }
+            continue;
+          }
           for (int h = h_lo; h < h_hi; ++h) {
             if (kb == sg.kb0 && au >= 1 && !pmbar_wait_warp(acc_empty + 8 * (acc0 + h), (au - 1) & 1, abort_flag)) { failed = true; break; }
             // (bf16: the de-quantisers waited for the activation box themselves and converted it)
