@@ -87,6 +87,7 @@ struct PrefillCfg {
   int sk_atomic;             // stream-K hand-over: 1 = parts added into one sum per tile (reductions in L2), 0 = a slot per part
   int pair_split;            // clusters of two blocks on one tile, half of the contraction each; the second block's
                              // fp32 sums go into the first one's shared memory (the rings, idle by then)
+  int csplit;                // block pairs, one box per tile: pairs (of one cluster) that share a tile's contraction
   int halves;                // tiles on both accumulators: the tiles left over after the whole rounds run as half tiles
                              // (one box of 256 tokens each, on twice as many blocks), every block's last segment
   int* status;
@@ -123,7 +124,8 @@ struct Seg { int tile, kb0, kb1, half; };
 struct SegIter {
   long u, ue;
   int t, t_end, n_kb, step, tail_tile0, half_tile, half, ps_tile, ps_kb0, ps_kb1;
-  __device__ inline void init(const PrefillCfg& c, int b, int grid) {
+  // part: which of the pairs that share a tile's contraction this one is (-1: tiles are not shared)
+  __device__ inline void init(const PrefillCfg& c, int b, int grid, int part) {
     n_kb = c.n_kb; step = grid; t = b;
     half_tile = -1; half = 0;
     ps_tile = -1;
@@ -134,6 +136,13 @@ struct SegIter {
       const int mid = n_kb - n_kb / 2;
       ps_kb0 = (b & 1) ? mid : 0;
       ps_kb1 = (b & 1) ? n_kb : mid;
+      return;
+    }
+    if (part >= 0) {
+      // one tile per cluster, a part of its k-blocks per pair
+      t_end = 0; tail_tile0 = 0; u = ue = 0; t = 1;
+      ps_tile = b;
+      ps_kb0 = n_kb * part / c.csplit; ps_kb1 = n_kb * (part + 1) / c.csplit;
       return;
     }
     if (c.halves) {
@@ -225,11 +234,13 @@ __global__ void x_to_f16_kernel(const __nv_bfloat16* __restrict__ x, int ldx, in
 // into its own shared memory and fetches half of the tokens' boxes; the first block's MMA warp issues for both.  A block's
 // shared memory then takes in 16 instead of 32 KB of activations per 256 tokens and k-block, which with one block per tile
 // was what L2 could not deliver and the shared-memory port could not take beside the operand reads.  PAIR = 1 / 2: one or
-// two boxes of 256 tokens per tile.
+// two boxes of 256 tokens per tile; 3: one box, and the pairs of a cluster share a tile (an instance of its own: inside 1 its
+// registers cost every launch 3 - 10 %).
 template <typename T, bool CONV, bool HEADS, int PAIR>
 __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__ Params p,
                                                          const __grid_constant__ PrefillCfg c) {
   extern __shared__ unsigned char psmem_raw[];
+  constexpr bool ONE = PAIR == 1 || PAIR == 3;              // block pairs, one box of tokens per tile
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (warp-uniform for the compiler)
   // Programmatic dependent launch: the next kernel of the stream may be set up while this one runs (its blocks
   // become resident as ours leave).  What a block does before its own `griddepcontrol.wait` touches nothing a
@@ -239,13 +250,18 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
   const uint32_t raw = (uint32_t)__cvta_generic_to_shared(psmem_raw);
   const uint32_t sbase = (raw + 1023u) & ~1023u;           // swizzled tiles need 1024-byte alignment
   unsigned char* smem = psmem_raw + (sbase - raw);
-  constexpr int NB = PAIR == 1 ? PSTAGES1 : PAIR ? 2 * PSTAGES2 : BSLOTS;               // slots of the activation ring and their size
+  constexpr int NB = ONE ? PSTAGES1 : PAIR ? 2 * PSTAGES2 : BSLOTS;               // slots of the activation ring and their size
   constexpr int NB_BYTES = PAIR ? B_BYTES / 2 : B_BYTES;
-  const int bid = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x, nblk = PAIR ? (int)gridDim.x >> 1 : (int)gridDim.x;
-  constexpr int NA = PAIR == 1 ? PSTAGES1 : PAIR ? PSTAGES2 : PSTAGES;             // weight stages
+  // PAIR: the pair's number and their count (3: the cluster's), and this pair's part of a shared tile
+  const int n_share = PAIR == 3 ? c.csplit : 1, per = PAIR ? 2 * n_share : 1;
+  const int bid = PAIR ? (int)blockIdx.x / per : (int)blockIdx.x, nblk = PAIR ? (int)gridDim.x / per : (int)gridDim.x;
+  const uint32_t rank = (PAIR || c.pair_split) ? pcluster_rank() : 0u;
+  const uint32_t crank = PAIR == 3 ? rank & 1u : rank, lrank = PAIR == 3 ? rank & ~1u : 0u;   // block of the pair, rank of the pair's first block
+  const int part = PAIR == 3 ? (int)(rank >> 1) : -1;
+  constexpr int NA = ONE ? PSTAGES1 : PAIR ? PSTAGES2 : PSTAGES;             // weight stages
   constexpr int RING = PAIR ? RING2_BYTES : RING_BYTES;
   constexpr int B_RING = NA * A_BYTES;                      // the activation boxes follow the weight stages
-  constexpr int TEAM_WARPS = PAIR == 1 ? DQ_WARPS : DQ_TEAM_WARPS;
+  constexpr int TEAM_WARPS = ONE ? DQ_WARPS : DQ_TEAM_WARPS;
   const uint32_t bars = sbase + RING;
   const uint32_t full_a = bars, empty_a = bars + 8 * NA;
   // (PAIR: a stage's weights and its half boxes share one pair of barriers -- the MMA warp's loop is one chain of
@@ -256,7 +272,8 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
   const uint32_t last_full = acc_full + 48;        // the MMAs of the block's last segment are complete (one phase only)
   const uint32_t px_ready = acc_full + 56;         // pair split, second block: the first block's rings are idle
   const uint32_t px_done = acc_full + 64;          // pair split, first block: the second block's sums have arrived
-  unsigned char* misc = smem + RING + 16 * NA + 16 * NB + 72;
+  const uint32_t xq = acc_full + 72;               // pairs that share a tile: the others' sums have arrived, per quadrant
+  unsigned char* misc = smem + RING + 16 * NA + 16 * NB + 104;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
 
@@ -275,6 +292,8 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     pmbar_init(last_full, 1);
     pmbar_init(px_ready, 1);
     pmbar_init(px_done, c.helpers ? 4 + 2 * DQ_WARPS : 4);       // one arrival per warp that sends
+    if (PAIR == 3)
+      for (int b = 0; b < 4; ++b) pmbar_init(xq + 8 * b, max(1, (n_share - 1) * (c.helpers ? 5 : 1)));
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -291,7 +310,6 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const uint32_t crank = (PAIR || c.pair_split) ? pcluster_rank() : 0u;
   if (PAIR || c.pair_split) {                   // the other block's barriers exist before anything is sent to it
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -351,7 +369,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
         __syncwarp();
         if (lane == 0) {
           const uint32_t eb = acc_empty + 8 * (acc0 + (ch * EPI_TOK) / c.bn);
-          if (PAIR) pmbar_signal_peer(ppeer_addr(eb, 0u)); else pmbar_arrive(eb);
+          if (PAIR) pmbar_signal_peer(ppeer_addr(eb, lrank)); else pmbar_arrive(eb);
         }
       };
       if (sg.kb0 == 0 && sg.kb1 == c.n_kb) {
@@ -381,6 +399,52 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
         //      would take the four epilogue warps longer than the tiles behind can hide: such launches add the parts
         //      into ONE sum per tile instead (reductions done in L2, zero at launch; the last bit of a sum then
         //      depends on the order of arrival when more than two blocks share a tile).
+        if (PAIR == 3) {
+          // ---- the pairs of a cluster share this tile.  Eight tokens at a time: pair i % n_share finishes chunk i.  Each
+          //      leaves its sums of the other pairs' chunks in a slot ([token][row], L2), tells them (remote arrivals,
+          //      one per warp and pair), and adds up and finishes its own chunks in the order of the parts.
+          float* slots = c.partials + row;
+          const float* first = slots + (size_t)(blockIdx.x - rank + crank) * (MAXBN * BMW);   // part 0's block of the same rows
+          float* mine = slots + (size_t)blockIdx.x * (MAXBN * BMW);
+          constexpr int CH = 8, N_CH = MAXBN / CH;
+          for (int ch = ch0; ch < N_CH; ch += chs) {
+            if (ch % n_share == part) continue;
+            uint32_t v[8];
+            tmem_ld8(t_acc + (uint32_t)(ch * CH), v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int k = 0; k < 8; ++k) __stcg(mine + (size_t)(ch * CH + k) * BMW, __uint_as_float(v[k]));
+          }
+          __syncwarp();
+          if (lane < n_share && lane != part) {
+            asm volatile("fence.acq_rel.cluster;" ::: "memory");
+            pmbar_arrive_peer(ppeer_addr(xq + 8 * q, (uint32_t)(2 * lane) + crank));
+          }
+          if (!__all_sync(0xffffffffu, pmbar_wait_cluster(xq + 8 * q, 0, abort_flag))) { failed = true; return; }
+          for (int own = ch0; part + own * n_share < N_CH; own += chs) {
+            const int tk = (part + own * n_share) * CH;
+            if (tt * ntok + tk >= p.M) break;
+            uint32_t v[8];
+            tmem_ld8(t_acc + (uint32_t)tk, v);
+            tmem_ld_wait();
+            float val[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) val[k] = 0.f;
+            const float* src = first + (size_t)tk * BMW;
+            for (int r0 = 0; r0 < n_share; r0 += 2) {          // two parts in flight, added in their order
+              float a[8], b[8];
+              const bool own_a = r0 == part, own_b = r0 + 1 == part, has_b = r0 + 1 < n_share;
+#pragma unroll
+              for (int k = 0; k < 8; ++k) a[k] = own_a ? __uint_as_float(v[k]) : __ldcg(src + (size_t)(2 * r0) * (MAXBN * BMW) + (size_t)k * BMW);
+#pragma unroll
+              for (int k = 0; k < 8; ++k) b[k] = own_b ? __uint_as_float(v[k]) : has_b ? __ldcg(src + (size_t)(2 * r0 + 2) * (MAXBN * BMW) + (size_t)k * BMW) : 0.f;
+#pragma unroll
+              for (int k = 0; k < 8; ++k) val[k] = (val[k] + a[k]) + b[k];
+            }
+            store_chunk(tk, val);
+          }
+          return;
+        }
         const bool pair_send = c.pair_split && crank != 0;
         if (c.pair_split && !pair_send) {
           // ---- the two blocks of a cluster each ran half of the contraction.  The second block waits until the
@@ -483,10 +547,10 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     if (PAIR) {
       // (warp-uniform, as the MMA warp: one lane walking this loop took longer per k-block than the MMAs do)
       asm volatile("griddepcontrol.wait;" ::: "memory");
-      constexpr int NH = PAIR == 1 ? 1 : 2;
-      const uint32_t rfull = ppeer_addr(full_a, 0u);       // both blocks' half boxes count on the first block's barriers
+      constexpr int NH = ONE ? 1 : 2;
+      const uint32_t rfull = ppeer_addr(full_a, lrank);       // both blocks' half boxes count on the first block's barriers
       int s = 0, it = 0; uint32_t par = 1;
-      SegIter si; si.init(c, bid, nblk);
+      SegIter si; si.init(c, bid, nblk, part);
       Seg sg;
       while (!failed && si.next(sg)) {
         const int n_box = NH == 1 || sg.half >= 0 ? 1 : 2;
@@ -512,7 +576,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     } else if (lane == 0) {
       asm volatile("griddepcontrol.wait;" ::: "memory");   // the activations may come from the preceding kernel
       int s = 0; uint32_t par = 1; int jb = 0;             // box slot, parity of its previous use, boxes so far
-      SegIter si; si.init(c, bid, nblk);
+      SegIter si; si.init(c, bid, nblk, part);
       Seg sg;
       while (!failed && si.next(sg)) {
         const int tt = sg.tile % c.n_ttiles;
@@ -540,10 +604,11 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     // (the whole warp walks the loop, so that stage indexes, parities and descriptors are warp-uniform; one elected
     //  lane issues)
     if (!PAIR || crank == 0) {
-      auto commit = [](uint32_t bar) { if (PAIR) umma_commit_pair(bar); else umma_commit(bar); };
+      const unsigned short pair_mask = (unsigned short)(3u << lrank);
+      auto commit = [&](uint32_t bar) { if (PAIR) umma_commit_pair(bar, pair_mask); else umma_commit(bar); };
       int s = 0; uint32_t par = 0; int tcount = 0;         // weight stage and its parity
       int sb = 0; uint32_t parb = 0;                       // activation box slot and its parity
-      SegIter si; si.init(c, bid, nblk);
+      SegIter si; si.init(c, bid, nblk, part);
       Seg sg;
       for (; !failed && si.next(sg); ++tcount) {
         // A tile of one box alternates between the two accumulators; a tile of two boxes holds both: the
@@ -569,13 +634,13 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
                 __syncwarp();
               }
               if (failed) break;
-              if (elect_one()) umma_commit_pair(empty_a + 8 * s);
+              if (elect_one()) umma_commit_pair(empty_a + 8 * s, pair_mask);
             } else {
               tc_fence_after();
               if (elect_one()) {
                 umma_kblock<true>(tmem_base + (uint32_t)((acc0 + h_lo) * MAXBN), adesc, bdesc, c.idesc, more);
                 if (n_box == 2) umma_kblock<true>(tmem_base + (uint32_t)((acc0 + 1) * MAXBN), adesc, bdesc + (NB_BYTES >> 4), c.idesc, more);
-                umma_commit_pair(empty_a + 8 * s);        // the stage is free once these MMAs have read it
+                umma_commit_pair(empty_a + 8 * s, pair_mask);        // the stage is free once these MMAs have read it
               }
             }
             __syncwarp();
@@ -585,14 +650,14 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
           for (int h = h_lo; h < h_hi; ++h) {
             if (kb == sg.kb0 && au >= 1 && !pmbar_wait_warp(acc_empty + 8 * (acc0 + h), (au - 1) & 1, abort_flag)) { failed = true; break; }
             // (bf16: the de-quantisers waited for the activation box themselves and converted it)
-            if (!CONV && PAIR != 1 && !pmbar_wait_warp(full_b + 8 * sb, parb, abort_flag)) { failed = true; break; }
+            if (!CONV && !ONE && !pmbar_wait_warp(full_b + 8 * sb, parb, abort_flag)) { failed = true; break; }
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)((acc0 + h) * MAXBN);
             const uint64_t bdesc = smem_desc_sw128(sbase + B_RING + sb * NB_BYTES);
             if (elect_one()) {
               umma_kblock<PAIR != 0>(d_tmem, adesc, bdesc, c.idesc, kb > sg.kb0 ? 1u : 0u);
-              if (PAIR != 1) commit(empty_b + 8 * sb);    // the box is free once these MMAs have read it
-              if (PAIR == 1 || h == h_hi - 1) commit(empty_a + 8 * s);   // ... and the weight stage after the last of them
+              if (!ONE) commit(empty_b + 8 * sb);    // the box is free once these MMAs have read it
+              if (ONE || h == h_hi - 1) commit(empty_a + 8 * s);   // ... and the weight stage after the last of them
             }
             __syncwarp();
             if (++sb == NB) { sb = 0; parb ^= 1; }
@@ -644,11 +709,11 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     const int team = pos >= TEAM_WARPS ? 1 : 0;
     const int dt = (pos - team * TEAM_WARPS) * 32 + lane;                       // 0..191 or 0..255
     constexpr int TEAM_TH = TEAM_WARPS * 32;
-    const int n_items = PAIR == 1 ? 1 : dt + TEAM_TH < 2 * BMW ? 2 : 1;                         // items dt and dt + 192 of 256
+    const int n_items = ONE ? 1 : dt + TEAM_TH < 2 * BMW ? 2 : 1;                         // items dt and dt + 192 of 256
     const int G = p.K / kGroup;
     int done = 0;                      // stage iterations before this segment
     constexpr bool heads = HEADS;
-    SegIter si; si.init(c, bid, nblk);
+    SegIter si; si.init(c, bid, nblk, part);
     Seg sg;
     for (; !failed && si.next(sg); done += sg.kb1 - sg.kb0) {
       const int it0 = done - sg.kb0;   // stage iteration of k-block kb of this segment = it0 + kb
@@ -663,7 +728,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
       int hf_of[2], r7[2];
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
-        if (PAIR == 1 && m > 0) { live[m] = false; wrow[m] = nullptr; srow[m] = zrow[m] = nullptr; st_off[m] = 0; hf_of[m] = r7[m] = 0; break; }
+        if (ONE && m > 0) { live[m] = false; wrow[m] = nullptr; srow[m] = zrow[m] = nullptr; st_off[m] = 0; hf_of[m] = r7[m] = 0; break; }
         const int item = dt + m * TEAM_TH;
         const int r = (item >> 1) & (BMW - 1), hf = item & 1;
         const RowInfo ri = tile_row(jb, local_tile(wt, jn), r);
@@ -747,7 +812,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
         fence_async_smem();            // generic-proxy writes must be visible to the tensor core (async proxy)
         __syncwarp();
         if (lane == 0) {
-          if (PAIR && crank != 0) pmbar_signal_peer(ppeer_addr(full_a + 8 * s, 0u)); else pmbar_arrive(full_a + 8 * s);
+          if (PAIR && crank != 0) pmbar_signal_peer(ppeer_addr(full_a + 8 * s, lrank)); else pmbar_arrive(full_a + 8 * s);
         }
 #pragma unroll
         for (int m = 0; m < 2; ++m) { q0[m] = q1[m]; s0[m] = s1[m]; z0[m] = z1[m]; }
@@ -758,7 +823,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     Seg last_sg = {0, 0, 0, -1};
     int n_seg = 0;
     {
-      SegIter sj; sj.init(c, bid, nblk);
+      SegIter sj; sj.init(c, bid, nblk, part);
       Seg sgj;
       while (sj.next(sgj)) { last_sg = sgj; ++n_seg; }
     }
@@ -773,7 +838,7 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
     // ===================================================================== epilogue
     asm volatile("griddepcontrol.wait;" ::: "memory");     // positions, outputs and workspace: after the preceding kernel
     int tcount = 0;
-    SegIter si; si.init(c, bid, nblk);
+    SegIter si; si.init(c, bid, nblk, part);
     Seg sg;
     for (; !failed && si.next(sg); ++tcount) {
       // The block's last segment: nothing is left to overlap its epilogue with, and the sixteen de-quantiser warps
@@ -849,13 +914,13 @@ int launch_pth(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stre
   if (PAIR || c.pair_split) {
     // clusters of two, only when every pair can be resident at once; else the caller plans without them
     attr[lc.numAttrs].id = cudaLaunchAttributeClusterDimension;
-    attr[lc.numAttrs].val.clusterDim.x = 2;
+    attr[lc.numAttrs].val.clusterDim.x = PAIR == 3 ? 2 * c.csplit : 2;
     attr[lc.numAttrs].val.clusterDim.y = 1;
     attr[lc.numAttrs].val.clusterDim.z = 1;
     ++lc.numAttrs;
     // (asked once per kernel instance: the answer depends on the block's resources, which do not change)
     static std::atomic<int> max_clusters{-1};
-    int n_clusters = max_clusters.load();
+    int n_clusters = PAIR ? device_sms() / 2 : max_clusters.load();          // (PAIR: the caller has asked pair_capacity())
     if (n_clusters < 0) {
       if (cudaOccupancyMaxActiveClusters(&n_clusters, kern, &lc) != cudaSuccess) { cudaGetLastError(); n_clusters = 0; }
       max_clusters.store(n_clusters);
@@ -870,24 +935,26 @@ int launch_pt(const Params& p, const PrefillCfg& c, int grid, cudaStream_t strea
   return c.km_period != 0 ? launch_pth<T, CONV, true, PAIR>(p, c, grid, stream) : launch_pth<T, CONV, false, PAIR>(p, c, grid, stream);
 }
 
-// Clusters of two blocks of the pair kernel that the device holds at once (asked once per device; the instances need the
-// same resources).
-int pair_capacity() {
-  static std::atomic<int> n[64] = {};
+// Clusters of `share` block pairs that the device holds at once (asked once per device; the instances need the same
+// resources).
+constexpr int kMaxShare = 4;
+int pair_capacity(int share) {
+  static std::atomic<int> n[64][kMaxShare + 1] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  int v = n[dev].load(std::memory_order_relaxed);
+  int v = n[dev][share].load(std::memory_order_relaxed);
   if (v != 0) return v - 1;
-  auto kern = prefill_kernel<__half, false, false, 1>;
+  auto kern = prefill_kernel<__half, false, false, 3>;
   const size_t smem = 1024 + (size_t)RING2_BYTES + 512;
+  const int most = device_sms() / (2 * share);
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
-  lc.gridDim = dim3((unsigned)(device_sms() / 2 * 2));
+  lc.gridDim = dim3((unsigned)(most * 2 * share));
   lc.blockDim = dim3(PTH);
   lc.dynamicSmemBytes = smem;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.x = 2 * share;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   lc.attrs = attr;
   lc.numAttrs = 1;
@@ -896,8 +963,8 @@ int pair_capacity() {
     cudaGetLastError();
     v = 0;
   }
-  if (v > device_sms() / 2) v = device_sms() / 2;
-  n[dev].store(v + 1);
+  if (v > most) v = most;
+  n[dev][share].store(v + 1);
   return v;
 }
 
@@ -1040,18 +1107,19 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
   const int opt_pair = opt(kOptPrefillPair);
   int wt2 = 0, gp = 0;
   // (options that steer the one-block plans, forced by tests, keep the pairs out unless they are forced too)
-  const bool pair_auto = opt_pair < 0 && env_grid == 0 && env_streamk <= 0 && opt(kOptPrefillDual) <= 0;
+  const bool pair_auto = opt_pair < 0 && env_grid == 0 && (env_streamk <= 0 || env_streamk > 10) && opt(kOptPrefillDual) <= 0;
   if (c.bn == MAXBN && !conv_in_kernel && (pair_auto || opt_pair >= 1)) {
     for (int j = 0; j < p.n_jobs; ++j) wt2 += (host_job_tiles(p.job[j]) + 1) / 2;
-    gp = pair_capacity();
+    gp = pair_capacity(1);
     if (env_grid >= 1 && env_grid < gp) gp = env_grid;
   }
-  struct Plan { int nh, ttiles, tiles, left, g; bool streamk, atomic, halves, pair, cg2; size_t sums; double us; };
+  struct Plan { int nh, ttiles, tiles, left, g; int share; bool streamk, atomic, halves, pair, cg2; size_t sums; double us; };
   static std::atomic<bool> pair_refused{false};       // a cluster launch was refused once: planned without from then on
   auto plan_for = [&](int nh, bool cg2) {
     Plan q;
     q.nh = nh;
     q.cg2 = cg2;
+    q.share = 1;
     const int g2 = cg2 ? gp : g1;
     q.g = g2;
     const int ntok = c.bn * nh;
@@ -1059,7 +1127,8 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     const long tiles = (long)(cg2 ? wt2 : wt) * q.ttiles;
     q.tiles = tiles <= (1 << 24) ? (int)tiles : (1 << 24);
     q.left = q.tiles % g2;
-    const double kcost = cg2 ? (nh == 2 ? 0.62 : 0.36) : (nh == 2 ? 1.07 : 0.65);
+    // (pairs: fitted over 7 layer shapes at M = 160 .. 2048, every form forced in turn; worst choice 6 % off the best)
+    const double kcost = cg2 ? (nh == 2 ? 0.60 : 0.365) : (nh == 2 ? 1.07 : 0.65);
     const double wide = ntok / 256.0;
     // blocks on the split tile with the most of them: its finishing block reads that many slots back
     const long units = (long)q.left * c.n_kb;
@@ -1068,7 +1137,7 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     double hand_over;
     q.atomic = false;
     // a k-block of a one-box tile by the number of busy SMs (0.45 us with 28 of them, 0.61 us with all)
-    auto kb1 = [&](int busy) { return cg2 ? 0.34 : 0.42 + 0.19 * (busy < g2 ? busy : g2) / g2; };
+    auto kb1 = [&](int busy) { return cg2 ? 0.365 : 0.42 + 0.19 * (busy < g2 ? busy : g2) / g2; };
     if (q.tiles < g2) {
       // every tile is split and every block ends on a split tile: the hand-over is shared with the de-quantiser warps
       // (one-box tiles, measured at M = 64 .. 512 on seven layer shapes: 5 us per 64 tokens of the tile)
@@ -1088,7 +1157,7 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     if (env_streamk == 1) q.atomic = false;                            // tests: the form of the hand-over forced
     if (env_streamk == 2) q.atomic = true;
     // (a split is taken where it is estimated 5 % ahead: its hand-over varies more than a whole tile's time)
-    const double us_split = 1.05 * ((double)q.tiles / g2 * c.n_kb * ((nh == 1 && q.tiles < g2) ? kb1(g2) : kcost) + hand_over);
+    double us_split = 1.05 * ((double)q.tiles / g2 * c.n_kb * ((nh == 1 && q.tiles < g2) ? kb1(g2) : kcost) + hand_over);
     // Whole tiles.  On both accumulators a k-block takes 0.84 us when every SM runs one and less when some have no
     // tile (0.79 us with 28 busy SMs: they share the activation traffic out of L2), and between two tiles of a block
     // the MMAs wait 7 - 10 us for the epilogue to drain the accumulators (in-kernel time stamps, Qwen2.5-7B gate at
@@ -1097,9 +1166,10 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     double us_whole = (double)rounds * c.n_kb * kcost;
     if (nh == 1 && q.tiles <= g2) us_whole = c.n_kb * kb1(q.tiles);
     if (nh == 2 && cg2)
-      us_whole = (double)rounds * (c.n_kb * 0.62 + 10.0);
+      us_whole = (double)rounds * (c.n_kb * 0.60 + 9.0);
     else if (nh == 2)
       us_whole = (double)(q.tiles / g2) * c.n_kb * 0.96 + (q.left ? c.n_kb * (0.90 + 0.06 * q.left / g2) : 0.0) + 10.0 * (rounds - 1);
+    if (cg2 && nh == 1) { us_whole += 5.5; us_split += 5.5; }                  // start and last epilogue
     // one fp32 slot per (left-over tile, block) piece, or one sum per left-over tile
     q.sums = (size_t)(q.atomic ? q.left : q.left + g2) * ntok * BMW * 4 * (cg2 ? 2 : 1);
     const bool want = env_streamk >= 0 ? (env_streamk >= 1) : (q.left != 0 && us_split < us_whole);
@@ -1110,7 +1180,7 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     // (0.45 - 0.6 us per k-block by the number of busy SMs) instead of a two-box tile's on a few SMs.
     q.halves = false;
     if (nh == 2 && q.left != 0 && 2 * q.left <= g2 && q.tiles > g2 && !conv_in_kernel && env_streamk < 1 && opt(kOptPrefillDual) != 2) {
-      const double us_halves = cg2 ? (double)(q.tiles / g2) * (c.n_kb * 0.62 + 10.0) + c.n_kb * 0.34
+      const double us_halves = cg2 ? (double)(q.tiles / g2) * (c.n_kb * 0.60 + 9.0) + c.n_kb * 0.365 + 5.5
                                    : (double)(q.tiles / g2) * (c.n_kb * 0.96 + 10.0) + c.n_kb * (0.45 + 0.15 * 2 * q.left / g2);
       if (us_halves < q.us || opt(kOptPrefillDual) == 3) { q.halves = true; q.streamk = false; q.us = us_halves; }
     }
@@ -1123,6 +1193,16 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
       // (against a split over all SMs it has to be 10 % ahead: with long contractions the two come out level and
       //  the split measured ahead, Qwen2.5-7B down projection at M = 512)
       if (us_pair * (q.streamk ? 1.10 : 1.0) < q.us || env_streamk == 3) { q.pair = true; q.streamk = false; q.us = us_pair; }
+    }
+    // Few tiles of a pair: a cluster of two to four pairs per tile, a part of the contraction each (0.34 us per k-block, 7 us
+    // for the exchange beside what a whole tile's start and end take; 4096 x 4096 at M = 256: 25.7 -> 19.0 us).
+    if (cg2 && nh == 1 && env_streamk != 0 && c.n_kb >= 8) {
+      for (int k = 2; k <= kMaxShare; ++k) {
+        const int cap = env_grid >= 1 ? env_grid / k : pair_capacity(k);
+        const bool fits = q.tiles <= cap && cfg.ws_bytes >= ws_used + (size_t)q.tiles * k * 2 * MAXBN * BMW * 4;
+        const double us = (c.n_kb + k - 1) / k * 0.34 + 12.5;
+        if (fits && (env_streamk == 10 + k || (env_streamk < 0 && us < q.us))) { q.share = k; q.streamk = false; q.us = us; }
+      }
     }
     return q;
   };
@@ -1147,6 +1227,7 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
   c.nh = pl.nh;
   c.halves = pl.halves ? 1 : 0;
   c.pair_split = pl.pair ? 1 : 0;
+  c.csplit = pl.share;
   c.n_ttiles = pl.ttiles;
   c.n_tiles = pl.tiles;
   if (pl.cg2) {
@@ -1172,18 +1253,21 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
       if (rc != UNIQL_OK) return rc;
     }
   }
-  if (pl.cg2) grid *= 2;
+  if (pl.cg2) grid *= 2 * pl.share;
+  if (pl.share > 1) c.partials = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(cfg.workspace) + ws_used);
   int rc = encode_x_map(&c.xmap, xsrc, p.k_in, p.M, ldxs, pl.cg2 ? c.bn / 2 : c.bn, conv_in_kernel);
   if (rc != UNIQL_OK) return rc;
   if (p.dt == UNIQL_BF16)
     rc = conv_in_kernel ? launch_pt<__nv_bfloat16, true, 0>(p, c, grid, cfg.stream)
          : !pl.cg2      ? launch_pt<__nv_bfloat16, false, 0>(p, c, grid, cfg.stream)
+         : c.csplit > 1 ? launch_pt<__nv_bfloat16, false, 3>(p, c, grid, cfg.stream)
          : c.nh == 1    ? launch_pt<__nv_bfloat16, false, 1>(p, c, grid, cfg.stream)
                         : launch_pt<__nv_bfloat16, false, 2>(p, c, grid, cfg.stream);
   else
-    rc = !pl.cg2     ? launch_pt<__half, false, 0>(p, c, grid, cfg.stream)
-         : c.nh == 1 ? launch_pt<__half, false, 1>(p, c, grid, cfg.stream)
-                     : launch_pt<__half, false, 2>(p, c, grid, cfg.stream);
+    rc = !pl.cg2        ? launch_pt<__half, false, 0>(p, c, grid, cfg.stream)
+         : c.csplit > 1 ? launch_pt<__half, false, 3>(p, c, grid, cfg.stream)
+         : c.nh == 1    ? launch_pt<__half, false, 1>(p, c, grid, cfg.stream)
+                        : launch_pt<__half, false, 2>(p, c, grid, cfg.stream);
   if (rc == UNIQL_ERR_UNSUPPORTED && c.pair_split) {
     // the pairs cannot all be resident (or clusters cannot be launched here): planned again without them
     pair_refused.store(true);

@@ -99,3 +99,32 @@ def test_half_tiles_and_gated_product(B, width):
     check_output(h, h_ref, "f16", TOL, "h")
     check_output(y, y_ref, "f16", 1e-3, "y")
     assert B.workspace_status() == 0
+
+
+@pytest.mark.parametrize("share", [2, 3, 4])
+@pytest.mark.parametrize("M", [129, 256, 300])
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+def test_tiles_shared_by_the_pairs_of_a_cluster(B, M, dtype, share):
+    """A part of the contraction per pair, sums exchanged inside the cluster: k-block counts that do not divide, ragged
+    rows and tokens, every epilogue, the same bits on every run."""
+    B.set_option("prefill_pair", 1)
+    B.set_option("prefill_streamk", 10 + share)
+    rng = np.random.default_rng(2300 + M)
+    qw = synth.draw_qweight(rng, 700, 1024)
+    dw = dev_weight(qw)
+    bias = synth.to_dtype_values(rng.standard_normal(700).astype(np.float32), dtype)
+    for (k_in, k_out) in ((1024, 700), (652, 132)):
+        x = synth.draw_x(rng, M, k_in, dtype)
+        y, ref = run_ex(B, qw, dw, x, dtype, None, k_in, None, k_out, bias=bias, ldx_pad=8 - k_in % 8 if k_in % 8 else 0, ldy_pad=3)
+        check_output(y, ref, dtype, TOL, "shared by %d M=%d %s k=(%d,%d)" % (share, M, dtype, k_in, k_out))
+        y2, _ = run_ex(B, qw, dw, x, dtype, None, k_in, None, k_out, bias=bias, ldx_pad=8 - k_in % 8 if k_in % 8 else 0, ldy_pad=3)
+        assert torch.equal(y, y2)
+    for helpers in (1, 0):
+        B.set_option("prefill_helpers", helpers)
+        for (g, r) in run_rope(B, rng, M, 512, 6, 2, 128, 84, 5e5, dtype, bias=True):
+            check_output(g, r, dtype, TOL, "rope shared by %d" % share)
+        im = synth.map_per_head(8, 128, 104)
+        x = synth.draw_x(rng, M, synth.map_size(im), dtype)
+        y, ref = run_ex(B, qw, dw, x, dtype, im, 0, None, 200, ldx_pad=8)
+        check_output(y, ref, dtype, TOL, "per-head input map shared by %d" % share)
+    assert B.workspace_status() == 0
