@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
       const uint32_t x_row = (uint32_t)(sr * 128), x_sw = (uint32_t)((half * 4) ^ (sr & 7)) * 16;   // piece i: x_sw ^ (16 i)
       uint32_t w[16];
       __half sc, zp;
-      auto fetch = [&]() -> bool {               // codes, scale and zero-point of the next stage of the ring; the slot is free again
+      auto fetch = [&]() -> bool {               // codes, scale and zero-point of the next stage of the ring
         if (!pmbar_wait_warp(w_full + 8 * ws, wpar, abort_flag)) return false;
         const uint32_t src = sbase + (uint32_t)(c.off_w + ws * WSTAGE);
 #pragma unroll
@@ -435,10 +435,14 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
         asm volatile("ld.shared.u16 %0, [%1];" : "=h"(sh) : "r"(src + s_off) : "memory");
         asm volatile("ld.shared.u16 %0, [%1];" : "=h"(zh) : "r"(src + s_off + BMW * 4) : "memory");
         sc = __ushort_as_half(sh); zp = __ushort_as_half(zh);
+        return true;
+      };
+      // The slot goes back only after its values were USED: an arrival issued behind the loads can overtake them, and the
+      // next stage's copy then lands under the reads (wrong rows in contractions long enough for the ring to wrap).
+      auto release = [&]() {
         __syncwarp();
         if (lane == 0) pmbar_arrive(w_empty + 8 * ws);
         if (++ws == c.wst) { ws = 0; wpar ^= 1; }
-        return true;
       };
       if (!fetch()) { failed = true; break; }
       for (int st = sg.s0; st < sg.s1; ++st) {
@@ -469,6 +473,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
         tmem_st32(a_lane + (uint32_t)(64 * as), o);
         convert(8);
         convert(12);
+        release();
         if (st + 1 < sg.s1 && !fetch()) { failed = true; break; }
         tmem_st32(a_lane + (uint32_t)(64 * as + 32), o);
         stored_as = as;

@@ -1,0 +1,33 @@
+"""Batch kernel (17 to 128 rows): contractions long enough that its rings wrap many times, alone and back to back."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import check_output, dev_weight
+from test_gpu_prefill import B, run_ex  # noqa: F401  (B: fixture)
+from paper_2512_03383_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+TOL = 5e-4       # as the other tensor-core tests: weights rounded once to fp16, fp32 sums
+
+
+@pytest.mark.parametrize("M", [17, 48, 64, 100, 128])
+@pytest.mark.parametrize("split", [0, -1])
+def test_long_contractions(B, M, split):
+    B.set_path(B.PATH_PREFILL)
+    B.set_option("prefill_streamk", split)
+    rng = np.random.default_rng(2400 + M)
+    for (N, K) in ((640, 8192), (1500, 4096)):
+        qw = synth.random_qweight_fast(rng, N, K)
+        dw = dev_weight(qw)
+        x = synth.draw_x(rng, M, K, "f16")
+        y, ref = run_ex(B, qw, dw, x, "f16", None, K, None, N)
+        check_output(y, ref, "f16", TOL, "M=%d N=%d K=%d" % (M, N, K))
+        first = y.clone()
+        for _ in range(20):                        # (launches behind one another: blocks of two launches share the SMs)
+            y, _ = run_ex(B, qw, dw, x, "f16", None, K, None, N)
+        assert torch.equal(y, first)
+    assert B.workspace_status() == 0
+    B.set_path(B.PATH_AUTO)
+    B.reset_options()
