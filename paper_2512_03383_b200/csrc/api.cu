@@ -26,7 +26,6 @@ const OptDesc kOpts[kOptCount] = {
     {"decode_narrow", "UNIQL_DECODE_NARROW", -1},       // narrow tiles: -1 automatic, 0 off, 1 on
     {"decode_xstream", "UNIQL_DECODE_XSTREAM", -1},     // streamed activations: -1 automatic, 0 off, 1 on
     {"decode_xcluster", "UNIQL_DECODE_XCLUSTER", -1},   // shared staging in clusters of two: -1 automatic, 0 off, 1 on
-    {"decode_half", "UNIQL_DECODE_HALF", -1},           // blocks of half an SM at one to four rows: -1 automatic, 0 off
     {"decode_i8", "UNIQL_DECODE_I8", 1},                // integer path (0: fp16 MMAs)
     {"decode_split_batch", "UNIQL_DECODE_SPLIT_BATCH", 2},   // batches of 9..16: one streamed launch where it applies
     {"prefill_grid", "UNIQL_PREFILL_GRID", 0},          // blocks of the tensor-core kernel (0: one per SM)

@@ -47,7 +47,6 @@ constexpr int CTH = CW * 32;            // consumer threads
 constexpr int EW = 4;                   // epilogue warps
 constexpr int ETH = EW * 32;
 constexpr int NTH = CTH + 32 + ETH;     // consumers + one producer warp + epilogue warps
-constexpr int NTH_HALF = CTH / 2 + 32 + ETH;   // ... of a block that shares its SM with the next launch's
 constexpr int RB = 64;                  // row slots per tile
 constexpr int CG = 8;                   // groups per chunk
 constexpr int BOX_COLS = CG / 2;        // 128-byte columns (two groups each) per chunk
@@ -61,7 +60,7 @@ constexpr int kStatusOff = kCounterInts * 4;   // status word right after the co
 constexpr int kGridSyncOff = kStatusOff + 64;   // the two counters of the barrier between phases
 constexpr int kWsHeader = kStatusOff + 256;
 constexpr int kMaxKParts = 16;
-constexpr int kSmemMax = 227 * 1024, kSmemHalf = 113 * 1024;
+constexpr int kSmemMax = 227 * 1024;
 constexpr int kWaitLimit = 1 << 18;
 constexpr int kGridWaitLimit = 1 << 21;   // polls (40 ns apart) of the barrier between the phases of a fused launch
 constexpr int BAR_BYTES = 256;
@@ -144,7 +143,6 @@ struct DecodeCfg {
   // batch row), and every stage of the ring carries the eight groups of its unit beside the weights.
   int x_cluster;         // blocks run as clusters of two that share the staging of the activations: each quantises
                          // half of the (row, group) pairs and writes them into both blocks' shared memory
-  int half;              // blocks of half an SM (see decode_kernel)
   int x_stream;
   int stage_bytes;       // STAGE_BYTES, plus vr * CG * 128 + 1024 when the activations are streamed
   int vr;                // virtual rows per group in a stage: 8 (up to four batch rows) or 16
@@ -530,14 +528,10 @@ struct UnitIter {
 // T: activation and output type (bf16: integer path only).  A template parameter although a model never mixes the two:
 // as a flag of the launch it cost the instance for nine to sixteen rows more spills in its loop (Llama-3-8B layer at
 // sixteen rows 79 -> 85 us).
-// HF: half an SM per block (eight consumer warps, at most kSmemHalf of shared memory), so that the next launch's block sits
-// beside this one with its first stages fetched when this one ends.  With a whole SM per block a launch of 7 - 60 MB spent
-// about 4 us between its predecessor's last byte and its own first.
-template <int MT, bool ONECOL, int NT, int NPH, bool XS, bool XC, typename T, bool HF>
-__global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel(const __grid_constant__ Params p,
+template <int MT, bool ONECOL, int NT, int NPH, bool XS, bool XC, typename T>
+__global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ Params p,
                                                         const __grid_constant__ DecodeCfg c) {
   extern __shared__ unsigned char smem_raw[];
-  constexpr int CWK = HF ? CW / 2 : CW, CTHK = CWK * 32;     // consumer warps and threads of this instance
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // the stage ring starts on a 1024-byte boundary (the swizzle pattern repeats every 1024 bytes)
   const uint32_t raw = (uint32_t)__cvta_generic_to_shared(smem_raw);
@@ -558,11 +552,11 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
   if (tid == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(bar_full + 8 * s, 33);      // one expect_tx arrival + 32 copy-completion arrivals
-      mbar_init(bar_empty + 8 * s, CWK);
+      mbar_init(bar_empty + 8 * s, CW);
     }
-    mbar_init(bar_cons, CWK);
+    mbar_init(bar_cons, CW);
     mbar_init(bar_epi, xc_on ? 2 * CW : EW);        // shared staging: the consumer warps of both blocks arrive
-    for (int b = 0; b < 2; ++b) { mbar_init(bar_pfull + 8 * b, CWK); mbar_init(bar_pfree + 8 * b, EW); }
+    for (int b = 0; b < 2; ++b) { mbar_init(bar_pfull + 8 * b, CW); mbar_init(bar_pfree + 8 * b, EW); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -575,16 +569,14 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
   if (c.n_kp > 1) { kp = rp / c.n_rp; rp -= kp * c.n_rp; }
   // Programmatic dependent launch: the next kernel of the stream may be set up while this one runs (its
   // blocks still need this block's resources, so they start as blocks here exit) ...
-  // (HF: the epilogue warps do this, once the predecessor is complete: a launch further on would take the slot that the next
-  //  one's block needs)
-  if (!HF) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const PhaseCtx pc0 = phase_ctx(c, 0, kp, rp);
   if (NPH == 1 && pc0.wk.n_units == 0) return;
 
   // ======================================================================================= producer
   // The ring runs on across phases: the weights of the next phase are fetched while the grid-wide barrier
   // between the phases is still being crossed (weights, scales and zero-points are never produced in here).
-  if (warp == CWK) {
+  if (warp == CW) {
     int it = 0, s = 0;
     uint32_t ring_parity = 1;      // parity of the previous use of ring position s
     bool ok = true;
@@ -733,15 +725,14 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
   // ======================================================================================= epilogue
   // Finishes the block's tiles in order, behind the consumers: sums the eight parked group partials of
   // every (row slot, batch row), then stores the tile, or parks the sum for the block that finishes it.
-  if (warp > CWK) {
-    const int etid = tid - (CWK + 1) * 32;
+  if (warp > CW) {
+    const int etid = tid - (CW + 1) * 32;
     auto give_up = [&]() { if (lane == 0) atomicExch(c.status, UNIQL_ERR_TIMEOUT); };
     int tiles_done = 0;
     // ... and this kernel may have been started before its predecessor finished: outputs, workspace, bias,
     // positions and indices are touched only after the predecessor is complete (the producer warp does not
     // wait: weights, scales and zero-points are not produced by a preceding decode launch)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (HF) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (int ph = 0; ph < NPH; ++ph) {
       const PhaseCtx pc = (NPH == 1 || ph == 0) ? pc0 : phase_ctx(c, ph, kp, rp);
       const Work& wk = pc.wk;
@@ -809,7 +800,7 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
             __threadfence();
             __syncwarp();
             int last_w = 0;
-            int* cnt = c.counters + tile * EW + (warp - CWK - 1);
+            int* cnt = c.counters + tile * EW + (warp - CW - 1);
             if (lane == 0) {
               last_w = atomicAdd(cnt, 1) == total - 1;
               __threadfence();
@@ -847,7 +838,7 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
   }
 
   // ======================================================================================= consumers
-  const int ctid = tid;                    // 0..CTHK-1
+  const int ctid = tid;                    // 0..CTH-1
   const int g = lane >> 2, t = lane & 3;
   const int kpw = warp & 7, rg = warp >> 3;
   // MMA row g of a sub-tile is row slot pg: lanes g = 2i and 2i+1 get slots that differ in bit 2, so that
@@ -899,7 +890,7 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
     auto row_of = [&](int pair) { int m = 0; while (pair >= Gn) { pair -= Gn; ++m; } return m; };
     auto needed_group = [&](int gn) { int ch = ch0 + (gn >> cg_sh); if (ch >= wk.Ck) ch -= wk.Ck; return (ch << cg_sh) + (gn & (cgz - 1)); };
     if (NT == 0) {          // (the integer path writes every entry it later reads)
-      for (int i = ctid; i < Gk * 8 * MT; i += CTHK) xg[i] = make_float2(0.f, 0.f);
+      for (int i = ctid; i < Gk * 8 * MT; i += CTH) xg[i] = make_float2(0.f, 0.f);
       if (!consumer_sync()) return false;
     }
     if constexpr (NT > 0) {
@@ -924,11 +915,11 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
         pxg = peer_addr(sbase + (uint32_t)c.off_xg, (uint32_t)(crank ^ 1));
       }
       constexpr int UN = 4;
-      for (int u0 = ctid; u0 < ((n_units + 31) & ~31); u0 += CTHK * UN) {
+      for (int u0 = ctid; u0 < ((n_units + 31) & ~31); u0 += CTH * UN) {
         uint4 in[UN];
 #pragma unroll
         for (int q4 = 0; q4 < UN; ++q4) {
-          const int u = u0 + q4 * CTHK;
+          const int u = u0 + q4 * CTH;
           in[q4] = make_uint4(0, 0, 0, 0);
           if (u < n_units) {
             const int pair = ((u >> 4) << csh) + crank, m = row_of(pair), lv = needed_group(pair - m * Gn);
@@ -938,7 +929,7 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
         }
 #pragma unroll
         for (int q4 = 0; q4 < UN; ++q4) {
-          const int u = u0 + q4 * CTHK;
+          const int u = u0 + q4 * CTH;
           if (u >= ((n_units + 31) & ~31)) break;                  // warp-uniform
           const int u16 = u & 15, pair = u < n_units ? ((u >> 4) << csh) + crank : 0;
           const int m = row_of(pair), lv = needed_group(pair - m * Gn);
@@ -984,11 +975,11 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
     if (c.x_vec) {
       const int n_units = Gn * p.M * 16;
       constexpr int UN = 4;                                        // loads in flight per thread
-      for (int u0 = ctid; u0 < ((n_units + 31) & ~31); u0 += CTHK * UN) {   // whole warps stay in the shuffles
+      for (int u0 = ctid; u0 < ((n_units + 31) & ~31); u0 += CTH * UN) {   // whole warps stay in the shuffles
         uint4 in[UN];
 #pragma unroll
         for (int q4 = 0; q4 < UN; ++q4) {
-          const int u = u0 + q4 * CTHK;
+          const int u = u0 + q4 * CTH;
           in[q4] = make_uint4(0, 0, 0, 0);
           if (u < n_units) {
             const int pair = u >> 4, m = row_of(pair), lv = needed_group(pair - m * Gn);
@@ -998,7 +989,7 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
         }
 #pragma unroll
         for (int q4 = 0; q4 < UN; ++q4) {
-          const int u = u0 + q4 * CTHK;
+          const int u = u0 + q4 * CTH;
           if (u >= ((n_units + 31) & ~31)) break;                  // warp-uniform
           const int u16 = u & 15, pair = u < n_units ? u >> 4 : 0;
           const int m = row_of(pair), lv = needed_group(pair - m * Gn);
@@ -1023,7 +1014,7 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
     } else {
       T* xh = reinterpret_cast<T*>(smem + c.off_x);
       const int n_pairs = Gk * p.M;
-      for (int pair = warp; pair < n_pairs; pair += CWK) {
+      for (int pair = warp; pair < n_pairs; pair += CW) {
         const int m = pair / Gk, lv = pair - m * Gk;
         const int kbase = (sg_lo + lv) * kGroup;
         float se = 0.f, so = 0.f;
@@ -1078,10 +1069,9 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
     const uint32_t xsg = (uint32_t)(STAGE_BYTES + c.vr * CG * 128 + kpw * 64 * MT + t * 8);
     const uint32_t wl_off = (uint32_t)((kpw >> 1) * BOX_BYTES + (rg * 32 + pg) * 128 + ((((kpw & 1) * 4 + t) ^ pg) * 16));
     const uint32_t sl_off = (uint32_t)(STAGE_W + (rg * 32 + pg) * (CG * 2) + kpw * 2);
-    constexpr int RGN = HF ? 2 : 1;                    // row halves of a stage that this warp works on
-    float out8[2 * RGN][NT][2];
+    float out8[2][NT][2];
 #pragma unroll
-    for (int sub = 0; sub < 2 * RGN; ++sub)
+    for (int sub = 0; sub < 2; ++sub)
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) out8[sub][nt][0] = out8[sub][nt][1] = 0.f;
     uint4 xr8[NT][2];
@@ -1134,12 +1124,10 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
         give_up();
         return;
       }
-#pragma unroll
-      for (int rh = 0; rh < RGN; ++rh) {
-      const int gi = ui.chunk * c.cgz + (HF && c.cgz > CG ? rh * CG + kpw : g_first);
+      const int gi = ui.chunk * c.cgz + g_first;
       if (gi < Gk) {
         const uint32_t st = sbase + (uint32_t)s * (xs_on ? (uint32_t)c.stage_bytes : (uint32_t)STAGE_BYTES);
-        const uint32_t wp = st + wl_off + (uint32_t)(rh * 32 * 128), sp = st + sl_off + (uint32_t)(rh * 32 * CG * 2);
+        const uint32_t wp = st + wl_off, sp = st + sl_off;
         if constexpr (NT <= 1) {
         uint4 wa[2], wb[2];
         wa[0] = lds128<0>(wp);
@@ -1188,8 +1176,8 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
             // 256 * (sum q*hi) + (sum q*lo) = sum q*x_i exactly, in integers; one conversion, one rounding
             const float y0 = (float)(d[sub][nt][0] * 256 + d[sub][nt][1]);
             const float y1 = (float)(d[sub][nt][2] * 256 + d[sub][nt][3]);
-            out8[2 * rh + sub][nt][0] = fmaf(sc[sub][0] * xs.y, fmaf(-zp[sub][0], xs.x, y0), out8[2 * rh + sub][nt][0]);
-            out8[2 * rh + sub][nt][1] = fmaf(sc[sub][1] * xs.y, fmaf(-zp[sub][1], xs.x, y1), out8[2 * rh + sub][nt][1]);
+            out8[sub][nt][0] = fmaf(sc[sub][0] * xs.y, fmaf(-zp[sub][0], xs.x, y0), out8[sub][nt][0]);
+            out8[sub][nt][1] = fmaf(sc[sub][1] * xs.y, fmaf(-zp[sub][1], xs.x, y1), out8[sub][nt][1]);
           }
         }
         } else {
@@ -1242,7 +1230,6 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
           }
         }
       }
-      }
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_empty + 8 * s);
       if (++s == S) { s = 0; ring_parity ^= 1; }
@@ -1252,7 +1239,7 @@ __global__ void __launch_bounds__(HF ? NTH_HALF : NTH, HF ? 2 : 1) decode_kernel
         if (use > 0 && !mbar_wait(bar_pfree + 8 * buf, (use - 1) & 1, abort_flag)) { give_up(); return; }
         float* pb = part + buf * part_stride + kpw * RM;
 #pragma unroll
-        for (int sub = 0; sub < 2 * RGN; ++sub)
+        for (int sub = 0; sub < 2; ++sub)
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt) {
             const int m = t + 4 * nt;
@@ -1541,9 +1528,9 @@ void fill_split(const DecodeCfg& c, Phase* P) {
   P->by_bt0 = fast_div((unsigned)P->bt0, ut * (unsigned long long)c.n_rp);
 }
 
-template <int MT, bool ONECOL, int NT, int NPH, bool XS, bool XC, typename T, bool HF>
+template <int MT, bool ONECOL, int NT, int NPH, bool XS, bool XC, typename T>
 int launch_as(const Params& p, const DecodeCfg& c, size_t smem, cudaStream_t stream) {
-  auto kern = decode_kernel<MT, ONECOL, NT, NPH, XS, XC, T, HF>;
+  auto kern = decode_kernel<MT, ONECOL, NT, NPH, XS, XC, T>;
   {
     // the shared-memory limit of this instance is raised once per device (the call costs about a microsecond)
     static std::mutex mu;
@@ -1560,7 +1547,7 @@ int launch_as(const Params& p, const DecodeCfg& c, size_t smem, cudaStream_t str
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
   lc.gridDim = dim3(c.n_kp * c.n_rp);
-  lc.blockDim = dim3(HF ? NTH_HALF : NTH);
+  lc.blockDim = dim3(NTH);
   lc.dynamicSmemBytes = smem;
   lc.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -1595,13 +1582,13 @@ int launch_as(const Params& p, const DecodeCfg& c, size_t smem, cudaStream_t str
   return as_clusters ? UNIQL_ERR_UNSUPPORTED : UNIQL_ERR_CUDA;
 }
 
-template <int MT, bool ONECOL, int NT, int NPH, bool XS = false, bool XC = false, bool HF = false>
+template <int MT, bool ONECOL, int NT, int NPH, bool XS = false, bool XC = false>
 int launch_t(const Params& p, const DecodeCfg& c, size_t smem, cudaStream_t stream) {
   if constexpr (NT > 0 && NPH == 1) {
-    if (p.dt == UNIQL_BF16) return launch_as<MT, ONECOL, NT, NPH, XS, XC, __nv_bfloat16, HF>(p, c, smem, stream);
+    if (p.dt == UNIQL_BF16) return launch_as<MT, ONECOL, NT, NPH, XS, XC, __nv_bfloat16>(p, c, smem, stream);
   }
   if (p.dt != UNIQL_F16) return UNIQL_ERR_UNSUPPORTED;
-  return launch_as<MT, ONECOL, NT, NPH, XS, XC, __half, HF>(p, c, smem, stream);
+  return launch_as<MT, ONECOL, NT, NPH, XS, XC, __half>(p, c, smem, stream);
 }
 
 // Visited groups of the input map: from the first to the last 128-channel group that holds a retained
@@ -1657,25 +1644,6 @@ size_t plan_split(DecodeCfg* c, int M, int g_total, int gran, bool i8) {
   // the kernel cuts the left-over units with 32-bit products of at most n_rp * n_rp * (chunks per tile)
   if ((long long)n_rp * n_rp * ((c->gp + CG - 1) / CG) >= (1ll << 31)) return 0;
   return smem;
-}
-
-// Plan for blocks of half an SM (one to four rows): two or three stages and the staged activations in kSmemHalf, the input
-// channels not split.  Returns 0 when that does not fit.
-size_t plan_half(DecodeCfg* c, int M, int g_total, int gran) {
-  const int gp = round_up(g_total, gran);
-  for (int stages = 3; stages >= 2; --stages)
-    for (int bufs = 2; bufs >= 1; --bufs) {
-      const size_t smem = plan_smem(c, M, 1, gp, stages, bufs, true);
-      if (smem > (size_t)kSmemHalf) continue;
-      c->gp = gp;
-      c->g_total = g_total;
-      c->gran = gran;
-      c->n_kp = 1;
-      c->n_rp = sm_count();
-      if ((long long)c->n_rp * c->n_rp * ((gp + CG - 1) / CG) >= (1ll << 31)) return 0;
-      return smem;
-    }
-  return 0;
 }
 
 // Shared-memory plan with streamed activations: no staged copy of x, every stage carries the unit's eight
@@ -1844,12 +1812,7 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
       }
     }
   }
-  const bool steered = opt(kOptDecodeKp) != 0 || opt(kOptDecodeRp) != 0 || opt(kOptDecodeStages) != 0 || opt(kOptDecodeXcluster) > 0;
-  if (!c.x_stream && i8 && p.M <= 4 && !steered && opt(kOptDecodeHalf) != 0) {
-    smem = plan_half(&c, p.M, g_total, gran);
-    c.half = smem != 0;
-  }
-  if (!c.x_stream && !c.half) smem = plan_split(&c, p.M, g_total, gran, i8);
+  if (!c.x_stream) smem = plan_split(&c, p.M, g_total, gran, i8);
   if (!smem) return UNIQL_ERR_UNSUPPORTED;
 
   // ---- narrow tiles (32 rows x 16 groups) when the schedule they give is shorter: matrices with fewer
@@ -1933,7 +1896,7 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
     // per thread (smaller batches would alternate between two kernel functions within a layer, which costs more
     // than the staging saved).
     const int force_xc = opt(kOptDecodeXcluster);
-    c.x_cluster = i8 && !c.x_stream && !c.half && c.n_kp == 1 && (c.n_rp % 2) == 0 && p.M <= 8 && all_stage_everything &&
+    c.x_cluster = i8 && !c.x_stream && c.n_kp == 1 && (c.n_rp % 2) == 0 && p.M <= 8 && all_stage_everything &&
                   pairs_alike && force_xc != 0 && (force_xc == 1 || (p.M >= 7 && g_total * p.M >= 256));
   }
   if (tiles < 1 || tiles * EW > kCounterInts) return UNIQL_ERR_UNSUPPORTED;
@@ -1977,7 +1940,6 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
     c.x_cluster = 0;
   }
   if (i8) {
-    if (c.half) return launch_t<1, false, 1, 1, false, false, true>(p, c, smem, cfg.stream);
     if (p.M <= 4) return launch_t<1, false, 1, 1>(p, c, smem, cfg.stream);
     return launch_t<2, false, 4, 1>(p, c, smem, cfg.stream);
   }
@@ -2045,11 +2007,7 @@ int launch_mlp_phases(const MlpDecode& d, int first, int count, const LaunchCfg&
   c.x_stream = smem != 0;
   if (!smem) {
     c.stage_bytes = STAGE_BYTES;
-    if (count == 1 && d.M <= 4 && opt(kOptDecodeHalf) != 0 && opt(kOptDecodeKp) == 0 && opt(kOptDecodeRp) == 0 && opt(kOptDecodeStages) == 0) {
-      smem = plan_half(&c, d.M, g_max, gran);
-      c.half = smem != 0;
-    }
-    if (!smem) smem = plan_split(&c, d.M, g_max, gran, true);
+    smem = plan_split(&c, d.M, g_max, gran, true);
   }
   if (!smem) return UNIQL_ERR_UNSUPPORTED;
   if (count > 1 && (c.n_kp != 1 || d.M > 8)) return UNIQL_ERR_UNSUPPORTED;
@@ -2126,7 +2084,6 @@ int launch_mlp_phases(const MlpDecode& d, int first, int count, const LaunchCfg&
     if (d.M <= 4) return launch_t<1, false, 1, 2>(p, c, smem, cfg.stream);
     return launch_t<1, false, 2, 2>(p, c, smem, cfg.stream);
   }
-  if (c.half) return launch_t<1, false, 1, 1, false, false, true>(p, c, smem, cfg.stream);
   if (d.M <= 4) return launch_t<1, false, 1, 1>(p, c, smem, cfg.stream);
   if (d.M <= 8) {
     // shared staging under the rule of the plain launches (every block of the gate|up launch has whole tiles)
