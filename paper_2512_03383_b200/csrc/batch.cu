@@ -220,30 +220,43 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
     const uint32_t t_acc = tmem + ((uint32_t)(32 * q) << 16);
     const int n_ch = c.n / kTokChunk;
     tc_fence_after();
+    if (c.p == 1) {                                            // nothing to exchange: sixteen tokens at a time
+      for (int tk = 16 * half; tk < c.n; tk += 32) {
+        uint32_t v[16];
+        tmem_ld16(t_acc + (uint32_t)tk, v);
+        tmem_ld_wait();
+        float val[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) val[k] = __uint_as_float(v[k]);
+        rs.store(p, tk, val);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) pmbar_arrive(acc_empty);
+      return;
+    }
     const size_t slot_f = (size_t)c.n * BMW;
     float* slots = c.partials + (size_t)(count & 1) * slot_f + 32 * q + lane;      // + block * 2 slots + token * BMW
     const float* block0 = slots + (size_t)((int)blockIdx.x - rank) * 2 * slot_f;
-    if (c.p > 1) {
-      // the sums of the chunks that other blocks finish
-      float* mine = slots + (size_t)blockIdx.x * 2 * slot_f;
-      for (int ch = half; ch < n_ch; ch += 2) {
-        if (ch % c.p == rank) continue;
-        uint32_t v[8];
-        tmem_ld8(t_acc + (uint32_t)(ch * kTokChunk), v);
-        tmem_ld_wait();
+    // the sums of the chunks that other blocks finish
+    float* mine = slots + (size_t)blockIdx.x * 2 * slot_f;
+    for (int ch = half; ch < n_ch; ch += 2) {
+      if (ch % c.p == rank) continue;
+      uint32_t v[8];
+      tmem_ld8(t_acc + (uint32_t)(ch * kTokChunk), v);
+      tmem_ld_wait();
 #pragma unroll
-        for (int k = 0; k < 8; ++k) __stcg(mine + (size_t)(ch * kTokChunk + k) * BMW, __uint_as_float(v[k]));
-      }
-      __syncwarp();
-      // (barriers alternate from tile to tile: a peer may be a tile ahead before another peer's arrival has come in)
-      const uint32_t xb = xbar + 32 * (count & 1) + 8 * q;
-      if (lane < c.p && lane != rank) {
-        asm volatile("fence.acq_rel.cluster;" ::: "memory");
-        pmbar_arrive_peer(ppeer_addr(xb, (uint32_t)lane));
-      }
-      const bool ok = __all_sync(0xffffffffu, pmbar_wait_cluster(xb, (count >> 1) & 1, abort_flag));
-      if (!ok) { failed = true; return; }
+      for (int k = 0; k < 8; ++k) __stcg(mine + (size_t)(ch * kTokChunk + k) * BMW, __uint_as_float(v[k]));
     }
+    __syncwarp();
+    // (barriers alternate from tile to tile: a peer may be a tile ahead before another peer's arrival has come in)
+    const uint32_t xb = xbar + 32 * (count & 1) + 8 * q;
+    if (lane < c.p && lane != rank) {
+      asm volatile("fence.acq_rel.cluster;" ::: "memory");
+      pmbar_arrive_peer(ppeer_addr(xb, (uint32_t)lane));
+    }
+    const bool ok = __all_sync(0xffffffffu, pmbar_wait_cluster(xb, (count >> 1) & 1, abort_flag));
+    if (!ok) { failed = true; return; }
     for (int own = half; rank + own * c.p < n_ch; own += 2) {
       const int ch = rank + own * c.p;
       uint32_t v[8];
