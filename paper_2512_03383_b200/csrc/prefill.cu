@@ -1172,7 +1172,8 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     if (cg2 && nh == 1) { us_whole += 5.5; us_split += 5.5; }                  // start and last epilogue
     // one fp32 slot per (left-over tile, block) piece, or one sum per left-over tile
     q.sums = (size_t)(q.atomic ? q.left : q.left + g2) * ntok * BMW * 4 * (cg2 ? 2 : 1);
-    const bool want = env_streamk >= 0 ? (env_streamk >= 1) : (q.left != 0 && us_split < us_whole);
+    // (pairs: only where forced -- with a k-block at 0.36 us no split of the left-over tiles measured ahead of whole tiles)
+    const bool want = env_streamk >= 0 ? (env_streamk >= 1 && env_streamk < 10) : (!cg2 && q.left != 0 && us_split < us_whole);
     q.streamk = want && q.left != 0 && cfg.ws_bytes >= ws_used + q.sums && q.tiles <= (1 << 15);
     q.us = q.streamk ? us_split : us_whole;
     // Tiles of two boxes left over after the whole rounds, when they are few: each runs as two half tiles (one box,
@@ -1215,6 +1216,8 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
       if (dual >= 1 || p2.us < pl.us) pl = p2;
     }
     if (gp >= 1 && env_streamk != 3) {
+      // (above 128 rows pairs measured ahead of every one-block plan on all 20 layer shapes tried, 10 - 40 %)
+      if (opt_pair < 0) pl.us = 1e30;
       // (tests: 1 / 2 force pairs with one or two boxes per tile)
       for (int nh = 1; nh <= 2; ++nh) {
         if ((nh == 2 && (p.M <= MAXBN || dual == 0)) || (nh == 1 && p.M > MAXBN && dual >= 1)) continue;
