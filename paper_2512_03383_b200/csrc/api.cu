@@ -144,16 +144,14 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
   // allow it: at 17..63 rows the generic kernel measured 13 to 26 times slower (930 us against 71 us for the
   // Llama-3-8B gate|up at M = 17)
   bool pre_ok = prefill_supported(p);
-  // One to four rows whose input map is on 4- but not 8-channel boundaries (head dims 108 and 84, 1740 of 2048
-  // channels): re-laid on 8-channel boundaries for the decode kernel's integer path where that is possible (with
-  // the small kernel in front under programmatic dependent launch: Llama-3-8B o_proj at head dim 108, M = 1 / 4:
-  // 5.9 / 8.4 us), else the streaming kernel, which stages activations in 8-byte units (8.7 / 13.1 us).
+  // The streaming kernel (one to four rows): where it is asked for, and where the decode kernel's integer path cannot run
+  // (scales on 8- but not 16-byte boundaries).
   bool gv = path == UNIQL_PATH_GEMV || (path == UNIQL_PATH_AUTO && gemv_supported(p) && opt(kOptGemvFirst) == 1);
   const bool gv_else = path == UNIQL_PATH_AUTO && !gv && gemv_supported(p) && !(dec_ok && decode_integer_path(p));
   bool relaid = false;
-  // Everything else that misses a fast kernel only because of where its activations lie (blocks of 108 or 84
-  // channels, an odd row pitch) gets them re-laid in the workspace by a small kernel in front: 5..16 rows then run
-  // on the integer path of the decode kernel, larger batches on the tensor cores.
+  // What misses a fast kernel only because of where its activations lie (above 16 rows blocks of 108 or 84 channels, at
+  // decode sizes blocks that are no multiple of 4, an odd row pitch) gets them re-laid in the workspace by a small kernel
+  // in front.
   if (!gv && path != UNIQL_PATH_GENERIC) {
     bool decode_size = p.M <= 16 && path != UNIQL_PATH_PREFILL;
     Params q;

@@ -104,7 +104,8 @@ struct Phase {
   const void* x;         // activations [M][ldx]
   long long ldx;
   int K;                 // stored input channels of the phase's matrices
-  int start, keep;       // the input family (128-bit staging): head h keeps [start + h*period, +keep)
+  int x4;                // kept blocks lie on 4- but not on 8-channel boundaries: units are loaded in two halves
+  int start, keep;       // the input family (vector staging): head h keeps [start + h*period, +keep)
   int period, count;     // count = 1: a leading block
   int g_total, v_first;  // visited groups and the first of them
   int tile0, tiles;      // global tiles [tile0, tile0 + tiles)
@@ -305,13 +306,24 @@ __device__ inline float2 lds64f(uint32_t addr) {
 }
 
 
-// stored input channel (a multiple of 8) -> compact activation column, or -1 when the channel is pruned
+// stored input channel (a multiple of 8, or of 4 with x4) -> compact activation column, or -1 when the channel is pruned
 __device__ inline int compact_channel(const Phase& P, int ch) {
   int r = ch - P.start;
   if (r < 0) return -1;
   int h = 0;
   if (P.count > 1) { h = r / P.period; r -= h * P.period; if (h >= P.count) return -1; }
   return r < P.keep ? h * P.keep + r : -1;
+}
+
+// The eight activations of channels ch .. ch + 7 of a row (zero where pruned), for maps on 4-channel boundaries: head dims
+// 108 and 84 on the input side of o_proj.  (A kernel in front that re-lays such activations on 8-channel boundaries cost
+// 3 us per launch.)
+template <typename T, typename F>
+__device__ inline uint4 load_halves(const T* row, int ch, F compact) {
+  const int t0 = compact(ch), t1 = compact(ch + 4);
+  const uint2 a = t0 >= 0 ? __ldg(reinterpret_cast<const uint2*>(row + t0)) : make_uint2(0u, 0u);
+  const uint2 b = t1 >= 0 ? __ldg(reinterpret_cast<const uint2*>(row + t1)) : make_uint2(0u, 0u);
+  return make_uint4(a.x, a.y, b.x, b.y);
 }
 
 // Quantises the activations of one launch once (streamed mode): half-warp (batch row m, visited group lv).
@@ -329,8 +341,13 @@ __global__ void __launch_bounds__(256) xquant_kernel(const Phase P, int M, int v
     const int lv = pair / rows, m = pair - lv * rows;
     uint4 in = make_uint4(0, 0, 0, 0);
     if (u < n_units && m < M) {
-      const int t0 = compact_channel(P, (P.v_first + lv) * kGroup + 8 * u16);
-      if (t0 >= 0) in = __ldg(reinterpret_cast<const uint4*>(x + (size_t)m * P.ldx + t0));
+      const int ch = (P.v_first + lv) * kGroup + 8 * u16;
+      if (P.x4) {
+        in = load_halves(x + (size_t)m * P.ldx, ch, [&](int k) { return compact_channel(P, k); });
+      } else {
+        const int t0 = compact_channel(P, ch);
+        if (t0 >= 0) in = __ldg(reinterpret_cast<const uint4*>(x + (size_t)m * P.ldx + t0));
+      }
     }
     uint2 hi2, lo2;
     int isum;
@@ -923,8 +940,13 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
           in[q4] = make_uint4(0, 0, 0, 0);
           if (u < n_units) {
             const int pair = ((u >> 4) << csh) + crank, m = row_of(pair), lv = needed_group(pair - m * Gn);
-            const int t0 = compact_of((sg_lo + lv) * kGroup + 8 * (u & 15));
-            if (lv < Gk && t0 >= 0) in[q4] = load16(x + (size_t)m * ldx + t0);
+            const int ch = (sg_lo + lv) * kGroup + 8 * (u & 15);
+            if (NPH == 1 && P.x4) {
+              if (lv < Gk) in[q4] = load_halves(x + (size_t)m * ldx, ch, compact_of);
+            } else {
+              const int t0 = compact_of(ch);
+              if (lv < Gk && t0 >= 0) in[q4] = load16(x + (size_t)m * ldx + t0);
+            }
           }
         }
 #pragma unroll
@@ -1743,12 +1765,17 @@ int decode_supported(const Params& p) {
   return 1;
 }
 
-// The integer path of this kernel applies: one input family, everything on 8-channel boundaries, 128-bit loads.
-int decode_integer_path(const Params& p) {
-  return p.imap.n_fam == 1 && (p.imap.fam[0].start % 8) == 0 && (p.imap.fam[0].keep % 8) == 0 &&
-         (p.imap.fam[0].count == 1 || (p.imap.fam[0].period % 8) == 0) && (p.ldx % 8) == 0 &&
-         ((((uintptr_t)p.x) & 15) == 0);
+namespace {
+// the input map, row pitch and base address allow loads of `n` channels
+bool x_aligned(const Params& p, int n) {
+  const Fam& a = p.imap.fam[0];
+  return p.imap.n_fam == 1 && a.start % n == 0 && a.keep % n == 0 && (a.count == 1 || a.period % n == 0) && p.ldx % n == 0 &&
+         (((uintptr_t)p.x) & (uintptr_t)(2 * n - 1)) == 0;
 }
+}  // namespace
+
+// The integer path of this kernel applies: one input family, everything on 4-channel boundaries (8: one load per unit).
+int decode_integer_path(const Params& p) { return x_aligned(p, 4) ? 1 : 0; }
 
 size_t decode_workspace_bytes(int M, int K, int N_total) {
   // header (arrival counters, status word) + fp32 partial sums [slots][M][64] per tile.  With many tiles
@@ -1778,11 +1805,11 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
   visited_range(p.imap, gran, &v_first, &g_total);
   const int MT = p.M <= 8 ? 1 : 2;
   // 128-bit staging: one leading family, everything 8-element aligned
-  c.x_vec = decode_integer_path(p);
+  c.x_vec = x_aligned(p, 8);
   if (count_tile_fams(p) > kMaxTF) return UNIQL_ERR_UNSUPPORTED;
 
   // integer path: fp16 activations staged with 128-bit loads (a leading input block); UNIQL_DECODE_I8=0: fp16 MMAs
-  const bool i8 = c.x_vec && opt(kOptDecodeI8) != 0;
+  const bool i8 = decode_integer_path(p) && opt(kOptDecodeI8) != 0;
   // Streamed activations for rows too long to stage whole beside the ring (which would otherwise split the input
   // channels over several groups of blocks and hand every tile over); UNIQL_DECODE_XSTREAM=0/1 forces.  Where the
   // staged copy fits the quantising kernel in front costs more than the staging it saves (measured 3.5 us), and
@@ -1881,6 +1908,7 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
   {
     Phase& P = c.ph[0];
     P.x = p.x; P.ldx = p.ldx; P.K = p.K;
+    P.x4 = c.x_vec ? 0 : 1;
     P.start = p.imap.fam[0].start; P.keep = p.imap.fam[0].keep;
     P.period = p.imap.fam[0].period; P.count = p.imap.fam[0].count;
     P.g_total = g_total; P.v_first = v_first;
