@@ -57,6 +57,7 @@ constexpr int kMaxBF = 8;                      // row families of a launch
 constexpr int MAX_WST = 6, MAX_BST = 4, MAX_AST = 3;
 constexpr int LOADERS = 2, LD_WARP0 = 2, DQ0 = 4, DQN = 8;
 constexpr int kSmemBatch = 113 * 1024;         // two blocks per SM
+constexpr int kSmemAlone = 118 * 1024;         // one (never beside another block of this kernel)
 constexpr int kTmemCols = 256;
 constexpr int kTokChunk = 8;                   // tokens per epilogue pass; chunk i is finished by block i % p of the cluster
 
@@ -594,7 +595,7 @@ int residency(Residency* out) {
   Residency& r = dev_res[dev];
   if (!r.known) {
     for (int k = 0; k < 4; ++k)
-      if (cudaFuncSetAttribute(batch_instance(k & 1, k & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBatch) != cudaSuccess)
+      if (cudaFuncSetAttribute(batch_instance(k & 1, k & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone) != cudaSuccess)
         return UNIQL_ERR_CUDA;
     const int sms = device_sms();
     r.clusters[0] = 0;
@@ -655,7 +656,7 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   const int room = kSmemBatch - 1024 - 512 - c.off_w;
   c.wst = room / WSTAGE < MAX_WST ? room / WSTAGE : MAX_WST;
   c.off_bar = c.off_w + c.wst * WSTAGE;
-  const size_t smem = 1024 + (size_t)c.off_bar + 512;
+  size_t smem = 1024 + (size_t)c.off_bar + 512;
   c.status = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(cfg.workspace) + decode_status_offset());
   size_t used = (decode_workspace_header_bytes() + 255) & ~(size_t)255;
   const void* x = p.x;
@@ -704,6 +705,12 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   }
   rc = encode_x_map(&c.xmap, x, p.k_in, p.M, ldx, c.n, false);
   if (rc != UNIQL_OK) return rc;
+  // Shared tiles of at most a block per SM, planned at the pace of one: where the launch before still holds half of some
+  // SMs, the other halves are free first and the blocks came in two to an SM, at 1.05 us per stage instead of 0.65, with
+  // half of the SMs empty (SwiGLU block of Llama-3-8B, M = 64, keep 0.85: 47.4 -> 43.6 us; Qwen2.5-7B layer, 100 rows 95 -> 88
+  // us).  Asking for a little more than half of the SM spreads them.  Ten stages are where that pays for the later start:
+  // with four to eight (q|k|v, o_proj) a launch gains more from loading beside its predecessor (9.0 against 11.5 us).
+  if (c.p > 1 && best_clusters * c.p <= device_sms() && c.spt >= 10 * c.p) smem = kSmemAlone;
   BLaunch l(best_clusters * c.p, c.p, smem, cfg.stream);
   if (cudaLaunchKernelEx(&l.lc, batch_instance(p.dt == UNIQL_BF16, c.head_kb != 0), p, c) != cudaSuccess) {
     cudaGetLastError();
