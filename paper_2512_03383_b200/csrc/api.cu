@@ -188,8 +188,11 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
   if (gv_else && !relaid) gv = true;
   // Nine to sixteen rows in bf16: the batch kernel, whose fp16 operands that type had at these sizes before the decode kernel
   // took it (Mamba2-2.7B mixer at 12 rows 28.9 -> 22.0 us).  fp16 stays on exact codes.
-  const bool batch = path == UNIQL_PATH_AUTO && p.dt == UNIQL_BF16 && p.M > 8 && p.M <= 16 && batch_supported(p) &&
-                     (!cfg.workspace || cfg.ws_bytes >= prefill_workspace_bytes(p.M, p.K));
+  // fp16: its instance that multiplies the codes themselves, by the rule of exact_batch().
+  const bool batch = path == UNIQL_PATH_AUTO &&
+                     (p.dt == UNIQL_BF16 ? p.M > 8 && p.M <= 16 && batch_supported(p) &&
+                                               (!cfg.workspace || cfg.ws_bytes >= prefill_workspace_bytes(p.M, p.K))
+                                         : exact_batch(p));
   if (path == UNIQL_PATH_AUTO)
     path = batch ? UNIQL_PATH_PREFILL : gv ? UNIQL_PATH_GEMV : dec_ok ? UNIQL_PATH_DECODE : (pre_ok ? UNIQL_PATH_PREFILL : UNIQL_PATH_GENERIC);
   if (path == UNIQL_PATH_GEMV) {
@@ -510,7 +513,7 @@ int mlp_tensor_core(const void* x, int ldx, int dt, const uint8_t* wg, const voi
     jd.y = h; jd.ldy = ldh; jd.N = inter; jd.k_out = k_int;
     jd.pair = j + 1;
   }
-  if (!prefill_supported(a)) return UNIQL_ERR_UNSUPPORTED;
+  if (!prefill_supported(a) || (M <= 16 && dt == UNIQL_F16 && !exact_batch(a))) return UNIQL_ERR_UNSUPPORTED;   // (nothing launched)
   int rc = launch_prefill(a, cfg);
   if (rc != UNIQL_OK) return rc;
   Params b;
@@ -580,6 +583,11 @@ int mlp_block(const void* x, int ldx, int dt, const uint8_t* wg, const void* sg,
     const bool too_small = workspace && ws_bytes < mlp_decode_workspace_bytes(M, hidden, inter);
     if ((g_path.load() != UNIQL_PATH_AUTO && g_path.load() != UNIQL_PATH_DECODE) || too_small || !mlp_decode_supported(d))
       return tensor_core();
+  }
+  // the batch kernel on exact codes, both products (a decode launch behind a batch launch cannot come in beside it)
+  if (dt == UNIQL_F16 && M > 8 && fuse != 1 && g_path.load() == UNIQL_PATH_AUTO && mlp_decode_supported(d)) {
+    rc = tensor_core();
+    if (rc != UNIQL_ERR_UNSUPPORTED) return rc;
   }
   // one to four rows: two launches of the streaming kernel (unless one launch or the persistent kernel is asked for)
   if (fuse != 1 && gemv_mlp_supported(d) &&

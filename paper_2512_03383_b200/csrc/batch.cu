@@ -26,6 +26,13 @@
 //                then the tile's epilogue (bias, rotation or gated product, store; RowStore)
 // Tensor memory (256 columns): an accumulator of N columns, two or three half-stage A operands of 64 columns.
 //
+// EXACT instance (fp16, up to 16 rows).  The decode kernel, which takes these sizes otherwise, multiplies the codes
+// themselves; rounding code x scale to fp16 would lose precision against it.  So here A holds codes - 8 (exact in fp16), a
+// half stage is one group of 128 channels with accumulators of its own (P = sum (q - 8) x of 16 tokens and, from an operand
+// of ones, X = sum x in every lane), and the de-quantiser thread that made the operand adds s P + s (8 - z) X to fp32
+// registers: activations and codes enter unrounded, all sums are fp32.  The group's accumulators are read where the
+// thread waits for its A slot anyway.  Two FMAs per token and group replace one per pair of codes.
+//
 // Work split: clusters of p blocks share a tile, every block a p-th of its stages; the cluster takes tiles round-robin.
 // Each block then owns every p-th chunk of 16 tokens: it leaves its fp32 sums of the other chunks in a slot of its own
 // ([token][row], L2), tells the peers (remote arrivals on a barrier in their shared memory), and adds up and finishes its
@@ -77,6 +84,7 @@ struct BatchCfg {
   CUtensorMap xmap;          // activations: (k, token), box 64 x n
   int n;                     // tokens of an MMA: M rounded up to 16
   int n_ast, a_base;         // tensor memory: half-stage A operands, their first column
+  int exact;                 // codes as operands, scales applied to the groups' sums
   int wst, bst, off_w, off_bar;                // ring depths and shared-memory offsets (the activation ring is first)
   BFam fam[kMaxBF];
   int n_fam;
@@ -105,6 +113,13 @@ __device__ inline void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
         "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]),
         "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]),
         "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]) : "memory");
+}
+__device__ inline void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
 }
 __device__ inline void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // (through L1: eight consecutive stages use the same 32-byte sector of a row's scales)
@@ -173,7 +188,11 @@ struct BSegIter {
   }
 };
 
-template <typename T, bool HEADS>
+// Tensor memory of the EXACT instance: [0, 32) the tile's sums of the two halves, then per half P and X of a group, then
+// the operand of ones (eight columns; four columns of zeros behind it, so that four columns on it covers 8 channels).
+constexpr uint32_t kExP = 32, kExOnes = 96, kExA = 112;
+
+template <typename T, bool HEADS, bool EXACT>
 __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ Params p, const __grid_constant__ BatchCfg c) {
   extern __shared__ unsigned char bsm_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
@@ -193,7 +212,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
     for (int s = 0; s < MAX_WST; ++s) { pmbar_init(w_full + 8 * s, LOADERS * 32 + 1); pmbar_init(w_empty + 8 * s, DQN); }
     for (int s = 0; s < MAX_BST; ++s) { pmbar_init(b_full + 8 * s, 1); pmbar_init(b_empty + 8 * s, 1); }
     for (int s = 0; s < MAX_AST; ++s) { pmbar_init(a_full + 8 * s, DQN / 2); pmbar_init(a_empty + 8 * s, 1); }
-    pmbar_init(acc_full, 1);
+    pmbar_init(acc_full, EXACT ? DQN : 1);
     pmbar_init(acc_empty, DQN);
     for (int q = 0; q < 8; ++q) pmbar_init(xbar + 8 * q, max(1, 2 * (c.p - 1)));
     *abort_flag = 0;
@@ -214,6 +233,17 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
   }
   bool failed = false;
 
+  // the sums of 8 or 16 tokens from column `col` of the accumulator
+  auto load8 = [&](uint32_t col, uint32_t (&v)[8]) {
+    tmem_ld8(col, v);
+    if (EXACT) {
+      uint32_t u[8];
+      tmem_ld8(col + 16, u);
+      tmem_ld_wait();
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = __float_as_uint(__uint_as_float(v[k]) + __uint_as_float(u[k]));
+    }
+  };
   // ---- epilogue of the block's tile number `count` for the de-quantiser warp that calls it; the two warps of a quadrant
   //      (`half`) share the chunks
   auto epilogue_tile = [&](const RowStore<T>& rs, int count, int half) {
@@ -229,6 +259,12 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
         float val[16];
 #pragma unroll
         for (int k = 0; k < 16; ++k) val[k] = __uint_as_float(v[k]);
+        if (EXACT) {
+          tmem_ld16(t_acc + 16, v);
+          tmem_ld_wait();
+#pragma unroll
+          for (int k = 0; k < 16; ++k) val[k] += __uint_as_float(v[k]);
+        }
         rs.store(p, tk, val);
       }
       tc_fence_before();
@@ -244,7 +280,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
     for (int ch = half; ch < n_ch; ch += 2) {
       if (ch % c.p == rank) continue;
       uint32_t v[8];
-      tmem_ld8(t_acc + (uint32_t)(ch * kTokChunk), v);
+      load8(t_acc + (uint32_t)(ch * kTokChunk), v);
       tmem_ld_wait();
 #pragma unroll
       for (int k = 0; k < 8; ++k) __stcg(mine + (size_t)(ch * kTokChunk + k) * BMW, __uint_as_float(v[k]));
@@ -261,7 +297,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
     for (int own = half; rank + own * c.p < n_ch; own += 2) {
       const int ch = rank + own * c.p;
       uint32_t v[8];
-      tmem_ld8(t_acc + (uint32_t)(ch * kTokChunk), v);
+      load8(t_acc + (uint32_t)(ch * kTokChunk), v);
       float val[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) val[k] = 0.f;
@@ -328,7 +364,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
     int as = 0, bs = 0, count = 0; uint32_t apar = 0, bpar = 0;
     const uint64_t box_step = (uint64_t)(c.n * 8);             // a box of n * 128 bytes, in the descriptor's 16-byte units
     for (; !failed && si.next(sg); ++count) {
-      if (count >= 1 && !pmbar_wait_warp(acc_empty, (count - 1) & 1, abort_flag)) { failed = true; break; }
+      if (!EXACT && count >= 1 && !pmbar_wait_warp(acc_empty, (count - 1) & 1, abort_flag)) { failed = true; break; }
       for (int v0 = sg.s0 * KS; v0 < sg.s1 * KS; v0 += KS / 2) {
         const int nv = c.n_kb - v0;                            // k-blocks of this half stage (none behind the last: only handed back)
         if ((nv > 0 && !pmbar_wait_warp(b_full + 8 * bs, bpar, abort_flag)) || !pmbar_wait_warp(a_full + 8 * as, apar, abort_flag)) {
@@ -342,6 +378,18 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
 #pragma unroll
           for (int i = 0; i < KS / 2; ++i) {
             if (i >= nv) break;
+            if (EXACT) {                                       // (slot = half = accumulator)
+              const uint32_t d = tmem + kExP + 32u * (uint32_t)as;
+              const int kept = HEADS ? c.head_keep - ((v0 + i) % c.head_kb) * BK : BK;
+#pragma unroll
+              for (int k = 0; k < BK / 16; ++k) {
+                const uint32_t more = (i > 0 || k > 0) ? 1u : 0u;
+                umma_ts(d, a0 + 32 * i + 8 * k, bd + i * box_step + 2 * k, c.idesc, more);
+                if (!HEADS || 16 * k < kept)                   // (kept channels are a multiple of 8)
+                  umma_ts(d + 16, tmem + kExOnes + (HEADS && 16 * k + 8 == kept ? 4u : 0u), bd + i * box_step + 2 * k, c.idesc, more);
+              }
+              continue;
+            }
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k)
               umma_ts(tmem, a0 + 32 * i + 8 * k, bd + i * box_step + 2 * k, c.idesc, (v0 > sg.s0 * KS || i > 0 || k > 0) ? 1u : 0u);
@@ -354,7 +402,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
         if (nv > 0 && ++bs == c.bst) { bs = 0; bpar ^= 1; }
       }
       if (failed) break;
-      if (elect_one()) umma_commit(acc_full);
+      if (!EXACT && elect_one()) umma_commit(acc_full);
       __syncwarp();
     }
   } else if (warp < DQ0) {
@@ -433,7 +481,33 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
       if (lane == 0) pmbar_arrive(a_full + 8 * stored_as);
       stored_as = -1;
     };
+    float sum[16], g_s = 0.f, g_cz = 0.f;        // EXACT: the tile's sums, scale and offset of the group whose sums are due
+    bool due = false;
+    auto add_group = [&]() {                     // (behind the wait for the slot whose MMAs these are)
+#pragma unroll
+      for (int k0 = 0; k0 < 16; k0 += 8) {
+        uint32_t v[8], u[8];
+        tmem_ld8(a_lane - (uint32_t)c.a_base + kExP + 32 * half + k0, v);
+        tmem_ld8(a_lane - (uint32_t)c.a_base + kExP + 32 * half + 16 + k0, u);
+        tmem_ld_wait();
+#pragma unroll
+        for (int k = 0; k < 8; ++k) sum[k0 + k] = fmaf(g_s, __uint_as_float(v[k]), fmaf(g_cz, __uint_as_float(u[k]), sum[k0 + k]));
+      }
+    };
+    if (EXACT && half == 0) {                    // (complete before this warp's first arrival for the MMA warp)
+      const uint32_t t = a_lane - (uint32_t)c.a_base + kExOnes;
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(t + 8 * k), "r"(k ? 0u : 0x3c003c00u) : "memory");
+      tmem_st_wait();
+      tc_fence_before();
+    }
     for (int count = 0; !failed && si.next(sg); ++count) {
+      if (EXACT) {
+        due = false;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) sum[k] = 0.f;
+      }
       const int sr = batch_row(c, p, fam_of_tile(c, sg.tile), sg.tile, r).smem_row;
       const uint32_t x_row = (uint32_t)(sr * 128), x_sw = (uint32_t)((half * 4) ^ (sr & 7)) * 16;   // piece i: x_sw ^ (16 i)
       uint32_t w[16];
@@ -473,7 +547,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
           for (int i = j0; i < j0 + 4; ++i) {
             const int k = i & 7;
             const bool kept = !HEADS || k * 8 < (i < 8 ? (valid & 255) : (valid >> 8));
-            const uint4 d = kept ? dequant_word(w[i], s2, cz2) : make_uint4(0, 0, 0, 0);
+            const uint4 d = !kept ? make_uint4(0, 0, 0, 0) : EXACT ? codes_word(w[i]) : dequant_word(w[i], s2, cz2);
             o[4 * k] = d.x; o[4 * k + 1] = d.y; o[4 * k + 2] = d.z; o[4 * k + 3] = d.w;
           }
         };
@@ -485,6 +559,12 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
         if (use > 0 && !pmbar_wait_warp(a_empty + 8 * as, (use - 1) & 1, abort_flag)) { failed = true; break; }
         tc_fence_after();
         tmem_st32(a_lane + (uint32_t)(64 * as), o);
+        if (EXACT) {
+          if (due) add_group();
+          g_s = __half2float(sc);
+          g_cz = (8.f - __half2float(zp)) * g_s;
+          due = st * KS + half * (KS / 2) < c.n_kb;
+        }
         convert(8);
         convert(12);
         release();
@@ -498,6 +578,21 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
       announce();
       asm volatile("griddepcontrol.wait;" ::: "memory");       // outputs, positions and workspace: after the preceding kernel
       const RowStore<T> rs = row_store(sg.tile);               // (several dependent loads, while the last MMAs run)
+      if (EXACT) {
+        if (!pmbar_wait_warp(a_empty + 8 * as, (use - 1) & 1, abort_flag)) { failed = true; break; }
+        tc_fence_after();
+        if (due) add_group();
+        if (count >= 1 && !pmbar_wait_warp(acc_empty, (count - 1) & 1, abort_flag)) { failed = true; break; }
+        tc_fence_after();
+        uint32_t v[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = __float_as_uint(sum[k]);
+        tmem_st16(a_lane - (uint32_t)c.a_base + 16 * half, v);
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) pmbar_arrive(acc_full);
+      }
       if (!pmbar_wait_warp(acc_full, count & 1, abort_flag)) { failed = true; break; }
       epilogue_tile(rs, count, half);
     }
@@ -554,9 +649,10 @@ int batch_families(const Params& p, BatchCfg* c) {
 }
 
 typedef void (*BatchKernel)(Params, BatchCfg);
-BatchKernel batch_instance(bool bf16, bool heads) {
-  if (bf16) return heads ? batch_kernel<__nv_bfloat16, true> : batch_kernel<__nv_bfloat16, false>;
-  return heads ? batch_kernel<__half, true> : batch_kernel<__half, false>;
+BatchKernel batch_instance(bool bf16, bool heads, bool exact) {
+  if (bf16) return heads ? batch_kernel<__nv_bfloat16, true, false> : batch_kernel<__nv_bfloat16, false, false>;
+  if (exact) return heads ? batch_kernel<__half, true, true> : batch_kernel<__half, false, true>;
+  return heads ? batch_kernel<__half, true, false> : batch_kernel<__half, false, false>;
 }
 
 struct BLaunch {
@@ -594,8 +690,8 @@ int residency(Residency* out) {
   std::lock_guard<std::mutex> lock(mu);
   Residency& r = dev_res[dev];
   if (!r.known) {
-    for (int k = 0; k < 4; ++k)
-      if (cudaFuncSetAttribute(batch_instance(k & 1, k & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone) != cudaSuccess)
+    for (int k = 0; k < 8; ++k)
+      if (cudaFuncSetAttribute(batch_instance(k & 1, k & 2, k & 4), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone) != cudaSuccess)
         return UNIQL_ERR_CUDA;
     const int sms = device_sms();
     r.clusters[0] = 0;
@@ -603,7 +699,7 @@ int residency(Residency* out) {
     for (int p = 2; p <= kMaxP; ++p) {
       BLaunch l(2 * sms / p * p, p, kSmemBatch, nullptr);
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, batch_instance(false, false), &l.lc) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      if (cudaOccupancyMaxActiveClusters(&n, batch_instance(false, false, false), &l.lc) != cudaSuccess) { cudaGetLastError(); n = 0; }
       r.clusters[p] = n < 2 * sms / p ? n : 2 * sms / p;
     }
     r.known = true;
@@ -630,6 +726,25 @@ int batch_supported(const Params& p) {
   return batch_families(p, nullptr) > 0;
 }
 
+// Whether an fp16 launch of up to 16 rows goes to the EXACT instance instead of the decode kernel.  From twelve rows: the
+// decode kernel's activation traffic grows with the rows (a layer 8 - 12 % from nine to sixteen), this instance's does not,
+// and they meet between nine and fifteen rows depending on the shape.  Measured at 12 / 16 rows, decode kernel -> here, the
+// whole layer in microseconds: Qwen2.5-7B 84 -> 75 / 90 -> 75, Mamba2-2.7B 29.1 -> 23.3 / 32.1 -> 23.2, Llama-3-8B 75.9 -> 75.2 /
+// 79.2 -> 74.9, at keep 0.75 - / 75.8 -> 66.5, at keep 0.65 68.3 -> 70.5 / 72.7 -> 70.3.
+// Not where kept blocks of output rows are no multiple of 8: the launch that reads those channels then stays on the decode
+// kernel (4-channel boundaries), whose blocks need a whole SM and cannot come in beside this kernel's (Mamba2 mixer at keep
+// 0.8 29.5 -> 30.7 us).  Rotated heads excepted: there the other four launches of a layer outweigh that.
+int exact_batch(const Params& p) {
+  if (p.dt != UNIQL_F16 || p.M < 12 || p.M > 16 || !batch_supported(p) || !prefill_supported(p)) return 0;
+  if (opt(kOptDecodeSplitBatch) != 2 || opt(kOptDecodeXstream) == 0 || opt(kOptDecodeI8) == 0) return 0;   // asked for by name
+  for (int j = 0; j < p.n_jobs; ++j) {
+    if (p.n_jobs > 1 && p.job[0].rope.enabled) break;
+    for (int k = 0; k < p.job[j].omap.n_fam; ++k)
+      if (p.job[j].omap.fam[k].count > 1 && p.job[j].omap.fam[k].keep % 8 != 0) return 0;
+  }
+  return 1;
+}
+
 // Measured (Llama-3-8B, M = 17 / 64 / 128, against the prefill kernel): q|k|v 18.5 / 21.5 / 21.4 -> 11.5 / 13.0 / 17.2 us, o_proj
 // 20.2 / 24.4 / 27.6 -> 9.1 / 13.2 / 12.0 us, down projection 36 / 36 / 40 -> 18 / 17 / 21 us, whole layer at M = 64 and keep
 // 0.85 137 -> 75 us.  What bounds it now: the issue slots of SMs that hold two tiles (0.65 us per stage and block alone on
@@ -648,8 +763,9 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   c.head_keep = a.keep;
   // fp32 accumulate, A and B fp16, both K-major, N tokens, 128 rows
   c.idesc = (1u << 4) | ((uint32_t)(c.n >> 3) << 17) | ((uint32_t)(BMW >> 4) << 24);
-  c.n_ast = c.n <= 64 ? 3 : 2;
-  c.a_base = c.n <= 64 ? 64 : 128;
+  c.exact = p.M <= 16 && p.dt != UNIQL_BF16;
+  c.n_ast = c.n <= 64 && !c.exact ? 3 : 2;
+  c.a_base = c.exact ? (int)kExA : c.n <= 64 ? 64 : 128;
   // shared memory: two to four half stages of activations, the rest for the codes (HBM's latency is theirs to cover)
   c.bst = c.n > 64 ? 2 : (c.n > 32 ? 3 : 4);
   c.off_w = c.bst * (KS / 2) * c.n * 128;
@@ -712,7 +828,7 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   // with four to eight (q|k|v, o_proj) a launch gains more from loading beside its predecessor (9.0 against 11.5 us).
   if (c.p > 1 && best_clusters * c.p <= device_sms() && c.spt >= 10 * c.p) smem = kSmemAlone;
   BLaunch l(best_clusters * c.p, c.p, smem, cfg.stream);
-  if (cudaLaunchKernelEx(&l.lc, batch_instance(p.dt == UNIQL_BF16, c.head_kb != 0), p, c) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&l.lc, batch_instance(p.dt == UNIQL_BF16, c.head_kb != 0, c.exact != 0), p, c) != cudaSuccess) {
     cudaGetLastError();
     return UNIQL_ERR_CUDA;
   }

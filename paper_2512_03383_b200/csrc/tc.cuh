@@ -295,7 +295,19 @@ __device__ inline uint4 dequant_word(uint32_t w, __half2 s2, __half2 cz2) {
   }
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
-
+// The codes themselves, less 8, as fp16 (exact), in channel order.
+__device__ inline uint4 codes_word(uint32_t w) {
+  uint32_t o[4];
+  const __half2 off = __halves2half2(__ushort_as_half(0x6408), __ushort_as_half(0x5480));
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const uint32_t t = __byte_perm(w, 0u, 0x4040u + 0x0101u * b);
+    const uint32_t v = pand_or(t, 0x00f0000fu, 0x54006400u);
+    const __half2 r = __hsub2(*reinterpret_cast<const __half2*>(&v), off);
+    o[b] = *reinterpret_cast<const uint32_t*>(&r);
+  }
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
 
 // ---------------------------------------------------------------------------------------- epilogue of a row
 // Bias, rotary embedding (Section 3.2, fused RoPE) or gated product, one rounding and the stores of a thread that owns

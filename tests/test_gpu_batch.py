@@ -31,3 +31,29 @@ def test_long_contractions(B, M, split):
     assert B.workspace_status() == 0
     B.set_path(B.PATH_AUTO)
     B.reset_options()
+
+
+@pytest.mark.parametrize("M", [1, 12, 15, 16])
+@pytest.mark.parametrize("N,K,take", [(8, 256, 256), (136, 1024, 1000), (640, 8192, 8192), (1500, 4096, 3976), (200, 1024, "72"),
+                                      (200, 1024, "104"), (328, 2048, "96"), (130, 1024, "128")])
+@pytest.mark.parametrize("split", [0, -1])
+def test_exact_codes(B, M, N, K, take, split):
+    """Up to 16 fp16 rows; `take`: leading channels, or the kept channels of heads of 128.  Codes and activations enter
+    unrounded, so beyond the output's rounding only fp32 sums remain: 8 + K / 128 <= 72 of them in a chain, 2^-23 each of
+    sum |terms|, which is up to 25 times the largest output: 2.2e-4."""
+    B.set_path(B.PATH_PREFILL)
+    B.set_option("prefill_streamk", split)
+    rng = np.random.default_rng(7 * M + N + K)
+    qw = synth.random_qweight_fast(rng, N, K)
+    dw = dev_weight(qw)
+    im = synth.map_per_head(K // 128, 128, int(take)) if isinstance(take, str) else None
+    k_in = 0 if im else take
+    x = synth.draw_x(rng, M, synth.map_size(im) if im else k_in, "f16")
+    y, ref = run_ex(B, qw, dw, x, "f16", im, k_in, None, N)
+    check_output(y, ref, "f16", 3e-4, "M=%d N=%d K=%d %s" % (M, N, K, take))
+    for _ in range(5):
+        again, _ = run_ex(B, qw, dw, x, "f16", im, k_in, None, N)
+        assert torch.equal(again, y)
+    assert B.workspace_status() == 0
+    B.set_path(B.PATH_AUTO)
+    B.reset_options()
