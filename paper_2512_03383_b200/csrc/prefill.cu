@@ -1144,7 +1144,9 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     if (q.tiles < g2) {
       // every tile is split and every block ends on a split tile: the hand-over is shared with the de-quantiser warps
       // (one-box tiles, measured at M = 64 .. 512 on seven layer shapes: 5 us per 64 tokens of the tile)
-      hand_over = nh == 2 ? 24.0 + 2.0 * pmax * wide : (14.0 + pmax) * wide;
+      // (64-token tiles, measured on four shapes with 3 to 52 tiles: 0.9 us for every part that the finishing block adds; a
+      //  contraction of 4744 channels and three tiles took 47 us split over all SMs and 24 us over pairs of blocks)
+      hand_over = nh == 2 ? 24.0 + 2.0 * pmax * wide : c.bn == 64 ? 5.0 + 0.9 * pmax : (14.0 + pmax) * wide;
     } else {
       // The split tiles come first and whole tiles follow.  Reading a tile's slots back takes the four epilogue
       // warps 11 us per slot of 256 tokens, and a split tile in front of whole tiles has three or more parts: that
