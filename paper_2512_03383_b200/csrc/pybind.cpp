@@ -65,10 +65,15 @@ struct Args {
     if (!THPVariable_Check(v[i])) { fail(PyExc_TypeError, "a torch tensor or None is expected", i); return nullptr; }
     return &THPVariable_Unpack(v[i]);
   }
-  // device address of a tensor, NULL for None
+  // device address of a tensor that the call reads, NULL for None
   void* ptr(int i) {
     const at::Tensor* t = tensor(i);
     return t ? const_cast<void*>(t->const_data_ptr()) : nullptr;
+  }
+  // ... that the call writes: a tensor that shares its storage until the first write (a lazy clone) gets its own here
+  void* out(int i) {
+    const at::Tensor* t = tensor(i);
+    return t ? t->mutable_data_ptr() : nullptr;
   }
   long long integer(int i, long long dflt = 0) {
     if (!v[i]) return dflt;
@@ -100,7 +105,7 @@ struct Args {
     const at::Tensor* t = tensor(i);
     if (!t) return nullptr;
     *bytes = (size_t)t->numel() * (size_t)t->element_size();
-    return const_cast<void*>(t->const_data_ptr());
+    return t->mutable_data_ptr();
   }
   void* stream(int i) {
     if (none(i)) return c10::cuda::getCurrentCUDAStream().stream();
@@ -174,7 +179,7 @@ typedef int (*QlinearFn)(const void*, const uint8_t*, const void*, const void*, 
 PyObject* qlinear_as(const char* fn, const char* what, QlinearFn call, PyObject* const* args, Py_ssize_t nargs, PyObject* kwnames) {
   SIGNATURE(R("x"), R("packed_w"), R("scales"), R("zeros"), R("M"), R("K"), R("N"), R("k_in"), R("k_out"), R("y"), O("stream"))
   PARSE(fn)
-  void *x = a.ptr(0), *w = a.ptr(1), *s = a.ptr(2), *z = a.ptr(3), *y = a.ptr(9);
+  void *x = a.ptr(0), *w = a.ptr(1), *s = a.ptr(2), *z = a.ptr(3), *y = a.out(9);
   const int M = a.i32(4), K = a.i32(5), N = a.i32(6), k_in = a.i32(7), k_out = a.i32(8);
   if (!a.ok) return nullptr;
   void* stream = a.stream(10);
@@ -190,7 +195,7 @@ FAST(qlinear_ex) {
   SIGNATURE(R("x"), R("ldx"), R("packed_w"), R("scales"), R("zeros"), R("bias"), R("M"), R("K"), R("N"), R("in_map"),
             R("k_in"), R("out_map"), R("k_out"), R("y"), R("ldy"), O("workspace"), O("stream"))
   PARSE("qlinear_ex")
-  void *x = a.ptr(0), *w = a.ptr(2), *s = a.ptr(3), *z = a.ptr(4), *b = a.ptr(5), *y = a.ptr(13);
+  void *x = a.ptr(0), *w = a.ptr(2), *s = a.ptr(3), *z = a.ptr(4), *b = a.ptr(5), *y = a.out(13);
   const int ldx = a.i32(1), M = a.i32(6), K = a.i32(7), N = a.i32(8), k_in = a.i32(10), k_out = a.i32(12), ldy = a.i32(14);
   const int dt = a.dtype(0);
   uniql_chanmap im, om;
@@ -231,7 +236,8 @@ FAST(qlinear_multi) {
       PyObject* o = item(key, required);
       if (!o || (o == Py_None && !required)) return nullptr;
       if (!THPVariable_Check(o)) { if (a.ok) PyErr_Format(PyExc_TypeError, "job %d: %s: a torch tensor is expected", j, key); a.ok = false; return nullptr; }
-      return const_cast<void*>(THPVariable_Unpack(o).const_data_ptr());
+      const at::Tensor& v = THPVariable_Unpack(o);
+      return strcmp(key, "y") == 0 ? v.mutable_data_ptr() : const_cast<void*>(v.const_data_ptr());
     };
     auto number = [&](const char* key, bool required) -> int32_t {
       PyObject* o = item(key, required);
@@ -267,7 +273,7 @@ FAST(qk_rope_proj) {
   void* p[10];
   for (int i = 0; i < 10; ++i) p[i] = i == 1 ? nullptr : a.ptr(i);
   const int ldx = a.i32(1), M = a.i32(10), K = a.i32(11), hq = a.i32(12), hkv = a.i32(13), hd = a.i32(14), keep = a.i32(15);
-  void *idx = a.ptr(16), *pos = a.ptr(17), *q = a.ptr(20), *k = a.ptr(22);
+  void *idx = a.ptr(16), *pos = a.ptr(17), *q = a.out(20), *k = a.out(22);
   const double theta = a.real(18);
   double buf[512] = {0};
   const double* f = a.table(19, buf, 512);
@@ -292,7 +298,7 @@ FAST(qkv_rope_proj) {
   for (int i = 0; i < 14; ++i) p[i] = i == 1 ? nullptr : a.ptr(i);
   const int ldx = a.i32(1), M = a.i32(14), K = a.i32(15), hq = a.i32(16), hkv = a.i32(17), hd = a.i32(18), keep = a.i32(19),
             vkeep = a.i32(20);
-  void *idx = a.ptr(21), *pos = a.ptr(22), *q = a.ptr(25), *k = a.ptr(27), *v = a.ptr(29);
+  void *idx = a.ptr(21), *pos = a.ptr(22), *q = a.out(25), *k = a.out(27), *v = a.out(29);
   const double theta = a.real(23);
   double buf[512] = {0};
   const double* f = a.table(24, buf, 512);
@@ -315,7 +321,7 @@ FAST(mlp_swiglu_decode) {
   void* p[11];
   for (int i = 0; i < 11; ++i) p[i] = i == 1 ? nullptr : a.ptr(i);
   const int ldx = a.i32(1), M = a.i32(11), hidden = a.i32(12), inter = a.i32(13), k_int = a.i32(14), ldh = a.i32(16), ldy = a.i32(18);
-  void *h = a.ptr(15), *y = a.ptr(17);
+  void *h = a.out(15), *y = a.out(17);
   const int fuse = a.i32(19, -1);
   for (int i : {0, 15, 17})
     if (a.ok && a.tensor(i) && a.tensor(i)->scalar_type() != at::kHalf) {
@@ -340,7 +346,7 @@ FAST(mlp_swiglu) {
   void* p[11];
   for (int i = 0; i < 11; ++i) p[i] = i == 1 ? nullptr : a.ptr(i);
   const int ldx = a.i32(1), M = a.i32(11), hidden = a.i32(12), inter = a.i32(13), k_int = a.i32(14), ldh = a.i32(16), ldy = a.i32(18);
-  void *h = a.ptr(15), *y = a.ptr(17);
+  void *h = a.out(15), *y = a.out(17);
   const int dt = a.dtype(0);
   for (int i : {15, 17})
     if (a.ok && a.tensor(i) && a.tensor(i)->scalar_type() != a.tensor(0)->scalar_type()) {
@@ -363,14 +369,14 @@ FAST(embed_rows) {
   for (int i : {0, 3, 4})
     if (!a.tensor(i)) { a.fail(PyExc_TypeError, "a torch tensor is expected", i); return nullptr; }
   const at::Tensor &packed = *a.tensor(0), &ids = *a.tensor(3), &out = *a.tensor(4);
-  void *s = a.ptr(1), *z = a.ptr(2), *bad = a.ptr(5);
+  void *s = a.ptr(1), *z = a.ptr(2), *bad = a.out(5);
   const int dt = a.dtype(4);
   if (!a.ok) return nullptr;
   if (packed.dim() != 2 || out.dim() < 1) { PyErr_SetString(PyExc_ValueError, "embed_rows: packed is [V][K/2], out [M][K]"); return nullptr; }
   void* stream = a.stream(6);
   if (!a.ok) return nullptr;
   return DONE(uniql_embed_rows((const uint8_t*)packed.const_data_ptr(), s, z, packed.size(0), packed.size(1) * 2,
-                               (const int32_t*)ids.const_data_ptr(), ids.numel(), dt, const_cast<void*>(out.const_data_ptr()),
+                               (const int32_t*)ids.const_data_ptr(), ids.numel(), dt, out.mutable_data_ptr(),
                                out.stride(0), (int*)bad, stream), "uniql_embed_rows");
 }
 

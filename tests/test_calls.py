@@ -37,3 +37,26 @@ def test_status_travels_with_the_error():
     with pytest.raises(B.UniqlError) as e:
         B.embed_rows(W, S, S, torch.zeros(2, dtype=torch.int32), X[:, :64].contiguous(), stream=0)      # rows narrower than K
     assert e.value.status == 2
+
+
+@pytest.mark.parametrize("fn, written", [
+    (lambda y, w: B.qlinear(X, W, S, S, 1, 100, 16, 100, 16, y, stream=0), 1),
+    (lambda y, w: B.qlinear_noalloc(X, W, S, S, 1, 100, 16, 100, 16, y, stream=0), 1),
+    (lambda y, w: B.qlinear_ex(X, 128, W, S, S, None, 1, 100, 16, None, 100, None, 16, y, 16, workspace=w, stream=0), 2),
+    (lambda y, w: B.qlinear_multi(X, 128, 1, 100, None, 100, [dict(packed_w=W, scales=S, zeros=S, N=16, k_out=16, y=y, ldy=16)],
+                                  workspace=w, stream=0), 2),
+    (lambda y, w: B.qk_rope_proj(X, 128, W, S, S, W, S, S, None, None, 1, 100, 1, 1, 16, 16, S, S, 1e4, None, y, 16, w, 16, stream=0), 2),
+    (lambda y, w: B.qkv_rope_proj(X, 128, W, S, S, W, S, S, W, S, S, None, None, None, 1, 100, 1, 1, 16, 16, 16, S, S, 1e4, None, y, 16,
+                                  y, 16, w, 16, stream=0), 2),
+    (lambda y, w: B.mlp_swiglu(X, 128, W, S, S, W, S, S, W, S, S, 0, 128, 128, 128, y, 128, w, 128, stream=0), 2),
+    (lambda y, w: B.mlp_swiglu_decode(X, 128, W, S, S, W, S, S, W, S, S, 0, 128, 128, 128, y, 128, w, 128, stream=0), 2),
+    (lambda y, w: B.embed_rows(W, S, S, torch.zeros(2, dtype=torch.int32), y[:, :64], bad_id=w, stream=0), 2),
+])
+def test_written_tensors_own_their_storage(fn, written):
+    """A lazy clone shares its storage until it is written to: what a call writes must not land in the tensor it was cloned
+    from.  (Every call here is refused for its shapes, after its addresses were taken.)"""
+    for w_only in range(written):
+        y, w = torch._lazy_clone(X), torch._lazy_clone(X)
+        with pytest.raises(B.UniqlError):
+            fn(y, w)
+        assert not torch._C._is_cow_tensor(w if w_only else y)
