@@ -57,3 +57,23 @@ def test_exact_codes(B, M, N, K, take, split):
     assert B.workspace_status() == 0
     B.set_path(B.PATH_AUTO)
     B.reset_options()
+
+
+@pytest.mark.parametrize("M,dtype", [(12, "f16"), (12, "bf16"), (40, "f16"), (40, "bf16"), (128, "f16"), (128, "bf16")])
+@pytest.mark.parametrize("heads", [False, True])
+def test_code_ring_wraps_in_every_instance(B, M, dtype, heads):
+    """A whole contraction per block (32 stages in rings of two to six), plain and per-head, both types, codes multiplied as
+    they are and rounded to fp16: a slot handed back before its codes were read shows as wrong rows."""
+    B.set_path(B.PATH_PREFILL)
+    B.set_option("prefill_streamk", 0)
+    rng = np.random.default_rng(2500 + M)
+    N, K = 700, 8192
+    qw = synth.random_qweight_fast(rng, N, K)
+    dw = dev_weight(qw)
+    im = synth.map_per_head(K // 128, 128, 104) if heads else None
+    x = synth.draw_x(rng, M, synth.map_size(im) if im else K, dtype)
+    y, ref = run_ex(B, qw, dw, x, dtype, im, 0 if im else K, None, N)
+    check_output(y, ref, dtype, TOL, "M=%d %s heads %d" % (M, dtype, heads))
+    assert B.workspace_status() == 0
+    B.set_path(B.PATH_AUTO)
+    B.reset_options()
