@@ -139,7 +139,17 @@ int relay_candidate(const Params& p, Params* q) {
 int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, void* stream) {
   LaunchCfg cfg{workspace, ws_bytes, (cudaStream_t)stream};
   Params p = p_in;
-  bool dec_ok = p.M <= 16 && decode_supported(p);
+  // The rows of a decode launch: option "decode_split_batch" (or streaming turned off) runs nine to sixteen rows as two
+  // launches, and what those can take is asked for them (five to eight rows need activations on 8-channel boundaries).
+  const bool streams = opt(kOptDecodeSplitBatch) == 2 && opt(kOptDecodeI8) != 0 && opt(kOptDecodeXstream) != 0;
+  auto as_launched = [&](const Params& a) {
+    Params q = a;
+    if (q.M > 8 && q.M <= 16 && !streams && opt(kOptDecodeSplitBatch) != 0) q.M = (q.M + 1) / 2;
+    return q;
+  };
+  auto decodes = [&](const Params& a) { return a.M <= 16 && decode_supported(as_launched(a)); };
+  auto on_integers = [&](const Params& a) { return decode_integer_path(as_launched(a)) != 0; };
+  bool dec_ok = decodes(p);
   // every batch the decode kernel does not take (more than 16 rows) goes to the tensor cores when the maps
   // allow it: at 17..63 rows the generic kernel measured 13 to 26 times slower (930 us against 71 us for the
   // Llama-3-8B gate|up at M = 17)
@@ -147,7 +157,7 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
   // The streaming kernel (one to four rows): where it is asked for, and where the decode kernel's integer path cannot run
   // (scales on 8- but not 16-byte boundaries).
   bool gv = path == UNIQL_PATH_GEMV || (path == UNIQL_PATH_AUTO && gemv_supported(p) && opt(kOptGemvFirst) == 1);
-  const bool gv_else = path == UNIQL_PATH_AUTO && !gv && gemv_supported(p) && !(dec_ok && decode_integer_path(p));
+  const bool gv_else = path == UNIQL_PATH_AUTO && !gv && gemv_supported(p) && !(dec_ok && on_integers(p));
   bool relaid = false;
   // What misses a fast kernel only because of where its activations lie (above 16 rows blocks of 108 or 84 channels, at
   // decode sizes blocks that are no multiple of 4, an odd row pitch) gets them re-laid in the workspace by a small kernel
@@ -158,11 +168,11 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
     int keep8 = 0;
     // (bf16 at decode sizes that the integer path cannot take even re-laid: the tensor cores, as larger batches)
     if (decode_size && p.dt != UNIQL_F16 && path == UNIQL_PATH_AUTO && !dec_ok &&
-        !(relay_candidate(p, &q) != 0 && decode_supported(q)))
+        !(relay_candidate(p, &q) != 0 && decodes(q)))
       decode_size = false;
-    const bool slow = decode_size ? !(dec_ok && decode_integer_path(p)) : !pre_ok;
+    const bool slow = decode_size ? !(dec_ok && on_integers(p)) : !pre_ok;
     if (slow && path != (decode_size ? UNIQL_PATH_PREFILL : UNIQL_PATH_DECODE) && (keep8 = relay_candidate(p, &q)) != 0 &&
-        (decode_size ? (decode_supported(q) && decode_integer_path(q)) : prefill_supported(q))) {
+        (decode_size ? (decodes(q) && on_integers(q)) : prefill_supported(q))) {
       if (!cfg.workspace) {
         int rc = lib_workspace(&cfg.workspace, &cfg.ws_bytes, cfg.stream);
         if (rc != UNIQL_OK) return rc;
@@ -180,7 +190,7 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
         p = q;
         relaid = true;
         cfg.ws_bytes = off;
-        dec_ok = p.M <= 16 && decode_supported(p);
+        dec_ok = decodes(p);
         pre_ok = prefill_supported(p);
       }
     }
@@ -204,7 +214,7 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
     return launch_gemv(p, cfg);
   }
   if (path == UNIQL_PATH_DECODE) {
-    if (!(p.M <= 16 && decode_supported(p))) return UNIQL_ERR_UNSUPPORTED;
+    if (!decodes(p)) return UNIQL_ERR_UNSUPPORTED;
     if (!cfg.workspace) {
       int rc = lib_workspace(&cfg.workspace, &cfg.ws_bytes, cfg.stream);
       if (rc != UNIQL_OK) return rc;

@@ -117,3 +117,21 @@ def test_fp16_mma_path_of_the_decode_kernel(B, M):
         x = synth.draw_x(rng, M, k_in, "f16")
         y, ref = run(B, qw, dw, x, "f16", None, k_in)
         check_output(y, ref, "f16", 4e-4, "fp16 MMA path k_in=%d M=%d" % (k_in, M))
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("option,value", [("decode_split_batch", 1), ("decode_split_batch", 0), ("decode_xstream", 0)])
+@pytest.mark.parametrize("M", [9, 13, 16])
+def test_batches_run_as_two_halves(B, M, option, value, dtype):
+    """Nine to sixteen rows on 4-channel boundaries with the options that turn the single launch off: what the halves (five to
+    eight rows) cannot take is re-laid for them, not refused."""
+    B.set_option(option, value)
+    rng = np.random.default_rng(860 + M)
+    qw = synth.draw_qweight(rng, 256, 1024)
+    dw = dev_weight(qw)
+    for path in (B.PATH_AUTO, B.PATH_DECODE):
+        B.set_path(path)
+        for in_map, k_in in ((synth.map_per_head(8, 128, 108), 0), (None, 876)):
+            x = synth.draw_x(rng, M, synth.map_size(in_map) if in_map else k_in, dtype)
+            y, ref = run(B, qw, dw, x, dtype, in_map, k_in, ldx_pad=4)
+            check_output(y, ref, dtype, TOL["decode"], "%s %s=%d M=%d %s" % (dtype, option, value, M, in_map))
