@@ -588,6 +588,7 @@ int mlp_block(const void* x, int ldx, int dt, const uint8_t* wg, const void* sg,
   d.sg = (const __half*)sg; d.zg = (const __half*)zg; d.su = (const __half*)su; d.zu = (const __half*)zu;
   d.sd = (const __half*)sd; d.zd = (const __half*)zd;
   d.h = h; d.ldh = ldh; d.y = y; d.ldy = ldy;
+  d.decode_only = g_path.load() == UNIQL_PATH_DECODE;
   if (dt != UNIQL_F16) {
     // bf16: the decode kernel where its rules and the workspace allow it, else the tensor cores as for larger batches
     const bool too_small = workspace && ws_bytes < mlp_decode_workspace_bytes(M, hidden, inter);

@@ -741,7 +741,10 @@ int batch_supported(const Params& p) {
 // 0.8 29.5 -> 30.7 us).  Rotated heads excepted: there the other four launches of a layer outweigh that.
 int exact_batch(const Params& p) {
   if (p.dt != UNIQL_F16 || p.M < 12 || p.M > 16 || !batch_supported(p) || !prefill_supported(p)) return 0;
-  if (opt(kOptDecodeSplitBatch) != 2 || opt(kOptDecodeXstream) == 0 || opt(kOptDecodeI8) == 0) return 0;   // asked for by name
+  // (an option of the decode kernel that is set asks for that kernel)
+  if (opt(kOptDecodeKp) != 0 || opt(kOptDecodeRp) != 0 || opt(kOptDecodeStages) != 0 || opt(kOptDecodeNarrow) != -1 || opt(kOptDecodeXstream) != -1 ||
+      opt(kOptDecodeXcluster) != -1 || opt(kOptDecodeI8) != 1 || opt(kOptDecodeSplitBatch) != 2)
+    return 0;
   for (int j = 0; j < p.n_jobs; ++j) {
     if (p.n_jobs > 1 && p.job[0].rope.enabled) break;
     for (int k = 0; k < p.job[j].omap.n_fam; ++k)

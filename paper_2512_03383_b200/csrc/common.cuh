@@ -175,6 +175,7 @@ struct MlpDecode {
   const __half *sg, *zg, *su, *zu, *sd, *zd;
   void* h; int ldh;            // [M][k_int]: the gated activations (written, then read)
   void* y; int ldy;            // [M][hidden]
+  int decode_only;             // the decode kernel was asked for: no product goes to another one
 };
 // fuse != 0: both products in one launch (UNIQL_ERR_UNSUPPORTED when the shapes do not allow it);
 // fuse == 0: two launches.

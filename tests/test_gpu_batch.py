@@ -77,3 +77,25 @@ def test_code_ring_wraps_in_every_instance(B, M, dtype, heads):
     assert B.workspace_status() == 0
     B.set_path(B.PATH_AUTO)
     B.reset_options()
+
+
+@pytest.mark.parametrize("option,value", [("decode_kp", 2), ("decode_rp", 20), ("decode_stages", 2), ("decode_xstream", 1),
+                                          ("decode_split_batch", 1), ("decode_i8", 0)])
+def test_options_of_the_decode_kernel_ask_for_it(B, option, value):
+    """The automatic choice at twelve to sixteen rows is the batch kernel, unless an option of the decode kernel is set: then
+    the bits are those of the decode kernel."""
+    rng = np.random.default_rng(2600)
+    qw = synth.random_qweight_fast(rng, 300, 2048)
+    dw = dev_weight(qw)
+    x = synth.draw_x(rng, 16, 2048, "f16")
+    B.set_option(option, value)
+    got = []
+    for path in (B.PATH_AUTO, B.PATH_DECODE):
+        B.set_path(path)
+        y, ref = run_ex(B, qw, dw, x, "f16", None, 2048, None, 300)
+        check_output(y, ref, "f16", TOL, "%s=%d path %d" % (option, value, path))
+        got.append(y.clone())
+    B.reset_options()
+    B.set_path(B.PATH_AUTO)
+    batch, _ = run_ex(B, qw, dw, x, "f16", None, 2048, None, 300)
+    assert torch.equal(got[0], got[1]) and not torch.equal(got[0], batch)

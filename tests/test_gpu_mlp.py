@@ -113,9 +113,10 @@ def test_typed_entry_point(B, small, M, dtype):
 @pytest.mark.parametrize("mode", [2, 1, 0])
 @pytest.mark.parametrize("M", [9, 11, 16])
 def test_batches_above_eight(B, small, M, mode):
-    """Nine to sixteen rows: one pass with streamed activations (2, the default), two passes over half the batch (1),
-    one pass with staged activations (0)."""
+    """Nine to sixteen rows on the decode kernel: one pass with streamed activations (2, the default), two passes over half
+    the batch (1), one pass with staged activations (0)."""
     B.set_option("decode_split_batch", mode)
+    B.set_path(B.PATH_DECODE)
     _, qs, ds = small
     x = synth.draw_x(np.random.default_rng(200 + M), M, 512, "f16")
     for fuse in (-1, 0):
@@ -123,8 +124,26 @@ def test_batches_above_eight(B, small, M, mode):
             h, h_ref, y, y_ref = run_mlp(B, qs, ds, x, k_int, fuse, pad=8)
             check_output(h, h_ref, "f16", TOL_H, "h M=%d mode %d k_int %d" % (M, mode, k_int))
             check_output(y, y_ref, "f16", TOL_Y, "y M=%d mode %d k_int %d" % (M, mode, k_int))
+    B.set_path(B.PATH_AUTO)
+    if mode == 2:                                          # (twelve rows and more: the batch kernel)
+        h, h_ref, y, y_ref = run_mlp(B, qs, ds, x, 872, -1, pad=8)
+        check_output(h, h_ref, "f16", TOL_H, "h M=%d automatic" % M)
+        check_output(y, y_ref, "f16", TOL_Y, "y M=%d automatic" % M)
     with pytest.raises(RuntimeError):                      # one launch holds at most eight batch rows
         run_mlp(B, qs, ds, x, 872, 1)
+
+
+@pytest.mark.parametrize("M", [9, 16])
+def test_forced_decode_path_keeps_both_products(B, small, M):
+    """bf16 at nine to sixteen rows: the automatic choice for the down projection is another kernel; the forced path is not."""
+    _, _, ((_, wg, sg, zg), (_, wu, su, zu), (_, wd, sd, zd)) = small
+    xd = dev_x(synth.draw_x(np.random.default_rng(500 + M), M, 512, "bf16"), "bf16")
+    h, y, y2 = (torch.zeros((M, n), device="cuda", dtype=torch.bfloat16) for n in (872, 512, 512))
+    B.set_path(B.PATH_DECODE)
+    B.mlp_swiglu(xd, 512, wg, sg, zg, wu, su, zu, wd, sd, zd, M, 512, 1024, 872, h, 872, y, 512)
+    B.qlinear_ex(h, 872, wd, sd, zd, None, M, 1024, 512, None, 872, None, 512, y2, 512)
+    B.set_path(B.PATH_AUTO)
+    assert B.workspace_status() == 0 and torch.equal(y, y2), "the down projection left the decode kernel"
 
 
 def test_repeated_calls_own_workspace_and_bitwise_repeatability(B, small):
