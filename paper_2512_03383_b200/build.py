@@ -10,7 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libuniql.so")
 CALLS = os.path.join(HERE, "_calls.so")
-SOURCES = ["api.cu", "util_kernels.cu", "generic.cu", "decode.cu", "gemv.cu", "prefill.cu", "batch.cu", "noalloc.cu"]
+SOURCES = ["api.cu", "util_kernels.cu", "generic.cu", "decode.cu", "gemv.cu", "prefill.cu", "single.cu", "batch.cu", "noalloc.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
               "-Xcompiler", "-fPIC", "--use_fast_math=false"]
 

@@ -1,189 +1,52 @@
-// Prefill kernel (more than 128 rows, and smaller batches that neither the decode nor the batch kernel takes) of the pruned 4-bit
-// linear layer, sm_100a: a dense contraction on
-// the fifth-generation tensor cores (tcgen05.mma, accumulators in tensor memory).
+// Block pairs (clusters of two blocks on tiles of 256 weight rows with cta_group::2 MMAs) and the planner of the tensor-core
+// kernels described in prefill.cuh.
 //
-// Orientation.  The packed weights are four times smaller than the activations, so the weight side
-// takes the MMA's M dimension (128 retained weight rows per tile, de-quantised once per tile and
-// k-block) and the tokens its N dimension (up to 256 per tile): D[row][token] += W[row][k] x[token][k].
-//
-// Roles inside a block (one persistent block per SM, tiles taken round-robin):
-//   warp 0       TMA producer: boxes [64 k x BN tokens] of activations into a ring of four (128-byte swizzle);
-//                one box per k-block, or two where a tile takes both accumulators (512 tokens)
-//   warp 1       allocates tensor memory; one lane issues the MMAs of a k-block (4 x K=16 per box) and commits
-//                them to the box's and the weight stage's "empty" barriers and, at the end of a tile, to
-//                "accumulator full"
-//   warps 4..7   epilogue: tcgen05.ld the fp32 accumulators (warp w owns TMEM lanes 32(w-4).., a lane
-//                is a tile row and holds 32 tokens of it per pass), bias, rotary embedding on the
-//                retained pair (Section 3.2; the pair's two rows are neighbouring lanes and swap
-//                values by shuffle), one rounding, stores of 32 consecutive outputs of a token per
-//                warp; two accumulator buffers of 256 columns let the epilogue of tile i overlap
-//                the MMAs of tile i+1 (tiles of 512 tokens use both and hand them back one by one);
-//                the epilogue of a block's last tile is shared with the de-quantiser warps, idle by then
-//   warps 8..23  de-quantisers: the twelve of them whose scheduler does not host the MMA warp (warp % 4 != 1), two
-//                teams of six warps on alternate stages; a thread converts 32 codes of a weight row per item --
-//                nibbles to fp16 by magic number, (q-8) exact, then one fp16 FMA (q-8)*s + fp16(s*(8-z))
-//                -- and writes them into the A-operand stage in the
-//                canonical K-major 128-byte-swizzled layout; the packed codes of the next k-block
-//                are already in registers.  All sixteen share the epilogue of the block's last segment.
-// Work split (chosen by the launcher from a cost model): whole tiles round-robin; tiles left over after the whole
-// rounds split along K over all blocks (stream-K: parts handed over through slots in the workspace, or added into
-// one sum per tile) or, for tiles of two boxes, run as half tiles on twice the blocks; launches with few tiles as
-// clusters of two blocks per tile, the second block's sums written into the first one's idle rings.
-// Above 128 rows (PAIR instances): clusters of two blocks run tiles of 256 weight rows with cta_group::2 MMAs, one or two boxes
-// of 256 tokens per tile; launches with few tiles as clusters of two to four such pairs per tile, a part of the contraction
-// each.  Measured: Qwen2.5-7B gate at M = 2048 227 -> 193 us (1.44 PFLOP/s), 4096 x 4096 at M = 256 27 -> 19 us.
-// Launched with programmatic stream serialization: what a block does before griddepcontrol.wait (barriers, tensor
-// memory, the first weight stages) touches nothing a preceding kernel may still read or write.
-// On-device pruning (Section 3.4) is index arithmetic: tile rows are compact output channels mapped to
-// stored rows per thread; the input side is the leading k_in channels (the TMA tensor ends at k_in, so
-// the tail of the last k-block is zero activations).
-// bf16 activations: bf16 weights would carry 2^-9 relative rounding error each, which alone spends the
-// 2e-3 error budget; instead the de-quantisers convert the activation tile to fp16 in place (exact in
-// fp16's range, saturating beyond) and both operands are fp16.
-//
-// Every mbarrier wait is bounded; on expiry the block raises a flag, every role leaves its loop, the
-// status word of the workspace is set, tensor memory is released and the block returns.
-#include <cuda.h>
-#include <stdlib.h>
+// Work split of the pairs (chosen by the launcher from a cost model): one or two boxes of 256 tokens per tile, whole tiles
+// round-robin; left-over tiles of two boxes as half tiles on twice the pairs; launches with few tiles as clusters of two to
+// four pairs per tile, a part of the contraction each.  Measured against one block per tile: Qwen2.5-7B gate at M = 2048
+// 227 -> 193 us (1.44 PFLOP/s), 4096 x 4096 at M = 256 27 -> 19 us.
 #include <string.h>
 
 #include <atomic>
 #include <mutex>
-#include <type_traits>
 
-#include "tc.cuh"
+#include "prefill.cuh"
 
 namespace uniql {
 namespace {
 
-constexpr int MAXBN = 256;          // tokens per tile (MMA N), at most
-constexpr int PSTAGES = 4;                   // ring of de-quantised weight stages (one k-block each)
-constexpr int BSLOTS = 4;                    // ring of activation boxes (one k-block of MAXBN tokens each)
-// block pairs: stages of weights and the k-block's half boxes (each block holds half of the tokens), one or two of them
+// stages of weights and the k-block's half boxes (each block holds half of the tokens), one or two of them
 constexpr int PSTAGES1 = 6, PSTAGES2 = 4;
-constexpr int A_BYTES = BMW * BK * 2;        // 16 KB
-constexpr int B_BYTES = MAXBN * BK * 2;      // 32 KB
-constexpr int RING_BYTES = PSTAGES * A_BYTES + BSLOTS * B_BYTES;
-constexpr int RING2_BYTES = PSTAGES2 * (A_BYTES + B_BYTES);
-static_assert(PSTAGES1 * (A_BYTES + B_BYTES / 2) == RING2_BYTES, "the pair instances use the same shared memory");
-constexpr int EPI_TOK = 32;                  // tokens per epilogue pass
-constexpr int NWARPS = 24;
-constexpr int PTH = NWARPS * 32;
-constexpr int DQ_WARP0 = 8, DQ_WARPS = 8;      // warps 8 .. 8 + 2 * DQ_WARPS - 1: the de-quantisers and epilogue helpers
-constexpr int DQ_TEAM_WARPS = 6;               // twelve of them convert: two teams of six warps on alternate stages
-constexpr int EPI_WARP0 = 4;
-constexpr int kMaxPJobs = kMaxJobs;
+constexpr int RING_BYTES = PSTAGES2 * (A_BYTES + B_BYTES);
+static_assert(PSTAGES1 * (A_BYTES + B_BYTES / 2) == RING_BYTES, "both widths use the same shared memory");
 
-struct PrefillCfg {
-  CUtensorMap xmap;          // activations: (k, token), box 64 x BN, 128-byte swizzle
-  int bn;                    // tokens per MMA and activation box: 64, 128 or 256
-  int nh;                    // boxes per tile: 2 when the tile takes both accumulators (512 tokens), else 1
-  int n_ttiles;              // token tiles
-  int wtile_begin[kMaxPJobs + 1];   // first weight tile of each job
-  int n_tiles;               // weight tiles (all jobs) x token tiles
-  int n_kb;                  // visited k-blocks of 64: kept blocks of every head, head after head
-  int km_start, km_period;   // input map in k-blocks: first stored block of head 0, stored blocks per head
-  int km_kbh, km_keep;       // kept k-blocks per head (the last may be partly kept), kept channels per head
-  uint32_t idesc;
-  int streamk;               // 1: contiguous ranges of (tile, k-block) units per block; 0: whole tiles round-robin
-  int helpers;               // 1: the de-quantiser warps share the epilogue of the block's last tile
-  int sk_atomic;             // stream-K hand-over: 1 = parts added into one sum per tile (reductions in L2), 0 = a slot per part
-  int pair_split;            // clusters of two blocks on one tile, half of the contraction each; the second block's
-                             // fp32 sums go into the first one's shared memory (the rings, idle by then)
-  int csplit;                // block pairs, one box per tile: pairs (of one cluster) that share a tile's contraction
-  int halves;                // tiles on both accumulators: the tiles left over after the whole rounds run as half tiles
-                             // (one box of 256 tokens each, on twice as many blocks), every block's last segment
-  int* status;
-  int* counters;             // stream-K: arrivals per tile
-  float* partials;           // stream-K: one slot [tokens / 32][128 rows][32 tokens] fp32 per (left-over tile, block) piece
-};
-
-// Work of a block as a sequence of segments (tile, k-blocks [kb0, kb1)): whole tiles t = b, b + grid, ...
-// With stream-K only for as many rounds as fill every block; the k-blocks of the tiles left over are
-// cut into equal contiguous ranges, one per block, so that every SM stays busy however few tiles remain.
-// A block runs its range of the split tiles FIRST: handing over the partial tile and finishing the split
-// tiles then overlap the main loop of the whole tiles that follow instead of standing at the kernel's end.  Blocks stay in step along k (few distinct k offsets are alive at a time, which keeps the
-// activation slices in L2).  Every block adds its fp32 partial tile to the tile's accumulation buffer in the
-// workspace (reductions done in L2); the last of the tile's blocks to arrive reads the sum
-// and finishes the tile.  With more than two blocks on a tile the order of the additions, and so the last
-// bit of the fp32 sum, depends on the order of arrival.
-// Visited k-block v of the input map -> stored k-block, first compact activation column, kept channels in it.
-// One family {start, period, keep, count}: head h keeps channels [0, keep) of its period; a leading block is
-// the case count = 1.  The activation box of a partly kept block also covers the first columns of the next
-// head: the de-quantisers write zeros for the pruned channels of the block, so those columns do not count.
-// Walked without a division per k-block (a division by the kept blocks per head cost the per-head launches 8 us
-// of 52): (head, kept block within the head) of a visited k-block, stepped.
-struct KWalk {
-  int h, r;
-  __device__ inline void start(const PrefillCfg& c, int v) { h = v / c.km_kbh; r = v - h * c.km_kbh; }
-  __device__ inline void step(const PrefillCfg& c, int n) { r += n; while (r >= c.km_kbh) { r -= c.km_kbh; ++h; } }
-  __device__ inline int stored(const PrefillCfg& c) const { return c.km_start + h * c.km_period + r; }
-  __device__ inline int xcol(const PrefillCfg& c) const { return h * c.km_keep + r * BK; }
-  __device__ inline int valid(const PrefillCfg& c) const { return min(BK, c.km_keep - r * BK); }
-};
-
-// half: -1 the whole tile; 0 / 1: only the first / second box of a tile of two boxes (into accumulator 0 / 1)
-struct Seg { int tile, kb0, kb1, half; };
+// Work of a pair as a sequence of segments: whole tiles t = b, b + grid, ..., the ones left over after the whole rounds as
+// halves, or a part of one tile's k-blocks (part >= 0: which of the pairs that share the tile this one is).
 struct SegIter {
-  long u, ue;
-  int t, t_end, n_kb, step, tail_tile0, half_tile, half, ps_tile, ps_kb0, ps_kb1;
-  // part: which of the pairs that share a tile's contraction this one is (-1: tiles are not shared)
+  int t, t_end, n_kb, step, half_tile, half, part_tile, part_kb0, part_kb1;
   __device__ inline void init(const PrefillCfg& c, int b, int grid, int part) {
-    n_kb = c.n_kb; step = grid; t = b;
-    half_tile = -1; half = 0;
-    ps_tile = -1;
-    if (c.pair_split) {
-      // block 2t takes the first k-blocks of tile t and finishes it, block 2t + 1 the rest (the smaller half)
-      t_end = 0; tail_tile0 = 0; u = ue = 0; t = 1;
-      ps_tile = b >> 1;
-      const int mid = n_kb - n_kb / 2;
-      ps_kb0 = (b & 1) ? mid : 0;
-      ps_kb1 = (b & 1) ? n_kb : mid;
-      return;
-    }
+    n_kb = c.n_kb; step = grid; t = b; t_end = c.n_tiles;
+    half_tile = part_tile = -1;
+    half = 0;
     if (part >= 0) {
-      // one tile per cluster, a part of its k-blocks per pair
-      t_end = 0; tail_tile0 = 0; u = ue = 0; t = 1;
-      ps_tile = b;
-      ps_kb0 = n_kb * part / c.csplit; ps_kb1 = n_kb * (part + 1) / c.csplit;
-      return;
-    }
-    if (c.halves) {
-      // whole rounds of whole tiles, then tile (rounds * grid + b / 2) as two halves on blocks b and b + 1
-      const int full = (c.n_tiles / grid) * grid;
-      t_end = full; tail_tile0 = full; u = ue = 0;
-      if (full + b / 2 < c.n_tiles) { half_tile = full + b / 2; half = b & 1; }
-      return;
-    }
-    const int base = c.streamk ? c.n_tiles / grid : (c.n_tiles + grid - 1) / grid;
-    t_end = c.streamk ? base * grid : c.n_tiles;
-    tail_tile0 = base * grid;
-    u = ue = 0;
-    if (c.streamk) {
-      const long Ut = (long)(c.n_tiles - tail_tile0) * c.n_kb;
-      const long Bt = grid < Ut ? grid : Ut;
-      if (b < Bt) { u = Ut * b / Bt; ue = Ut * (b + 1) / Bt; }
+      t_end = 0;
+      part_tile = b;
+      part_kb0 = n_kb * part / c.csplit; part_kb1 = n_kb * (part + 1) / c.csplit;
+    } else if (c.halves) {
+      // whole rounds of whole tiles, then tile (rounds * grid + b / 2) as two halves on pairs b and b + 1
+      t_end = (c.n_tiles / grid) * grid;
+      if (t_end + b / 2 < c.n_tiles) { half_tile = t_end + b / 2; half = b & 1; }
     }
   }
   __device__ inline bool next(Seg& sg) {
-    if (u < ue) {
-      const int tt = (int)(u / n_kb);
-      sg.tile = tail_tile0 + tt;
-      sg.kb0 = (int)(u - (long)tt * n_kb);
-      const long len = (n_kb - sg.kb0) < (ue - u) ? (n_kb - sg.kb0) : (ue - u);
-      sg.kb1 = sg.kb0 + (int)len;
-      sg.half = -1;
-      u += len;
-      return true;
-    }
     if (t < t_end) {
       sg.tile = t; sg.kb0 = 0; sg.kb1 = n_kb; sg.half = -1;
       t += step;
       return true;
     }
-    if (ps_tile >= 0) {
-      sg.tile = ps_tile; sg.kb0 = ps_kb0; sg.kb1 = ps_kb1; sg.half = -1;
-      ps_tile = -1;
+    if (part_tile >= 0) {
+      sg.tile = part_tile; sg.kb0 = part_kb0; sg.kb1 = part_kb1; sg.half = -1;
+      part_tile = -1;
       return true;
     }
     if (half_tile >= 0) {
@@ -194,10 +57,6 @@ struct SegIter {
     return false;
   }
 };
-// block whose range [U*b/B, U*(b+1)/B) of the left-over units holds unit u (exact in fp64 for these magnitudes)
-__device__ inline int sk_owner(long u, long B, long U) {
-  return (int)floor(((double)(u + 1) * (double)B - 1.0) / (double)U);
-}
 
 // bf16 activations -> fp16 copy in the workspace, once per call (every weight tile re-reads the tile of
 // activations, so converting there would repeat the work once per 128 weight rows).
@@ -230,18 +89,16 @@ __global__ void x_to_f16_kernel(const __nv_bfloat16* __restrict__ x, int ldx, in
   }
 }
 
-// T: activation / output type.  CONV: the activation tiles arrive as bf16 and are converted to fp16 in
-// shared memory by the de-quantisers (used when the workspace cannot hold a converted copy).
-// HEADS: the input map is a family of per-head blocks (else a leading block).
-// PAIR: clusters of two blocks work on tiles of 256 weight rows with cta_group::2 MMAs.  Each block de-quantises 128 rows
-// into its own shared memory and fetches half of the tokens' boxes; the first block's MMA warp issues for both.  A block's
-// shared memory then takes in 16 instead of 32 KB of activations per 256 tokens and k-block, which with one block per tile
-// was what L2 could not deliver and the shared-memory port could not take beside the operand reads.  PAIR = 1 / 2: one or
-// two boxes of 256 tokens per tile; 3: one box, and the pairs of a cluster share a tile (an instance of its own: inside 1 its
-// registers cost every launch 3 - 10 %).
-template <typename T, bool CONV, bool HEADS, int PAIR>
-__global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__ Params p,
-                                                         const __grid_constant__ PrefillCfg c) {
+// T: activation / output type.  HEADS: the input map is a family of per-head blocks (else a leading block).
+// Clusters of two blocks work on tiles of 256 weight rows with cta_group::2 MMAs.  Each block de-quantises 128 rows into its own
+// shared memory and fetches half of the tokens' boxes; the first block's MMA warp issues for both.  A block's shared memory then
+// takes in 16 instead of 32 KB of activations per 256 tokens and k-block, which with one block per tile was what L2 could not
+// deliver and the shared-memory port could not take beside the operand reads.  PAIR = 1 / 2: one or two boxes of 256 tokens per
+// tile; 3: one box, and the pairs of a cluster share a tile (an instance of its own: inside 1 its registers cost every launch
+// 3 - 10 %).
+template <typename T, bool HEADS, int PAIR>
+__global__ void __launch_bounds__(PTH, 1) pair_kernel(const __grid_constant__ Params p,
+                                                      const __grid_constant__ PrefillCfg c) {
   extern __shared__ unsigned char psmem_raw[];
   constexpr bool ONE = PAIR == 1 || PAIR == 3;              // block pairs, one box of tokens per tile
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (warp-uniform for the compiler)
@@ -253,99 +110,60 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
   const uint32_t raw = (uint32_t)__cvta_generic_to_shared(psmem_raw);
   const uint32_t sbase = (raw + 1023u) & ~1023u;           // swizzled tiles need 1024-byte alignment
   unsigned char* smem = psmem_raw + (sbase - raw);
-  constexpr int NB = ONE ? PSTAGES1 : PAIR ? 2 * PSTAGES2 : BSLOTS;               // slots of the activation ring and their size
-  constexpr int NB_BYTES = PAIR ? B_BYTES / 2 : B_BYTES;
-  // PAIR: the pair's number and their count (3: the cluster's), and this pair's part of a shared tile
-  const int n_share = PAIR == 3 ? c.csplit : 1, per = PAIR ? 2 * n_share : 1;
-  const int bid = PAIR ? (int)blockIdx.x / per : (int)blockIdx.x, nblk = PAIR ? (int)gridDim.x / per : (int)gridDim.x;
-  const uint32_t rank = (PAIR || c.pair_split) ? pcluster_rank() : 0u;
+  constexpr int NA = ONE ? PSTAGES1 : PSTAGES2;             // weight stages, each with the k-block's half boxes
+  constexpr int NB_BYTES = B_BYTES / 2;
+  // this pair's number and their count (3: the cluster's), and this pair's part of a shared tile
+  const int n_share = PAIR == 3 ? c.csplit : 1, per = 2 * n_share;
+  const int bid = (int)blockIdx.x / per, nblk = (int)gridDim.x / per;
+  const uint32_t rank = pcluster_rank();
   const uint32_t crank = PAIR == 3 ? rank & 1u : rank, lrank = PAIR == 3 ? rank & ~1u : 0u;   // block of the pair, rank of the pair's first block
   const int part = PAIR == 3 ? (int)(rank >> 1) : -1;
-  constexpr int NA = ONE ? PSTAGES1 : PAIR ? PSTAGES2 : PSTAGES;             // weight stages
-  constexpr int RING = PAIR ? RING2_BYTES : RING_BYTES;
   constexpr int B_RING = NA * A_BYTES;                      // the activation boxes follow the weight stages
   constexpr int TEAM_WARPS = ONE ? DQ_WARPS : DQ_TEAM_WARPS;
-  const uint32_t bars = sbase + RING;
+  const uint32_t bars = sbase + RING_BYTES;
+  // (a stage's weights and its half boxes share one pair of barriers -- the MMA warp's loop is one chain of dependent
+  //  instructions, 890 cycles per k-block of one box with two waits and two commits where the MMAs take 512)
   const uint32_t full_a = bars, empty_a = bars + 8 * NA;
-  // (PAIR: a stage's weights and its half boxes share one pair of barriers -- the MMA warp's loop is one chain of
-  //  dependent instructions, 890 cycles per k-block of one box with two waits and two commits where the MMAs take 512)
-  const uint32_t full_b = PAIR ? full_a : bars + 16 * NA, empty_b = PAIR ? empty_a : full_b + 8 * NB;
-  const uint32_t acc_full = bars + 16 * NA + 16 * NB, acc_empty = acc_full + 16, epi_bar = acc_full + 32;
-  const uint32_t help_bar = acc_full + 40;         // the epilogue warps and the de-quantiser warps that help them
-  const uint32_t last_full = acc_full + 48;        // the MMAs of the block's last segment are complete (one phase only)
-  const uint32_t px_ready = acc_full + 56;         // pair split, second block: the first block's rings are idle
-  const uint32_t px_done = acc_full + 64;          // pair split, first block: the second block's sums have arrived
-  const uint32_t xq = acc_full + 72;               // pairs that share a tile: the others' sums have arrived, per quadrant
-  unsigned char* misc = smem + RING + 16 * NA + 16 * NB + 104;
+  const uint32_t acc_full = bars + 16 * NA, acc_empty = acc_full + 16;
+  const uint32_t last_full = acc_full + 32;        // the MMAs of the block's last segment are complete (one phase only)
+  const uint32_t xq = acc_full + 40;               // pairs that share a tile: the others' sums have arrived, per quadrant
+  unsigned char* misc = smem + RING_BYTES + 16 * NA + 72;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
 
   if (tid == 0) {
     for (int s = 0; s < NA; ++s) {
-      pmbar_init(full_a + 8 * s, PAIR ? 2 * TEAM_WARPS + 1 : TEAM_WARPS);
+      pmbar_init(full_a + 8 * s, 2 * TEAM_WARPS + 1);
       pmbar_init(empty_a + 8 * s, 1);
     }
-    for (int s = 0; s < NB && !PAIR; ++s) {
-      pmbar_init(full_b + 8 * s, 1);
-      pmbar_init(empty_b + 8 * s, 1);
-    }
-    for (int b = 0; b < 2; ++b) { pmbar_init(acc_full + 8 * b, 1); pmbar_init(acc_empty + 8 * b, PAIR ? 8 : 4); }
-    pmbar_init(epi_bar, 4);
-    pmbar_init(help_bar, 4 + 2 * DQ_WARPS);
+    for (int b = 0; b < 2; ++b) { pmbar_init(acc_full + 8 * b, 1); pmbar_init(acc_empty + 8 * b, 8); }
     pmbar_init(last_full, 1);
-    pmbar_init(px_ready, 1);
-    pmbar_init(px_done, c.helpers ? 4 + 2 * DQ_WARPS : 4);       // one arrival per warp that sends
     if (PAIR == 3)
       for (int b = 0; b < 4; ++b) pmbar_init(xq + 8 * b, max(1, (n_share - 1) * (c.helpers ? 5 : 1)));
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) {                      // the whole tensor memory of the SM: two accumulators of 256 columns
-    const uint32_t slot = (uint32_t)__cvta_generic_to_shared(const_cast<uint32_t*>(tmem_slot));
-    if (PAIR) {
-      tmem_alloc_pair(slot, 512);
-    } else {
-      tmem_alloc(slot, 512);
-      tmem_relinquish();
-    }
-  }
+  // the whole tensor memory of the SM: two accumulators of 256 columns
+  if (warp == 1) tmem_alloc_pair((uint32_t)__cvta_generic_to_shared(const_cast<uint32_t*>(tmem_slot)), 512);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  if (PAIR || c.pair_split) {                   // the other block's barriers exist before anything is sent to it
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  }
+  // the other blocks' barriers exist before anything is sent to them
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
-  // 128-row tile of its job that this block holds (PAIR: tiles are counted in pairs)
-  auto local_tile = [&](int wt, int jn) { return PAIR ? 2 * (wt - c.wtile_begin[jn]) + (int)crank : wt - c.wtile_begin[jn]; };
+  // 128-row tile of its job that this block holds (tiles are counted in pairs)
+  auto local_tile = [&](int wt, int jn) { return 2 * (wt - c.wtile_begin[jn]) + (int)crank; };
   auto job_of_wt = [&](int wt) { int j = 0; while (j + 1 < p.n_jobs && wt >= c.wtile_begin[j + 1]) ++j; return j; };
   bool failed = false;
 
   // ---- the epilogue of one segment, for the warp that calls it: accumulator -> bias, rotary embedding or gated
   //      product, rounding, store.  A warp reaches the tensor-memory lanes 32 (warp % 4) .. + 31 (a lane is a tile
   //      row); it takes the chunks ch0, ch0 + chs, ... of 32 tokens.  chs == 1: the epilogue warp on its own (it
-  //      also hands the accumulators back and runs the hand-over of a tile split along K).
+  //      also hands the accumulators back).
   const int q = warp & 3;                          // TMEM lanes 32q .. 32q+31
   const int etid = 32 * q + lane;                  // tile row handled in the store phase
-  uint32_t epar = 0;
-  auto epi_sync = [&]() -> bool {
-    __syncwarp();
-    if (lane == 0) pmbar_arrive(epi_bar);
-    const bool ok = pmbar_wait(epi_bar, epar, abort_flag);
-    epar ^= 1;
-    return ok;
-  };
-  volatile int* last_flag = reinterpret_cast<volatile int*>(misc + 8);
-  uint32_t hpar = 0;
-  auto help_sync = [&]() -> bool {
-    __syncwarp();
-    if (lane == 0) pmbar_arrive(help_bar);
-    const bool ok = pmbar_wait(help_bar, hpar, abort_flag);
-    hpar ^= 1;
-    return ok;
-  };
   auto epilogue_segment = [&](const Seg& sg, int tcount, int ch0, int chs, bool acc_known_full) {
       const int acc0 = c.nh == 2 ? 0 : (tcount & 1);     // as in the MMA warp
       const int au = c.nh == 2 ? tcount : (tcount >> 1);
@@ -372,10 +190,54 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
         __syncwarp();
         if (lane == 0) {
           const uint32_t eb = acc_empty + 8 * (acc0 + (ch * EPI_TOK) / c.bn);
-          if (PAIR) pmbar_signal_peer(ppeer_addr(eb, lrank)); else pmbar_arrive(eb);
+          pmbar_signal_peer(ppeer_addr(eb, lrank));
         }
       };
-      if (sg.kb0 == 0 && sg.kb1 == c.n_kb) {
+      if constexpr (PAIR == 3) {
+        // ---- the pairs of a cluster share this tile.  Eight tokens at a time: pair i % n_share finishes chunk i.  Each
+        //      leaves its sums of the other pairs' chunks in a slot ([token][row], L2), tells them (remote arrivals,
+        //      one per warp and pair), and adds up and finishes its own chunks in the order of the parts.
+        float* slots = c.partials + row;
+        const float* first = slots + (size_t)(blockIdx.x - rank + crank) * (MAXBN * BMW);   // part 0's block of the same rows
+        float* mine = slots + (size_t)blockIdx.x * (MAXBN * BMW);
+        constexpr int CH = 8, N_CH = MAXBN / CH;
+        for (int ch = ch0; ch < N_CH; ch += chs) {
+          if (ch % n_share == part) continue;
+          uint32_t v[8];
+          tmem_ld8(t_acc + (uint32_t)(ch * CH), v);
+          tmem_ld_wait();
+#pragma unroll
+          for (int k = 0; k < 8; ++k) __stcg(mine + (size_t)(ch * CH + k) * BMW, __uint_as_float(v[k]));
+        }
+        __syncwarp();
+        if (lane < n_share && lane != part) {
+          asm volatile("fence.acq_rel.cluster;" ::: "memory");
+          pmbar_arrive_peer(ppeer_addr(xq + 8 * q, (uint32_t)(2 * lane) + crank));
+        }
+        if (!__all_sync(0xffffffffu, pmbar_wait_cluster(xq + 8 * q, 0, abort_flag))) { failed = true; return; }
+        for (int own = ch0; part + own * n_share < N_CH; own += chs) {
+          const int tk = (part + own * n_share) * CH;
+          if (tt * ntok + tk >= p.M) break;
+          uint32_t v[8];
+          tmem_ld8(t_acc + (uint32_t)tk, v);
+          tmem_ld_wait();
+          float val[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) val[k] = 0.f;
+          const float* src = first + (size_t)tk * BMW;
+          for (int r0 = 0; r0 < n_share; r0 += 2) {          // two parts in flight, added in their order
+            float a[8], b[8];
+            const bool own_a = r0 == part, own_b = r0 + 1 == part, has_b = r0 + 1 < n_share;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) a[k] = own_a ? __uint_as_float(v[k]) : __ldcg(src + (size_t)(2 * r0) * (MAXBN * BMW) + (size_t)k * BMW);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) b[k] = own_b ? __uint_as_float(v[k]) : has_b ? __ldcg(src + (size_t)(2 * r0 + 2) * (MAXBN * BMW) + (size_t)k * BMW) : 0.f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) val[k] = (val[k] + a[k]) + b[k];
+          }
+          store_chunk(tk, val);
+        }
+      } else {
         // ---- the whole contraction of this tile ran here (this warp takes every chs-th chunk of 32 tokens;
         //      of a half tile only the chunks of its box)
         const int cpb = c.bn / EPI_TOK;
@@ -389,228 +251,46 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
           for (int k = 0; k < 32; ++k) val[k] = __uint_as_float(v[k]);
           store_chunk(ch * EPI_TOK, val);
         }
-      } else {
-        // ---- a part of the contraction (stream-K): the fp32 partial tile goes to a slot of its own in the
-        //      workspace, [token][row] (a warp writes and later reads 32 consecutive rows of a token: whole
-        //      128-byte lines); the last of the tile's blocks to arrive adds the slots of all of them in block
-        //      order (the same sum whatever the order of arrival) and finishes the tile.
-        //      The pieces (tile, block) of the cut unit line are numbered lt + block: both grow along the line and
-        //      one of them grows from each piece to the next, so no two pieces share a number.
-        //      chs > 1: the block's last segment, shared with the de-quantiser warps (twenty warps write, meet at a
-        //      barrier of their own, and -- in the last block to arrive -- read back and finish).
-        //      Where a few split tiles in front of whole tiles have many parts each, reading all the slots back
-        //      would take the four epilogue warps longer than the tiles behind can hide: such launches add the parts
-        //      into ONE sum per tile instead (reductions done in L2, zero at launch; the last bit of a sum then
-        //      depends on the order of arrival when more than two blocks share a tile).
-        if (PAIR == 3) {
-          // ---- the pairs of a cluster share this tile.  Eight tokens at a time: pair i % n_share finishes chunk i.  Each
-          //      leaves its sums of the other pairs' chunks in a slot ([token][row], L2), tells them (remote arrivals,
-          //      one per warp and pair), and adds up and finishes its own chunks in the order of the parts.
-          float* slots = c.partials + row;
-          const float* first = slots + (size_t)(blockIdx.x - rank + crank) * (MAXBN * BMW);   // part 0's block of the same rows
-          float* mine = slots + (size_t)blockIdx.x * (MAXBN * BMW);
-          constexpr int CH = 8, N_CH = MAXBN / CH;
-          for (int ch = ch0; ch < N_CH; ch += chs) {
-            if (ch % n_share == part) continue;
-            uint32_t v[8];
-            tmem_ld8(t_acc + (uint32_t)(ch * CH), v);
-            tmem_ld_wait();
-#pragma unroll
-            for (int k = 0; k < 8; ++k) __stcg(mine + (size_t)(ch * CH + k) * BMW, __uint_as_float(v[k]));
-          }
-          __syncwarp();
-          if (lane < n_share && lane != part) {
-            asm volatile("fence.acq_rel.cluster;" ::: "memory");
-            pmbar_arrive_peer(ppeer_addr(xq + 8 * q, (uint32_t)(2 * lane) + crank));
-          }
-          if (!__all_sync(0xffffffffu, pmbar_wait_cluster(xq + 8 * q, 0, abort_flag))) { failed = true; return; }
-          for (int own = ch0; part + own * n_share < N_CH; own += chs) {
-            const int tk = (part + own * n_share) * CH;
-            if (tt * ntok + tk >= p.M) break;
-            uint32_t v[8];
-            tmem_ld8(t_acc + (uint32_t)tk, v);
-            tmem_ld_wait();
-            float val[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) val[k] = 0.f;
-            const float* src = first + (size_t)tk * BMW;
-            for (int r0 = 0; r0 < n_share; r0 += 2) {          // two parts in flight, added in their order
-              float a[8], b[8];
-              const bool own_a = r0 == part, own_b = r0 + 1 == part, has_b = r0 + 1 < n_share;
-#pragma unroll
-              for (int k = 0; k < 8; ++k) a[k] = own_a ? __uint_as_float(v[k]) : __ldcg(src + (size_t)(2 * r0) * (MAXBN * BMW) + (size_t)k * BMW);
-#pragma unroll
-              for (int k = 0; k < 8; ++k) b[k] = own_b ? __uint_as_float(v[k]) : has_b ? __ldcg(src + (size_t)(2 * r0 + 2) * (MAXBN * BMW) + (size_t)k * BMW) : 0.f;
-#pragma unroll
-              for (int k = 0; k < 8; ++k) val[k] = (val[k] + a[k]) + b[k];
-            }
-            store_chunk(tk, val);
-          }
-          return;
-        }
-        const bool pair_send = c.pair_split && crank != 0;
-        if (c.pair_split && !pair_send) {
-          // ---- the two blocks of a cluster each ran half of the contraction.  The second block waits until the
-          //      first one's MMAs are complete (its rings are idle then), writes its fp32 sums into them ([token][row]:
-          //      a warp stores 32 consecutive rows of a token) and arrives, one arrival per warp, at the first block's
-          //      barrier; the first block adds them to its own sums (always own + other: the same bits every run)
-          //      and finishes the tile.  No traffic through L2, no counter, nothing to clear.
-          {
-            if (!pmbar_wait_cluster(px_done, 0, abort_flag)) { failed = true; return; }
-            // (16 tokens at a time, as the read-back of the slots: what the registers of a thread hold)
-            for (int tk = 16 * ch0; tk < ntok; tk += 16 * chs) {
-              uint32_t v[16];
-              tmem_ld16(t_acc + (uint32_t)tk, v);
-              tmem_ld_wait();
-              const uint32_t src = sbase + (uint32_t)((tk * BMW + row) * 4);
-              float val[16];
-              pld_add_f32x16<BMW * 4>(src, v, val);
-              store_chunk(tk, val);
-            }
-          }
-          return;
-        }
-        const bool main_lane = warp == EPI_WARP0 && lane == 0;
-        const size_t slot_f = (size_t)ntok * BMW;
-        const int T0 = (c.n_tiles / nblk) * nblk;              // first left-over tile
-        // (PAIR: two slots side by side, a block's own 128 rows in each)
-        auto slot_of = [&](int n) { return c.partials + (PAIR ? 2 * (size_t)n + crank : (size_t)n) * slot_f; };
-        float* mine = slot_of((t - T0) + (c.sk_atomic ? 0 : bid));
-        int* arrivals = &c.counters[PAIR ? 2 * t + (int)crank : t];
-        if (pair_send) {
-          // (the second block of a pair: its "slot" is the first block's rings, once they are idle)
-          if (!pmbar_wait_cluster(px_ready, 0, abort_flag)) { failed = true; return; }
-          mine = ppeer_generic(smem, 0u);
-        }
-        for (int ch = ch0; ch < ntok / EPI_TOK; ch += chs) {
-          uint32_t v[32];
-          tmem_ld32(t_acc + (uint32_t)(ch * EPI_TOK), v);
-          tmem_ld_wait();
-          if (chs == 1) release_after(ch);                     // the accumulator is free for the next segment
-          float* dst = mine + (size_t)(ch * EPI_TOK) * BMW + row;
-          if (pair_send) {
-#pragma unroll
-            for (int k = 0; k < 32; ++k) dst[(size_t)k * BMW] = __uint_as_float(v[k]);
-          } else if (c.sk_atomic) {
-#pragma unroll
-            for (int k = 0; k < 32; ++k) atomicAdd(dst + (size_t)k * BMW, __uint_as_float(v[k]));
-          } else {
-#pragma unroll
-            for (int k = 0; k < 32; ++k) __stcg(dst + (size_t)k * BMW, __uint_as_float(v[k]));
-          }
-        }
-        if (pair_send) {
-          __syncwarp();
-          if (lane == 0) {
-            asm volatile("fence.acq_rel.cluster;" ::: "memory");
-            pmbar_arrive_peer(ppeer_addr(px_done, 0u));
-          }
-          return;
-        }
-        __threadfence();                                       // this thread's part is in place before ...
-        if (!(chs == 1 ? epi_sync() : help_sync())) { failed = true; return; }
-        const long U = (long)(c.n_tiles - T0) * c.n_kb, Bn = (long)nblk < U ? (long)nblk : U;
-        const long tu = (long)(t - T0) * c.n_kb;                               // the tile's first left-over unit
-        const int first = sk_owner(tu, Bn, U), last = sk_owner(tu + c.n_kb - 1, Bn, U);
-        if (main_lane) {
-          const int arrived = atomicAdd(arrivals, 1);          // ... the block's arrival shows
-          *last_flag = arrived == last - first;
-          __threadfence();
-        }
-        if (!(chs == 1 ? epi_sync() : help_sync())) { failed = true; return; }
-        if (*last_flag) {
-          const float* base = slot_of((t - T0) + (c.sk_atomic ? 0 : first));
-          const size_t part_f = PAIR ? 2 * slot_f : slot_f;    // from one block's part to the next one's
-          const int parts = c.sk_atomic ? 1 : last - first + 1;
-          // 16 tokens at a time, the loads of two slots in flight together (what the registers of a thread hold)
-          for (int tk = 16 * ch0; tk < ntok; tk += 16 * chs) {
-            float val[16];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) val[k] = 0.f;
-            const float* src = base + (size_t)tk * BMW + row;
-            for (int s2 = 0; s2 < parts; s2 += 2) {
-              const bool two = s2 + 1 < parts;
-              float a[16], b[16];
-#pragma unroll
-              for (int k = 0; k < 16; ++k) a[k] = __ldcg(src + (size_t)s2 * part_f + (size_t)k * BMW);
-#pragma unroll
-              for (int k = 0; k < 16; ++k) b[k] = two ? __ldcg(src + (size_t)(s2 + 1) * part_f + (size_t)k * BMW) : 0.f;
-#pragma unroll
-              for (int k = 0; k < 16; ++k) val[k] = (val[k] + a[k]) + b[k];
-            }
-            store_chunk(tk, val);
-          }
-          if (main_lane) *arrivals = 0;                  // ready for the next call
-        }
       }
   };
 
   if (warp == 0) {
     // ===================================================================== activations by TMA
-    if (PAIR) {
-      // (warp-uniform, as the MMA warp: one lane walking this loop took longer per k-block than the MMAs do)
-      asm volatile("griddepcontrol.wait;" ::: "memory");
-      constexpr int NH = ONE ? 1 : 2;
-      const uint32_t rfull = ppeer_addr(full_a, lrank);       // both blocks' half boxes count on the first block's barriers
-      int s = 0, it = 0; uint32_t par = 1;
-      SegIter si; si.init(c, bid, nblk, part);
-      Seg sg;
-      while (!failed && si.next(sg)) {
-        const int n_box = NH == 1 || sg.half >= 0 ? 1 : 2;
-        const int y0 = ((sg.tile % c.n_ttiles) * NH + (NH == 2 && sg.half > 0 ? 1 : 0)) * MAXBN + (int)crank * (MAXBN / 2);
-        KWalk kw;
-        if (HEADS) kw.start(c, sg.kb0);
-        for (int kb = sg.kb0; kb < sg.kb1; ++kb, ++it) {
-          const int x = HEADS ? kw.xcol(c) : kb * BK;
-          if (HEADS) kw.step(c, 1);
-          if (it >= NA && !pmbar_wait_warp(empty_a + 8 * s, par, abort_flag)) { failed = true; break; }
-          if (elect_one()) {
-            if (crank == 0) pmbar_expect_tx(full_a + 8 * s, (uint32_t)(n_box * MAXBN * BK * 2));
-            const uint32_t dst = sbase + B_RING + s * NH * NB_BYTES;
-            tma_box2_pair(dst, &c.xmap, x, y0, rfull + 8 * s);
-            if (n_box == 2) tma_box2_pair(dst + NB_BYTES, &c.xmap, x, y0 + MAXBN, rfull + 8 * s);
-          }
-          __syncwarp();
-          if (++s == NA) { s = 0; par ^= 1; }
+    // (warp-uniform, as the MMA warp: one lane walking this loop took longer per k-block than the MMAs do)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    constexpr int NH = ONE ? 1 : 2;
+    const uint32_t rfull = ppeer_addr(full_a, lrank);       // both blocks' half boxes count on the first block's barriers
+    int s = 0, it = 0; uint32_t par = 1;
+    SegIter si; si.init(c, bid, nblk, part);
+    Seg sg;
+    while (!failed && si.next(sg)) {
+      const int n_box = NH == 1 || sg.half >= 0 ? 1 : 2;
+      const int y0 = ((sg.tile % c.n_ttiles) * NH + (NH == 2 && sg.half > 0 ? 1 : 0)) * MAXBN + (int)crank * (MAXBN / 2);
+      KWalk kw;
+      if (HEADS) kw.start(c, sg.kb0);
+      for (int kb = sg.kb0; kb < sg.kb1; ++kb, ++it) {
+        const int x = HEADS ? kw.xcol(c) : kb * BK;
+        if (HEADS) kw.step(c, 1);
+        if (it >= NA && !pmbar_wait_warp(empty_a + 8 * s, par, abort_flag)) { failed = true; break; }
+        if (elect_one()) {
+          if (crank == 0) pmbar_expect_tx(full_a + 8 * s, (uint32_t)(n_box * MAXBN * BK * 2));
+          const uint32_t dst = sbase + B_RING + s * NH * NB_BYTES;
+          tma_box2_pair(dst, &c.xmap, x, y0, rfull + 8 * s);
+          if (n_box == 2) tma_box2_pair(dst + NB_BYTES, &c.xmap, x, y0 + MAXBN, rfull + 8 * s);
         }
+        __syncwarp();
+        if (++s == NA) { s = 0; par ^= 1; }
       }
-      if (failed)                           // copies may still be on their way into this block's shared memory: they land well
-        for (int i = 0; i < 1000; ++i) __nanosleep(200);        // within this time
-    } else if (lane == 0) {
-      asm volatile("griddepcontrol.wait;" ::: "memory");   // the activations may come from the preceding kernel
-      int s = 0; uint32_t par = 1; int jb = 0;             // box slot, parity of its previous use, boxes so far
-      SegIter si; si.init(c, bid, nblk, part);
-      Seg sg;
-      while (!failed && si.next(sg)) {
-        const int tt = sg.tile % c.n_ttiles;
-        KWalk kw;
-        if (HEADS) kw.start(c, sg.kb0);
-        for (int kb = sg.kb0; kb < sg.kb1 && !failed; ++kb) {
-          const int xcol = HEADS ? kw.xcol(c) : kb * BK;
-          if (HEADS) kw.step(c, 1);
-          const int h_lo = sg.half < 0 ? 0 : sg.half, h_hi = sg.half < 0 ? c.nh : sg.half + 1;
-          for (int h = h_lo; h < h_hi; ++h, ++jb) {
-            if (jb >= NB && !pmbar_wait(empty_b + 8 * s, par, abort_flag, true)) { failed = true; break; }
-            const uint32_t fb = full_b + 8 * s;
-            // (a box that starts at or beyond the last token is all zeros: the tensor map ends at M)
-            pmbar_expect_tx(fb, (uint32_t)(c.bn * BK * 2));
-            tma_box2(sbase + B_RING + s * NB_BYTES, &c.xmap, xcol, (tt * c.nh + h) * c.bn, fb);
-            if (++s == NB) { s = 0; par ^= 1; }
-          }
-        }
-      }
-      if (failed)                           // copies may still be on their way into this block's shared memory: they land well
-        for (int i = 0; i < 1000; ++i) __nanosleep(200);        // within this time
     }
+    if (failed)                           // copies may still be on their way into this block's shared memory: they land well
+      for (int i = 0; i < 1000; ++i) __nanosleep(200);        // within this time
   } else if (warp == 1) {
     // ===================================================================== MMA issue
     // (the whole warp walks the loop, so that stage indexes, parities and descriptors are warp-uniform; one elected
     //  lane issues)
-    if (!PAIR || crank == 0) {
+    if (crank == 0) {
       const unsigned short pair_mask = (unsigned short)(3u << lrank);
-      auto commit = [&](uint32_t bar) { if (PAIR) umma_commit_pair(bar, pair_mask); else umma_commit(bar); };
       int s = 0; uint32_t par = 0; int tcount = 0;         // weight stage and its parity
-      int sb = 0; uint32_t parb = 0;                       // activation box slot and its parity
       SegIter si; si.init(c, bid, nblk, part);
       Seg sg;
       for (; !failed && si.next(sg); ++tcount) {
@@ -650,22 +330,13 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
             if (++s == NA) { s = 0; par ^= 1; }
             continue;
           }
-          for (int h = h_lo; h < h_hi; ++h) {
-            if (kb == sg.kb0 && au >= 1 && !pmbar_wait_warp(acc_empty + 8 * (acc0 + h), (au - 1) & 1, abort_flag)) { failed = true; break; }
-            // (bf16: the de-quantisers waited for the activation box themselves and converted it)
-            if (!CONV && !ONE && !pmbar_wait_warp(full_b + 8 * sb, parb, abort_flag)) { failed = true; break; }
-            tc_fence_after();
-            const uint32_t d_tmem = tmem_base + (uint32_t)((acc0 + h) * MAXBN);
-            const uint64_t bdesc = smem_desc_sw128(sbase + B_RING + sb * NB_BYTES);
-            if (elect_one()) {
-              umma_kblock<PAIR != 0>(d_tmem, adesc, bdesc, c.idesc, kb > sg.kb0 ? 1u : 0u);
-              if (!ONE) commit(empty_b + 8 * sb);    // the box is free once these MMAs have read it
-              if (ONE || h == h_hi - 1) commit(empty_a + 8 * s);   // ... and the weight stage after the last of them
-            }
-            __syncwarp();
-            if (++sb == NB) { sb = 0; parb ^= 1; }
+          if (kb == sg.kb0 && au >= 1 && !pmbar_wait_warp(acc_empty + 8 * acc0, (au - 1) & 1, abort_flag)) { failed = true; break; }
+          tc_fence_after();
+          if (elect_one()) {
+            umma_kblock<true>(tmem_base + (uint32_t)(acc0 * MAXBN), adesc, smem_desc_sw128(sbase + B_RING + s * NB_BYTES), c.idesc, kb > sg.kb0 ? 1u : 0u);
+            umma_commit_pair(empty_a + 8 * s, pair_mask);        // the stage is free once these MMAs have read it
           }
-          if (failed) break;
+          __syncwarp();
           if (++s == NA) { s = 0; par ^= 1; }
         }
         if (failed) break;
@@ -676,21 +347,10 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
         Seg nxt;
         const bool last = !peek.next(nxt);
         if (elect_one()) {
-          for (int h = h_lo; h < h_hi; ++h) commit(acc_full + 8 * (acc0 + h));
-          if (last) commit(last_full);
+          for (int h = h_lo; h < h_hi; ++h) umma_commit_pair(acc_full + 8 * (acc0 + h), pair_mask);
+          if (last) umma_commit_pair(last_full, pair_mask);
         }
         __syncwarp();
-      }
-      if (c.pair_split && crank == 0 && !failed) {
-        // the first block of a pair: once its own MMAs are complete nothing reads its rings any more
-        if (pmbar_wait_warp(last_full, 0, abort_flag)) {
-          if (lane == 0) {
-            asm volatile("fence.acq_rel.cluster;" ::: "memory");
-            pmbar_arrive_peer(ppeer_addr(px_ready, 1u));
-          }
-        } else {
-          failed = true;
-        }
       }
     }
   } else if (warp >= DQ_WARP0) {
@@ -795,27 +455,10 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
             asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(a_st + (uint32_t)(((hf_of[m] * 4 + j) ^ r7[m]) * 16)), "r"(o.x), "r"(o.y), "r"(o.z), "r"(o.w) : "memory");
           }
         }
-        if constexpr (CONV) {
-          // bf16 activations: the tensor cores run on fp16 (8 more mantissa bits for the weights than bf16
-          // would leave them); the activation tile that TMA delivered is converted in place
-          for (int h = 0; h < c.nh && !failed; ++h) {
-            const int jb2 = it * c.nh + h;                 // the k-block's boxes in the order the producer issued them
-            const int sb = jb2 % BSLOTS;
-            if (!pmbar_wait(full_b + 8 * sb, (uint32_t)(jb2 / BSLOTS) & 1, abort_flag)) { failed = true; break; }
-            const uint32_t b_st = sbase + B_RING + sb * B_BYTES;
-            for (int ci = dt; ci < c.bn * 8; ci += TEAM_TH) {
-              uint32_t v0, v1, v2, v3;
-              asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v0), "=r"(v1), "=r"(v2), "=r"(v3) : "r"(b_st + ci * 16));
-              v0 = bf16x2_to_f16x2(v0); v1 = bf16x2_to_f16x2(v1); v2 = bf16x2_to_f16x2(v2); v3 = bf16x2_to_f16x2(v3);
-              asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(b_st + ci * 16), "r"(v0), "r"(v1), "r"(v2), "r"(v3) : "memory");
-            }
-          }
-          if (failed) break;
-        }
         fence_async_smem();            // generic-proxy writes must be visible to the tensor core (async proxy)
         __syncwarp();
         if (lane == 0) {
-          if (PAIR && crank != 0) pmbar_signal_peer(ppeer_addr(full_a + 8 * s, lrank)); else pmbar_arrive(full_a + 8 * s);
+          if (crank != 0) pmbar_signal_peer(ppeer_addr(full_a + 8 * s, lrank)); else pmbar_arrive(full_a + 8 * s);
         }
 #pragma unroll
         for (int m = 0; m < 2; ++m) { q0[m] = q1[m]; s0[m] = s1[m]; z0[m] = z1[m]; }
@@ -857,17 +500,12 @@ __global__ void __launch_bounds__(PTH, 1) prefill_kernel(const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (PAIR) {                           // (tensor memory of both blocks is given back together, after the last MMA)
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    if (warp == 1) tmem_dealloc_pair(tmem_base, 512);
-  } else if (warp == 1) {
-    tmem_dealloc(tmem_base, 512);
-  }
-  if (PAIR || c.pair_split) {                   // neither block of a pair leaves while the other may still send to it
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  }
+  // (tensor memory of both blocks is given back together, after the last MMA; no block leaves while another may still send to it)
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (warp == 1) tmem_dealloc_pair(tmem_base, 512);
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // -------------------------------------------------------------------------------- host side
@@ -897,10 +535,11 @@ int host_job_tiles(const JobDev& j) {
   return (j.k_out + BMW - 1) / BMW;
 }
 
-template <typename T, bool CONV, bool HEADS, int PAIR>
-int launch_pth(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stream) {
-  const size_t smem = 1024 + (size_t)(PAIR ? RING2_BYTES : RING_BYTES) + 512;
-  auto kern = prefill_kernel<T, CONV, HEADS, PAIR>;
+// UNIQL_ERR_UNSUPPORTED: the clusters were refused, and nothing was launched.
+template <typename T, bool HEADS, int PAIR>
+int launch_as(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stream) {
+  const size_t smem = 1024 + (size_t)RING_BYTES + 512;
+  auto kern = pair_kernel<T, HEADS, PAIR>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return UNIQL_ERR_CUDA;
   cudaLaunchConfig_t lc;
@@ -914,28 +553,17 @@ int launch_pth(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stre
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = attr;
   lc.numAttrs = opt(kOptPdl) ? 1 : 0;
-  if (PAIR || c.pair_split) {
-    // clusters of two, only when every pair can be resident at once; else the caller plans without them
-    attr[lc.numAttrs].id = cudaLaunchAttributeClusterDimension;
-    attr[lc.numAttrs].val.clusterDim.x = PAIR == 3 ? 2 * c.csplit : 2;
-    attr[lc.numAttrs].val.clusterDim.y = 1;
-    attr[lc.numAttrs].val.clusterDim.z = 1;
-    ++lc.numAttrs;
-    // (asked once per kernel instance: the answer depends on the block's resources, which do not change)
-    static std::atomic<int> max_clusters{-1};
-    int n_clusters = PAIR ? device_sms() / 2 : max_clusters.load();          // (PAIR: the caller has asked pair_capacity())
-    if (n_clusters < 0) {
-      if (cudaOccupancyMaxActiveClusters(&n_clusters, kern, &lc) != cudaSuccess) { cudaGetLastError(); n_clusters = 0; }
-      max_clusters.store(n_clusters);
-    }
-    if (n_clusters * 2 < grid) return UNIQL_ERR_UNSUPPORTED;
-  }
-  if (cudaLaunchKernelEx(&lc, kern, p, c) != cudaSuccess) { cudaGetLastError(); return PAIR || c.pair_split ? UNIQL_ERR_UNSUPPORTED : UNIQL_ERR_CUDA; }
+  attr[lc.numAttrs].id = cudaLaunchAttributeClusterDimension;
+  attr[lc.numAttrs].val.clusterDim.x = PAIR == 3 ? 2 * c.csplit : 2;
+  attr[lc.numAttrs].val.clusterDim.y = 1;
+  attr[lc.numAttrs].val.clusterDim.z = 1;
+  ++lc.numAttrs;
+  if (cudaLaunchKernelEx(&lc, kern, p, c) != cudaSuccess) { cudaGetLastError(); return UNIQL_ERR_UNSUPPORTED; }
   return UNIQL_OK;
 }
-template <typename T, bool CONV, int PAIR>
-int launch_pt(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stream) {
-  return c.km_period != 0 ? launch_pth<T, CONV, true, PAIR>(p, c, grid, stream) : launch_pth<T, CONV, false, PAIR>(p, c, grid, stream);
+template <typename T, int PAIR>
+int launch_pair(const Params& p, const PrefillCfg& c, int grid, cudaStream_t stream) {
+  return c.km_period != 0 ? launch_as<T, true, PAIR>(p, c, grid, stream) : launch_as<T, false, PAIR>(p, c, grid, stream);
 }
 
 // Clusters of `share` block pairs that the device holds at once (asked once per device; the instances need the same
@@ -947,8 +575,8 @@ int pair_capacity(int share) {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   int v = n[dev][share].load(std::memory_order_relaxed);
   if (v != 0) return v - 1;
-  auto kern = prefill_kernel<__half, false, false, 3>;
-  const size_t smem = 1024 + (size_t)RING2_BYTES + 512;
+  auto kern = pair_kernel<__half, false, 3>;
+  const size_t smem = 1024 + (size_t)RING_BYTES + 512;
   const int most = device_sms() / (2 * share);
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
@@ -1140,7 +768,7 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     double hand_over;
     q.atomic = false;
     // a k-block of a one-box tile by the number of busy SMs (0.45 us with 28 of them, 0.61 us with all)
-    auto kb1 = [&](int busy) { return cg2 ? 0.365 : 0.42 + 0.19 * (busy < g2 ? busy : g2) / g2; };
+    auto kb1 = [&](int busy) { return 0.42 + 0.19 * (busy < g2 ? busy : g2) / g2; };
     if (q.tiles < g2) {
       // every tile is split and every block ends on a split tile: the hand-over is shared with the de-quantiser warps
       // (one-box tiles, measured at M = 64 .. 512 on seven layer shapes: 5 us per 64 tokens of the tile)
@@ -1162,24 +790,24 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     if (env_streamk == 1) q.atomic = false;                            // tests: the form of the hand-over forced
     if (env_streamk == 2) q.atomic = true;
     // (a split is taken where it is estimated 5 % ahead: its hand-over varies more than a whole tile's time)
-    double us_split = 1.05 * ((double)q.tiles / g2 * c.n_kb * ((nh == 1 && q.tiles < g2) ? kb1(g2) : kcost) + hand_over);
+    const double us_split = 1.05 * ((double)q.tiles / g2 * c.n_kb * ((nh == 1 && q.tiles < g2) ? kb1(g2) : kcost) + hand_over);
     // Whole tiles.  On both accumulators a k-block takes 0.84 us when every SM runs one and less when some have no
     // tile (0.79 us with 28 busy SMs: they share the activation traffic out of L2), and between two tiles of a block
     // the MMAs wait 7 - 10 us for the epilogue to drain the accumulators (in-kernel time stamps, Qwen2.5-7B gate at
     // M = 2048); fitted over 48 launches (16 shapes at M = 512, 1024, 2048, every width and hand-over forced in turn).
     const int rounds = (q.tiles + g2 - 1) / g2;
     double us_whole = (double)rounds * c.n_kb * kcost;
-    if (nh == 1 && q.tiles <= g2) us_whole = c.n_kb * kb1(q.tiles);
+    if (nh == 1 && !cg2 && q.tiles <= g2) us_whole = c.n_kb * kb1(q.tiles);
     if (nh == 2 && cg2)
       us_whole = (double)rounds * (c.n_kb * 0.60 + 9.0);
     else if (nh == 2)
       us_whole = (double)(q.tiles / g2) * c.n_kb * 0.96 + (q.left ? c.n_kb * (0.90 + 0.06 * q.left / g2) : 0.0) + 10.0 * (rounds - 1);
-    if (cg2 && nh == 1) { us_whole += 5.5; us_split += 5.5; }                  // start and last epilogue
+    if (cg2 && nh == 1) us_whole += 5.5;                                       // start and last epilogue
     // one fp32 slot per (left-over tile, block) piece, or one sum per left-over tile
-    q.sums = (size_t)(q.atomic ? q.left : q.left + g2) * ntok * BMW * 4 * (cg2 ? 2 : 1);
-    // (pairs: only where forced -- with a k-block at 0.36 us no split of the left-over tiles measured ahead of whole tiles)
-    const bool want = env_streamk >= 0 ? (env_streamk >= 1 && env_streamk < 10) : (!cg2 && q.left != 0 && us_split < us_whole);
-    q.streamk = want && q.left != 0 && cfg.ws_bytes >= ws_used + q.sums && q.tiles <= (1 << 15);
+    q.sums = (size_t)(q.atomic ? q.left : q.left + g2) * ntok * BMW * 4;
+    // (pairs: never -- with a k-block at 0.36 us no split of the left-over tiles measured ahead of whole tiles)
+    const bool want = env_streamk >= 0 ? (env_streamk >= 1 && env_streamk < 10) : us_split < us_whole;
+    q.streamk = want && !cg2 && q.left != 0 && cfg.ws_bytes >= ws_used + q.sums && q.tiles <= (1 << 15);
     q.us = q.streamk ? us_split : us_whole;
     // Tiles of two boxes left over after the whole rounds, when they are few: each runs as two half tiles (one box,
     // 256 tokens) on two blocks, a block's last segment -- no hand-over, and the round takes a one-box tile's time
@@ -1265,17 +893,16 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
   if (pl.share > 1) c.partials = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(cfg.workspace) + ws_used);
   int rc = encode_x_map(&c.xmap, xsrc, p.k_in, p.M, ldxs, pl.cg2 ? c.bn / 2 : c.bn, conv_in_kernel);
   if (rc != UNIQL_OK) return rc;
-  if (p.dt == UNIQL_BF16)
-    rc = conv_in_kernel ? launch_pt<__nv_bfloat16, true, 0>(p, c, grid, cfg.stream)
-         : !pl.cg2      ? launch_pt<__nv_bfloat16, false, 0>(p, c, grid, cfg.stream)
-         : c.csplit > 1 ? launch_pt<__nv_bfloat16, false, 3>(p, c, grid, cfg.stream)
-         : c.nh == 1    ? launch_pt<__nv_bfloat16, false, 1>(p, c, grid, cfg.stream)
-                        : launch_pt<__nv_bfloat16, false, 2>(p, c, grid, cfg.stream);
+  if (!pl.cg2)
+    rc = launch_one_block(p, c, grid, conv_in_kernel, cfg.stream);
+  else if (p.dt == UNIQL_BF16)
+    rc = c.csplit > 1 ? launch_pair<__nv_bfloat16, 3>(p, c, grid, cfg.stream)
+         : c.nh == 1  ? launch_pair<__nv_bfloat16, 1>(p, c, grid, cfg.stream)
+                      : launch_pair<__nv_bfloat16, 2>(p, c, grid, cfg.stream);
   else
-    rc = !pl.cg2        ? launch_pt<__half, false, 0>(p, c, grid, cfg.stream)
-         : c.csplit > 1 ? launch_pt<__half, false, 3>(p, c, grid, cfg.stream)
-         : c.nh == 1    ? launch_pt<__half, false, 1>(p, c, grid, cfg.stream)
-                        : launch_pt<__half, false, 2>(p, c, grid, cfg.stream);
+    rc = c.csplit > 1 ? launch_pair<__half, 3>(p, c, grid, cfg.stream)
+         : c.nh == 1  ? launch_pair<__half, 1>(p, c, grid, cfg.stream)
+                      : launch_pair<__half, 2>(p, c, grid, cfg.stream);
   if (rc == UNIQL_ERR_UNSUPPORTED && c.pair_split) {
     // the pairs cannot all be resident (or clusters cannot be launched here): planned again without them
     pair_refused.store(true);
