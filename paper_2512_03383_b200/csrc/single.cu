@@ -104,7 +104,7 @@ template <typename T, bool CONV, bool HEADS>
 __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant__ Params p,
                                                          const __grid_constant__ PrefillCfg c) {
   extern __shared__ unsigned char psmem_raw[];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (warp-uniform for the compiler)
   // Programmatic dependent launch: the next kernel of the stream may be set up while this one runs (its blocks
   // become resident as ours leave).  What a block does before its own `griddepcontrol.wait` touches nothing a
   // predecessor may still write or read: barriers, tensor memory, and the weights, which no kernel writes (the
@@ -466,53 +466,61 @@ __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant
     }
   } else if (warp == 1) {
     // ===================================================================== MMA issue
-    if (lane == 0) {
-      int s = 0; uint32_t par = 0; int tcount = 0;         // weight stage and its parity
-      int sb = 0; uint32_t parb = 0;                       // activation box slot and its parity
-      SegIter si; si.init(c, blockIdx.x, gridDim.x);
-      Seg sg;
-      for (; !failed && si.next(sg); ++tcount) {
-        // A tile of one box alternates between the two accumulators; a tile of two boxes holds both: the
-        // de-quantised weight stage then serves 512 tokens, and the accumulator of the first 256 is drained by
-        // the epilogue while the MMAs of the next tile already run on ... once it is free again (per-accumulator waits).
-        const int acc0 = c.nh == 2 ? 0 : (tcount & 1);
-        const int au = c.nh == 2 ? tcount : (tcount >> 1);   // earlier tiles that used this tile's accumulator(s)
-        const int h_lo = sg.half < 0 ? 0 : sg.half, h_hi = sg.half < 0 ? c.nh : sg.half + 1;   // (a half tile is a block's last)
-        for (int kb = sg.kb0; kb < sg.kb1 && !failed; ++kb) {
-          if (!pmbar_wait(full_a + 8 * s, par, abort_flag)) { failed = true; break; }
-          const uint64_t adesc = smem_desc_sw128(sbase + s * A_BYTES);
-          for (int h = h_lo; h < h_hi; ++h) {
-            if (kb == sg.kb0 && au >= 1 && !pmbar_wait(acc_empty + 8 * (acc0 + h), (au - 1) & 1, abort_flag)) { failed = true; break; }
-            // (bf16: the de-quantisers waited for the activation box themselves and converted it)
-            if (!CONV && !pmbar_wait(full_b + 8 * sb, parb, abort_flag)) { failed = true; break; }
-            tc_fence_after();
-            const uint32_t d_tmem = tmem_base + (uint32_t)((acc0 + h) * MAXBN);
-            const uint64_t bdesc = smem_desc_sw128(sbase + B_RING + sb * B_BYTES);
-            umma_kblock<false>(d_tmem, adesc, bdesc, c.idesc, kb > sg.kb0 ? 1u : 0u);
+    // (the whole warp walks the loop, so that stage indexes, parities and descriptors are warp-uniform; one elected
+    //  lane issues)
+    int s = 0; uint32_t par = 0; int tcount = 0;         // weight stage and its parity
+    int sb = 0; uint32_t parb = 0;                       // activation box slot and its parity
+    SegIter si; si.init(c, blockIdx.x, gridDim.x);
+    Seg sg;
+    for (; !failed && si.next(sg); ++tcount) {
+      // A tile of one box alternates between the two accumulators; a tile of two boxes holds both: the
+      // de-quantised weight stage then serves 512 tokens, and the accumulator of the first 256 is drained by
+      // the epilogue while the MMAs of the next tile already run on ... once it is free again (per-accumulator waits).
+      const int acc0 = c.nh == 2 ? 0 : (tcount & 1);
+      const int au = c.nh == 2 ? tcount : (tcount >> 1);   // earlier tiles that used this tile's accumulator(s)
+      const int h_lo = sg.half < 0 ? 0 : sg.half, h_hi = sg.half < 0 ? c.nh : sg.half + 1;   // (a half tile is a block's last)
+      for (int kb = sg.kb0; kb < sg.kb1 && !failed; ++kb) {
+        if (!pmbar_wait_warp(full_a + 8 * s, par, abort_flag)) { failed = true; break; }
+        const uint64_t adesc = smem_desc_sw128(sbase + s * A_BYTES);
+        for (int h = h_lo; h < h_hi; ++h) {
+          if (kb == sg.kb0 && au >= 1 && !pmbar_wait_warp(acc_empty + 8 * (acc0 + h), (au - 1) & 1, abort_flag)) { failed = true; break; }
+          // (bf16: the de-quantisers waited for the activation box themselves and converted it)
+          if (!CONV && !pmbar_wait_warp(full_b + 8 * sb, parb, abort_flag)) { failed = true; break; }
+          tc_fence_after();
+          const uint64_t bdesc = smem_desc_sw128(sbase + B_RING + sb * B_BYTES);
+          if (elect_one()) {
+            umma_kblock<false>(tmem_base + (uint32_t)((acc0 + h) * MAXBN), adesc, bdesc, c.idesc, kb > sg.kb0 ? 1u : 0u);
             umma_commit(empty_b + 8 * sb);              // the box is free once these MMAs have read it
-            if (++sb == BSLOTS) { sb = 0; parb ^= 1; }
+            if (h == h_hi - 1) umma_commit(empty_a + 8 * s);   // ... and the weight stage after the last of them
           }
-          if (failed) break;
-          umma_commit(empty_a + 8 * s);                 // ... and the weight stage after the last of them
-          if (++s == PSTAGES) { s = 0; par ^= 1; }
+          __syncwarp();
+          if (++sb == BSLOTS) { sb = 0; parb ^= 1; }
         }
         if (failed) break;
-        for (int h = h_lo; h < h_hi; ++h) umma_commit(acc_full + 8 * (acc0 + h));
-        // (the de-quantiser warps that help with the last segment's epilogue cannot follow the phases of the
-        //  accumulator barriers -- a parity wait cannot tell "not yet" from "two phases ago" -- so the last
-        //  segment completes a barrier of its own, which has this one phase)
-        SegIter peek = si;
-        Seg nxt;
-        if (!peek.next(nxt)) umma_commit(last_full);
+        if (++s == PSTAGES) { s = 0; par ^= 1; }
       }
-      if (c.pair_split && crank == 0 && !failed) {
-        // the first block of a pair: once its own MMAs are complete nothing reads its rings any more
-        if (pmbar_wait(last_full, 0, abort_flag)) {
+      if (failed) break;
+      // (the de-quantiser warps that help with the last segment's epilogue cannot follow the phases of the
+      //  accumulator barriers -- a parity wait cannot tell "not yet" from "two phases ago" -- so the last
+      //  segment completes a barrier of its own, which has this one phase)
+      SegIter peek = si;
+      Seg nxt;
+      const bool last = !peek.next(nxt);
+      if (elect_one()) {
+        for (int h = h_lo; h < h_hi; ++h) umma_commit(acc_full + 8 * (acc0 + h));
+        if (last) umma_commit(last_full);
+      }
+      __syncwarp();
+    }
+    if (c.pair_split && crank == 0 && !failed) {
+      // the first block of a pair: once its own MMAs are complete nothing reads its rings any more
+      if (pmbar_wait_warp(last_full, 0, abort_flag)) {
+        if (lane == 0) {
           asm volatile("fence.acq_rel.cluster;" ::: "memory");
           pmbar_arrive_peer(ppeer_addr(px_ready, 1u));
-        } else {
-          failed = true;
         }
+      } else {
+        failed = true;
       }
     }
   } else if (warp >= DQ_WARP0) {
