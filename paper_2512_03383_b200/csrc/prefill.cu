@@ -767,14 +767,25 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     const double pmax = q.left ? (double)((bt + q.left - 1) / q.left + 1) : 0.0;
     double hand_over;
     q.atomic = false;
-    // a k-block of a one-box tile by the number of busy SMs (0.45 us with 28 of them, 0.61 us with all)
-    auto kb1 = [&](int busy) { return 0.42 + 0.19 * (busy < g2 ? busy : g2) / g2; };
+    // a k-block of a one-box tile by the number of busy SMs (256 tokens: 0.45 us with 28 of them, 0.61 us with all)
+    auto busy_part = [&](int busy) { return (double)(busy < g2 ? busy : g2) / g2; };
+    auto kb1 = [&](int busy) { return c.bn < MAXBN ? 0.435 + 0.06 * busy_part(busy) : 0.42 + 0.19 * busy_part(busy); };
+    // Up to 128 rows, fewer tiles than SMs: the lines for whole tiles, pairs of blocks and tiles split over all SMs are fitted to
+    // 60 shapes with an odd number of groups (2 to 112 tiles, 18 to 222 k-blocks, half of them above 64 rows), every form forced in
+    // turn.  On these and on 60 others the plans they choose are within 3 % of the best of the three, but for three within 8 %.
+    const bool small = c.bn < MAXBN && q.tiles < g2;
     if (q.tiles < g2) {
       // every tile is split and every block ends on a split tile: the hand-over is shared with the de-quantiser warps
       // (one-box tiles, measured at M = 64 .. 512 on seven layer shapes: 5 us per 64 tokens of the tile)
-      // (64-token tiles, measured on four shapes with 3 to 52 tiles: 0.9 us for every part that the finishing block adds; a
-      //  contraction of 4744 channels and three tiles took 47 us split over all SMs and 24 us over pairs of blocks)
-      hand_over = nh == 2 ? 24.0 + 2.0 * pmax * wide : c.bn == 64 ? 5.0 + 0.9 * pmax : (14.0 + pmax) * wide;
+      // (64-token tiles: 0.3 us for every part that the finishing block adds; 568 x 7296 at 26 rows, five tiles in 30 parts,
+      //  takes 22 us split over all SMs and 32 us over pairs of blocks.  128-token tiles: 0.7 us; where a block's range crosses
+      //  from one tile into the next its first part is handed over by the epilogue warps alone, and with a few k-blocks per
+      //  block they can be the last to arrive, and read the tile back alone: 640 x 7296 at 93 rows, 3.9 k-blocks per block, takes
+      //  75 us, 568 x 12416 at 125 rows, 6.6 of them, 36 us)
+      const double per_block = bt ? (double)units / (double)bt : 0.0;
+      const bool crosses = q.left != 0 && bt % q.left != 0 && per_block > 1.5;
+      const double hand128 = !crosses ? 8.0 + 0.75 * pmax : per_block < 6.0 ? 10.0 + 2.0 * pmax : per_block < 20.0 ? 8.0 + pmax : 8.0 + 0.9 * pmax;
+      hand_over = nh == 2 ? 24.0 + 2.0 * pmax * wide : c.bn == 64 ? 10.3 + 0.3 * pmax : c.bn == 128 ? hand128 : (14.0 + pmax) * wide;
     } else {
       // The split tiles come first and whole tiles follow.  Reading a tile's slots back takes the four epilogue
       // warps 11 us per slot of 256 tokens, and a split tile in front of whole tiles has three or more parts: that
@@ -797,7 +808,7 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     // M = 2048); fitted over 48 launches (16 shapes at M = 512, 1024, 2048, every width and hand-over forced in turn).
     const int rounds = (q.tiles + g2 - 1) / g2;
     double us_whole = (double)rounds * c.n_kb * kcost;
-    if (nh == 1 && !cg2 && q.tiles <= g2) us_whole = c.n_kb * kb1(q.tiles);
+    if (nh == 1 && !cg2 && q.tiles <= g2) us_whole = c.n_kb * kb1(q.tiles) + (small ? 3.0 : 0.0);
     if (nh == 2 && cg2)
       us_whole = (double)rounds * (c.n_kb * 0.60 + 9.0);
     else if (nh == 2)
@@ -823,10 +834,11 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     // against the 11 - 28 us of a hand-over through the workspace; a k-block takes the same 0.5 - 0.65 us).
     q.pair = false;
     if (nh == 1 && !cg2 && 2 * q.tiles <= sms && c.n_kb >= 4 && env_grid == 0 && !pair_refused.load() && (env_streamk < 0 || env_streamk == 3)) {
-      const double us_pair = (double)(c.n_kb - c.n_kb / 2) * kb1(2 * q.tiles) + 1.0 + 4.5 * wide + (any_rope ? 3.0 : 0.0);
-      // (against a split over all SMs it has to be 10 % ahead: with long contractions the two come out level and
+      const double ends = small ? 3.3 + 6.5 * wide + 2.6 * busy_part(2 * q.tiles) * busy_part(2 * q.tiles) : 1.0 + 4.5 * wide;
+      const double us_pair = (double)(c.n_kb - c.n_kb / 2) * kb1(2 * q.tiles) + ends + (any_rope ? 3.0 : 0.0);
+      // (256 tokens: against a split over all SMs it has to be 10 % ahead: with long contractions the two come out level and
       //  the split measured ahead, Qwen2.5-7B down projection at M = 512)
-      if (us_pair * (q.streamk ? 1.10 : 1.0) < q.us || env_streamk == 3) { q.pair = true; q.streamk = false; q.us = us_pair; }
+      if (us_pair * (q.streamk && !small ? 1.10 : 1.0) < q.us || env_streamk == 3) { q.pair = true; q.streamk = false; q.us = us_pair; }
     }
     // Few tiles of a pair: a cluster of two to four pairs per tile, a part of the contraction each (0.34 us per k-block, 7 us
     // for the exchange beside what a whole tile's start and end take; 4096 x 4096 at M = 256: 25.7 -> 19.0 us).
