@@ -141,7 +141,8 @@ int uniql_set_path(int path);
  *                      pairs ("prefill_pair"): whole tiles, or with few tiles two to four pairs of a cluster per tile (forced
  *                      by 12 .. 14); up to 128 rows the blocks of a cluster share a tile.  Both are bit-reproducible.
  *   "prefill_pair"     -1 / 0: tiles of 256 weight rows over clusters of two blocks above 128 rows; 1 / 2 force them with one
- *                      or two boxes of 256 tokens per tile (tests)
+ *                      or two boxes of 256 tokens per tile (tests); 3 chooses as -1 and refuses every launch as clusters
+ *                      of this and of the batch kernel, as a device without room for them would (tests)
  *   "prefill_dual"     -1 / 0: above 256 tokens a tile of the tensor-core kernel takes both accumulators (512
  *                      tokens per de-quantised weight stage); 0 keeps tiles of 256 tokens; 1 forces tiles of 512 tokens
  *                      wherever M > 256 (tests: 2 the same without half tiles for the left-over round, 3 with them

@@ -33,7 +33,7 @@ const OptDesc kOpts[kOptCount] = {
     {"prefill_streamk", "UNIQL_PREFILL_STREAMK", -1},   // split tiles: -1 automatic, 0 never, 1 always (a slot per part), 2 always (one sum per tile), 3 pairs of blocks
     {"prefill_dual", "UNIQL_PREFILL_DUAL", -1},         // tiles of 512 tokens on both accumulators: -1 by cost, 0 never, 1 always (2 / 3: without / with half tiles)
     {"prefill_helpers", "UNIQL_PREFILL_HELPERS", 1},    // de-quantiser warps share the epilogue of a block's last tile
-    {"prefill_pair", "UNIQL_PREFILL_PAIR", -1},         // block pairs (cta_group::2): -1 by cost, 0 never, 1 / 2 always, with 256 / 512 tokens per tile
+    {"prefill_pair", "UNIQL_PREFILL_PAIR", -1},         // block pairs (cta_group::2): -1 by cost, 0 never, 1 / 2 always, with 256 / 512 tokens per tile, 3 by cost and refused at launch
     {"gemv_first", "UNIQL_GEMV_FIRST", 0},              // 1: the streaming kernel wherever it applies (M <= 4)
     {"gemv_depth", "UNIQL_GEMV_DEPTH", 0},              // ring slots per warp of the streaming kernel (0: automatic)
     {"wait_shift", "UNIQL_WAIT_SHIFT", 0},              // bounded device waits: limits divided by 2^shift (tests)

@@ -835,12 +835,16 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   // us).  Asking for a little more than half of the SM spreads them.  Ten stages are where that pays for the later start:
   // with four to eight (q|k|v, o_proj) a launch gains more from loading beside its predecessor (9.0 against 11.5 us).
   if (c.p > 1 && best_clusters * c.p <= device_sms() && c.spt >= 10 * c.p) smem = kSmemAlone;
-  BLaunch l(best_clusters * c.p, c.p, smem, cfg.stream);
-  if (cudaLaunchKernelEx(&l.lc, batch_instance(p.dt == UNIQL_BF16, c.head_kb != 0, c.exact != 0), p, c) != cudaSuccess) {
+  for (;;) {
+    BLaunch l(best_clusters * c.p, c.p, smem, cfg.stream);
+    const bool refused = c.p > 1 && opt(kOptPrefillPair) == 3;                 // tests
+    if (!refused && cudaLaunchKernelEx(&l.lc, batch_instance(p.dt == UNIQL_BF16, c.head_kb != 0, c.exact != 0), p, c) == cudaSuccess) return UNIQL_OK;
     cudaGetLastError();
-    return UNIQL_ERR_CUDA;
+    if (c.p == 1) return UNIQL_ERR_CUDA;
+    c.p = 1;                                                                   // clusters cannot be launched here: whole tiles
+    best_clusters = c.n_tiles < res.clusters[1] ? c.n_tiles : res.clusters[1];
+    smem = 1024 + (size_t)c.off_bar + 512;
   }
-  return UNIQL_OK;
 }
 
 }  // namespace uniql

@@ -558,6 +558,7 @@ int launch_as(const Params& p, const PrefillCfg& c, int grid, cudaStream_t strea
   attr[lc.numAttrs].val.clusterDim.y = 1;
   attr[lc.numAttrs].val.clusterDim.z = 1;
   ++lc.numAttrs;
+  if (opt(kOptPrefillPair) == 3) return UNIQL_ERR_UNSUPPORTED;             // tests
   if (cudaLaunchKernelEx(&lc, kern, p, c) != cudaSuccess) { cudaGetLastError(); return UNIQL_ERR_UNSUPPORTED; }
   return UNIQL_OK;
 }
@@ -665,13 +666,10 @@ int prefill_supported(const Params& p) {
   return 1;
 }
 
-int launch_prefill(const Params& p, const LaunchCfg& cfg) {
-  if (!cfg.workspace || cfg.ws_bytes < decode_workspace_header_bytes()) return UNIQL_ERR_WORKSPACE;   // status word
-  // up to 128 rows: the batch kernel (bf16: where the workspace has room for the fp16 copy)
-  if (batch_supported(p) &&
-      (p.dt != UNIQL_BF16 || (opt(kOptPrefillConvert) != 1 && cfg.ws_bytes >= ((decode_workspace_header_bytes() + 255) & ~(size_t)255) +
-                                                                               (size_t)p.M * ((p.k_in + 63) / 64 * 64) * 2 + 256)))
-    return launch_batch(p, cfg);
+namespace {
+
+// clusters: false after a launch as clusters was refused
+int launch_planned(const Params& p, const LaunchCfg& cfg, bool clusters) {
   const int env_grid = opt(kOptPrefillGrid), env_streamk = opt(kOptPrefillStreamk);
   PrefillCfg c;
   memset(&c, 0, sizeof(c));
@@ -735,17 +733,16 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
   bool any_rope = false;
   for (int j = 0; j < p.n_jobs; ++j) any_rope = any_rope || p.job[j].rope.enabled != 0;
   // Block pairs (cta_group::2): tiles of 256 rows, a cluster of two blocks where the other plans have one block.
-  const int opt_pair = opt(kOptPrefillPair);
+  const int opt_pair = opt(kOptPrefillPair) == 3 ? -1 : opt(kOptPrefillPair);
   int wt2 = 0, gp = 0;
   // (options that steer the one-block plans, forced by tests, keep the pairs out unless they are forced too)
   const bool pair_auto = opt_pair < 0 && env_grid == 0 && (env_streamk <= 0 || env_streamk > 10) && opt(kOptPrefillDual) <= 0;
-  if (c.bn == MAXBN && !conv_in_kernel && (pair_auto || opt_pair >= 1)) {
+  if (clusters && c.bn == MAXBN && !conv_in_kernel && (pair_auto || opt_pair >= 1)) {
     for (int j = 0; j < p.n_jobs; ++j) wt2 += (host_job_tiles(p.job[j]) + 1) / 2;
     gp = pair_capacity(1);
     if (env_grid >= 1 && env_grid < gp) gp = env_grid;
   }
   struct Plan { int nh, ttiles, tiles, left, g; int share; bool streamk, atomic, halves, pair, cg2; size_t sums; double us; };
-  static std::atomic<bool> pair_refused{false};       // a cluster launch was refused once: planned without from then on
   auto plan_for = [&](int nh, bool cg2) {
     Plan q;
     q.nh = nh;
@@ -833,7 +830,7 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     // contraction each, the second block's sums handed over through the first one's shared memory (about 5 us
     // against the 11 - 28 us of a hand-over through the workspace; a k-block takes the same 0.5 - 0.65 us).
     q.pair = false;
-    if (nh == 1 && !cg2 && 2 * q.tiles <= sms && c.n_kb >= 4 && env_grid == 0 && !pair_refused.load() && (env_streamk < 0 || env_streamk == 3)) {
+    if (nh == 1 && !cg2 && 2 * q.tiles <= sms && c.n_kb >= 4 && env_grid == 0 && clusters && (env_streamk < 0 || env_streamk == 3)) {
       const double ends = small ? 3.3 + 6.5 * wide + 2.6 * busy_part(2 * q.tiles) * busy_part(2 * q.tiles) : 1.0 + 4.5 * wide;
       const double us_pair = (double)(c.n_kb - c.n_kb / 2) * kb1(2 * q.tiles) + ends + (any_rope ? 3.0 : 0.0);
       // (256 tokens: against a split over all SMs it has to be 10 % ahead: with long contractions the two come out level and
@@ -915,12 +912,20 @@ int launch_prefill(const Params& p, const LaunchCfg& cfg) {
     rc = c.csplit > 1 ? launch_pair<__half, 3>(p, c, grid, cfg.stream)
          : c.nh == 1  ? launch_pair<__half, 1>(p, c, grid, cfg.stream)
                       : launch_pair<__half, 2>(p, c, grid, cfg.stream);
-  if (rc == UNIQL_ERR_UNSUPPORTED && c.pair_split) {
-    // the pairs cannot all be resident (or clusters cannot be launched here): planned again without them
-    pair_refused.store(true);
-    return launch_prefill(p, cfg);
-  }
-  return rc;
+  // (the clusters cannot all be resident, or cannot be launched here: planned again without them)
+  return rc == UNIQL_ERR_UNSUPPORTED && clusters ? launch_planned(p, cfg, false) : rc;
+}
+
+}  // namespace
+
+int launch_prefill(const Params& p, const LaunchCfg& cfg) {
+  if (!cfg.workspace || cfg.ws_bytes < decode_workspace_header_bytes()) return UNIQL_ERR_WORKSPACE;   // status word
+  // up to 128 rows: the batch kernel (bf16: where the workspace has room for the fp16 copy)
+  if (batch_supported(p) &&
+      (p.dt != UNIQL_BF16 || (opt(kOptPrefillConvert) != 1 && cfg.ws_bytes >= ((decode_workspace_header_bytes() + 255) & ~(size_t)255) +
+                                                                               (size_t)p.M * ((p.k_in + 63) / 64 * 64) * 2 + 256)))
+    return launch_batch(p, cfg);
+  return launch_planned(p, cfg, true);
 }
 
 size_t prefill_workspace_bytes(int M, int K) {

@@ -720,7 +720,7 @@ int launch_as(const Params& p, const PrefillCfg& c, int grid, cudaStream_t strea
       if (cudaOccupancyMaxActiveClusters(&n_clusters, kern, &lc) != cudaSuccess) { cudaGetLastError(); n_clusters = 0; }
       max_clusters.store(n_clusters);
     }
-    if (n_clusters * 2 < grid) return UNIQL_ERR_UNSUPPORTED;
+    if (n_clusters * 2 < grid || opt(kOptPrefillPair) == 3) return UNIQL_ERR_UNSUPPORTED;
   }
   if (cudaLaunchKernelEx(&lc, kern, p, c) != cudaSuccess) { cudaGetLastError(); return c.pair_split ? UNIQL_ERR_UNSUPPORTED : UNIQL_ERR_CUDA; }
   return UNIQL_OK;

@@ -128,3 +128,20 @@ def test_tiles_shared_by_the_pairs_of_a_cluster(B, M, dtype, share):
         y, ref = run_ex(B, qw, dw, x, dtype, im, 0, None, 200, ldx_pad=8)
         check_output(y, ref, dtype, TOL, "per-head input map shared by %d" % share)
     assert B.workspace_status() == 0
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("M,N,K", [(300, 700, 512), (200, 300, 1024), (1100, 1500, 128), (48, 300, 2048), (12, 300, 2048), (100, 300, 1920)])
+def test_refused_cluster_launches(B, M, N, K, dtype):
+    """A device that does not take the clusters a plan asks for: the call runs on single blocks instead of failing (pairs of
+    one and two boxes, pairs that share a tile, the batch kernel's shared tiles, tiles shared by two blocks)."""
+    rng = np.random.default_rng(2350 + M)
+    qw = synth.draw_qweight(rng, N, K)
+    dw = dev_weight(qw)
+    x = synth.draw_x(rng, M, K, dtype)
+    B.set_option("prefill_pair", 3)
+    for split in (-1, 3, 12):
+        B.set_option("prefill_streamk", split)
+        y, ref = run_ex(B, qw, dw, x, dtype, None, K, None, N)
+        check_output(y, ref, dtype, TOL, "refused clusters M=%d %s split %d" % (M, dtype, split))
+    assert B.workspace_status() == 0
