@@ -201,7 +201,7 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
   // fp16: its instance that multiplies the codes themselves, by the rule of exact_batch().
   const bool batch = path == UNIQL_PATH_AUTO &&
                      (p.dt == UNIQL_BF16 ? p.M > 8 && p.M <= 16 && batch_supported(p) &&
-                                               (!cfg.workspace || cfg.ws_bytes >= prefill_workspace_bytes(p.M, p.K))
+                                               (!cfg.workspace || cfg.ws_bytes >= batch_workspace_min(p.dt, p.M, p.k_in))
                                          : exact_batch(p));
   if (path == UNIQL_PATH_AUTO)
     path = batch ? UNIQL_PATH_PREFILL : gv ? UNIQL_PATH_GEMV : dec_ok ? UNIQL_PATH_DECODE : (pre_ok ? UNIQL_PATH_PREFILL : UNIQL_PATH_GENERIC);
@@ -304,7 +304,8 @@ extern "C" size_t uniql_workspace_bytes(int M, int K, int N_total) {
   // (+ room for the activations re-laid on 8-channel boundaries, see dispatch())
   const size_t relay = (((size_t)M * (size_t)(K + 8) * 2) + 255) / 256 * 256 + 512;
   if (M > 16) return prefill_workspace_bytes(M, K) + relay;
-  const size_t a = decode_workspace_bytes(M, K, N_total), b = M <= 4 ? gemv_workspace_bytes(M, K, N_total) : 0;
+  const size_t a = decode_workspace_bytes(M, K, N_total);
+  const size_t b = M <= 4 ? gemv_workspace_bytes(M, K, N_total) : M > 8 ? batch_workspace_bytes(M, K) : 0;
   return (a > b ? a : b) + relay;
 }
 

@@ -731,6 +731,16 @@ int batch_supported(const Params& p) {
   return batch_families(p, nullptr) > 0;
 }
 
+// What a launch cannot do without (the header and the fp16 copy of bf16 activations), and with room for every split.
+size_t batch_workspace_min(int dt, int M, int k_in) {
+  const size_t header = (decode_workspace_header_bytes() + 255) & ~(size_t)255;
+  return dt == UNIQL_BF16 ? header + (size_t)M * ((k_in + 63) / 64 * 64) * 2 + 256 : header;
+}
+size_t batch_workspace_bytes(int M, int K) {
+  const size_t n = (M + 15) / 16 * 16;
+  return batch_workspace_min(UNIQL_BF16, M, K) + (size_t)2 * device_sms() * 2 * n * BMW * 4;
+}
+
 // Whether an fp16 launch of up to 16 rows goes to the EXACT instance instead of the decode kernel.  From twelve rows: the
 // decode kernel's activation traffic grows with the rows (a layer 8 - 12 % from nine to sixteen), this instance's does not,
 // and they meet between nine and fifteen rows depending on the shape.  Measured at 12 / 16 rows, decode kernel -> here, the
@@ -802,8 +812,8 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
     int fit = res.clusters[k];
     if (env_grid >= 1 && env_grid / k < fit) fit = env_grid / k;              // tests: several tiles per block on small problems
     if (fit < 1 || k > c.spt) continue;
-    if (k > 1 && (env_split == 0 || cfg.ws_bytes < used + (size_t)fit * k * 2 * c.n * BMW * 4)) continue;
     const int clusters = c.n_tiles < fit ? c.n_tiles : fit;
+    if (k > 1 && (env_split == 0 || cfg.ws_bytes < used + (size_t)clusters * k * 2 * c.n * BMW * 4)) continue;
     const int rounds = (c.n_tiles + fit - 1) / fit;
     double cost = rounds * ((double)c.spt / k * (clusters * k > device_sms() ? 1.05 : 0.65) + (k > 1 ? 3.0 : 1.0));
     if (env_split >= 1 && env_split <= 3 && k > 1) cost *= 1e-3;              // tests: split wherever it is possible

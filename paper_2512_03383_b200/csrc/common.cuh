@@ -191,6 +191,8 @@ int gemv_mlp_supported(const MlpDecode& d);
 // tensor-core kernel for up to 128 rows (csrc/batch.cu), taken by launch_prefill where its rules hold
 int launch_batch(const Params& p, const LaunchCfg& cfg);
 int batch_supported(const Params& p);
+size_t batch_workspace_min(int dt, int M, int k_in);
+size_t batch_workspace_bytes(int M, int K);
 int exact_batch(const Params& p);             // twelve to sixteen fp16 rows on its exact-code instance
 // fp16 copy of bf16 activations [M][k_in], row pitch ldo (a multiple of 8; the columns from k_in on are zeros)
 int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo, cudaStream_t stream);

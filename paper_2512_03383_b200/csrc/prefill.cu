@@ -921,9 +921,7 @@ int launch_planned(const Params& p, const LaunchCfg& cfg, bool clusters) {
 int launch_prefill(const Params& p, const LaunchCfg& cfg) {
   if (!cfg.workspace || cfg.ws_bytes < decode_workspace_header_bytes()) return UNIQL_ERR_WORKSPACE;   // status word
   // up to 128 rows: the batch kernel (bf16: where the workspace has room for the fp16 copy)
-  if (batch_supported(p) &&
-      (p.dt != UNIQL_BF16 || (opt(kOptPrefillConvert) != 1 && cfg.ws_bytes >= ((decode_workspace_header_bytes() + 255) & ~(size_t)255) +
-                                                                               (size_t)p.M * ((p.k_in + 63) / 64 * 64) * 2 + 256)))
+  if (batch_supported(p) && (p.dt != UNIQL_BF16 || (opt(kOptPrefillConvert) != 1 && cfg.ws_bytes >= batch_workspace_min(p.dt, p.M, p.k_in))))
     return launch_batch(p, cfg);
   return launch_planned(p, cfg, true);
 }

@@ -103,3 +103,21 @@ def test_mlp_block_stays_inside(B, M):
         check_output(h, h_ref, "f16", TOL_H if M <= 16 else 6e-4, "h M=%d" % M)
         check_output(y, y_ref, "f16", TOL_Y, "y M=%d" % M)
         assert band_intact(buf, nbytes), "wrote behind the workspace: MLP M=%d" % M
+
+
+@pytest.mark.parametrize("M,dtype", [(9, "bf16"), (16, "bf16"), (12, "f16"), (16, "f16")])
+def test_advertised_workspace_gives_the_bits_of_the_librarys_own(B, M, dtype):
+    """Nine to sixteen rows: the kernel and the split of a tile depend on the room in the workspace; the advertised size has
+    room for what the library's own buffer gives."""
+    rng = np.random.default_rng(1500 + M)
+    for (N, K) in ((256, 1024), (4096, 4096)):
+        qw = synth.random_qweight_fast(rng, N, K)
+        dw = dev_weight(qw)
+        nbytes = B.workspace_bytes(M, K, N)
+        buf, ws = guarded(B, nbytes)
+        x = dev_x(synth.draw_x(rng, M, K, dtype), dtype)
+        y = [torch.zeros((M, N), dtype=x.dtype, device="cuda") for _ in range(2)]
+        for out, w in zip(y, (None, ws)):
+            B.qlinear_ex(x, K, *dw[1:], None, M, K, N, None, K, None, N, out, N, workspace=w)
+        assert band_intact(buf, nbytes) and B.workspace_status(ws) == 0
+        assert torch.equal(y[0], y[1]), "M=%d %s %s" % (M, dtype, (N, K))
