@@ -1818,7 +1818,9 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
   if (count_tile_fams(p) > kMaxTF) return UNIQL_ERR_UNSUPPORTED;
 
   // integer path: fp16 activations staged with 128-bit loads (a leading input block); UNIQL_DECODE_I8=0: fp16 MMAs
-  const bool i8 = decode_integer_path(p) && opt(kOptDecodeI8) != 0;
+  // (the launches of uniql_qlinear_noalloc, which clear the header, are never re-laid: on 4-channel boundaries that entry point
+  //  has unrounded activations on the fp16 MMAs, and keeps them)
+  const bool i8 = decode_integer_path(p) && (c.x_vec || !cfg.clear_header) && opt(kOptDecodeI8) != 0;
   // Streamed activations for rows too long to stage whole beside the ring (which would otherwise split the input
   // channels over several groups of blocks and hand every tile over); UNIQL_DECODE_XSTREAM=0/1 forces.  Where the
   // staged copy fits the quantising kernel in front costs more than the staging it saves (measured 3.5 us), and

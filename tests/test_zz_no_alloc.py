@@ -47,6 +47,27 @@ def test_noalloc_matches_oracle_and_regular_entry_point_twice_in_a_row():
         B.set_path(B.PATH_AUTO)
 
 
+@pytest.mark.parametrize("M", [1, 4, 12])
+def test_noalloc_on_four_channel_boundaries_is_not_quantised(M):
+    """1740 channels are no multiple of 8: the fixed-scratch entry point multiplies the fp16 activations themselves there.  What
+    keeps an output from being the correctly rounded one is then the fp32 sums, which carry the codes' offset of 1024: about
+    25000 per group of 128 (1032 times a sum of activations of rms 2), 2^-24 of it per addition and 112 additions, times a
+    scale of 0.008: 1e-4 at most beside a spacing of 1e-3, so one or two outputs in ten.  Activations in 16-bit fixed point
+    (2^-17 of a group's maximum of 60, times weights of 0.02, over 1740 channels: 2e-4) make it three in ten."""
+    from paper_2512_03383_b200 import binding as B
+    rng = np.random.default_rng(127)
+    qw = synth.draw_qweight(rng, 512, 2048)
+    packed, wp, ws, wz = dev_weight(qw)
+    k = synth.keep_count(0.85, 2048)
+    x32 = synth.draw_x(rng, M, k, "f16")
+    y = torch.zeros((M, 512), dtype=torch.float16, device="cuda")
+    B.qlinear_noalloc(dev_x(x32, "f16"), wp, ws, wz, M, 2048, 512, k, 512, y)
+    torch.cuda.synchronize()
+    assert B.noalloc_status() == 0
+    o = oracle.qlinear(x32, packed, qw.scales, qw.zeros, oracle.leading(512), oracle.leading(k))
+    assert (y.cpu().numpy() != o.astype(np.float16)).mean() < 0.2
+
+
 @pytest.mark.parametrize("rate", [1.0, 0.65])
 def test_noalloc_llama_mlp_matrices_at_sixteen_rows(rate):
     """The header promises that the Llama-3-8B MLP matrices fit the fixed array for every M <= 16."""
