@@ -3,13 +3,26 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import check_output, dev_weight
+import oracle
+from helpers import check_output, dev_weight, dev_x
 from test_gpu_prefill import B, run_ex  # noqa: F401  (B: fixture)
 from paper_2512_03383_b200 import synth
 
 pytestmark = pytest.mark.gpu
 
 TOL = 5e-4       # as the other tensor-core tests: weights rounded once to fp16, fp32 sums
+
+
+def in_flight(B, dw, x, dtype, in_map, k_in, N, K, count):
+    """`count` launches behind one another with nothing between them, each into an output of its own: blocks of two launches
+    share the SMs and their tensor memory, codes are fetched before the launch in front is complete, and every launch uses
+    the slots of the one in front."""
+    xd = dev_x(x, dtype)
+    out = [torch.full((x.shape[0], N), -77.0, device="cuda", dtype=xd.dtype) for _ in range(count)]
+    for y in out:
+        B.qlinear_ex(xd, xd.shape[1], *dw[1:], None, x.shape[0], K, N, in_map, k_in, None, N, y, N)
+    torch.cuda.synchronize()
+    return out
 
 
 @pytest.mark.parametrize("M", [17, 48, 64, 100, 128])
@@ -24,10 +37,8 @@ def test_long_contractions(B, M, split):
         x = synth.draw_x(rng, M, K, "f16")
         y, ref = run_ex(B, qw, dw, x, "f16", None, K, None, N)
         check_output(y, ref, "f16", TOL, "M=%d N=%d K=%d" % (M, N, K))
-        first = y.clone()
-        for _ in range(20):                        # (launches behind one another: blocks of two launches share the SMs)
-            y, _ = run_ex(B, qw, dw, x, "f16", None, K, None, N)
-        assert torch.equal(y, first)
+        for again in in_flight(B, dw, x, "f16", None, K, N, K, 20):
+            assert torch.equal(again, y)
     assert B.workspace_status() == 0
     B.set_path(B.PATH_AUTO)
     B.reset_options()
@@ -51,8 +62,7 @@ def test_exact_codes(B, M, N, K, take, split):
     x = synth.draw_x(rng, M, synth.map_size(im) if im else k_in, "f16")
     y, ref = run_ex(B, qw, dw, x, "f16", im, k_in, None, N)
     check_output(y, ref, "f16", 3e-4, "M=%d N=%d K=%d %s" % (M, N, K, take))
-    for _ in range(5):
-        again, _ = run_ex(B, qw, dw, x, "f16", im, k_in, None, N)
+    for again in in_flight(B, dw, x, "f16", im, k_in, N, K, 20):
         assert torch.equal(again, y)
     assert B.workspace_status() == 0
     B.set_path(B.PATH_AUTO)
@@ -74,6 +84,8 @@ def test_code_ring_wraps_in_every_instance(B, M, dtype, heads):
     x = synth.draw_x(rng, M, synth.map_size(im) if im else K, dtype)
     y, ref = run_ex(B, qw, dw, x, dtype, im, 0 if im else K, None, N)
     check_output(y, ref, dtype, TOL, "M=%d %s heads %d" % (M, dtype, heads))
+    for again in in_flight(B, dw, x, dtype, im, 0 if im else K, N, K, 20):
+        assert torch.equal(again, y)
     assert B.workspace_status() == 0
     B.set_path(B.PATH_AUTO)
     B.reset_options()
@@ -99,3 +111,43 @@ def test_options_of_the_decode_kernel_ask_for_it(B, option, value):
     B.set_path(B.PATH_AUTO)
     batch, _ = run_ex(B, qw, dw, x, "f16", None, 2048, None, 300)
     assert torch.equal(got[0], got[1]) and not torch.equal(got[0], batch)
+
+
+@pytest.mark.parametrize("M,dtype", [(12, "f16"), (16, "f16"), (12, "bf16"), (40, "f16"), (128, "f16"), (128, "bf16")])
+@pytest.mark.parametrize("split", [0, -1])
+def test_chain_of_dependent_launches(B, M, dtype, split):
+    """Every launch reads what the one in front wrote, and its matrix has another shape, so that the number of blocks that
+    share a tile changes from launch to launch: the bits are those without programmatic dependent launch."""
+    B.set_path(B.PATH_PREFILL)
+    B.set_option("prefill_streamk", split)
+    rng = np.random.default_rng(2700 + M)
+    sizes = [(1536, 512), (4096, 1536), (512, 4096)]               # (N, K), in turn
+    ws = [synth.draw_qweight(rng, n, k) for n, k in sizes]
+    ds = [dev_weight(w) for w in ws]
+    x = synth.draw_x(rng, M, 512, dtype) * np.float32(2.0 ** -6)
+    xd = torch.from_numpy(x).cuda().to(torch.float16 if dtype == "f16" else torch.bfloat16)
+
+    def chain(pdl):
+        B.set_option("pdl", pdl)
+        outs, src = [], xd
+        for i in range(9):
+            (n, k), d = sizes[i % 3], ds[i % 3]
+            y = torch.zeros((M, n), dtype=xd.dtype, device="cuda")
+            B.qlinear_ex(src, k, *d[1:], None, M, k, n, None, k, None, n, y, n)
+            outs.append(y)
+            src = y
+            if i % 3 == 2:                                         # (kept in range, on the same stream)
+                src = y * (2.0 ** -6 / y.abs().amax().clamp_min(1e-3)).to(y.dtype)
+        torch.cuda.synchronize()
+        return outs
+
+    off = chain(0)
+    assert all(torch.isfinite(y.float()).all() and y.abs().amax() > 0 for y in off)
+    for rep in range(5):
+        for i, (a, b) in enumerate(zip(chain(1), off)):
+            assert torch.equal(a, b), "link %d repeat %d" % (i, rep)
+    ref = oracle.qlinear(xd.float().cpu().numpy(), ds[0][0], ws[0].scales, ws[0].zeros, oracle.leading(1536), oracle.leading(512))
+    check_output(off[0], ref, dtype, TOL, "first link M=%d %s" % (M, dtype))
+    assert B.workspace_status() == 0
+    B.set_path(B.PATH_AUTO)
+    B.reset_options()
