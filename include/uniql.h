@@ -76,17 +76,21 @@ typedef enum {
 
 typedef enum { UNIQL_F16 = 0, UNIQL_BF16 = 1 } uniql_dtype;
 
-/* Kernel selection, for A/B tests.  AUTO: batches of M <= 16 take the persistent decode kernel
- * (UNIQL_PATH_DECODE; bf16 wherever its 16-byte loads apply: input blocks on 8-channel boundaries, or re-laid on them); where the input map lies on 4- but not on 8-channel boundaries (head dims 108 and 84 on the
- * input side of o_proj, 1740 of 2048 leading channels) a small kernel in front re-lays the activations on
- * 8-channel boundaries in the workspace, and batches of M <= 4 for which that is not possible (no room in the
- * workspace, blocks that do not start on 8-channel boundaries) take the streaming kernel (UNIQL_PATH_GEMV:
- * every warp copies its own share of the codes through a private shared-memory ring) when its rules hold (one
- * input family, every start / keep / period a multiple of 4, K a multiple of 512, x 8-byte aligned with ldx a
- * multiple of 4, scale and zero-point arrays 8-byte aligned); everything
- * else the tensor-core (prefill) kernel when its alignment rules hold (activations 16-byte
- * aligned with a row pitch that is a multiple of 8, input map a leading block or one family of per-head
- * blocks on 64-channel boundaries with keep % 8 == 0), otherwise the generic kernel. */
+/* Kernel selection, for A/B tests.  AUTO:
+ *  - batches of M <= 16 take the persistent decode kernel (UNIQL_PATH_DECODE).  Its integer path (bf16: the only one) wants
+ *    one input family on 8-channel boundaries, or on 4-channel ones at one to four and nine to sixteen rows; at five to
+ *    eight rows, and wherever blocks are no multiple of 4 (head dims 108 and 84 on the input side of o_proj, 870 leading
+ *    channels), a small kernel in front re-lays the activations on 8-channel boundaries in the workspace.  Batches of
+ *    M <= 4 that the integer path cannot take even so go to the streaming kernel (UNIQL_PATH_GEMV: every warp copies its own
+ *    share of the codes through a private shared-memory ring) when its rules hold (one input family, every start / keep /
+ *    period a multiple of 4, K a multiple of 512, x 8-byte aligned with ldx a multiple of 4, scale and zero-point arrays
+ *    8-byte aligned);
+ *  - fp16 at twelve to sixteen rows and bf16 at nine to sixteen go to the batch kernel instead where its rules hold, unless an
+ *    option of the decode kernel ("decode_*") is off its default (fp16);
+ *  - everything else goes to the tensor cores (UNIQL_PATH_PREFILL: the batch kernel up to 128 rows, block pairs above,
+ *    single blocks for what neither takes) when their alignment rules hold (activations 16-byte aligned, or re-laid, with
+ *    a row pitch that is a multiple of 8, input map a leading block or one family of per-head blocks on 64-channel
+ *    boundaries with keep % 8 == 0), otherwise to the generic kernel. */
 typedef enum { UNIQL_PATH_AUTO = 0, UNIQL_PATH_GENERIC = 1, UNIQL_PATH_DECODE = 2,
                UNIQL_PATH_PREFILL = 3, UNIQL_PATH_GEMV = 4 } uniql_path;
 

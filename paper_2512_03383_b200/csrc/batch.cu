@@ -742,10 +742,10 @@ size_t batch_workspace_bytes(int M, int K) {
 }
 
 // Whether an fp16 launch of up to 16 rows goes to the EXACT instance instead of the decode kernel.  From twelve rows: the
-// decode kernel's activation traffic grows with the rows (a layer 8 - 12 % from nine to sixteen), this instance's does not,
-// and they meet between nine and fifteen rows depending on the shape.  Measured at 12 / 16 rows, decode kernel -> here, the
-// whole layer in microseconds: Qwen2.5-7B 84 -> 75 / 90 -> 75, Mamba2-2.7B 29.1 -> 23.3 / 32.1 -> 23.2, Llama-3-8B 75.9 -> 75.2 /
-// 79.2 -> 74.9, at keep 0.75 - / 75.8 -> 66.5, at keep 0.65 68.3 -> 70.5 / 72.7 -> 70.3.
+// decode kernel's activation traffic grows with the rows (a layer 8 - 12 % from nine to sixteen), this instance's does not.
+// Measured at 12 / 16 rows, decode kernel -> here, the whole layer in microseconds: Qwen2.5-7B 84.2 -> 71.7 / 90.6 -> 71.4,
+// Mamba2-2.7B 29.0 -> 22.5 / 31.4 -> 22.5, Llama-3-8B 76.0 -> 71.6 / 79.6 -> 71.7, at keep 0.75 71.9 -> 63.6 / 74.9 -> 63.5, at keep
+// 0.65 68.6 -> 66.6 / 72.9 -> 67.2; over five keep rates from 0.55 the decode kernel is nowhere ahead by more than 1 %.
 // Not where kept blocks of output rows are no multiple of 8: the launch that reads those channels then stays on the decode
 // kernel (4-channel boundaries), whose blocks need a whole SM and cannot come in beside this kernel's (Mamba2 mixer at keep
 // 0.8 29.5 -> 30.7 us).  Rotated heads excepted: there the other four launches of a layer outweigh that.
@@ -765,7 +765,7 @@ int exact_batch(const Params& p) {
 
 // Measured (Llama-3-8B, M = 17 / 64 / 128, against the prefill kernel): q|k|v 18.5 / 21.5 / 21.4 -> 11.5 / 13.0 / 17.2 us, o_proj
 // 20.2 / 24.4 / 27.6 -> 9.1 / 13.2 / 12.0 us, down projection 36 / 36 / 40 -> 18 / 17 / 21 us, whole layer at M = 64 and keep
-// 0.85 137 -> 75 us.  What bounds it now: the issue slots of SMs that hold two tiles (0.65 us per stage and block alone on
+// 0.85 137 -> 69 us.  What bounds it now: the issue slots of SMs that hold two tiles (0.65 us per stage and block alone on
 // its SM, 1.05 us for two), and 7 us per launch before the first and after the last stage.
 int launch_batch(const Params& p, const LaunchCfg& cfg) {
   BatchCfg c;
