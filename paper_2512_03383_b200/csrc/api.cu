@@ -142,13 +142,15 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
   // The rows of a decode launch: option "decode_split_batch" (or streaming turned off) runs nine to sixteen rows as two
   // launches, and what those can take is asked for them (five to eight rows need activations on 8-channel boundaries).
   const bool streams = opt(kOptDecodeSplitBatch) == 2 && opt(kOptDecodeI8) != 0 && opt(kOptDecodeXstream) != 0;
-  auto as_launched = [&](const Params& a) {
+  const bool halves = p.M > 8 && p.M <= 16 && !streams && opt(kOptDecodeSplitBatch) != 0;
+  auto as_launched = [&](const Params& a, int (*holds)(const Params&)) {
+    if (!halves) return holds(a) != 0;
     Params q = a;
-    if (q.M > 8 && q.M <= 16 && !streams && opt(kOptDecodeSplitBatch) != 0) q.M = (q.M + 1) / 2;
-    return q;
+    q.M = (q.M + 1) / 2;
+    return holds(q) != 0;
   };
-  auto decodes = [&](const Params& a) { return a.M <= 16 && decode_supported(as_launched(a)); };
-  auto on_integers = [&](const Params& a) { return decode_integer_path(as_launched(a)) != 0; };
+  auto decodes = [&](const Params& a) { return a.M <= 16 && as_launched(a, decode_supported); };
+  auto on_integers = [&](const Params& a) { return as_launched(a, decode_integer_path); };
   bool dec_ok = decodes(p);
   // every batch the decode kernel does not take (more than 16 rows) goes to the tensor cores when the maps
   // allow it: at 17..63 rows the generic kernel measured 13 to 26 times slower (930 us against 71 us for the
