@@ -35,6 +35,7 @@
 #include <string.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "quant.cuh"
@@ -349,14 +350,14 @@ __global__ void __launch_bounds__(256) xquant_kernel(const Phase P, int M, int v
         if (t0 >= 0) in = __ldg(reinterpret_cast<const uint4*>(x + (size_t)m * P.ldx + t0));
       }
     }
-    uint2 hi2, lo2;
+    const uint4 unit[1] = {in};
+    uint2 hi2[1], lo2[1];
     int isum;
     float inv_scale;
-    quantise16<T>(in, hi2, lo2, isum, inv_scale);
+    quantise_units<T, 1>(unit, hi2, lo2, isum, inv_scale);
     if (u < n_units) {
-      const int off = (u16 >> 2) * 32 + (u16 & 3) * 8;
-      *reinterpret_cast<uint2*>(xq + ((size_t)lv * vr + 2 * m) * 128 + off) = hi2;
-      *reinterpret_cast<uint2*>(xq + ((size_t)lv * vr + 2 * m + 1) * 128 + off) = lo2;
+      *reinterpret_cast<uint2*>(xq + ((size_t)lv * vr + 2 * m) * 128 + u16 * 8) = hi2[0];
+      *reinterpret_cast<uint2*>(xq + ((size_t)lv * vr + 2 * m + 1) * 128 + u16 * 8) = lo2[0];
       if (u16 == 0) xg[lv * xg_stride + m] = make_float2((float)isum, inv_scale);
     }
   }
@@ -923,7 +924,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
       const bool xc = xc_on;
       const int crank = xc ? (int)cluster_rank() : 0, csh = xc ? 1 : 0;
       const int n_pairs = Gn * p.M;
-      const int n_units = ((n_pairs - crank + csh) >> csh) * 16;     // units of this block's pairs
+      const int my_pairs = (n_pairs - crank + csh) >> csh;            // this block's pairs
       unsigned char* xb = smem + c.off_x;
       uint32_t px = 0, pxg = 0;                                      // the other block's x and xg regions
       if (xc) {
@@ -931,57 +932,72 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
         px = peer_addr(sbase + (uint32_t)c.off_x, (uint32_t)(crank ^ 1));
         pxg = peer_addr(sbase + (uint32_t)c.off_xg, (uint32_t)(crank ^ 1));
       }
-      constexpr int UN = 4;
-      for (int u0 = ctid; u0 < ((n_units + 31) & ~31); u0 += CTH * UN) {
-        uint4 in[UN];
-        if (NPH == 1 && NT != 2 && P.x4) {
+      // U units of eight activations per thread, 16 / U lanes per (row, group).  Lane l takes the units l, l + 16 / U, ... of
+      // its group's sixteen (consecutive 16 bytes of x from lane to lane), the U groups of a half-warp beginning at different
+      // ones: their 8-byte stores, 128 bytes apart from group to group, then hit distinct banks.  UN: threads' worth in flight.
+      auto quantise = [&](auto units, auto in_flight) {
+        constexpr int U = decltype(units)::value, UN = decltype(in_flight)::value, LG = 16 / U;
+        const int l = lane & (LG - 1), rot = (lane / LG) & (U - 1);
+        const int n = my_pairs * LG, n32 = (n + 31) & ~31;
+        for (int u0 = ctid; u0 < n32; u0 += CTH * UN) {
+          uint4 in[UN][U];
+          int lvs[UN], row[UN];
 #pragma unroll
-          for (int q4 = 0; q4 < UN; ++q4) {
-            const int u = u0 + q4 * CTH;
-            in[q4] = make_uint4(0, 0, 0, 0);
-            if (u < n_units) {
-              const int pair = u >> 4, m = row_of(pair), lv = needed_group(pair - m * Gn);
-              if (lv < Gk) in[q4] = load_halves(x + (size_t)m * ldx, (sg_lo + lv) * kGroup + 8 * (u & 15), compact_of);
+          for (int j = 0; j < UN; ++j) {
+            const int u = u0 + j * CTH;
+            lvs[j] = -1; row[j] = 0;
+#pragma unroll
+            for (int k = 0; k < U; ++k) in[j][k] = make_uint4(0, 0, 0, 0);
+            if (u < n) {
+              const int pair = ((u / LG) << csh) + crank, m = row_of(pair), lv = needed_group(pair - m * Gn);
+              if (lv < Gk) {
+                lvs[j] = lv; row[j] = m;
+                const T* xrow = x + (size_t)m * ldx;
+#pragma unroll
+                for (int k = 0; k < U; ++k) {
+                  const int ch = (sg_lo + lv) * kGroup + 8 * (l + LG * ((k + rot) & (U - 1)));
+                  if (NPH == 1 && NT != 2 && P.x4) {
+                    in[j][k] = load_halves(xrow, ch, compact_of);
+                  } else {
+                    const int t0 = compact_of(ch);
+                    if (t0 >= 0) in[j][k] = load16(xrow + t0);
+                  }
+                }
+              }
             }
           }
-        } else {
 #pragma unroll
-          for (int q4 = 0; q4 < UN; ++q4) {
-            const int u = u0 + q4 * CTH;
-            in[q4] = make_uint4(0, 0, 0, 0);
-            if (u < n_units) {
-              const int pair = ((u >> 4) << csh) + crank, m = row_of(pair), lv = needed_group(pair - m * Gn);
-              const int t0 = compact_of((sg_lo + lv) * kGroup + 8 * (u & 15));
-              if (lv < Gk && t0 >= 0) in[q4] = load16(x + (size_t)m * ldx + t0);
+          for (int j = 0; j < UN; ++j) {
+            if (u0 + j * CTH >= n32) break;                          // warp-uniform
+            uint2 hi[U], lo[U];
+            int isum;
+            float inv_scale;
+            quantise_units<T, U>(in[j], hi, lo, isum, inv_scale);
+            if (lvs[j] >= 0) {
+              // unit c'*4 + i (word i of lane quarter c'): 8 bytes at c'*32 + i*8 of the group's 128 bytes
+              const int m = row[j], at = (2 * m) * c.xrow + lvs[j] * 128 + l * 8;
+#pragma unroll
+              for (int k = 0; k < U; ++k) {
+                const int o = at + ((k + rot) & (U - 1)) * (LG * 8);
+                *reinterpret_cast<uint2*>(xb + o) = hi[k];
+                *reinterpret_cast<uint2*>(xb + o + c.xrow) = lo[k];
+                if (xc) {
+                  st_peer_v2(px + (uint32_t)o, hi[k].x, hi[k].y);
+                  st_peer_v2(px + (uint32_t)(o + c.xrow), lo[k].x, lo[k].y);
+                }
+              }
+              if (l == 0) {
+                xg[lvs[j] * 8 * MT + m] = make_float2((float)isum, inv_scale);
+                if (xc) st_peer_v2(pxg + (uint32_t)((lvs[j] * 8 * MT + m) * 8), (uint32_t)__float_as_int((float)isum), (uint32_t)__float_as_int(inv_scale));
+              }
             }
           }
         }
-#pragma unroll
-        for (int q4 = 0; q4 < UN; ++q4) {
-          const int u = u0 + q4 * CTH;
-          if (u >= ((n_units + 31) & ~31)) break;                  // warp-uniform
-          const int u16 = u & 15, pair = u < n_units ? ((u >> 4) << csh) + crank : 0;
-          const int m = row_of(pair), lv = needed_group(pair - m * Gn);
-          const bool in_range = u < n_units && lv < Gk;
-          uint2 hi2, lo2;
-          int isum;
-          float inv_scale;
-          quantise16<T>(in[q4], hi2, lo2, isum, inv_scale);
-          if (in_range) {
-            // word j of lane quarter c' (u16 = c'*4 + j): 8 bytes at c'*32 + j*8 of the group's 128 bytes
-            const int off = lv * 128 + (u16 >> 2) * 32 + (u16 & 3) * 8;
-            *reinterpret_cast<uint2*>(xb + (size_t)(2 * m) * c.xrow + off) = hi2;
-            *reinterpret_cast<uint2*>(xb + (size_t)(2 * m + 1) * c.xrow + off) = lo2;
-            if (u16 == 0) xg[lv * 8 * MT + m] = make_float2((float)isum, inv_scale);
-            if (xc) {
-              st_peer_v2(px + (uint32_t)((2 * m) * c.xrow + off), hi2.x, hi2.y);
-              st_peer_v2(px + (uint32_t)((2 * m + 1) * c.xrow + off), lo2.x, lo2.y);
-              if (u16 == 0) st_peer_v2(pxg + (uint32_t)((lv * 8 * MT + m) * 8), (uint32_t)__float_as_int((float)isum),
-                                       (uint32_t)__float_as_int(inv_scale));
-            }
-          }
-        }
-      }
+      };
+      using std::integral_constant;
+      if (my_pairs * 16 <= CTH) quantise(integral_constant<int, 1>(), integral_constant<int, 1>());
+      else if (my_pairs * 16 <= 2 * CTH) quantise(integral_constant<int, 2>(), integral_constant<int, 1>());
+      else quantise(integral_constant<int, 4>(), integral_constant<int, 2>());
       if (xc) {
         // both halves are in place once the sixteen consumer warps of each block have arrived at this block's
         // barrier (bounded wait; the other block cannot leave before it has seen this block's arrivals, and this

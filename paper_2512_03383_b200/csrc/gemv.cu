@@ -310,14 +310,15 @@ __global__ void __launch_bounds__(GTH, 1) gemv_kernel(const __grid_constant__ Gv
       for (int k = 0; k < UN; ++k) {
         const int u = u0 + k * GTH;
         if (u >= n_units) break;                        // warp-uniform (n_units and GTH are multiples of 32)
-        uint2 hi2, lo2;
+        const uint4 unit[1] = {in[k]};
+        uint2 hi2[1], lo2[1];
         int isum;
         float inv_scale;
-        quantise16<__half>(in[k], hi2, lo2, isum, inv_scale);
+        quantise_units<__half, 1>(unit, hi2, lo2, isum, inv_scale);
         const int u16 = u & 15;
-        const int off = lvv[k] * 128 + (u16 >> 2) * 32 + (u16 & 3) * 8;
-        *reinterpret_cast<uint2*>(xb + (size_t)(2 * mm[k]) * xrow + off) = hi2;
-        *reinterpret_cast<uint2*>(xb + (size_t)(2 * mm[k] + 1) * xrow + off) = lo2;
+        const int off = lvv[k] * 128 + u16 * 8;
+        *reinterpret_cast<uint2*>(xb + (size_t)(2 * mm[k]) * xrow + off) = hi2[0];
+        *reinterpret_cast<uint2*>(xb + (size_t)(2 * mm[k] + 1) * xrow + off) = lo2[0];
         if (u16 == 0) xg[lvv[k] * 4 + mm[k]] = make_float2((float)isum, inv_scale);
       }
     }
