@@ -179,16 +179,22 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
         int rc = lib_workspace(&cfg.workspace, &cfg.ws_bytes, cfg.stream);
         if (rc != UNIQL_OK) return rc;
       }
-      const size_t bytes = (((size_t)p.M * (size_t)q.ldx * 2) + 255) & ~(size_t)255;
       const size_t floor_bytes = decode_size ? decode_workspace_bytes(p.M, p.K, 1) : decode_workspace_header_bytes();
+      // (tensor cores: rows of whole 128-byte lines, as launch_planned() has them, where there is room)
+      const int lines = (q.ldx + 63) / 64 * 64;
+      if (!decode_size && cfg.ws_bytes >= (size_t)p.M * (size_t)lines * 2 + 255 + floor_bytes + 256) q.ldx = lines;
+      const size_t bytes = (((size_t)p.M * (size_t)q.ldx * 2) + 255) & ~(size_t)255;
       if (cfg.ws_bytes >= bytes + floor_bytes + 256) {
         // the copy lives at the end of the workspace; the kernels get what lies before it
         const size_t off = (cfg.ws_bytes - bytes) & ~(size_t)255;
         void* xr = reinterpret_cast<unsigned char*>(cfg.workspace) + off;
         const Fam& a = p.imap.fam[0];
-        int rc = launch_relay_x(p.x, p.ldx, p.M, a.count, a.keep, keep8, xr, cfg.stream);
+        // (bf16 above 16 rows goes to the tensor cores, whose operands are fp16: converted on the way)
+        const bool to_f16 = p.dt == UNIQL_BF16 && p.M > 16 && opt(kOptPrefillConvert) != 1;
+        int rc = launch_relay_x(p.x, p.ldx, p.M, a.count, a.keep, keep8, xr, q.ldx, to_f16, cfg.stream);
         if (rc != UNIQL_OK) return rc;
         q.x = xr;
+        q.x_f16 = to_f16 ? 1 : 0;
         p = q;
         relaid = true;
         cfg.ws_bytes = off;
@@ -203,7 +209,7 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
   // fp16: its instance that multiplies the codes themselves, by the rule of exact_batch().
   const bool batch = path == UNIQL_PATH_AUTO &&
                      (p.dt == UNIQL_BF16 ? p.M > 8 && p.M <= 16 && batch_supported(p) &&
-                                               (!cfg.workspace || cfg.ws_bytes >= batch_workspace_min(p.dt, p.M, p.k_in))
+                                               (!cfg.workspace || cfg.ws_bytes >= batch_workspace_min(true, p.M, p.k_in))
                                          : exact_batch(p));
   if (path == UNIQL_PATH_AUTO)
     path = batch ? UNIQL_PATH_PREFILL : gv ? UNIQL_PATH_GEMV : dec_ok ? UNIQL_PATH_DECODE : (pre_ok ? UNIQL_PATH_PREFILL : UNIQL_PATH_GENERIC);
@@ -510,7 +516,7 @@ namespace {
 // projection over the leading k_int channels of h.
 int mlp_tensor_core(const void* x, int ldx, int dt, const uint8_t* wg, const void* sg, const void* zg, const uint8_t* wu,
                     const void* su, const void* zu, const uint8_t* wd, const void* sd, const void* zd, int M, int hidden,
-                    int inter, int k_int, void* h, int ldh, void* y, int ldy, const LaunchCfg& cfg) {
+                    int inter, int k_int, void* h, int ldh, void* y, int ldy, const LaunchCfg& cfg_in) {
   if ((hidden % kGroup) != 0 || (inter % kGroup) != 0) return UNIQL_ERR_SHAPE;
   Params a;
   memset(&a, 0, sizeof(a));
@@ -526,6 +532,19 @@ int mlp_tensor_core(const void* x, int ldx, int dt, const uint8_t* wg, const voi
     jd.y = h; jd.ldy = ldh; jd.N = inter; jd.k_out = k_int;
     jd.pair = j + 1;
   }
+  // bf16: the gated launch leaves h as fp16 too, in rows of whole 128-byte lines at the end of the workspace, and the down
+  // projection reads that copy (a pass over h in between took 28 of 840 us at 2048 rows of Qwen2.5-7B).  Where there is room
+  // for it beside everything that the two launches may use.
+  const int ld16 = (k_int + 63) / 64 * 64, path = g_path.load();
+  const size_t h16_bytes = ((size_t)M * ld16 * 2 + 255) & ~(size_t)255;
+  const bool h16 = dt == UNIQL_BF16 && M > 16 && (path == UNIQL_PATH_AUTO || path == UNIQL_PATH_PREFILL) && opt(kOptPrefillConvert) != 1 &&
+                   cfg_in.ws_bytes >= h16_bytes + prefill_workspace_bytes(M, hidden) + 256;
+  LaunchCfg cfg = cfg_in;
+  if (h16) {
+    cfg.ws_bytes = (cfg_in.ws_bytes - h16_bytes) & ~(size_t)255;
+    a.job[0].y16 = reinterpret_cast<__half*>(reinterpret_cast<unsigned char*>(cfg_in.workspace) + cfg.ws_bytes);
+    a.job[0].ld16 = ld16;
+  }
   if (!prefill_supported(a) || (M <= 16 && dt == UNIQL_F16 && !exact_batch(a))) return UNIQL_ERR_UNSUPPORTED;   // (nothing launched)
   int rc = launch_prefill(a, cfg);
   if (rc != UNIQL_OK) return rc;
@@ -533,6 +552,7 @@ int mlp_tensor_core(const void* x, int ldx, int dt, const uint8_t* wg, const voi
   memset(&b, 0, sizeof(b));
   compile_map(nullptr, k_int, inter, &b.imap);
   b.x = h; b.ldx = ldh; b.dt = dt; b.M = M; b.K = inter; b.k_in = k_int;
+  if (h16) { b.x = a.job[0].y16; b.ldx = ld16; b.x_f16 = 1; }
   b.n_jobs = 1;
   JobDev& jd = b.job[0];
   compile_map(nullptr, hidden, hidden, &jd.omap);
@@ -545,7 +565,9 @@ int mlp_tensor_core(const void* x, int ldx, int dt, const uint8_t* wg, const voi
 
 extern "C" size_t uniql_mlp_workspace_bytes(int M, int hidden, int inter) {
   if (M < 1 || hidden < 1 || inter < 1) return 0;
-  if (M > 16) return prefill_workspace_bytes(M, hidden > inter ? hidden : inter);     // tensor-core kernel, two launches
+  // tensor-core kernel, two launches (+ the fp16 copies of both activations of bf16 at once)
+  if (M > 16)
+    return prefill_workspace_bytes(M, hidden > inter ? hidden : inter) + (size_t)M * (((hidden < inter ? hidden : inter) + 63) / 64 * 64) * 2 + 512;
   // (16 rows or fewer in bf16 also run on the tensor-core kernel: room for its fp16 copy of the activations)
   const size_t a = mlp_decode_workspace_bytes(M, hidden, inter), b = prefill_workspace_bytes(M, hidden > inter ? hidden : inter);
   size_t c = 0;

@@ -733,13 +733,13 @@ int batch_supported(const Params& p) {
 }
 
 // What a launch cannot do without (the header and the fp16 copy of bf16 activations), and with room for every split.
-size_t batch_workspace_min(int dt, int M, int k_in) {
+size_t batch_workspace_min(bool copy_x, int M, int k_in) {
   const size_t header = (decode_workspace_header_bytes() + 255) & ~(size_t)255;
-  return dt == UNIQL_BF16 ? header + (size_t)M * ((k_in + 63) / 64 * 64) * 2 + 256 : header;
+  return copy_x ? header + (size_t)M * ((k_in + 63) / 64 * 64) * 2 + 256 : header;
 }
 size_t batch_workspace_bytes(int M, int K) {
   const size_t n = (M + 15) / 16 * 16;
-  return batch_workspace_min(UNIQL_BF16, M, K) + (size_t)2 * device_sms() * 2 * n * BMW * 4;
+  return batch_workspace_min(true, M, K) + (size_t)2 * device_sms() * 2 * n * BMW * 4;
 }
 
 // Whether an fp16 launch of up to 16 rows goes to the EXACT instance instead of the decode kernel.  From twelve rows: the
@@ -796,7 +796,8 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   size_t used = (decode_workspace_header_bytes() + 255) & ~(size_t)255;
   const void* x = p.x;
   int ldx = p.ldx;
-  if (p.dt == UNIQL_BF16) {                     // (room for the copy was checked by the caller)
+  const bool copy_x = p.dt == UNIQL_BF16 && !p.x_f16;
+  if (copy_x) {                                 // (room for the copy was checked by the caller)
     ldx = (p.k_in + 63) / 64 * 64;
     x = reinterpret_cast<unsigned char*>(cfg.workspace) + used;
     used = (used + (size_t)p.M * ldx * 2 + 255) & ~(size_t)255;
@@ -823,7 +824,7 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   }
   c.p = best;
   c.partials = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(cfg.workspace) + used);
-  if (p.dt == UNIQL_BF16) {
+  if (copy_x) {
     rc = launch_x_to_f16(p.x, p.ldx, p.M, p.k_in, const_cast<void*>(x), ldx, cfg.stream);
     if (rc != UNIQL_OK) return rc;
   }

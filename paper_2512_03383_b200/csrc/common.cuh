@@ -48,12 +48,15 @@ struct JobDev {
                       // rows 2i, 2i+1 of a tile are retained row i of this matrix and of the NEXT job's (the up
                       // matrix), and the epilogue stores silu(g_i) * u_i at column i of this job's output.
                       // 2: that next job (it has no tiles of its own).
+  __half* y16;        // job 0, pair == 1, bf16: the stored outputs once more as fp16 (the operands of the launch behind), or null
+  int ld16;
 };
 
 struct Params {
   const void* x;
   int ldx;
   int dt;             // uniql_dtype
+  int x_f16;          // tensor-core kernels: the activations are fp16 whatever dt says (outputs and bias are dt)
   int M;
   int K;              // stored input channels
   int k_in;           // retained input channels
@@ -156,8 +159,9 @@ struct LaunchCfg {
                          // once the launch is certain (a workspace that may hold what an unfinished call left)
 };
 int launch_generic(const Params& p, const LaunchCfg& cfg);
-// out[m][h * keep8 + r] = r < keep ? x[m][h * keep + r] : 0  (2-byte elements; out 16-byte aligned, keep8 % 8 == 0)
-int launch_relay_x(const void* x, long long ldx, int M, int count, int keep, int keep8, void* out, cudaStream_t stream);
+// out[m][h * keep8 + r] = r < keep ? x[m][h * keep + r] : 0  (2-byte elements; out 16-byte aligned, keep8 and ldo multiples
+// of 8); to_f16: from bf16 to fp16 on the way
+int launch_relay_x(const void* x, long long ldx, int M, int count, int keep, int keep8, void* out, int ldo, bool to_f16, cudaStream_t stream);
 int launch_decode(const Params& p, const LaunchCfg& cfg);
 int decode_supported(const Params& p);
 int decode_integer_path(const Params& p);
@@ -191,7 +195,7 @@ int gemv_mlp_supported(const MlpDecode& d);
 // tensor-core kernel for up to 128 rows (csrc/batch.cu), taken by launch_prefill where its rules hold
 int launch_batch(const Params& p, const LaunchCfg& cfg);
 int batch_supported(const Params& p);
-size_t batch_workspace_min(int dt, int M, int k_in);
+size_t batch_workspace_min(bool copy_x, int M, int k_in);   // copy_x: bf16 activations, to be copied to fp16
 size_t batch_workspace_bytes(int M, int K);
 int exact_batch(const Params& p);             // twelve to sixteen fp16 rows on its exact-code instance
 // fp16 copy of bf16 activations [M][k_in], row pitch ldo (a multiple of 8; the columns from k_in on are zeros)
@@ -204,5 +208,17 @@ int device_sms();             // SMs of the current device
 int launch_prefill(const Params& p, const LaunchCfg& cfg);
 int prefill_supported(const Params& p);
 size_t prefill_workspace_bytes(int M, int K);
+
+
+// ---------------------------------------------------------------- bf16 -> fp16
+// Two bf16 values of a word as two fp16 values (exact for magnitudes in fp16's normal range, which
+// holds LLM activations; larger magnitudes saturate at +-65504 instead of becoming infinite).
+__device__ inline uint32_t bf16x2_to_f16x2(uint32_t w) {
+  uint32_t d;
+  asm("cvt.rn.satfinite.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(__uint_as_float(w & 0xffff0000u)), "f"(__uint_as_float(w << 16)));
+  return d;
+}
+__device__ inline __half f16_of(__nv_bfloat16 v) { return __ushort_as_half((unsigned short)bf16x2_to_f16x2(__bfloat16_as_ushort(v))); }
+__device__ inline __half f16_of(__half v) { return v; }
 
 }  // namespace uniql

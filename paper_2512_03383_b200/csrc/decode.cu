@@ -2173,7 +2173,7 @@ int launch_mlp_decode(const MlpDecode& d, int fuse, const LaunchCfg& cfg) {
   jd.w = d.wd; jd.scales = d.sd; jd.zeros = d.zd; jd.y = d.y; jd.ldy = d.ldy; jd.N = d.hidden; jd.k_out = d.hidden;
   jd.omap.n_fam = 1; jd.omap.total = d.hidden; jd.omap.fam[0] = Fam{0, d.hidden, d.hidden, 1}; jd.omap.base[0] = 0;
   // (bf16 at nine to sixteen rows: the batch kernel, as any plain launch of that kind)
-  if (!d.decode_only && p.dt == UNIQL_BF16 && p.M > 8 && batch_supported(p) && cfg.ws_bytes >= batch_workspace_min(p.dt, p.M, p.k_in)) return launch_prefill(p, cfg);
+  if (!d.decode_only && p.dt == UNIQL_BF16 && p.M > 8 && batch_supported(p) && cfg.ws_bytes >= batch_workspace_min(true, p.M, p.k_in)) return launch_prefill(p, cfg);
   return launch_decode(p, cfg);
 }
 

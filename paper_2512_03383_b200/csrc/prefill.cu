@@ -65,10 +65,9 @@ __global__ void x_to_f16_kernel(const __nv_bfloat16* __restrict__ x, int ldx, in
   //  waits for its own predecessor before it reads x or overwrites the copy that predecessor may still read)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int units = ldo / 8;                         // 16-byte units per output row (ldo is a multiple of 8)
-  const long total = (long)M * units;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const int m = (int)(i / units), u = (int)(i - (long)m * units);
+  const int u = blockIdx.x * blockDim.x + threadIdx.x;        // 16-byte unit of the output row (ldo is a multiple of 8)
+  if (u * 8 >= ldo) return;
+  for (int m = blockIdx.y; m < M; m += gridDim.y) {
     const __nv_bfloat16* src = x + (size_t)m * ldx + u * 8;
     uint32_t w[4];
     if (u * 8 + 8 <= k_in && ((ldx & 7) == 0) && ((((uintptr_t)x) & 15) == 0)) {
@@ -613,12 +612,11 @@ int device_sms() {
 }
 
 int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo, cudaStream_t stream) {
-  const long units = (long)M * (ldo / 8), most = (long)device_sms() * 8;
-  const long blocks = (units + 255) / 256;
+  const unsigned cols = (unsigned)(ldo / 8 + 127) / 128, rows = (unsigned)device_sms() * 32 / cols + 1;
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
-  lc.gridDim = dim3((unsigned)(blocks < most ? blocks : most));
-  lc.blockDim = dim3(256);
+  lc.gridDim = dim3(cols, (unsigned)M < rows ? (unsigned)M : rows);
+  lc.blockDim = dim3(128);
   lc.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -700,7 +698,7 @@ int launch_planned(const Params& p, const LaunchCfg& cfg, bool clusters) {
   bool conv_in_kernel = false;
   __half* x16 = nullptr;              // fp16 copy to be written by the pre-pass
   int x16_ld = 0;
-  if (p.dt == UNIQL_BF16) {
+  if (p.dt == UNIQL_BF16 && !p.x_f16) {
     // (a row pitch of whole 128-byte lines: a box row that straddles two lines costs a second L2 request, measured
     //  as 1.09 instead of 0.85 us per k-block on the Qwen2.5-7B down projection at 12312 of 18944 input channels)
     int ldo = (p.k_in + 63) / 64 * 64;
@@ -921,7 +919,8 @@ int launch_planned(const Params& p, const LaunchCfg& cfg, bool clusters) {
 int launch_prefill(const Params& p, const LaunchCfg& cfg) {
   if (!cfg.workspace || cfg.ws_bytes < decode_workspace_header_bytes()) return UNIQL_ERR_WORKSPACE;   // status word
   // up to 128 rows: the batch kernel (bf16: where the workspace has room for the fp16 copy)
-  if (batch_supported(p) && (p.dt != UNIQL_BF16 || (opt(kOptPrefillConvert) != 1 && cfg.ws_bytes >= batch_workspace_min(p.dt, p.M, p.k_in))))
+  if (batch_supported(p) &&
+      (p.dt != UNIQL_BF16 || p.x_f16 || (opt(kOptPrefillConvert) != 1 && cfg.ws_bytes >= batch_workspace_min(true, p.M, p.k_in))))
     return launch_batch(p, cfg);
   return launch_planned(p, cfg, true);
 }

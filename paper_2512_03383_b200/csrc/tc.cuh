@@ -3,6 +3,8 @@
 #pragma once
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace uniql {
@@ -270,14 +272,6 @@ __device__ inline RowInfo tile_row(const JobDev& jb, int tl, int r) {
   return o;
 }
 
-// Two bf16 values of a word as two fp16 values (exact for magnitudes in fp16's normal range, which
-// holds LLM activations; larger magnitudes saturate at +-65504 instead of becoming infinite).
-__device__ inline uint32_t bf16x2_to_f16x2(uint32_t w) {
-  uint32_t d;
-  asm("cvt.rn.satfinite.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(__uint_as_float(w & 0xffff0000u)), "f"(__uint_as_float(w << 16)));
-  return d;
-}
-
 // Eight codes of one 32-bit word, in input-channel order, as eight fp16 values packed in a uint4:
 // byte b -> (1024 + c_even, 64 + c_odd) as an fp16 pair (one PRMT, one LOP3), minus (1032, 72) = the
 // exact (c-8) pair, then one fp16 FMA per pair: (c-8)*s + cz with cz = fp16(s*(8-z)).  s is the stored
@@ -397,6 +391,16 @@ struct RowStore {
           for (int k = 0; k < H; ++k) {
             if (k < n) *yp = r[k];
             yp += step;
+          }
+          if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+            if (p.job[0].y16 != nullptr) {
+              __half* hp = p.job[0].y16 + (live ? ri.out_col : 0) + (size_t)(m0 + b + odd) * p.job[0].ld16;
+#pragma unroll
+              for (int k = 0; k < H; ++k) {
+                if (k < n) *hp = f16_of(r[k]);
+                hp += 2 * (size_t)p.job[0].ld16;
+              }
+            }
           }
         }
       }

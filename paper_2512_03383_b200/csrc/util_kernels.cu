@@ -77,31 +77,36 @@ __global__ void embed_kernel(const uint8_t* __restrict__ packed, const __half* _
 
 // Activations re-laid with every kept block padded to a multiple of 8 channels (zeros in the padding): the fast
 // kernels read activations in 16-byte units, which blocks of 108 or 84 channels (multiples of 4) do not give.
-// One thread per 4 output channels (8 bytes); x needs 2-byte alignment only.
-__global__ void relay_x_kernel(const unsigned short* __restrict__ x, long long ldx, int M, int count, int keep, int keep8,
-                               unsigned short* __restrict__ out) {
+// One thread per 8 output channels (16 bytes) of one or more rows; x needs 2-byte alignment only.  F16: bf16 activations on
+// their way to the tensor cores become fp16 here instead of in a pass of their own.
+template <bool F16>
+__global__ void __launch_bounds__(128) relay_x_kernel(const unsigned short* __restrict__ x, long long ldx, int M, int count, int keep,
+                                                      int keep8, unsigned short* __restrict__ out, int ldo) {
   // (programmatic dependent launch: the kernel behind this one may set itself up meanwhile; this one waits for its
   //  own predecessor before it reads x or overwrites the copy that predecessor may still read)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int units_row = count * (keep8 >> 2);
-  const long long total = (long long)M * units_row;
+  const int u = blockIdx.x * blockDim.x + threadIdx.x, per = keep8 >> 3;
+  if (u >= count * per) return;
+  const int h = u / per, r = (u - h * per) * 8;
   const bool vec = ((ldx & 3) == 0) && ((((uintptr_t)x) & 7) == 0) && ((keep & 3) == 0);
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int m = (int)(i / units_row), u = (int)(i - (long long)m * units_row);
-    const int h = u / (keep8 >> 2), r = (u - h * (keep8 >> 2)) * 4;
+  const int left = keep - r;                         // kept channels of this unit: eight, or the last few of the block
+  for (int m = blockIdx.y; m < M; m += gridDim.y) {
     const unsigned short* src = x + (size_t)m * ldx + (size_t)h * keep + r;
-    uint2 v = make_uint2(0u, 0u);
-    if (vec && r + 4 <= keep) {
-      v = *reinterpret_cast<const uint2*>(src);
+    uint2 v[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
+    if (vec) {
+      if (left >= 4) v[0] = *reinterpret_cast<const uint2*>(src);
+      if (left >= 8) v[1] = *reinterpret_cast<const uint2*>(src + 4);
     } else {
-      unsigned short e[4];
+      unsigned short e[8];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) e[k] = r + k < keep ? src[k] : (unsigned short)0;
-      v.x = (uint32_t)e[0] | ((uint32_t)e[1] << 16);
-      v.y = (uint32_t)e[2] | ((uint32_t)e[3] << 16);
+      for (int k = 0; k < 8; ++k) e[k] = k < left ? src[k] : (unsigned short)0;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) v[k] = make_uint2((uint32_t)e[4 * k] | ((uint32_t)e[4 * k + 1] << 16), (uint32_t)e[4 * k + 2] | ((uint32_t)e[4 * k + 3] << 16));
     }
-    *reinterpret_cast<uint2*>(out + (size_t)m * ((size_t)count * keep8) + (size_t)h * keep8 + r) = v;
+    uint4 o = make_uint4(v[0].x, v[0].y, v[1].x, v[1].y);
+    if (F16) o = make_uint4(bf16x2_to_f16x2(o.x), bf16x2_to_f16x2(o.y), bf16x2_to_f16x2(o.z), bf16x2_to_f16x2(o.w));
+    *reinterpret_cast<uint4*>(out + (size_t)m * ldo + (size_t)h * keep8 + r) = o;
   }
 }
 
@@ -121,20 +126,21 @@ inline int grid_for(int64_t n, int threads) {
 }  // namespace
 }  // namespace uniql
 
-int uniql::launch_relay_x(const void* x, long long ldx, int M, int count, int keep, int keep8, void* out, cudaStream_t stream) {
-  const int64_t units = (int64_t)M * count * (keep8 / 4);
+int uniql::launch_relay_x(const void* x, long long ldx, int M, int count, int keep, int keep8, void* out, int ldo, bool to_f16,
+                          cudaStream_t stream) {
+  const unsigned cols = (unsigned)(count * (keep8 / 8) + 127) / 128, rows = (unsigned)device_sms() * 32 / cols + 1;
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
-  lc.gridDim = dim3((unsigned)grid_for(units, 256));
-  lc.blockDim = dim3(256);
+  lc.gridDim = dim3(cols, (unsigned)M < rows ? (unsigned)M : rows);
+  lc.blockDim = dim3(128);
   lc.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = attr;
   lc.numAttrs = opt(kOptPdl) ? 1 : 0;
-  if (cudaLaunchKernelEx(&lc, relay_x_kernel, reinterpret_cast<const unsigned short*>(x), ldx, M, count, keep, keep8,
-                         reinterpret_cast<unsigned short*>(out)) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&lc, to_f16 ? relay_x_kernel<true> : relay_x_kernel<false>, reinterpret_cast<const unsigned short*>(x), ldx, M, count,
+                         keep, keep8, reinterpret_cast<unsigned short*>(out), ldo) != cudaSuccess) {
     cudaGetLastError();
     return UNIQL_ERR_CUDA;
   }
