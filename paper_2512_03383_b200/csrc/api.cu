@@ -155,7 +155,9 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
   // every batch the decode kernel does not take (more than 16 rows) goes to the tensor cores when the maps
   // allow it: at 17..63 rows the generic kernel measured 13 to 26 times slower (930 us against 71 us for the
   // Llama-3-8B gate|up at M = 17)
-  bool pre_ok = prefill_supported(p);
+  // (fp16 up to 128 rows: the batch kernel also takes heads that keep 4 (mod 8) channels)
+  auto on_tensor_cores = [](const Params& a) { return prefill_supported(a) != 0 || (a.dt == UNIQL_F16 && batch_supported(a) != 0); };
+  bool pre_ok = on_tensor_cores(p);
   // The streaming kernel (one to four rows): where it is asked for, and where the decode kernel's integer path cannot run
   // (scales on 8- but not 16-byte boundaries).
   bool gv = path == UNIQL_PATH_GEMV || (path == UNIQL_PATH_AUTO && gemv_supported(p) && opt(kOptGemvFirst) == 1);
@@ -199,7 +201,7 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
         relaid = true;
         cfg.ws_bytes = off;
         dec_ok = decodes(p);
-        pre_ok = prefill_supported(p);
+        pre_ok = on_tensor_cores(p);
       }
     }
   }
@@ -252,7 +254,7 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
     return launch_decode(p, cfg);
   }
   if (path == UNIQL_PATH_PREFILL) {
-    if (!prefill_supported(p)) return UNIQL_ERR_UNSUPPORTED;
+    if (!on_tensor_cores(p)) return UNIQL_ERR_UNSUPPORTED;
     if (!cfg.workspace) {      // only the status word of the workspace is used
       int rc = lib_workspace(&cfg.workspace, &cfg.ws_bytes, cfg.stream);
       if (rc != UNIQL_OK) return rc;

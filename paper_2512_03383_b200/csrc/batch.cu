@@ -92,6 +92,7 @@ struct BatchCfg {
   int n_tiles, n_kb, spt;    // weight tiles of 128 rows, k-blocks, stages per tile
   int kb_first;              // first stored k-block
   int head_kb, head_keep;    // per-head maps: k-blocks and kept channels per head (0: leading block)
+  int head_4;                // 4: kept blocks are no multiple of 8 channels (but of 4)
   uint32_t idesc;
   int p;                     // blocks per tile (cluster size)
   int* status;
@@ -189,9 +190,25 @@ struct BSegIter {
   }
 };
 
+// Heads that keep 4 (mod 8) channels.  A box of activations starts on a 16-byte boundary, and every second head's first column
+// lies 4 channels behind one: its boxes begin those 4 columns early, and the de-quantisers move the codes of the head up by as
+// many, with zero weights under what the boxes hold of the neighbours.  A copy of the activations re-laid by a kernel in front
+// took 2.8 us of the 69 us of a Llama-3-8B layer at 64 rows (head dim 108).  Channels of k-block r of head h in its box:
+// [lead, end).
+struct HeadSpan { int shift, lead, end; };
+__device__ inline HeadSpan head_span(const BatchCfg& c, int v) {
+  const int h = v / c.head_kb, r = v - h * c.head_kb;
+  HeadSpan s;
+  s.shift = (h & 1) ? c.head_4 : 0;
+  s.lead = r == 0 ? s.shift : 0;
+  s.end = min(BK, c.head_keep + s.shift - r * BK);
+  return s;
+}
+
 // Tensor memory of the EXACT instance: [0, 32) the tile's sums of the two halves, then per half P and X of a group, then
-// the operand of ones (eight columns; four columns of zeros behind it, so that four columns on it covers 8 channels).
-constexpr uint32_t kExP = 32, kExOnes = 96, kExA = 112;
+// the operand of ones (eight columns, eight of zeros behind it: n columns on it covers 16 - 2 n channels), and behind the A
+// operands the one that leaves out the first 4 of 16 channels.
+constexpr uint32_t kExP = 32, kExOnes = 96, kExA = 112, kExLate = 240;
 
 template <typename T, bool HEADS, bool EXACT>
 __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ Params p, const __grid_constant__ BatchCfg c) {
@@ -348,7 +365,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
           pmbar_expect_tx(fb, (uint32_t)nv * box);
           for (int i = 0; i < nv; ++i) {
             const int v = v0 + i;
-            const int x = HEADS ? (v / c.head_kb) * c.head_keep + (v % c.head_kb) * BK : v * BK;
+              const int x = HEADS ? (((v / c.head_kb) * c.head_keep) & ~7) + (v % c.head_kb) * BK : v * BK;
             tma_box2(sbase + (uint32_t)(s * (KS / 2) + i) * box, &c.xmap, x, 0, fb);
           }
         }
@@ -381,13 +398,15 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
             if (i >= nv) break;
             if (EXACT) {                                       // (slot = half = accumulator)
               const uint32_t d = tmem + kExP + 32u * (uint32_t)as;
-              const int kept = HEADS ? c.head_keep - ((v0 + i) % c.head_kb) * BK : BK;
+              HeadSpan hs = {0, 0, BK};
+              if (HEADS) hs = head_span(c, v0 + i);
 #pragma unroll
               for (int k = 0; k < BK / 16; ++k) {
                 const uint32_t more = (i > 0 || k > 0) ? 1u : 0u;
                 umma_ts(d, a0 + 32 * i + 8 * k, bd + i * box_step + 2 * k, c.idesc, more);
-                if (!HEADS || 16 * k < kept)                   // (kept channels are a multiple of 8)
-                  umma_ts(d + 16, tmem + kExOnes + (HEADS && 16 * k + 8 == kept ? 4u : 0u), bd + i * box_step + 2 * k, c.idesc, more);
+                if (!HEADS || 16 * k < hs.end)                 // (a head keeps at least 12 channels where one has a lead)
+                  umma_ts(d + 16, tmem + (!HEADS ? kExOnes : k == 0 && hs.lead ? kExLate : kExOnes + (uint32_t)max(0, 16 * (k + 1) - hs.end) / 2),
+                          bd + i * box_step + 2 * k, c.idesc, more);
               }
               continue;
             }
@@ -499,6 +518,9 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
 #pragma unroll
       for (int k = 0; k < 2; ++k)
         asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(t + 8 * k), "r"(k ? 0u : 0x3c003c00u) : "memory");
+      if (HEADS)
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %2, %2, %2, %2, %2, %2};"
+                     ::"r"(a_lane - (uint32_t)c.a_base + kExLate), "r"(0u), "r"(0x3c003c00u) : "memory");
       tmem_st_wait();
       tc_fence_before();
     }
@@ -543,18 +565,18 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
         const __half2 s2 = __half2half2(sc);
         const __half2 cz2 = __float2half2_rn((8.f - __half2float(zp)) * __half2float(sc));
         uint32_t o[32];
-        int valid = 2 * BK;                      // kept channels of the half stage's k-blocks, one bit field each
-        if (HEADS) {
-          const int v = st * KS + 2 * half;
-          valid = min(BK, c.head_keep - (v % c.head_kb) * BK) | (min(BK, c.head_keep - ((v + 1) % c.head_kb) * BK) << 8);
-        }
+        HeadSpan hs[2] = {{0, 0, BK}, {0, 0, BK}};                 // of the half stage's k-blocks
+        if (HEADS) { hs[0] = head_span(c, st * KS + 2 * half); hs[1] = head_span(c, st * KS + 2 * half + 1); }
         auto convert = [&](int j0) {             // words j0 .. j0 + 3 of the sixteen
 #pragma unroll
           for (int i = j0; i < j0 + 4; ++i) {
-            const int k = i & 7;
-            const bool kept = !HEADS || k * 8 < (i < 8 ? (valid & 255) : (valid >> 8));
-            const uint4 d = !kept ? make_uint4(0, 0, 0, 0) : EXACT ? codes_word(w[i]) : dequant_word(w[i], s2, cz2);
-            o[4 * k] = d.x; o[4 * k + 1] = d.y; o[4 * k + 2] = d.z; o[4 * k + 3] = d.w;
+            const int k = i & 7, b = i >> 3;
+            uint32_t wi = w[i];
+            if (HEADS)                           // (k-block b is a head's first unless heads have two and b is 1)
+              wi = __funnelshift_l(k > 0 || (b == 1 && hs[1].lead != hs[1].shift) ? w[i > 0 ? i - 1 : 0] : 0u, w[i], 4 * hs[b].shift);
+            const uint4 d = HEADS && k * 8 >= hs[b].end ? make_uint4(0, 0, 0, 0) : EXACT ? codes_word(wi) : dequant_word(wi, s2, cz2);
+            const bool no_lo = HEADS && k == 0 && hs[b].lead != 0, no_hi = HEADS && k * 8 + 4 == hs[b].end;
+            o[4 * k] = no_lo ? 0u : d.x; o[4 * k + 1] = no_lo ? 0u : d.y; o[4 * k + 2] = no_hi ? 0u : d.z; o[4 * k + 3] = no_hi ? 0u : d.w;
           }
         };
         convert(0);
@@ -723,8 +745,10 @@ int batch_supported(const Params& p) {
   const Fam& a = p.imap.fam[0];
   if (a.count == 1) {
     if (a.start != 0) return 0;
-  } else if (a.start % (KS * BK) != 0 || a.period % BK != 0 || a.keep % 8 != 0 || a.keep <= a.period - BK) {
+  } else if (a.start % (KS * BK) != 0 || a.period % BK != 0 || a.keep % 4 != 0 || a.keep <= a.period - BK) {
     return 0;
+  } else if (a.keep % 8 != 0 && (p.dt != UNIQL_F16 || a.period > 2 * BK || a.keep < 12)) {
+    return 0;                            // (heads of one or two k-blocks, read in place: bf16 activations are copied anyway)
   }
   if ((p.ldx % 8) != 0 || (((uintptr_t)p.x) & 15) != 0) return 0;
   for (int j = 0; j < p.n_jobs; ++j)
@@ -747,20 +771,12 @@ size_t batch_workspace_bytes(int M, int K) {
 // Measured at 12 / 16 rows, decode kernel -> here, the whole layer in microseconds: Qwen2.5-7B 84.2 -> 71.7 / 90.6 -> 71.4,
 // Mamba2-2.7B 29.0 -> 22.5 / 31.4 -> 22.5, Llama-3-8B 76.0 -> 71.6 / 79.6 -> 71.7, at keep 0.75 71.9 -> 63.6 / 74.9 -> 63.5, at keep
 // 0.65 68.6 -> 66.6 / 72.9 -> 67.2; over five keep rates from 0.55 the decode kernel is nowhere ahead by more than 1 %.
-// Not where kept blocks of output rows are no multiple of 8: the launch that reads those channels then stays on the decode
-// kernel (4-channel boundaries), whose blocks need a whole SM and cannot come in beside this kernel's (Mamba2 mixer at keep
-// 0.8 29.5 -> 30.7 us).  Rotated heads excepted: there the other four launches of a layer outweigh that.
 int exact_batch(const Params& p) {
-  if (p.dt != UNIQL_F16 || p.M < 12 || p.M > 16 || !batch_supported(p) || !prefill_supported(p)) return 0;
+  if (p.dt != UNIQL_F16 || p.M < 12 || p.M > 16 || !batch_supported(p)) return 0;
   // (an option of the decode kernel that is set asks for that kernel)
   if (opt(kOptDecodeKp) != 0 || opt(kOptDecodeRp) != 0 || opt(kOptDecodeStages) != 0 || opt(kOptDecodeNarrow) != -1 || opt(kOptDecodeXstream) != -1 ||
       opt(kOptDecodeXcluster) != -1 || opt(kOptDecodeI8) != 1 || opt(kOptDecodeSplitBatch) != 2)
     return 0;
-  for (int j = 0; j < p.n_jobs; ++j) {
-    if (p.n_jobs > 1 && p.job[0].rope.enabled) break;
-    for (int k = 0; k < p.job[j].omap.n_fam; ++k)
-      if (p.job[j].omap.fam[k].count > 1 && p.job[j].omap.fam[k].keep % 8 != 0) return 0;
-  }
   return 1;
 }
 
@@ -780,6 +796,7 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   c.kb_first = a.start / BK;
   c.head_kb = a.count > 1 ? kbh : 0;
   c.head_keep = a.keep;
+  c.head_4 = a.count > 1 ? a.keep & 4 : 0;
   // fp32 accumulate, A and B fp16, both K-major, N tokens, 128 rows
   c.idesc = (1u << 4) | ((uint32_t)(c.n >> 3) << 17) | ((uint32_t)(BMW >> 4) << 24);
   c.exact = p.M <= 16 && p.dt != UNIQL_BF16;
