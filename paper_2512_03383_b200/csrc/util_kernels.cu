@@ -48,6 +48,10 @@ template <typename T>
 __global__ void embed_kernel(const uint8_t* __restrict__ packed, const __half* __restrict__ scales,
                              const __half* __restrict__ zeros, int64_t V, int64_t K, const int32_t* __restrict__ ids,
                              T* __restrict__ out, int64_t ldo, int* __restrict__ bad) {
+  // (programmatic dependent launch, as the kernels of the layers: this one's blocks come in as the preceding launch's leave,
+  //  and the next launch sets itself up and fetches its first weights meanwhile; ids and out are touched behind the wait)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t m = blockIdx.y;
   int64_t row = ids[m];
   const bool in_range = row >= 0 && row < V;
@@ -198,12 +202,20 @@ extern "C" int uniql_embed_rows(const uint8_t* packed, const void* scales, const
   const int threads = 128;
   int bx = (int)((K / 8 + threads - 1) / threads);
   if (bx > 64) bx = 64;
-  dim3 grid(bx, (unsigned)M);
-  if (dt == UNIQL_F16)
-    embed_kernel<__half><<<grid, threads, 0, (cudaStream_t)stream>>>(packed, (const __half*)scales, (const __half*)zeros,
-                                                                      V, K, ids, (__half*)out, ldo, bad_id);
-  else
-    embed_kernel<__nv_bfloat16><<<grid, threads, 0, (cudaStream_t)stream>>>(
-        packed, (const __half*)scales, (const __half*)zeros, V, K, ids, (__nv_bfloat16*)out, ldo, bad_id);
-  return cudaGetLastError() == cudaSuccess ? UNIQL_OK : UNIQL_ERR_CUDA;
+  cudaLaunchConfig_t lc;
+  cudaLaunchAttribute attr[1];
+  memset(&lc, 0, sizeof(lc));
+  lc.gridDim = dim3(bx, (unsigned)M);
+  lc.blockDim = dim3(threads);
+  lc.stream = (cudaStream_t)stream;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = attr;
+  lc.numAttrs = opt(kOptPdl) ? 1 : 0;
+  const cudaError_t e =
+      dt == UNIQL_F16 ? cudaLaunchKernelEx(&lc, embed_kernel<__half>, packed, (const __half*)scales, (const __half*)zeros, V, K, ids, (__half*)out, ldo, bad_id)
+                      : cudaLaunchKernelEx(&lc, embed_kernel<__nv_bfloat16>, packed, (const __half*)scales, (const __half*)zeros, V, K, ids,
+                                           (__nv_bfloat16*)out, ldo, bad_id);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess ? UNIQL_OK : UNIQL_ERR_CUDA;
 }
