@@ -28,10 +28,10 @@
 //
 // EXACT instance (fp16, up to 16 rows).  The decode kernel, which takes these sizes otherwise, multiplies the codes
 // themselves; rounding code x scale to fp16 would lose precision against it.  So here A holds codes - 8 (exact in fp16), a
-// half stage is one group of 128 channels with an accumulator of its own (P = sum (q - 8) x of 16 tokens), warp 3 adds up the
-// activations of the group (X = sum x) from the boxes in shared memory, and the de-quantiser thread that made the operand
-// adds s P + s (8 - z) X to fp32 registers: activations and codes enter unrounded, all sums are fp32.  Two FMAs per token
-// and group replace one per pair of codes.
+// half stage is one group of 128 channels with accumulators of its own (P = sum (q - 8) x of 16 tokens and, from an operand
+// of ones, X = sum x in every lane), and the de-quantiser thread that made the operand adds s P + s (8 - z) X to fp32
+// registers: activations and codes enter unrounded, all sums are fp32.  The group's accumulators are read where the
+// thread waits for its A slot anyway.  Two FMAs per token and group replace one per pair of codes.
 //
 // Work split: clusters of p blocks share a tile, every block a p-th of its stages; the cluster takes tiles round-robin.
 // Each block then owns every p-th chunk of 16 tokens: it leaves its fp32 sums of the other chunks in a slot of its own
@@ -99,19 +99,10 @@ struct BatchCfg {
   float* partials;           // two slots [n tokens][128 rows] fp32 per block (p > 1)
 };
 
-// D[tmem] (+)= A[tmem] * B[smem desc] over a k-block of 64: four MMAs, 8 columns of A and 32 bytes of B (+2 in the descriptor's
-// address field) each; accumulate == 0: the first one overwrites D.  One block of code, as umma_kblock(): the issuing warp's
-// loop is a chain of dependent instructions that shares its scheduler with four de-quantisers, and a half stage of eight
-// MMAs written one by one took it a thousand cycles where they run in 340 (64 tokens).
-__device__ inline void umma_ts_kblock(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+__device__ inline void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p, t;\n\t.reg .b32 a1, a2, a3;\n\t.reg .b64 b1, b2, b3;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
-      "add.u32 a1, %1, 8;\n\tadd.s64 b1, %2, 2;\n\tadd.u32 a2, %1, 16;\n\tadd.s64 b2, %2, 4;\n\tadd.u32 a3, %1, 24;\n\tadd.s64 b3, %2, 6;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a2], b2, %3, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a3], b3, %3, t;\n\t}"
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
       ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
 // 32 columns of this thread's lane
@@ -214,12 +205,9 @@ __device__ inline HeadSpan head_span(const BatchCfg& c, int v) {
   return s;
 }
 
-// Tensor memory of the EXACT instance: [0, 32) the tile's sums of the two halves, then P of a group per half, the A operands.
-// (X from an operand of ones took as many MMAs as P, and the columns of a third A operand.)
-constexpr uint32_t kExP = 32;
-constexpr int kBarBytes = 1536;                  // barriers and flags, then X of the last groups
-constexpr int kXsOff = 512;                      // their place behind the barriers
-constexpr int kExRing = 16;                      // groups whose X is kept: the boxes run up to four ahead, every second may be empty
+// Tensor memory of the EXACT instance: [0, 32) the tile's sums of the two halves, then per half P and X of a group, then
+// the operand of ones (eight columns; four columns of zeros behind it, so that four columns on it covers 8 channels).
+constexpr uint32_t kExP = 32, kExOnes = 96, kExA = 112;
 
 template <typename T, bool HEADS, bool EXACT>
 __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ Params p, const __grid_constant__ BatchCfg c) {
@@ -233,16 +221,13 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
   const uint32_t a_full = b_empty + 8 * MAX_BST, a_empty = a_full + 8 * MAX_AST;
   const uint32_t acc_full = a_empty + 8 * MAX_AST, acc_empty = acc_full + 8;
   const uint32_t xbar = acc_empty + 8;             // exchange between the blocks of a cluster: two per quadrant
-  const uint32_t xs_full = xbar + 64;              // EXACT: X of a group is in shared memory
-  unsigned char* misc = smem + c.off_bar + 8 * (2 * MAX_WST + 2 * MAX_BST + 2 * MAX_AST + 2 + 8 + kExRing);
+  unsigned char* misc = smem + c.off_bar + 8 * (2 * MAX_WST + 2 * MAX_BST + 2 * MAX_AST + 2 + 8);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
-  const uint32_t xs_sum = bars + kXsOff;           // EXACT: [group % 16][16 tokens] fp32
 
   if (tid == 0) {
-    for (int s = 0; s < MAX_WST; ++s) { pmbar_init(w_full + 8 * s, (EXACT ? 1 : LOADERS) * 32 + 1); pmbar_init(w_empty + 8 * s, DQN); }
-    for (int s = 0; s < MAX_BST; ++s) { pmbar_init(b_full + 8 * s, 1); pmbar_init(b_empty + 8 * s, EXACT ? 2 : 1); }
-    for (int s = 0; s < kExRing; ++s) pmbar_init(xs_full + 8 * s, 1);
+    for (int s = 0; s < MAX_WST; ++s) { pmbar_init(w_full + 8 * s, LOADERS * 32 + 1); pmbar_init(w_empty + 8 * s, DQN); }
+    for (int s = 0; s < MAX_BST; ++s) { pmbar_init(b_full + 8 * s, 1); pmbar_init(b_empty + 8 * s, 1); }
     for (int s = 0; s < MAX_AST; ++s) { pmbar_init(a_full + 8 * s, DQN / 2); pmbar_init(a_empty + 8 * s, 1); }
     pmbar_init(acc_full, EXACT ? DQN : 1);
     pmbar_init(acc_empty, DQN);
@@ -379,7 +364,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
           pmbar_expect_tx(fb, (uint32_t)nv * box);
           for (int i = 0; i < nv; ++i) {
             const int v = v0 + i;
-              const int x = HEADS ? (((v / c.head_kb) * c.head_keep) & ~7) + (v % c.head_kb) * BK : v * BK;
+            const int x = HEADS ? (((v / c.head_kb) * c.head_keep) & ~7) + (v % c.head_kb) * BK : v * BK;
             tma_box2(sbase + (uint32_t)(s * (KS / 2) + i) * box, &c.xmap, x, 0, fb);
           }
         }
@@ -395,11 +380,8 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
     // ===================================================================== MMA issue
     int as = 0, bs = 0, count = 0; uint32_t apar = 0, bpar = 0;
     const uint64_t box_step = (uint64_t)(c.n * 8);             // a box of n * 128 bytes, in the descriptor's 16-byte units
-    const uint64_t b_desc0 = smem_desc_sw128(sbase);           // (the activation ring is first)
-    const uint32_t slot_step = (uint32_t)(c.n * 8 * (KS / 2));
     for (; !failed && si.next(sg); ++count) {
       if (!EXACT && count >= 1 && !pmbar_wait_warp(acc_empty, (count - 1) & 1, abort_flag)) { failed = true; break; }
-      uint32_t more = 0, hh = 0;                               // not the tile's first half stage; EXACT: the half
       for (int v0 = sg.s0 * KS; v0 < sg.s1 * KS; v0 += KS / 2) {
         const int nv = c.n_kb - v0;                            // k-blocks of this half stage (none behind the last: only handed back)
         if ((nv > 0 && !pmbar_wait_warp(b_full + 8 * bs, bpar, abort_flag)) || !pmbar_wait_warp(a_full + 8 * as, apar, abort_flag)) {
@@ -407,18 +389,32 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
           break;
         }
         tc_fence_after();
+        const uint32_t a0 = tmem + (uint32_t)(c.a_base + 64 * as);
+        const uint64_t bd = smem_desc_sw128(sbase + (uint32_t)(bs * (KS / 2) * c.n) * 128u);
         if (elect_one()) {
-          const uint32_t d = EXACT ? tmem + kExP + 16u * hh : tmem;
-          const uint32_t a0 = tmem + (uint32_t)(c.a_base + 64 * as);
-          const uint64_t bd = b_desc0 + (uint64_t)((uint32_t)bs * slot_step);
-          if (nv > 0) umma_ts_kblock(d, a0, bd, c.idesc, more);
-          if (nv > 1) umma_ts_kblock(d, a0 + 32, bd + box_step, c.idesc, 1u);
+#pragma unroll
+          for (int i = 0; i < KS / 2; ++i) {
+            if (i >= nv) break;
+            if (EXACT) {                                       // (slot = half = accumulator)
+              const uint32_t d = tmem + kExP + 32u * (uint32_t)as;
+              const int kept = HEADS ? c.head_keep - ((v0 + i) % c.head_kb) * BK : BK;
+#pragma unroll
+              for (int k = 0; k < BK / 16; ++k) {
+                const uint32_t more = (i > 0 || k > 0) ? 1u : 0u;
+                umma_ts(d, a0 + 32 * i + 8 * k, bd + i * box_step + 2 * k, c.idesc, more);
+                if (!HEADS || 16 * k < kept)                   // (kept channels are a multiple of 8)
+                  umma_ts(d + 16, tmem + kExOnes + (HEADS && 16 * k + 8 == kept ? 4u : 0u), bd + i * box_step + 2 * k, c.idesc, more);
+              }
+              continue;
+            }
+#pragma unroll
+            for (int k = 0; k < BK / 16; ++k)
+              umma_ts(tmem, a0 + 32 * i + 8 * k, bd + i * box_step + 2 * k, c.idesc, (v0 > sg.s0 * KS || i > 0 || k > 0) ? 1u : 0u);
+          }
           umma_commit(a_empty + 8 * as);
           if (nv > 0) umma_commit(b_empty + 8 * bs);
         }
         __syncwarp();
-        more = EXACT ? 0u : 1u;
-        hh ^= 1u;
         if (++as == c.n_ast) { as = 0; apar ^= 1; }
         if (nv > 0 && ++bs == c.bst) { bs = 0; bpar ^= 1; }
       }
@@ -426,66 +422,22 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
       if (!EXACT && elect_one()) umma_commit(acc_full);
       __syncwarp();
     }
-  } else if (EXACT && warp == LD_WARP0 + 1) {
-    // ===================================================================== EXACT: sums of the activations, group by group
-    // Lane 2 t + u adds up channels 32 u .. + 31 of token t in each of the half stage's two boxes (16-byte pieces, swizzled).
-    const int t = lane >> 1, u = lane & 1;
-    const uint32_t box = (uint32_t)c.n * 128u;
-    int s = 0; uint32_t par = 0, it = 0;
-    while (!failed && si.next(sg)) {
-      for (int v0 = sg.s0 * KS; v0 < sg.s1 * KS; v0 += KS / 2, ++it) {
-        const int nv = c.n_kb - v0;
-        if (nv > 0) {
-          if (!pmbar_wait_warp(b_full + 8 * s, par, abort_flag)) { failed = true; break; }
-          float sum = 0.f;
-          for (int i = 0; i < min(nv, KS / 2); ++i) {
-            HeadSpan hs = {0, 0, BK};
-            if (HEADS) hs = head_span(c, v0 + i);
-            const uint32_t row = sbase + (uint32_t)(s * (KS / 2) + i) * box + (uint32_t)(t * 128);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              uint32_t w[4];
-              asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
-                           : "r"(row + (uint32_t)(((4 * u + k) ^ (t & 7)) * 16)) : "memory");
-              const int ch = 32 * u + 8 * k;
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {                    // (channels of a head come and go in fours)
-                const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[e]));
-                if (!HEADS || (ch + 2 * e >= hs.lead && ch + 2 * e < hs.end)) sum += f.x + f.y;
-              }
-            }
-          }
-          sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-          if (u == 0) asm volatile("st.shared.f32 [%0], %1;" ::"r"(xs_sum + (it & (kExRing - 1)) * 64u + (uint32_t)t * 4u), "f"(sum) : "memory");
-          __syncwarp();
-          if (lane == 0) { pmbar_arrive(xs_full + 8 * (it & (kExRing - 1))); pmbar_arrive(b_empty + 8 * s); }
-          if (++s == c.bst) { s = 0; par ^= 1; }
-        } else if (lane == 0) {
-          pmbar_arrive(xs_full + 8 * (it & (kExRing - 1)));
-        }
-      }
-    }
   } else if (warp < DQ0) {
     // ===================================================================== loaders
     // Codes by TMA, issued by warp 2 (a box per lane).  (The first version copied them with cp.async, sixteen 16-byte
     // pieces per lane and stage: 1100 cycles of issue per stage and loader warp, which set the pace.)  Scales and
     // zero-points are two fp16 per row and stage at any row pitch: cp.async of 4 bytes, 64 rows per warp.
-    // (EXACT: one warp has all 128 rows.)
-    constexpr int NR = EXACT ? 4 : 2;                                            // rows per lane
-    const int r0 = EXACT ? 0 : (warp - LD_WARP0) * 64;
+    const int r0 = (warp - LD_WARP0) * 64;
     const int G = p.K / kGroup;
     int s = 0, it = 0; uint32_t par = 1;
     while (!failed && si.next(sg)) {
       const BFam& f = fam_of_tile(c, sg.tile);
       const JobDev& js = p.job[f.job + ((f.mode == kBSwiglu && (lane & 1)) ? 1 : 0)];   // odd rows of a SwiGLU pair: the up matrix
-      const __half* sp[NR];
-      const __half* zp[NR];
-#pragma unroll
-      for (int k = 0; k < NR; ++k) {
-        const int row = batch_row(c, p, f, sg.tile, r0 + 32 * k + lane).info.stored;
-        sp[k] = row < 0 ? nullptr : js.scales + c.kb_first / 2 + (size_t)row * G;
-        zp[k] = js.zeros + c.kb_first / 2 + (size_t)max(row, 0) * G;
-      }
+      const int row0 = batch_row(c, p, f, sg.tile, r0 + lane).info.stored, row1 = batch_row(c, p, f, sg.tile, r0 + 32 + lane).info.stored;
+      const __half* s0 = js.scales + c.kb_first / 2 + (size_t)max(row0, 0) * G;
+      const __half* z0 = js.zeros + c.kb_first / 2 + (size_t)max(row0, 0) * G;
+      const __half* s1 = js.scales + c.kb_first / 2 + (size_t)max(row1, 0) * G;
+      const __half* z1 = js.zeros + c.kb_first / 2 + (size_t)max(row1, 0) * G;
       // this lane's box (warp 2): blocks beyond the family's last are left out
       const int tl = sg.tile - f.tile_begin;
       const CUtensorMap* tm = &c.wmap[&f - c.fam];
@@ -510,12 +462,14 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
           if (lane < boxes) tma_box_3d(dst + (uint32_t)(lane * f.box_rows) * 128u, tm, c.kb_first * 32 + st * 128, by, bz, w_full + 8 * s);
         }
         const uint32_t sd = dst + WST_BYTES + (uint32_t)((r0 + lane) * 4);
-#pragma unroll
-        for (int k = 0; k < NR; ++k)
-          if (sp[k]) {
-            bcp_async4(sd + 128 * k, sp[k] + st * 2);
-            bcp_async4(sd + BMW * 4 + 128 * k, zp[k] + st * 2);
-          }
+        if (row0 >= 0) {
+          bcp_async4(sd, s0 + st * 2);
+          bcp_async4(sd + BMW * 4, z0 + st * 2);
+        }
+        if (row1 >= 0) {
+          bcp_async4(sd + 128, s1 + st * 2);
+          bcp_async4(sd + BMW * 4 + 128, z1 + st * 2);
+        }
         bcp_async_arrive(w_full + 8 * s);
         if (++s == c.wst) { s = 0; par ^= 1; }
       }
@@ -545,27 +499,25 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
     };
     float sum[16], g_s = 0.f, g_cz = 0.f;        // EXACT: the tile's sums, scale and offset of the group whose sums are due
     bool due = false;
-    int g_as = 0;                                // ... its A slot and the phase in which its MMAs complete, its place in the X ring
-    uint32_t g_par = 0, g_it = 0, my_it = (uint32_t)half;
-    auto add_group = [&]() -> bool {             // (before the next operand of this half is announced: its MMAs overwrite P)
-      const uint32_t xr = g_it & (kExRing - 1);
-      if (!pmbar_wait_warp(xs_full + 8 * xr, (g_it / kExRing) & 1, abort_flag) || !pmbar_wait_warp(a_empty + 8 * g_as, g_par, abort_flag)) return false;
-      tc_fence_after();
+    auto add_group = [&]() {                     // (behind the wait for the slot whose MMAs these are)
 #pragma unroll
       for (int k0 = 0; k0 < 16; k0 += 8) {
-        uint32_t v[8];
-        float u[8];
-        tmem_ld8(a_lane - (uint32_t)c.a_base + kExP + 16 * half + k0, v);
-#pragma unroll
-        for (int k = 0; k < 8; k += 4)
-          asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(u[k]), "=f"(u[k + 1]), "=f"(u[k + 2]), "=f"(u[k + 3]) : "r"(xs_sum + xr * 64u + (k0 + k) * 4u) : "memory");
+        uint32_t v[8], u[8];
+        tmem_ld8(a_lane - (uint32_t)c.a_base + kExP + 32 * half + k0, v);
+        tmem_ld8(a_lane - (uint32_t)c.a_base + kExP + 32 * half + 16 + k0, u);
         tmem_ld_wait();
 #pragma unroll
-        for (int k = 0; k < 8; ++k) sum[k0 + k] = fmaf(g_s, __uint_as_float(v[k]), fmaf(g_cz, u[k], sum[k0 + k]));
+        for (int k = 0; k < 8; ++k) sum[k0 + k] = fmaf(g_s, __uint_as_float(v[k]), fmaf(g_cz, __uint_as_float(u[k]), sum[k0 + k]));
       }
-      tc_fence_before();
-      return true;
     };
+    if (EXACT && half == 0) {                    // (complete before this warp's first arrival for the MMA warp)
+      const uint32_t t = a_lane - (uint32_t)c.a_base + kExOnes;
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(t + 8 * k), "r"(k ? 0u : 0x3c003c00u) : "memory");
+      tmem_st_wait();
+      tc_fence_before();
+    }
     for (int count = 0; !failed && si.next(sg); ++count) {
       if (EXACT) {
         due = false;
@@ -614,36 +566,33 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
           for (int i = j0; i < j0 + 4; ++i) {
             const int k = i & 7, b = i >> 3;
             uint32_t wi = w[i];
-            if (HEADS)                           // (k-block b is a head's first unless heads have two and b is 1)
+            if (HEADS && !EXACT)                 // (k-block b is a head's first unless heads have two and b is 1)
               wi = __funnelshift_l(k > 0 || (b == 1 && hs[1].lead != hs[1].shift) ? w[i > 0 ? i - 1 : 0] : 0u, w[i], 4 * hs[b].shift);
             const uint4 d = HEADS && k * 8 >= hs[b].end ? make_uint4(0, 0, 0, 0) : EXACT ? codes_word(wi) : dequant_word(wi, s2, cz2);
-            const bool no_lo = HEADS && k == 0 && hs[b].lead != 0, no_hi = HEADS && k * 8 + 4 == hs[b].end;
+            const bool no_lo = HEADS && !EXACT && k == 0 && hs[b].lead != 0, no_hi = HEADS && !EXACT && k * 8 + 4 == hs[b].end;
             o[4 * k] = no_lo ? 0u : d.x; o[4 * k + 1] = no_lo ? 0u : d.y; o[4 * k + 2] = no_hi ? 0u : d.z; o[4 * k + 3] = no_hi ? 0u : d.w;
           }
         };
         convert(0);
-        if (!EXACT) announce();
+        announce();
         convert(4);
         // (the slot's previous user: the half stage n_ast earlier.  This warp wrote the half stage two earlier after a wait
         //  that implies every half stage up to 2 + n_ast earlier is done, so the parity cannot be two phases old.)
         if (use > 0 && !pmbar_wait_warp(a_empty + 8 * as, (use - 1) & 1, abort_flag)) { failed = true; break; }
         tc_fence_after();
         tmem_st32(a_lane + (uint32_t)(64 * as), o);
-        convert(8);
-        convert(12);
-        tmem_st32(a_lane + (uint32_t)(64 * as + 32), o);
         if (EXACT) {
-          if (due && !add_group()) { failed = true; break; }
+          if (due) add_group();
           g_s = __half2float(sc);
           g_cz = (8.f - __half2float(zp)) * g_s;
           due = st * KS + half * (KS / 2) < c.n_kb;
-          g_as = as; g_par = (uint32_t)use & 1u; g_it = my_it;
-          my_it += 2;
         }
-        stored_as = as;
-        if (EXACT) announce();
+        convert(8);
+        convert(12);
+        tmem_st32(a_lane + (uint32_t)(64 * as + 32), o);
         release();
         if (st + 1 < sg.s1 && !fetch()) { failed = true; break; }
+        stored_as = as;
         as += 2;
         if (as >= c.n_ast) { as -= c.n_ast; ++use; }
       }
@@ -652,7 +601,9 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
       asm volatile("griddepcontrol.wait;" ::: "memory");       // outputs, positions and workspace: after the preceding kernel
       const RowStore<T> rs = row_store(sg.tile);               // (several dependent loads, while the last MMAs run)
       if (EXACT) {
-        if (due && !add_group()) { failed = true; break; }
+        if (!pmbar_wait_warp(a_empty + 8 * as, (use - 1) & 1, abort_flag)) { failed = true; break; }
+        tc_fence_after();
+        if (due) add_group();
         if (count >= 1 && !pmbar_wait_warp(acc_empty, (count - 1) & 1, abort_flag)) { failed = true; break; }
         tc_fence_after();
         uint32_t v[16];
@@ -790,7 +741,7 @@ int batch_supported(const Params& p) {
     if (a.start != 0) return 0;
   } else if (a.start % (KS * BK) != 0 || a.period % BK != 0 || a.keep % 4 != 0 || a.keep <= a.period - BK) {
     return 0;
-  } else if (a.keep % 8 != 0 && (p.dt != UNIQL_F16 || a.period > 2 * BK || a.keep < 12)) {
+  } else if (a.keep % 8 != 0 && (p.M <= 16 || p.dt != UNIQL_F16 || a.period > 2 * BK)) {
     return 0;                            // (heads of one or two k-blocks, read in place: bf16 activations are copied anyway)
   }
   if ((p.ldx % 8) != 0 || (((uintptr_t)p.x) & 15) != 0) return 0;
@@ -814,12 +765,20 @@ size_t batch_workspace_bytes(int M, int K) {
 // Measured at 12 / 16 rows, decode kernel -> here, the whole layer in microseconds: Qwen2.5-7B 84.2 -> 71.7 / 90.6 -> 71.4,
 // Mamba2-2.7B 29.0 -> 22.5 / 31.4 -> 22.5, Llama-3-8B 76.0 -> 71.6 / 79.6 -> 71.7, at keep 0.75 71.9 -> 63.6 / 74.9 -> 63.5, at keep
 // 0.65 68.6 -> 66.6 / 72.9 -> 67.2; over five keep rates from 0.55 the decode kernel is nowhere ahead by more than 1 %.
+// Not where kept blocks of output rows are no multiple of 8: the launch that reads those channels then stays on the decode
+// kernel (4-channel boundaries), whose blocks need a whole SM and cannot come in beside this kernel's (Mamba2 mixer at keep
+// 0.8 29.5 -> 30.7 us).  Rotated heads excepted: there the other four launches of a layer outweigh that.
 int exact_batch(const Params& p) {
-  if (p.dt != UNIQL_F16 || p.M < 12 || p.M > 16 || !batch_supported(p)) return 0;
+  if (p.dt != UNIQL_F16 || p.M < 12 || p.M > 16 || !batch_supported(p) || !prefill_supported(p)) return 0;
   // (an option of the decode kernel that is set asks for that kernel)
   if (opt(kOptDecodeKp) != 0 || opt(kOptDecodeRp) != 0 || opt(kOptDecodeStages) != 0 || opt(kOptDecodeNarrow) != -1 || opt(kOptDecodeXstream) != -1 ||
       opt(kOptDecodeXcluster) != -1 || opt(kOptDecodeI8) != 1 || opt(kOptDecodeSplitBatch) != 2)
     return 0;
+  for (int j = 0; j < p.n_jobs; ++j) {
+    if (p.n_jobs > 1 && p.job[0].rope.enabled) break;
+    for (int k = 0; k < p.job[j].omap.n_fam; ++k)
+      if (p.job[j].omap.fam[k].count > 1 && p.job[j].omap.fam[k].keep % 8 != 0) return 0;
+  }
   return 1;
 }
 
@@ -843,15 +802,15 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   // fp32 accumulate, A and B fp16, both K-major, N tokens, 128 rows
   c.idesc = (1u << 4) | ((uint32_t)(c.n >> 3) << 17) | ((uint32_t)(BMW >> 4) << 24);
   c.exact = p.M <= 16 && p.dt != UNIQL_BF16;
-  c.n_ast = c.n <= 64 ? 3 : 2;
-  c.a_base = c.n <= 64 ? 64 : 128;
+  c.n_ast = c.n <= 64 && !c.exact ? 3 : 2;
+  c.a_base = c.exact ? (int)kExA : c.n <= 64 ? 64 : 128;
   // shared memory: two to four half stages of activations, the rest for the codes (HBM's latency is theirs to cover)
   c.bst = c.n > 64 ? 2 : (c.n > 32 ? 3 : 4);
   c.off_w = c.bst * (KS / 2) * c.n * 128;
-  const int room = kSmemBatch - 1024 - kBarBytes - c.off_w;
+  const int room = kSmemBatch - 1024 - 512 - c.off_w;
   c.wst = room / WSTAGE < MAX_WST ? room / WSTAGE : MAX_WST;
   c.off_bar = c.off_w + c.wst * WSTAGE;
-  size_t smem = 1024 + (size_t)c.off_bar + kBarBytes;
+  size_t smem = 1024 + (size_t)c.off_bar + 512;
   c.status = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(cfg.workspace) + decode_status_offset());
   size_t used = (decode_workspace_header_bytes() + 255) & ~(size_t)255;
   const void* x = p.x;
@@ -915,7 +874,7 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
     if (c.p == 1) return UNIQL_ERR_CUDA;
     c.p = 1;                                                                   // clusters cannot be launched here: whole tiles
     best_clusters = c.n_tiles < res.clusters[1] ? c.n_tiles : res.clusters[1];
-    smem = 1024 + (size_t)c.off_bar + kBarBytes;
+    smem = 1024 + (size_t)c.off_bar + 512;
   }
 }
 
