@@ -1653,7 +1653,9 @@ void visited_range(const ChanMap& m, int gran, int* first, int* total) {
 
 // Split of the visited groups into k-parts and the shared-memory plan: as few k-parts as let the staged
 // activations fit beside a deep enough ring of stages.  Returns 0 when nothing fits.
-size_t plan_split(DecodeCfg* c, int M, int g_total, int gran, bool i8) {
+// A fourth stage before the second buffer of parked sums (one_buf): the bytes in flight are what a launch streams with, while
+// the epilogue warps drain a buffer in a fraction of a tile's time.
+size_t plan_split(DecodeCfg* c, int M, int g_total, int gran, bool i8, bool one_buf = true) {
   const int MT = M <= 8 ? 1 : 2;
   const int part_bufs = M <= 8 ? 2 : 1;
   int n_kp = opt(kOptDecodeKp);
@@ -1673,8 +1675,10 @@ size_t plan_split(DecodeCfg* c, int M, int g_total, int gran, bool i8) {
     for (n_kp = 1; n_kp <= kMaxKParts && !fits; ++n_kp)
       for (int s = want; s >= 3 && !fits; --s) {
         const int gp = round_up((g_total + n_kp - 1) / n_kp, gran);
-        smem = plan_smem(c, M, MT, gp, s, part_bufs, i8);
-        fits = smem <= (size_t)kSmemMax;
+        for (int bufs = part_bufs; bufs >= (one_buf ? 1 : part_bufs) && !fits; --bufs) {
+          smem = plan_smem(c, M, MT, gp, s, bufs, i8);
+          fits = smem <= (size_t)kSmemMax;
+        }
         c->gp = gp;
       }
   }
@@ -1811,7 +1815,7 @@ size_t decode_workspace_bytes(int M, int K, int N_total) {
   DecodeCfg c;
   memset(&c, 0, sizeof(c));
   const int G = (K + kGroup - 1) / kGroup;
-  if (!plan_split(&c, M, G, 2, false)) return (size_t)kWsHeader;
+  if (!plan_split(&c, M, G, 2, false, false)) return (size_t)kWsHeader;
   const size_t chunks = (size_t)(G + CG - 1) / CG;
   const size_t tiles = (size_t)(N_total + RB - 1) / RB + (size_t)N_total / 32 + 2 * kMaxJobs;
   const size_t slots = tiles * 2 * c.n_kp + (size_t)c.n_rp * c.n_kp * (chunks + 2 * c.n_kp);
