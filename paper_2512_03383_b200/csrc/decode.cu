@@ -996,7 +996,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
       };
       using std::integral_constant;
       if (my_pairs * 16 <= CTH) quantise(integral_constant<int, 1>(), integral_constant<int, 1>());
-      else if (my_pairs * 16 <= 2 * CTH) quantise(integral_constant<int, 2>(), integral_constant<int, 1>());
+      else if (my_pairs * 32 <= 3 * CTH) quantise(integral_constant<int, 2>(), integral_constant<int, 1>());
       else quantise(integral_constant<int, 4>(), integral_constant<int, 2>());
       if (xc) {
         // both halves are in place once the sixteen consumer warps of each block have arrived at this block's
