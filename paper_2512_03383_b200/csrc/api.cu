@@ -206,6 +206,44 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
     }
   }
   if (gv_else && !relaid) gv = true;
+  // Decode sizes with an odd number of groups: the decode kernel on a copy of the scales and zero-points with padded rows, a
+  // sixteenth of the weight's bytes (on single blocks of the tensor-core kernel, which took them before, 10192 x 10624 at two
+  // rows was 52 us where its bytes take 9).  Not under options that run a batch as two halves.
+  if (path == UNIQL_PATH_AUTO && !gv && !dec_ok && p.M <= 16 && !halves && (p.K / kGroup) % 2 != 0) {
+    Params q = p;
+    const int G = p.K / kGroup;
+    q.sz_pitch = (G + 7) / 8 * 8;
+    size_t at[kMaxJobs + 1] = {0};
+    int rows[kMaxJobs] = {0}, n_total = 0;
+    bool small = true;
+    for (int j = 0; j < p.n_jobs; ++j) {                     // (rows up to the last kept one)
+      const Fam& f = p.job[j].omap.fam[p.job[j].omap.n_fam - 1];
+      rows[j] = f.start + (f.count - 1) * f.period + f.keep;
+      n_total += p.job[j].k_out;
+      small = small && (int64_t)rows[j] * (q.sz_pitch / 8) < (1 << 30);
+      at[j + 1] = at[j] + (((size_t)rows[j] * q.sz_pitch * 4 + 255) & ~(size_t)255);
+      q.job[j].scales = q.job[j].zeros = nullptr;            // (aligned as the copies will be)
+    }
+    if (small && decodes(q) && on_integers(q)) {
+      if (!cfg.workspace) {
+        int rc = lib_workspace(&cfg.workspace, &cfg.ws_bytes, cfg.stream);
+        if (rc != UNIQL_OK) return rc;
+      }
+      if (cfg.ws_bytes >= at[p.n_jobs] + decode_workspace_bytes(p.M, p.K + kGroup, n_total) + 256) {
+        LaunchCfg dc = cfg;
+        dc.ws_bytes = (cfg.ws_bytes - at[p.n_jobs]) & ~(size_t)255;
+        for (int j = 0; j < p.n_jobs; ++j) {
+          __half* o = reinterpret_cast<__half*>(reinterpret_cast<unsigned char*>(cfg.workspace) + dc.ws_bytes + at[j]);
+          int rc = launch_pad_scales(p.job[j].scales, p.job[j].zeros, rows[j], G, q.sz_pitch, o, cfg.stream);
+          if (rc != UNIQL_OK) return rc;
+          q.job[j].scales = o;
+          q.job[j].zeros = o + (size_t)rows[j] * q.sz_pitch;
+        }
+        const int rc = launch_decode(q, dc);
+        if (rc != UNIQL_ERR_WORKSPACE && rc != UNIQL_ERR_UNSUPPORTED) return rc;      // (those: nothing was launched)
+      }
+    }
+  }
   // Nine to sixteen rows in bf16: the batch kernel, whose fp16 operands that type had at these sizes before the decode kernel
   // took it (Mamba2-2.7B mixer at 12 rows 28.9 -> 22.0 us).  fp16 stays on exact codes.
   // fp16: its instance that multiplies the codes themselves, by the rule of exact_batch().
@@ -314,7 +352,10 @@ extern "C" size_t uniql_workspace_bytes(int M, int K, int N_total) {
   // (+ room for the activations re-laid on 8-channel boundaries, see dispatch())
   const size_t relay = (((size_t)M * (size_t)(K + 8) * 2) + 255) / 256 * 256 + 512;
   if (M > 16) return prefill_workspace_bytes(M, K) + relay;
-  const size_t a = decode_workspace_bytes(M, K, N_total);
+  const int G = (K + kGroup - 1) / kGroup;
+  // (an odd number of groups: the copy of the scales and zero-points, see dispatch_as())
+  const size_t pad = G % 2 != 0 ? (size_t)N_total * ((G + 7) / 8 * 8) * 4 + 256 * (kMaxJobs + 1) : 0;
+  const size_t a = (pad ? decode_workspace_bytes(M, K + kGroup, N_total) : decode_workspace_bytes(M, K, N_total)) + pad;
   const size_t b = M <= 4 ? gemv_workspace_bytes(M, K, N_total) : M > 8 ? batch_workspace_bytes(M, K) : 0;
   return (a > b ? a : b) + relay;
 }

@@ -56,6 +56,8 @@ struct Params {
   const void* x;
   int ldx;
   int dt;             // uniql_dtype
+  int sz_pitch;       // decode kernel: groups per row of the jobs' scales and zero-points where that is not K / 128 (a copy with
+                      // padded rows that the kernel in front makes), else 0
   int x_f16;          // tensor-core kernels: the activations are fp16 whatever dt says (outputs and bias are dt)
   int M;
   int K;              // stored input channels
@@ -162,6 +164,8 @@ int launch_generic(const Params& p, const LaunchCfg& cfg);
 // out[m][h * keep8 + r] = r < keep ? x[m][h * keep + r] : 0  (2-byte elements; out 16-byte aligned, keep8 and ldo multiples
 // of 8); to_f16: from bf16 to fp16 on the way
 int launch_relay_x(const void* x, long long ldx, int M, int count, int keep, int keep8, void* out, int ldo, bool to_f16, cudaStream_t stream);
+// scales and zero-points [rows][G] -> out[rows][pitch], then the same of the zero-points (pitch a multiple of 8, out 16-byte aligned)
+int launch_pad_scales(const void* scales, const void* zeros, int rows, int G, int pitch, void* out, cudaStream_t stream);
 int launch_decode(const Params& p, const LaunchCfg& cfg);
 int decode_supported(const Params& p);
 int decode_integer_path(const Params& p);

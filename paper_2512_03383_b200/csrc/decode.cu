@@ -105,6 +105,7 @@ struct Phase {
   const void* x;         // activations [M][ldx]
   long long ldx;
   int K;                 // stored input channels of the phase's matrices
+  int G;                 // groups per row of their scales and zero-points
   int x4;                // kept blocks lie on 4- but not on 8-channel boundaries: units are loaded in two halves
   int start, keep;       // the input family (vector staging): head h keeps [start + h*period, +keep)
   int period, count;     // count = 1: a leading block
@@ -143,6 +144,7 @@ struct DecodeCfg {
   // Streamed activations (rows too long to stage whole beside the ring): a small kernel quantises x once
   // into the layout the consumers read, [group][virtual row][128 bytes] plus (integer sum, 2^-e) per (group,
   // batch row), and every stage of the ring carries the eight groups of its unit beside the weights.
+  int sz_wait;           // scales and zero-points are a copy made by the kernel in front
   int x_cluster;         // blocks run as clusters of two that share the staging of the activations: each quantises
                          // half of the (row, group) pairs and writes them into both blocks' shared memory
   int x_stream;
@@ -502,7 +504,7 @@ __device__ inline PhaseCtx phase_ctx(const DecodeCfg& c, int ph, int kp, int rp)
   const int v_lo = kp * c.gp;                                   // first visit index of this k-part
   k.Gk = min(c.gp, P.g_total - v_lo);
   k.sg_lo = P.v_first + v_lo;
-  k.G = P.K / kGroup;
+  k.G = P.G;
   int Ck = P.ck0, Bt = P.bt0;
   FastDiv by_ck = P.by_ck0, by_bt = P.by_bt0;
   if (k.Gk != P.gk0) {                                          // a shorter last k-part
@@ -602,7 +604,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
     // fill of the ring do not wait for it: their stages are armed with the weight bytes only, and once the ring
     // is full (or the block's units are all issued) the producer waits for the predecessor and sends the
     // activations of those stages after them, with the arrival the stages' barriers still lack.
-    bool x_waited = !xs_on;
+    bool x_waited = !xs_on, sz_waited = c.sz_wait == 0;
     int x_lv0[MAX_STAGES];
     auto send_x = [&](int stage, int lv0) {                          // lane 31: arrival + the unit's activations
       const uint32_t full = bar_full + 8 * stage;
@@ -700,6 +702,10 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
           }
         }
         if (new_tile) setup_rows();
+        if (!sz_waited) {
+          asm volatile("griddepcontrol.wait;" ::: "memory");
+          sz_waited = true;
+        }
 #pragma unroll
         for (int r2 = 0; r2 < 2; ++r2) {
           const int ngr = (mode == kNarrow && r2) ? ng2 : ng;      // groups of this half of the row slots
@@ -1782,9 +1788,9 @@ int decode_supported(const Params& p) {
   if (p.M < 1 || p.M > 16) return 0;
   // (bf16 activations: the integer path only, whose staging takes either type to the same 16-bit fixed point)
   if (p.dt != UNIQL_F16 && (opt(kOptDecodeI8) == 0 || !decode_integer_path(p))) return 0;
-  if ((p.K % (2 * kGroup)) != 0) return 0;
+  if ((p.K % (2 * kGroup)) != 0 && p.sz_pitch == 0) return 0;
   if (count_tile_fams(p) > kMaxTF) return 0;
-  const int gran = copy_granule(p.K / kGroup);
+  const int gran = copy_granule(p.sz_pitch ? p.sz_pitch : p.K / kGroup);
   for (int j = 0; j < p.n_jobs; ++j) {
     // scale / zero-point rows are copied in granules of 2, 4 or 8 fp16 values
     if (((uintptr_t)p.job[j].scales | (uintptr_t)p.job[j].zeros) & (uintptr_t)(gran * 2 - 1)) return 0;
@@ -1828,7 +1834,7 @@ size_t decode_workspace_bytes(int M, int K, int N_total) {
 int launch_decode(const Params& p, const LaunchCfg& cfg) {
   DecodeCfg c;
   memset(&c, 0, sizeof(c));
-  const int G = p.K / kGroup;
+  const int G = p.sz_pitch ? p.sz_pitch : p.K / kGroup;
   const int gran = copy_granule(G);
   int g_total = 0, v_first = 0;
   visited_range(p.imap, gran, &v_first, &g_total);
@@ -1938,7 +1944,8 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
   c.n_ph = 1;
   {
     Phase& P = c.ph[0];
-    P.x = p.x; P.ldx = p.ldx; P.K = p.K;
+    P.x = p.x; P.ldx = p.ldx; P.K = p.K; P.G = G;
+    c.sz_wait = p.sz_pitch != 0;
     P.x4 = c.x_vec ? 0 : 1;
     P.start = p.imap.fam[0].start; P.keep = p.imap.fam[0].keep;
     P.period = p.imap.fam[0].period; P.count = p.imap.fam[0].count;
@@ -2091,14 +2098,14 @@ int launch_mlp_phases(const MlpDecode& d, int first, int count, const LaunchCfg&
     P.tile0 = tiles; P.v_first = 0;
     int rc;
     if (ph == 0) {
-      P.x = d.x; P.ldx = d.ldx; P.K = d.hidden; P.start = 0; P.keep = d.hidden; P.g_total = d.hidden / kGroup;
+      P.x = d.x; P.ldx = d.ldx; P.K = d.hidden; P.G = d.hidden / kGroup; P.start = 0; P.keep = d.hidden; P.g_total = d.hidden / kGroup;
       P.period = d.hidden; P.count = 1;
       f.mode = kSwiglu; f.job = 0; f.job2 = 1; f.keep = d.k_int; f.period = d.inter;
       f.tpb = (d.k_int + RB / 2 - 1) / (RB / 2);
       rc = encode_w_map(&c.wmap[n_tf], d.wg, d.hidden, d.hidden / 2, d.k_int, 1, d.k_int, RB / 2);
       if (!rc) rc = encode_w_map(&c.wmap_up, d.wu, d.hidden, d.hidden / 2, d.k_int, 1, d.k_int, RB / 2);
     } else {
-      P.x = d.h; P.ldx = d.ldh; P.K = d.inter; P.start = 0; P.keep = d.k_int; P.period = d.inter; P.count = 1;
+      P.x = d.h; P.ldx = d.ldh; P.K = d.inter; P.G = d.inter / kGroup; P.start = 0; P.keep = d.k_int; P.period = d.inter; P.count = 1;
       P.g_total = (d.k_int + kGroup - 1) / kGroup;
       const int rows = narrow ? RB / 2 : RB;
       f.mode = narrow ? kNarrow : kPlain; f.job = 2; f.job2 = 2; f.keep = d.hidden; f.period = d.hidden;

@@ -114,6 +114,23 @@ __global__ void __launch_bounds__(128) relay_x_kernel(const unsigned short* __re
   }
 }
 
+// Scales and zero-points with rows padded to whole 16-byte pieces: with an odd number of groups a row begins on any 2-byte
+// boundary, and the decode kernel copies its rows asynchronously, four bytes at the least.  A thread has eight groups of a row.
+__global__ void __launch_bounds__(128) pad_scales_kernel(const unsigned short* __restrict__ scales, const unsigned short* __restrict__ zeros,
+                                                         int rows, int G, int pieces, uint4* __restrict__ out) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool live = i < rows * pieces;
+  const int r = live ? i / pieces : 0, g = (i - r * pieces) * 8;
+  const unsigned short* src = (blockIdx.y ? zeros : scales) + (size_t)r * G + g;
+  uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (live && g + k < G) w[k >> 1] |= (uint32_t)__ldg(src + k) << (16 * (k & 1));
+  asm volatile("griddepcontrol.wait;" ::: "memory");          // (weights are written by no kernel; the workspace is)
+  if (live) out[(size_t)blockIdx.y * rows * pieces + i] = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 inline int grid_for(int64_t n, int threads) {
   static const int sms = [] {
     int dev = 0, v = 0;
@@ -145,6 +162,25 @@ int uniql::launch_relay_x(const void* x, long long ldx, int M, int count, int ke
   lc.numAttrs = opt(kOptPdl) ? 1 : 0;
   if (cudaLaunchKernelEx(&lc, to_f16 ? relay_x_kernel<true> : relay_x_kernel<false>, reinterpret_cast<const unsigned short*>(x), ldx, M, count,
                          keep, keep8, reinterpret_cast<unsigned short*>(out), ldo) != cudaSuccess) {
+    cudaGetLastError();
+    return UNIQL_ERR_CUDA;
+  }
+  return UNIQL_OK;
+}
+
+int uniql::launch_pad_scales(const void* scales, const void* zeros, int rows, int G, int pitch, void* out, cudaStream_t stream) {
+  cudaLaunchConfig_t lc;
+  memset(&lc, 0, sizeof(lc));
+  lc.gridDim = dim3((unsigned)(((int64_t)rows * (pitch / 8) + 127) / 128), 2);
+  lc.blockDim = dim3(128);
+  lc.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = attr;
+  lc.numAttrs = opt(kOptPdl) ? 1 : 0;
+  if (cudaLaunchKernelEx(&lc, pad_scales_kernel, reinterpret_cast<const unsigned short*>(scales), reinterpret_cast<const unsigned short*>(zeros),
+                         rows, G, pitch / 8, reinterpret_cast<uint4*>(out)) != cudaSuccess) {
     cudaGetLastError();
     return UNIQL_ERR_CUDA;
   }
