@@ -575,13 +575,15 @@ int mlp_tensor_core(const void* x, int ldx, int dt, const uint8_t* wg, const voi
     jd.y = h; jd.ldy = ldh; jd.N = inter; jd.k_out = k_int;
     jd.pair = j + 1;
   }
-  // bf16: the gated launch leaves h as fp16 too, in rows of whole 128-byte lines at the end of the workspace, and the down
-  // projection reads that copy (a pass over h in between took 28 of 840 us at 2048 rows of Qwen2.5-7B).  Where there is room
-  // for it beside everything that the two launches may use.
+  // bf16 on the batch kernel: the gated launch leaves h as fp16 too, in rows of whole 128-byte lines at the end of the workspace,
+  // and the down projection reads that copy: a pass over h in between is a launch of its own (Llama-3-8B layer at 34 rows, with
+  // the kept blocks converted on their way, 77.3 -> 72.0 us).  Where there is room beside everything that the two launches may use.
+  // Not above 128 rows: there the second store of every output cost the gated launch what the pass takes (Qwen2.5-7B at 2048
+  // rows 730 -> 744 us, at 677 336 -> 339 us).
   const int ld16 = (k_int + 63) / 64 * 64, path = g_path.load();
   const size_t h16_bytes = ((size_t)M * ld16 * 2 + 255) & ~(size_t)255;
-  const bool h16 = dt == UNIQL_BF16 && M > 16 && (path == UNIQL_PATH_AUTO || path == UNIQL_PATH_PREFILL) && opt(kOptPrefillConvert) != 1 &&
-                   cfg_in.ws_bytes >= h16_bytes + prefill_workspace_bytes(M, hidden) + 256;
+  const bool h16 = dt == UNIQL_BF16 && M > 16 && batch_supported(a) && (path == UNIQL_PATH_AUTO || path == UNIQL_PATH_PREFILL) &&
+                   opt(kOptPrefillConvert) != 1 && cfg_in.ws_bytes >= h16_bytes + prefill_workspace_bytes(M, hidden) + 256;
   LaunchCfg cfg = cfg_in;
   if (h16) {
     cfg.ws_bytes = (cfg_in.ws_bytes - h16_bytes) & ~(size_t)255;
@@ -608,9 +610,10 @@ int mlp_tensor_core(const void* x, int ldx, int dt, const uint8_t* wg, const voi
 
 extern "C" size_t uniql_mlp_workspace_bytes(int M, int hidden, int inter) {
   if (M < 1 || hidden < 1 || inter < 1) return 0;
-  // tensor-core kernel, two launches (+ the fp16 copies of both activations of bf16 at once)
+  // tensor-core kernel, two launches (+ up to 128 rows the fp16 copies of both activations of bf16 at once)
   if (M > 16)
-    return prefill_workspace_bytes(M, hidden > inter ? hidden : inter) + (size_t)M * (((hidden < inter ? hidden : inter) + 63) / 64 * 64) * 2 + 512;
+    return prefill_workspace_bytes(M, hidden > inter ? hidden : inter) +
+           (M <= 128 ? (size_t)M * (((hidden < inter ? hidden : inter) + 63) / 64 * 64) * 2 + 512 : 0);
   // (16 rows or fewer in bf16 also run on the tensor-core kernel: room for its fp16 copy of the activations)
   const size_t a = mlp_decode_workspace_bytes(M, hidden, inter), b = prefill_workspace_bytes(M, hidden > inter ? hidden : inter);
   size_t c = 0;

@@ -49,6 +49,7 @@
 
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
 #include "tc.cuh"
 
@@ -263,7 +264,8 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
   };
   // ---- epilogue of the block's tile number `count` for the de-quantiser warp that calls it; the two warps of a quadrant
   //      (`half`) share the chunks
-  auto epilogue_tile = [&](const RowStore<T>& rs, int count, int half) {
+  using Store = RowStore<T, !std::is_same<T, __half>::value>;
+  auto epilogue_tile = [&](const Store& rs, int count, int half) {
     const int q = warp & 3;
     const uint32_t t_acc = tmem + ((uint32_t)(32 * q) << 16);
     const int n_ch = c.n / kTokChunk;
@@ -341,7 +343,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
   auto row_store = [&](int tile) {
     const BFam& f = fam_of_tile(c, tile);
     const int r = 32 * (warp & 3) + lane;
-    return RowStore<T>(p, f.job, batch_row(c, p, f, tile, r).info, (r & 1) != 0);
+    return Store(p, f.job, batch_row(c, p, f, tile, r).info, (r & 1) != 0);
   };
 
   BSegIter si;
@@ -600,7 +602,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
       if (failed) break;
       announce();
       asm volatile("griddepcontrol.wait;" ::: "memory");       // outputs, positions and workspace: after the preceding kernel
-      const RowStore<T> rs = row_store(sg.tile);               // (several dependent loads, while the last MMAs run)
+      const Store rs = row_store(sg.tile);               // (several dependent loads, while the last MMAs run)
       if (EXACT) {
         if (!pmbar_wait_warp(a_empty + 8 * as, (use - 1) & 1, abort_flag)) { failed = true; break; }
         tc_fence_after();

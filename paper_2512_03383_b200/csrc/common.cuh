@@ -48,8 +48,8 @@ struct JobDev {
                       // rows 2i, 2i+1 of a tile are retained row i of this matrix and of the NEXT job's (the up
                       // matrix), and the epilogue stores silu(g_i) * u_i at column i of this job's output.
                       // 2: that next job (it has no tiles of its own).
-  __half* y16;        // job 0, pair == 1, bf16: the stored outputs once more as fp16 (the operands of the launch behind), or null
-  int ld16;
+  __half* y16;        // batch kernel, job 0, pair == 1, bf16: the stored outputs once more as fp16 (the operands of the launch
+  int ld16;           // behind), or null
 };
 
 struct Params {
@@ -223,6 +223,5 @@ __device__ inline uint32_t bf16x2_to_f16x2(uint32_t w) {
   return d;
 }
 __device__ inline __half f16_of(__nv_bfloat16 v) { return __ushort_as_half((unsigned short)bf16x2_to_f16x2(__bfloat16_as_ushort(v))); }
-__device__ inline __half f16_of(__half v) { return v; }
 
 }  // namespace uniql

@@ -275,12 +275,7 @@ __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant
             for (int k = 0; k < NV; k += 2) {
               const float got = __shfl_xor_sync(0xffffffffu, second ? val[k] : val[k + 1], 1);
               const float g = (second ? got : val[k]) + b_g, u = (second ? val[k + 1] : got) + b_u;
-              if (live) {
-                const T r = DT<T>::from_f(__fdividef(g, 1.f + __expf(-g)) * u);
-                *yp = r;
-                if constexpr (std::is_same<T, __nv_bfloat16>::value)
-                  if (p.job[0].y16 != nullptr) p.job[0].y16[ri.out_col + (size_t)(m0 + odd + k) * p.job[0].ld16] = f16_of(r);
-              }
+              if (live) *yp = DT<T>::from_f(__fdividef(g, 1.f + __expf(-g)) * u);
               yp += step;
             }
           } else {
@@ -289,12 +284,7 @@ __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant
               if (k >= left) break;
               const float got = __shfl_xor_sync(0xffffffffu, second ? val[k] : val[k + 1], 1);
               const float g = (second ? got : val[k]) + b_g, u = (second ? val[k + 1] : got) + b_u;
-              if (live && k + odd < left) {
-                const T r = DT<T>::from_f(__fdividef(g, 1.f + __expf(-g)) * u);
-                *yp = r;
-                if constexpr (std::is_same<T, __nv_bfloat16>::value)
-                  if (p.job[0].y16 != nullptr) p.job[0].y16[ri.out_col + (size_t)(m0 + odd + k) * p.job[0].ld16] = f16_of(r);
-              }
+              if (live && k + odd < left) *yp = DT<T>::from_f(__fdividef(g, 1.f + __expf(-g)) * u);
               yp += step;
             }
           }

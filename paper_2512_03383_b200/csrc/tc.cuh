@@ -3,8 +3,6 @@
 #pragma once
 #include <stdint.h>
 
-#include <type_traits>
-
 #include "common.cuh"
 
 namespace uniql {
@@ -309,7 +307,8 @@ __device__ inline uint4 codes_word(uint32_t w) {
 // Bias, rotary embedding (Section 3.2, fused RoPE) or gated product, one rounding and the stores of a thread that owns
 // one row of a tile of job `jn` (`info`: which; odd: the up row of a SwiGLU pair); the two members of a pair sit in lanes
 // 2i and 2i + 1.
-template <typename T>
+// Y16: a gated product of bf16 is stored as fp16 too where the job asks for it.
+template <typename T, bool Y16 = false>
 struct RowStore {
   RowInfo ri;
   T* y;
@@ -394,7 +393,7 @@ struct RowStore {
             if (k < n) *yp = r[k];
             yp += step;
           }
-          if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+          if constexpr (Y16) {
             if (p.job[0].y16 != nullptr) {
               __half* hp = p.job[0].y16 + (live ? ri.out_col : 0) + (size_t)(m0 + b + odd) * p.job[0].ld16;
 #pragma unroll

@@ -48,10 +48,11 @@ template <typename T>
 __global__ void embed_kernel(const uint8_t* __restrict__ packed, const __half* __restrict__ scales,
                              const __half* __restrict__ zeros, int64_t V, int64_t K, const int32_t* __restrict__ ids,
                              T* __restrict__ out, int64_t ldo, int* __restrict__ bad) {
-  // (programmatic dependent launch, as the kernels of the layers: this one's blocks come in as the preceding launch's leave,
-  //  and the next launch sets itself up and fetches its first weights meanwhile; ids and out are touched behind the wait)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // (programmatic dependent launch: this one's blocks come in as the preceding launch's leave, and the next launch's beside
+  //  them -- only now: let in at entry, they took the places that the preceding launch's blocks freed one by one, two to an SM
+  //  with other SMs empty: lm_head at 24 rows 94.5 -> 98.7 us)
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int64_t m = blockIdx.y;
   int64_t row = ids[m];
   const bool in_range = row >= 0 && row < V;
