@@ -216,15 +216,19 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
     size_t at[kMaxJobs + 1] = {0};
     int rows[kMaxJobs] = {0}, n_total = 0;
     bool small = true;
+    int64_t codes = 0;
     for (int j = 0; j < p.n_jobs; ++j) {                     // (rows up to the last kept one)
       const Fam& f = p.job[j].omap.fam[p.job[j].omap.n_fam - 1];
       rows[j] = f.start + (f.count - 1) * f.period + f.keep;
       n_total += p.job[j].k_out;
+      codes += (int64_t)p.job[j].k_out * p.k_in;
       small = small && (int64_t)rows[j] * (q.sz_pitch / 8) < (1 << 30);
       at[j + 1] = at[j] + (((size_t)rows[j] * q.sz_pitch * 4 + 255) & ~(size_t)255);
       q.job[j].scales = q.job[j].zeros = nullptr;            // (aligned as the copies will be)
     }
-    if (small && decodes(q) && on_integers(q)) {
+    // (nine to sixteen rows have a second kernel in front, which quantises the activations: worth it from ten million codes on --
+    //  9 million 11.5 -> 11.6 us, half a million 9.2 -> 10.2 us, 17 million 18.5 -> 14.9 us)
+    if (small && (p.M <= 8 || codes >= 10000000) && decodes(q) && on_integers(q)) {
       if (!cfg.workspace) {
         int rc = lib_workspace(&cfg.workspace, &cfg.ws_bytes, cfg.stream);
         if (rc != UNIQL_OK) return rc;
