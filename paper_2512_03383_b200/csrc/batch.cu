@@ -93,7 +93,7 @@ struct BatchCfg {
   int n_tiles, n_kb, spt;    // weight tiles of 128 rows, k-blocks, stages per tile
   int kb_first;              // first stored k-block
   int head_kb, head_keep;    // per-head maps: k-blocks and kept channels per head (0: leading block)
-  int head_4;                // 4: kept blocks are no multiple of 8 channels (but of 4)
+  int heads;                 // the instance: see batch_kernel()
   uint32_t idesc;
   int p;                     // blocks per tile (cluster size)
   int* status;
@@ -197,11 +197,14 @@ struct BSegIter {
 // took 2.8 us of the 69 us of a Llama-3-8B layer at 64 rows (head dim 108).  Channels of k-block r of head h in its box:
 // [lead, end).
 struct HeadSpan { int shift, lead, end; };
+template <bool FOURS>
 __device__ inline HeadSpan head_span(const BatchCfg& c, int v) {
+  HeadSpan s = {0, 0, BK};
   const int h = v / c.head_kb, r = v - h * c.head_kb;
-  HeadSpan s;
-  s.shift = (h & 1) ? c.head_4 : 0;
-  s.lead = r == 0 ? s.shift : 0;
+  if (FOURS) {
+    s.shift = (h & 1) ? 4 : 0;
+    s.lead = r == 0 ? s.shift : 0;
+  }
   s.end = min(BK, c.head_keep + s.shift - r * BK);
   return s;
 }
@@ -210,7 +213,9 @@ __device__ inline HeadSpan head_span(const BatchCfg& c, int v) {
 // the operand of ones (eight columns; four columns of zeros behind it, so that four columns on it covers 8 channels).
 constexpr uint32_t kExP = 32, kExOnes = 96, kExA = 112;
 
-template <typename T, bool HEADS, bool EXACT>
+// HEADS: 0 a leading block of input channels, 1 heads that keep a multiple of 8 channels, 2 heads that keep 4 (mod 8) (an
+// instance of its own: inside 1 the shifts and selects per word cost a Bamba-v2-9B mixer at 30 rows 32.2 -> 32.7 us).
+template <typename T, int HEADS, bool EXACT>
 __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ Params p, const __grid_constant__ BatchCfg c) {
   extern __shared__ unsigned char bsm_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
@@ -563,16 +568,16 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
         const __half2 cz2 = __float2half2_rn((8.f - __half2float(zp)) * __half2float(sc));
         uint32_t o[32];
         HeadSpan hs[2] = {{0, 0, BK}, {0, 0, BK}};                 // of the half stage's k-blocks
-        if (HEADS) { hs[0] = head_span(c, st * KS + 2 * half); hs[1] = head_span(c, st * KS + 2 * half + 1); }
+        if (HEADS) { hs[0] = head_span<HEADS == 2>(c, st * KS + 2 * half); hs[1] = head_span<HEADS == 2>(c, st * KS + 2 * half + 1); }
         auto convert = [&](int j0) {             // words j0 .. j0 + 3 of the sixteen
 #pragma unroll
           for (int i = j0; i < j0 + 4; ++i) {
             const int k = i & 7, b = i >> 3;
             uint32_t wi = w[i];
-            if (HEADS && !EXACT)                 // (k-block b is a head's first unless heads have two and b is 1)
+            if (HEADS == 2)                      // (k-block b is a head's first unless heads have two and b is 1)
               wi = __funnelshift_l(k > 0 || (b == 1 && hs[1].lead != hs[1].shift) ? w[i > 0 ? i - 1 : 0] : 0u, w[i], 4 * hs[b].shift);
             const uint4 d = HEADS && k * 8 >= hs[b].end ? make_uint4(0, 0, 0, 0) : EXACT ? codes_word(wi) : dequant_word(wi, s2, cz2);
-            const bool no_lo = HEADS && !EXACT && k == 0 && hs[b].lead != 0, no_hi = HEADS && !EXACT && k * 8 + 4 == hs[b].end;
+            const bool no_lo = HEADS == 2 && k == 0 && hs[b].lead != 0, no_hi = HEADS == 2 && k * 8 + 4 == hs[b].end;
             o[4 * k] = no_lo ? 0u : d.x; o[4 * k + 1] = no_lo ? 0u : d.y; o[4 * k + 2] = no_hi ? 0u : d.z; o[4 * k + 3] = no_hi ? 0u : d.w;
           }
         };
@@ -674,10 +679,10 @@ int batch_families(const Params& p, BatchCfg* c) {
 }
 
 typedef void (*BatchKernel)(Params, BatchCfg);
-BatchKernel batch_instance(bool bf16, bool heads, bool exact) {
-  if (bf16) return heads ? batch_kernel<__nv_bfloat16, true, false> : batch_kernel<__nv_bfloat16, false, false>;
-  if (exact) return heads ? batch_kernel<__half, true, true> : batch_kernel<__half, false, true>;
-  return heads ? batch_kernel<__half, true, false> : batch_kernel<__half, false, false>;
+BatchKernel batch_instance(bool bf16, int heads, bool exact) {
+  if (bf16) return heads ? batch_kernel<__nv_bfloat16, 1, false> : batch_kernel<__nv_bfloat16, 0, false>;
+  if (exact) return heads ? batch_kernel<__half, 1, true> : batch_kernel<__half, 0, true>;
+  return heads == 2 ? batch_kernel<__half, 2, false> : heads ? batch_kernel<__half, 1, false> : batch_kernel<__half, 0, false>;
 }
 
 struct BLaunch {
@@ -715,8 +720,8 @@ int residency(Residency* out) {
   std::lock_guard<std::mutex> lock(mu);
   Residency& r = dev_res[dev];
   if (!r.known) {
-    for (int k = 0; k < 8; ++k)
-      if (cudaFuncSetAttribute(batch_instance(k & 1, k & 2, k & 4), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone) != cudaSuccess)
+    for (int k = 0; k < 12; ++k)
+      if (cudaFuncSetAttribute(batch_instance(k & 1, k >> 2, k & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone) != cudaSuccess)
         return UNIQL_ERR_CUDA;
     const int sms = device_sms();
     r.clusters[0] = 0;
@@ -724,7 +729,7 @@ int residency(Residency* out) {
     for (int p = 2; p <= kMaxP; ++p) {
       BLaunch l(2 * sms / p * p, p, kSmemBatch, nullptr);
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, batch_instance(false, false, false), &l.lc) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      if (cudaOccupancyMaxActiveClusters(&n, batch_instance(false, 0, false), &l.lc) != cudaSuccess) { cudaGetLastError(); n = 0; }
       r.clusters[p] = n < 2 * sms / p ? n : 2 * sms / p;
     }
     r.known = true;
@@ -801,7 +806,7 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   c.kb_first = a.start / BK;
   c.head_kb = a.count > 1 ? kbh : 0;
   c.head_keep = a.keep;
-  c.head_4 = a.count > 1 ? a.keep & 4 : 0;
+  c.heads = a.count == 1 ? 0 : a.keep % 8 == 0 ? 1 : 2;
   // fp32 accumulate, A and B fp16, both K-major, N tokens, 128 rows
   c.idesc = (1u << 4) | ((uint32_t)(c.n >> 3) << 17) | ((uint32_t)(BMW >> 4) << 24);
   c.exact = p.M <= 16 && p.dt != UNIQL_BF16;
@@ -872,7 +877,7 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   for (;;) {
     BLaunch l(best_clusters * c.p, c.p, smem, cfg.stream);
     const bool refused = c.p > 1 && opt(kOptPrefillPair) == 3;                 // tests
-    if (!refused && cudaLaunchKernelEx(&l.lc, batch_instance(p.dt == UNIQL_BF16, c.head_kb != 0, c.exact != 0), p, c) == cudaSuccess) return UNIQL_OK;
+    if (!refused && cudaLaunchKernelEx(&l.lc, batch_instance(p.dt == UNIQL_BF16, c.heads, c.exact != 0), p, c) == cudaSuccess) return UNIQL_OK;
     cudaGetLastError();
     if (c.p == 1) return UNIQL_ERR_CUDA;
     c.p = 1;                                                                   // clusters cannot be launched here: whole tiles
