@@ -206,10 +206,10 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
     }
   }
   if (gv_else && !relaid) gv = true;
-  // Decode sizes with an odd number of groups: the decode kernel on a copy of the scales and zero-points with padded rows, a
-  // sixteenth of the weight's bytes (on single blocks of the tensor-core kernel, which took them before, 10192 x 10624 at two
-  // rows was 52 us where its bytes take 9).  Not under options that run a batch as two halves.
-  if (path == UNIQL_PATH_AUTO && !gv && !dec_ok && p.M <= 16 && !halves && (p.K / kGroup) % 2 != 0) {
+  // An odd number of groups: the decode kernel or, above sixteen rows, the batch kernel on a copy of the scales and zero-points
+  // with padded rows, a sixteenth of the weight's bytes (on single blocks of the tensor-core kernel, which took them before,
+  // 10192 x 10624 at two rows was 41 us where its bytes take 7).  Not under options that run a batch as two halves.
+  if (path == UNIQL_PATH_AUTO && !gv && !dec_ok && p.M <= 128 && !halves && (p.K / kGroup) % 2 != 0) {
     Params q = p;
     const int G = p.K / kGroup;
     q.sz_pitch = (G + 7) / 8 * 8;
@@ -228,12 +228,14 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
     }
     // (nine to sixteen rows have a second kernel in front, which quantises the activations: worth it from ten million codes on --
     //  9 million 11.5 -> 11.6 us, half a million 9.2 -> 10.2 us, 17 million 18.5 -> 14.9 us)
-    if (small && (p.M <= 8 || codes >= 10000000) && decodes(q) && on_integers(q)) {
+    const bool dec = p.M <= 16 && (p.M <= 8 || codes >= 10000000) && decodes(q) && on_integers(q);
+    if (small && (dec || (p.M > 16 && batch_supported(q) && (p.dt != UNIQL_BF16 || opt(kOptPrefillConvert) != 1)))) {
       if (!cfg.workspace) {
         int rc = lib_workspace(&cfg.workspace, &cfg.ws_bytes, cfg.stream);
         if (rc != UNIQL_OK) return rc;
       }
-      if (cfg.ws_bytes >= at[p.n_jobs] + decode_workspace_bytes(p.M, p.K + kGroup, n_total) + 256) {
+      const size_t own = dec ? decode_workspace_bytes(p.M, p.K + kGroup, n_total) : prefill_workspace_bytes(p.M, p.K);
+      if (cfg.ws_bytes >= at[p.n_jobs] + own + 256) {
         LaunchCfg dc = cfg;
         dc.ws_bytes = (cfg.ws_bytes - at[p.n_jobs]) & ~(size_t)255;
         for (int j = 0; j < p.n_jobs; ++j) {
@@ -243,6 +245,7 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
           q.job[j].scales = o;
           q.job[j].zeros = o + (size_t)rows[j] * q.sz_pitch;
         }
+        if (!dec) return launch_batch(q, dc);
         const int rc = launch_decode(q, dc);
         if (rc != UNIQL_ERR_WORKSPACE && rc != UNIQL_ERR_UNSUPPORTED) return rc;      // (those: nothing was launched)
       }
@@ -355,10 +358,10 @@ extern "C" size_t uniql_workspace_bytes(int M, int K, int N_total) {
   if (M < 1 || K < 1 || N_total < 1) return 0;
   // (+ room for the activations re-laid on 8-channel boundaries, see dispatch())
   const size_t relay = (((size_t)M * (size_t)(K + 8) * 2) + 255) / 256 * 256 + 512;
-  if (M > 16) return prefill_workspace_bytes(M, K) + relay;
   const int G = (K + kGroup - 1) / kGroup;
   // (an odd number of groups: the copy of the scales and zero-points, see dispatch_as())
   const size_t pad = G % 2 != 0 ? (size_t)N_total * ((G + 7) / 8 * 8) * 4 + 256 * (kMaxJobs + 1) : 0;
+  if (M > 16) return prefill_workspace_bytes(M, K) + relay + (M <= 128 ? pad : 0);
   const size_t a = (pad ? decode_workspace_bytes(M, K + kGroup, N_total) : decode_workspace_bytes(M, K, N_total)) + pad;
   const size_t b = M <= 4 ? gemv_workspace_bytes(M, K, N_total) : M > 8 ? batch_workspace_bytes(M, K) : 0;
   return (a > b ? a : b) + relay;

@@ -436,7 +436,8 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
     // pieces per lane and stage: 1100 cycles of issue per stage and loader warp, which set the pace.)  Scales and
     // zero-points are two fp16 per row and stage at any row pitch: cp.async of 4 bytes, 64 rows per warp.
     const int r0 = (warp - LD_WARP0) * 64;
-    const int G = p.K / kGroup;
+    const int G = p.sz_pitch ? p.sz_pitch : p.K / kGroup;
+    bool sz_waited = p.sz_pitch == 0;              // (else the kernel in front makes the copy that these rows are)
     int s = 0, it = 0; uint32_t par = 1;
     while (!failed && si.next(sg)) {
       const BFam& f = fam_of_tile(c, sg.tile);
@@ -468,6 +469,10 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
           if (lane == 0) pmbar_expect_tx(w_full + 8 * s, (uint32_t)(boxes * f.box_rows) * 128u);
           __syncwarp();
           if (lane < boxes) tma_box_3d(dst + (uint32_t)(lane * f.box_rows) * 128u, tm, c.kb_first * 32 + st * 128, by, bz, w_full + 8 * s);
+        }
+        if (!sz_waited) {
+          asm volatile("griddepcontrol.wait;" ::: "memory");
+          sz_waited = true;
         }
         const uint32_t sd = dst + WST_BYTES + (uint32_t)((r0 + lane) * 4);
         if (row0 >= 0) {
@@ -743,7 +748,7 @@ int residency(Residency* out) {
 // Up to 128 rows; an input map whose k-blocks are all visited from a 256-channel boundary on (a leading block, or heads
 // that keep a part of every k-block); scale rows that can be copied two groups at a time.
 int batch_supported(const Params& p) {
-  if (p.M < 1 || p.M > 128 || p.K % (2 * kGroup) != 0 || p.imap.n_fam != 1) return 0;
+  if (p.M < 1 || p.M > 128 || (p.K % (2 * kGroup) != 0 && p.sz_pitch == 0) || p.imap.n_fam != 1) return 0;
   const Fam& a = p.imap.fam[0];
   if (a.count == 1) {
     if (a.start != 0) return 0;

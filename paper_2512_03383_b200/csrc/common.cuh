@@ -56,7 +56,7 @@ struct Params {
   const void* x;
   int ldx;
   int dt;             // uniql_dtype
-  int sz_pitch;       // decode kernel: groups per row of the jobs' scales and zero-points where that is not K / 128 (a copy with
+  int sz_pitch;       // decode and batch kernel: groups per row of the jobs' scales and zero-points where that is not K / 128 (a copy with
                       // padded rows that the kernel in front makes), else 0
   int x_f16;          // tensor-core kernels: the activations are fp16 whatever dt says (outputs and bias are dt)
   int M;

@@ -557,11 +557,12 @@ def test_llama_mlp_full_size(B, M):
         check_output(y, ref, "f16", TIGHT, "down keep %.2f" % rate)
 
 
-@pytest.mark.parametrize("M", [1, 2, 4, 5, 8, 9, 16])
-@pytest.mark.parametrize("N,K,k_in,k_out", [(72, 128, 128, 72), (200, 384, 384, 200), (300, 1152, 1032, 259), (520, 2176, 2176, 64), (64, 3968, 3840, 64)])
+@pytest.mark.parametrize("M", [1, 2, 4, 5, 8, 9, 16, 17, 64, 128])
+@pytest.mark.parametrize("N,K,k_in,k_out", [(2650, 3968, 3960, 2600), (72, 128, 128, 72), (200, 384, 384, 200), (300, 1152, 1032, 259), (520, 2176, 2176, 64), (64, 3968, 3840, 64)])
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
-def test_odd_number_of_groups_at_decode_sizes(B, M, N, K, k_in, k_out, dtype):
-    """Rows of scales on 2-byte boundaries: the decode kernel on a copy with padded rows (its own tolerance), also in a caller
+def test_odd_number_of_groups(B, M, N, K, k_in, k_out, dtype):
+    """Rows of scales on 2-byte boundaries: the decode kernel on a copy with padded rows (its own tolerance; from ten million codes
+    on also at nine to sixteen rows), above sixteen rows the batch kernel (weights rounded once to fp16), also in a caller
     workspace of the advertised size, with the same bits; a workspace without room for the copy takes the general path."""
     rng = np.random.default_rng(M + N + K)
     qw = synth.draw_qweight(rng, N, K)
@@ -569,7 +570,7 @@ def test_odd_number_of_groups_at_decode_sizes(B, M, N, K, k_in, k_out, dtype):
     bias = synth.to_dtype_values(rng.standard_normal(N).astype(np.float32), dtype)
     x = synth.draw_x(rng, M, k_in, dtype)
     y, ref = run_ex(B, qw, dw, x, dtype, None, k_in, None, k_out, bias=bias, ldx_pad=-k_in % 8, ldy_pad=1)
-    check_output(y, ref, dtype, 4e-4, "M=%d %dx%d" % (M, N, K))
+    check_output(y, ref, dtype, 4e-4 if M <= 8 else 5e-4, "M=%d %dx%d" % (M, N, K))
     big = torch.empty(B.workspace_bytes(M, K, N), dtype=torch.uint8, device="cuda")
     B.workspace_init(big)
     y2, _ = run_ex(B, qw, dw, x, dtype, None, k_in, None, k_out, bias=bias, ldx_pad=-k_in % 8, ldy_pad=1, workspace=big)
