@@ -193,7 +193,7 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
         const Fam& a = p.imap.fam[0];
         // (bf16 above 16 rows goes to the tensor cores, whose operands are fp16: converted on the way)
         const bool to_f16 = p.dt == UNIQL_BF16 && p.M > 16 && opt(kOptPrefillConvert) != 1;
-        int rc = launch_relay_x(p.x, p.ldx, p.M, a.count, a.keep, keep8, xr, q.ldx, to_f16, cfg.stream);
+        int rc = launch_relay_x(p.x, p.ldx, p.M, a.count, a.keep, keep8, xr, q.ldx, to_f16, p.M > 16 && p.M <= 128, cfg.stream);
         if (rc != UNIQL_OK) return rc;
         q.x = xr;
         q.x_f16 = to_f16 ? 1 : 0;
@@ -240,7 +240,7 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
         dc.ws_bytes = (cfg.ws_bytes - at[p.n_jobs]) & ~(size_t)255;
         for (int j = 0; j < p.n_jobs; ++j) {
           __half* o = reinterpret_cast<__half*>(reinterpret_cast<unsigned char*>(cfg.workspace) + dc.ws_bytes + at[j]);
-          int rc = launch_pad_scales(p.job[j].scales, p.job[j].zeros, rows[j], G, q.sz_pitch, o, cfg.stream);
+          int rc = launch_pad_scales(p.job[j].scales, p.job[j].zeros, rows[j], G, q.sz_pitch, o, !dec, cfg.stream);
           if (rc != UNIQL_OK) return rc;
           q.job[j].scales = o;
           q.job[j].zeros = o + (size_t)rows[j] * q.sz_pitch;

@@ -163,9 +163,9 @@ struct LaunchCfg {
 int launch_generic(const Params& p, const LaunchCfg& cfg);
 // out[m][h * keep8 + r] = r < keep ? x[m][h * keep + r] : 0  (2-byte elements; out 16-byte aligned, keep8 and ldo multiples
 // of 8); to_f16: from bf16 to fp16 on the way
-int launch_relay_x(const void* x, long long ldx, int M, int count, int keep, int keep8, void* out, int ldo, bool to_f16, cudaStream_t stream);
+int launch_relay_x(const void* x, long long ldx, int M, int count, int keep, int keep8, void* out, int ldo, bool to_f16, bool late, cudaStream_t stream);
 // scales and zero-points [rows][G] -> out[rows][pitch], then the same of the zero-points (pitch a multiple of 8, out 16-byte aligned)
-int launch_pad_scales(const void* scales, const void* zeros, int rows, int G, int pitch, void* out, cudaStream_t stream);
+int launch_pad_scales(const void* scales, const void* zeros, int rows, int G, int pitch, void* out, bool late, cudaStream_t stream);
 int launch_decode(const Params& p, const LaunchCfg& cfg);
 int decode_supported(const Params& p);
 int decode_integer_path(const Params& p);
@@ -203,7 +203,8 @@ size_t batch_workspace_min(bool copy_x, int M, int k_in);   // copy_x: bf16 acti
 size_t batch_workspace_bytes(int M, int K);
 int exact_batch(const Params& p);             // twelve to sixteen fp16 rows on its exact-code instance
 // fp16 copy of bf16 activations [M][k_in], row pitch ldo (a multiple of 8; the columns from k_in on are zeros)
-int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo, cudaStream_t stream);
+// late (here and below): the next launch is let in behind the kernel's wait for the one in front, see x_to_f16_kernel()
+int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo, bool late, cudaStream_t stream);
 // tensor map over activations [M][k_in] for boxes of 64 channels x `rows` tokens, 128-byte swizzle
 int encode_x_map(void* map, const void* x, int k_in, int M, int ldx, int rows, bool bf16);
 // tensor map over a family of kept row blocks of packed weights: (byte in row, row in block, block), 128-byte columns

@@ -86,11 +86,12 @@ __global__ void embed_kernel(const uint8_t* __restrict__ packed, const __half* _
 // their way to the tensor cores become fp16 here instead of in a pass of their own.
 template <bool F16>
 __global__ void __launch_bounds__(128) relay_x_kernel(const unsigned short* __restrict__ x, long long ldx, int M, int count, int keep,
-                                                      int keep8, unsigned short* __restrict__ out, int ldo) {
+                                                      int keep8, unsigned short* __restrict__ out, int ldo, int late) {
   // (programmatic dependent launch: the kernel behind this one may set itself up meanwhile; this one waits for its
   //  own predecessor before it reads x or overwrites the copy that predecessor may still read)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int u = blockIdx.x * blockDim.x + threadIdx.x, per = keep8 >> 3;
   if (u >= count * per) return;
   const int h = u / per, r = (u - h * per) * 8;
@@ -118,8 +119,8 @@ __global__ void __launch_bounds__(128) relay_x_kernel(const unsigned short* __re
 // Scales and zero-points with rows padded to whole 16-byte pieces: with an odd number of groups a row begins on any 2-byte
 // boundary, and the decode kernel copies its rows asynchronously, four bytes at the least.  A thread has eight groups of a row.
 __global__ void __launch_bounds__(128) pad_scales_kernel(const unsigned short* __restrict__ scales, const unsigned short* __restrict__ zeros,
-                                                         int rows, int G, int pieces, uint4* __restrict__ out) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+                                                         int rows, int G, int pieces, uint4* __restrict__ out, int late) {
+  if (!late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const bool live = i < rows * pieces;
   const int r = live ? i / pieces : 0, g = (i - r * pieces) * 8;
@@ -129,6 +130,7 @@ __global__ void __launch_bounds__(128) pad_scales_kernel(const unsigned short* _
   for (int k = 0; k < 8; ++k)
     if (live && g + k < G) w[k >> 1] |= (uint32_t)__ldg(src + k) << (16 * (k & 1));
   asm volatile("griddepcontrol.wait;" ::: "memory");          // (weights are written by no kernel; the workspace is)
+  if (late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (live) out[(size_t)blockIdx.y * rows * pieces + i] = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
@@ -149,7 +151,7 @@ inline int grid_for(int64_t n, int threads) {
 }  // namespace uniql
 
 int uniql::launch_relay_x(const void* x, long long ldx, int M, int count, int keep, int keep8, void* out, int ldo, bool to_f16,
-                          cudaStream_t stream) {
+                          bool late, cudaStream_t stream) {
   const unsigned cols = (unsigned)(count * (keep8 / 8) + 127) / 128, rows = (unsigned)device_sms() * 32 / cols + 1;
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
@@ -162,14 +164,14 @@ int uniql::launch_relay_x(const void* x, long long ldx, int M, int count, int ke
   lc.attrs = attr;
   lc.numAttrs = opt(kOptPdl) ? 1 : 0;
   if (cudaLaunchKernelEx(&lc, to_f16 ? relay_x_kernel<true> : relay_x_kernel<false>, reinterpret_cast<const unsigned short*>(x), ldx, M, count,
-                         keep, keep8, reinterpret_cast<unsigned short*>(out), ldo) != cudaSuccess) {
+                         keep, keep8, reinterpret_cast<unsigned short*>(out), ldo, late ? 1 : 0) != cudaSuccess) {
     cudaGetLastError();
     return UNIQL_ERR_CUDA;
   }
   return UNIQL_OK;
 }
 
-int uniql::launch_pad_scales(const void* scales, const void* zeros, int rows, int G, int pitch, void* out, cudaStream_t stream) {
+int uniql::launch_pad_scales(const void* scales, const void* zeros, int rows, int G, int pitch, void* out, bool late, cudaStream_t stream) {
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
   lc.gridDim = dim3((unsigned)(((int64_t)rows * (pitch / 8) + 127) / 128), 2);
@@ -181,7 +183,7 @@ int uniql::launch_pad_scales(const void* scales, const void* zeros, int rows, in
   lc.attrs = attr;
   lc.numAttrs = opt(kOptPdl) ? 1 : 0;
   if (cudaLaunchKernelEx(&lc, pad_scales_kernel, reinterpret_cast<const unsigned short*>(scales), reinterpret_cast<const unsigned short*>(zeros),
-                         rows, G, pitch / 8, reinterpret_cast<uint4*>(out)) != cudaSuccess) {
+                         rows, G, pitch / 8, reinterpret_cast<uint4*>(out), late ? 1 : 0) != cudaSuccess) {
     cudaGetLastError();
     return UNIQL_ERR_CUDA;
   }
