@@ -356,7 +356,6 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
   BSeg sg;
   if (warp == 0) {
     // ===================================================================== activations
-    if (elect_one()) prefetch_map(&c.xmap);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // Only now may the next launch's blocks come in: as two launches fit an SM, triggering at entry let the launch after
     // the next one in as well, whose blocks then sat in slots that this launch's blocks needed.

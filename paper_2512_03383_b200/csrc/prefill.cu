@@ -261,7 +261,6 @@ __global__ void __launch_bounds__(PTH, 1) pair_kernel(const __grid_constant__ Pa
   if (warp == 0) {
     // ===================================================================== activations by TMA
     // (warp-uniform, as the MMA warp: one lane walking this loop took longer per k-block than the MMAs do)
-    if (elect_one()) prefetch_map(&c.xmap);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     constexpr int NH = ONE ? 1 : 2;
     const uint32_t rfull = ppeer_addr(full_a, lrank);       // both blocks' half boxes count on the first block's barriers

@@ -113,8 +113,6 @@ __device__ inline bool pmbar_wait_cluster(uint32_t bar, uint32_t parity, volatil
   *abort_flag = 1;
   return false;
 }
-// a tensor map on its way to the SM before the first copy that needs it (read cold, the map delays that copy)
-__device__ inline void prefetch_map(const CUtensorMap* tm) { asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory"); }
 __device__ inline void tma_box2(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
