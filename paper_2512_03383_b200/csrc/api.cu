@@ -229,7 +229,12 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
     // (nine to sixteen rows have a second kernel in front, which quantises the activations: worth it from ten million codes on --
     //  9 million 11.5 -> 11.6 us, half a million 9.2 -> 10.2 us, 17 million 18.5 -> 14.9 us)
     const bool dec = p.M <= 16 && (p.M <= 8 || codes >= 10000000) && decodes(q) && on_integers(q);
-    if (small && (dec || (p.M > 16 && batch_supported(q) && (p.dt != UNIQL_BF16 || opt(kOptPrefillConvert) != 1)))) {
+    // (above 64 rows the exchange of shared tiles takes its share: single blocks -> batch kernel at 128 rows 0.5 million codes 9.7 ->
+    //  13.2 us, 9 million 12.3 -> 10.5, 17 million 23.2 -> 16.9, 78 million 43.3 -> 45.3; at 48 rows 9.4 -> 7.5, 11.7 -> 8.6, 18.7 ->
+    //  13.7, 41.3 -> 26.5)
+    const bool bat = p.M > 16 && (p.M <= 64 || (codes >= 5000000 && codes <= 40000000)) && (p.dt != UNIQL_BF16 || opt(kOptPrefillConvert) != 1) &&
+                     batch_supported(q);
+    if (small && (dec || bat)) {
       if (!cfg.workspace) {
         int rc = lib_workspace(&cfg.workspace, &cfg.ws_bytes, cfg.stream);
         if (rc != UNIQL_OK) return rc;
