@@ -856,7 +856,7 @@ int launch_batch(const Params& p, const LaunchCfg& cfg) {
   c.p = best;
   c.partials = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(cfg.workspace) + used);
   if (copy_x) {
-    rc = launch_x_to_f16(p.x, p.ldx, p.M, p.k_in, const_cast<void*>(x), ldx, true, cfg.stream);
+    rc = launch_x_to_f16(p.x, p.ldx, p.M, p.k_in, const_cast<void*>(x), ldx, cfg.stream);
     if (rc != UNIQL_OK) return rc;
   }
   const int x_extent = (c.kb_first + c.n_kb) * (BK / 2);     // bytes of a row up to the last visited k-block

@@ -161,6 +161,7 @@ struct LaunchCfg {
                          // once the launch is certain (a workspace that may hold what an unfinished call left)
 };
 int launch_generic(const Params& p, const LaunchCfg& cfg);
+// late (here and below): the next launch is let in behind the kernel's wait for the one in front, see relay_x_kernel()
 // out[m][h * keep8 + r] = r < keep ? x[m][h * keep + r] : 0  (2-byte elements; out 16-byte aligned, keep8 and ldo multiples
 // of 8); to_f16: from bf16 to fp16 on the way
 int launch_relay_x(const void* x, long long ldx, int M, int count, int keep, int keep8, void* out, int ldo, bool to_f16, bool late, cudaStream_t stream);
@@ -203,8 +204,7 @@ size_t batch_workspace_min(bool copy_x, int M, int k_in);   // copy_x: bf16 acti
 size_t batch_workspace_bytes(int M, int K);
 int exact_batch(const Params& p);             // twelve to sixteen fp16 rows on its exact-code instance
 // fp16 copy of bf16 activations [M][k_in], row pitch ldo (a multiple of 8; the columns from k_in on are zeros)
-// late (here and below): the next launch is let in behind the kernel's wait for the one in front, see x_to_f16_kernel()
-int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo, bool late, cudaStream_t stream);
+int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo, cudaStream_t stream);
 // tensor map over activations [M][k_in] for boxes of 64 channels x `rows` tokens, 128-byte swizzle
 int encode_x_map(void* map, const void* x, int k_in, int M, int ldx, int rows, bool bf16);
 // tensor map over a family of kept row blocks of packed weights: (byte in row, row in block, block), 128-byte columns

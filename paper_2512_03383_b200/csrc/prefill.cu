@@ -60,16 +60,11 @@ struct SegIter {
 
 // bf16 activations -> fp16 copy in the workspace, once per call (every weight tile re-reads the tile of
 // activations, so converting there would repeat the work once per 128 weight rows).
-// late: the next launch comes in behind this one's wait.  For the batch kernel (two blocks per SM): let in at entry, its blocks took
-// the places that the launch in front freed one by one, two to an SM with other SMs empty (Llama-3-8B layer in bf16 at 34 rows
-// 71.8 -> 65.7 us, at 124 rows 99.4 -> 89.0 us).  Blocks of a whole SM gain from the earlier entry (Qwen2.5-7B at 677 rows 254.7
-// against 257.1 us).
-__global__ void x_to_f16_kernel(const __nv_bfloat16* __restrict__ x, int ldx, int M, int k_in, __half* __restrict__ o, int ldo, int late) {
+__global__ void x_to_f16_kernel(const __nv_bfloat16* __restrict__ x, int ldx, int M, int k_in, __half* __restrict__ o, int ldo) {
   // (programmatic dependent launch: the tensor-core kernel behind this one may set itself up meanwhile; this one
   //  waits for its own predecessor before it reads x or overwrites the copy that predecessor may still read)
-  if (!late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int u = blockIdx.x * blockDim.x + threadIdx.x;        // 16-byte unit of the output row (ldo is a multiple of 8)
   if (u * 8 >= ldo) return;
   for (int m = blockIdx.y; m < M; m += gridDim.y) {
@@ -616,7 +611,7 @@ int device_sms() {
   return v;
 }
 
-int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo, bool late, cudaStream_t stream) {
+int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo, cudaStream_t stream) {
   const unsigned cols = (unsigned)(ldo / 8 + 127) / 128, rows = (unsigned)device_sms() * 32 / cols + 1;
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
@@ -628,7 +623,7 @@ int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = attr;
   lc.numAttrs = opt(kOptPdl) ? 1 : 0;
-  if (cudaLaunchKernelEx(&lc, x_to_f16_kernel, reinterpret_cast<const __nv_bfloat16*>(x), ldx, M, k_in, reinterpret_cast<__half*>(out), ldo, late ? 1 : 0) !=
+  if (cudaLaunchKernelEx(&lc, x_to_f16_kernel, reinterpret_cast<const __nv_bfloat16*>(x), ldx, M, k_in, reinterpret_cast<__half*>(out), ldo) !=
       cudaSuccess) {
     cudaGetLastError();
     return UNIQL_ERR_CUDA;
@@ -897,7 +892,7 @@ int launch_planned(const Params& p, const LaunchCfg& cfg, bool clusters) {
       if (pl.atomic && cudaMemsetAsync(c.partials, 0, pl.sums, cfg.stream) != cudaSuccess) return UNIQL_ERR_CUDA;
     }
     if (x16) {
-      const int rc = launch_x_to_f16(p.x, p.ldx, p.M, p.k_in, x16, x16_ld, false, cfg.stream);
+      const int rc = launch_x_to_f16(p.x, p.ldx, p.M, p.k_in, x16, x16_ld, cfg.stream);
       if (rc != UNIQL_OK) return rc;
     }
   }

@@ -84,6 +84,11 @@ __global__ void embed_kernel(const uint8_t* __restrict__ packed, const __half* _
 // kernels read activations in 16-byte units, which blocks of 108 or 84 channels (multiples of 4) do not give.
 // One thread per 8 output channels (16 bytes) of one or more rows; x needs 2-byte alignment only.  F16: bf16 activations on
 // their way to the tensor cores become fp16 here instead of in a pass of their own.
+// late: the next launch comes in behind this one's wait.  For the batch kernel (two blocks per SM): let in at entry, its blocks took
+// the places that the launch in front freed one by one, two to an SM with other SMs empty (Qwen2.5-7B layer in bf16 at 34 rows, keep
+// 0.65, 72.5 -> 67.9 us with the conversion on the way).  Not so in front of block pairs (677 rows 254.7 against 257.1 us), nor for the
+// copy of plain bf16 activations (x_to_f16_kernel: 17 rows, keep 1, 72.7 against 75.4 us; ahead only at 100 rows, keep 0.65, 91.8
+// against 83.5 us for the Llama-3-8B layer).
 template <bool F16>
 __global__ void __launch_bounds__(128) relay_x_kernel(const unsigned short* __restrict__ x, long long ldx, int M, int count, int keep,
                                                       int keep8, unsigned short* __restrict__ out, int ldo, int late) {
