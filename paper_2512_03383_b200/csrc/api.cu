@@ -155,8 +155,12 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
   // every batch the decode kernel does not take (more than 16 rows) goes to the tensor cores when the maps
   // allow it: at 17..63 rows the generic kernel measured 13 to 26 times slower (930 us against 71 us for the
   // Llama-3-8B gate|up at M = 17)
-  // (fp16 up to 128 rows: the batch kernel also takes heads that keep 4 (mod 8) channels)
-  auto on_tensor_cores = [](const Params& a) { return prefill_supported(a) != 0 || (a.dt == UNIQL_F16 && batch_supported(a) != 0); };
+  // (fp16 up to 128 rows: the batch kernel also takes heads that keep 4 (mod 8) channels, where the workspace has its header: such a
+  //  call is re-laid with more room and ran on the generic kernel, which needs none, with less)
+  auto on_tensor_cores = [&](const Params& a) {
+    return prefill_supported(a) != 0 || (a.dt == UNIQL_F16 && batch_supported(a) != 0 &&
+                                         (!cfg.workspace || cfg.ws_bytes >= decode_workspace_header_bytes()));
+  };
   bool pre_ok = on_tensor_cores(p);
   // The streaming kernel (one to four rows): where it is asked for, and where the decode kernel's integer path cannot run
   // (scales on 8- but not 16-byte boundaries).

@@ -104,6 +104,23 @@ def test_workspace_without_room_still_correct(B):
         check_output(y2, ref, "f16", 5e-4, "full workspace M=%d" % M)
 
 
+@pytest.mark.parametrize("M", [17, 128])
+@pytest.mark.parametrize("nbytes", [1024, (1 << 18) + 255])
+def test_workspace_smaller_than_its_header_is_no_reason_to_refuse(B, M, nbytes):
+    """Heads that keep 4 (mod 8) channels above 16 rows: read in place by the batch kernel, whose launch wants the header of the
+    workspace; with less the generic kernel, which needs no workspace, takes the call."""
+    rng = np.random.default_rng(870 + M)
+    qw = synth.draw_qweight(rng, 96, 1024)
+    packed, wp, ws, wz = dev_weight(qw)
+    in_map = synth.map_per_head(8, 128, 108)
+    x = synth.draw_x(rng, M, 8 * 108, "f16")
+    small = torch.zeros(nbytes, dtype=torch.uint8, device="cuda")
+    y = torch.full((M, 96), -77.0, device="cuda", dtype=torch.float16)
+    B.qlinear_ex(dev_x(x, "f16"), 8 * 108, wp, ws, wz, None, M, 1024, 96, in_map, 0, None, 96, y, 96, workspace=small)
+    ref = oracle.qlinear(x, packed, qw.scales, qw.zeros, oracle.leading(96), oracle.expand_map(in_map))
+    check_output(y, ref, "f16", TOL["decode"], "workspace of %d bytes M=%d" % (nbytes, M))
+
+
 @pytest.mark.parametrize("M", [1, 7, 16])
 def test_fp16_mma_path_of_the_decode_kernel(B, M):
     """The second arithmetic path of the persistent decode kernel (fp16 MMAs on exact fp16 operands), switched on for
