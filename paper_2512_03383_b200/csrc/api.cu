@@ -320,9 +320,8 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
 
 // bf16 at decode sizes ran on the tensor-core kernel until the decode kernel took that type (Qwen2.5-7B layer at two
 // rows: 146 us), and it still does where the caller's workspace holds that kernel's scratch but not the decode kernel's.
-int dispatch(const Params& p, void* workspace, size_t ws_bytes, void* stream) {
+int dispatch(const Params& p, void* workspace, size_t ws_bytes, void* stream, int path = g_path.load()) {
   if (cudaPeekAtLastError() != cudaSuccess) return UNIQL_ERR_CUDA;
-  const int path = g_path.load();
   const int rc = dispatch_as(p, path, workspace, ws_bytes, stream);
   if (rc == UNIQL_ERR_WORKSPACE && path == UNIQL_PATH_AUTO && p.dt != UNIQL_F16 && p.M <= 16)
     return dispatch_as(p, UNIQL_PATH_PREFILL, workspace, ws_bytes, stream);
@@ -596,6 +595,8 @@ int mlp_tensor_core(const void* x, int ldx, int dt, const uint8_t* wg, const voi
   // the kept blocks converted on their way, 77.3 -> 72.0 us).  Where there is room beside everything that the two launches may use.
   // Not above 128 rows: there the second store of every output cost the gated launch what the pass takes (Qwen2.5-7B at 2048
   // rows 730 -> 744 us, at 677 336 -> 339 us).
+  // (path and option are read here once for both launches: a switch set by another thread in between must not send the down
+  //  projection to a copy that was not written, nor the copy to a kernel that takes it for bf16)
   const int ld16 = (k_int + 63) / 64 * 64, path = g_path.load();
   const size_t h16_bytes = ((size_t)M * ld16 * 2 + 255) & ~(size_t)255;
   const bool h16 = dt == UNIQL_BF16 && M > 16 && batch_supported(a) && (path == UNIQL_PATH_AUTO || path == UNIQL_PATH_PREFILL) &&
@@ -607,7 +608,7 @@ int mlp_tensor_core(const void* x, int ldx, int dt, const uint8_t* wg, const voi
     a.job[0].ld16 = ld16;
   }
   if (!prefill_supported(a) || (M <= 16 && dt == UNIQL_F16 && !exact_batch(a))) return UNIQL_ERR_UNSUPPORTED;   // (nothing launched)
-  int rc = launch_prefill(a, cfg);
+  int rc = h16 ? launch_batch(a, cfg) : launch_prefill(a, cfg);
   if (rc != UNIQL_OK) return rc;
   Params b;
   memset(&b, 0, sizeof(b));
@@ -619,7 +620,7 @@ int mlp_tensor_core(const void* x, int ldx, int dt, const uint8_t* wg, const voi
   compile_map(nullptr, hidden, hidden, &jd.omap);
   jd.w = wd; jd.scales = (const __half*)sd; jd.zeros = (const __half*)zd;
   jd.y = y; jd.ldy = ldy; jd.N = hidden; jd.k_out = hidden;
-  return dispatch(b, cfg.workspace, cfg.ws_bytes, cfg.stream);
+  return dispatch(b, cfg.workspace, cfg.ws_bytes, cfg.stream, path);
 }
 
 }  // namespace

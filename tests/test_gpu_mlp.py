@@ -146,6 +146,58 @@ def test_forced_decode_path_keeps_both_products(B, small, M):
     assert B.workspace_status() == 0 and torch.equal(y, y2), "the down projection left the decode kernel"
 
 
+SWITCH_C = """
+int run(int (*set_option)(const char*, int), int (*set_path)(int), const char* name, volatile int* stop) {
+  int i = 0;
+  while (!*stop) { i ^= 1; if (name) set_option(name, i); else set_path(i); }
+  return i;
+}
+"""
+
+
+@pytest.mark.parametrize("name", [b"prefill_convert", None])
+def test_switches_set_by_another_thread(B, small, name, tmp_path):
+    """bf16 above 16 rows leaves h as fp16 for the down projection.  An option (or, None, the path) that another thread switches
+    while calls are being made changes which kernels run, never the result: 1500 calls on four inputs in turn, each against
+    the result without the other thread.  Two kernels differ by the rounding of h (see test_typed_entry_point) and of the output:
+    1e-2 of the largest output, where another input's h is off by all of it."""
+    import ctypes
+    import subprocess
+    import threading
+    (tmp_path / "switch.c").write_text(SWITCH_C)           # (a native loop: it runs while this thread holds the interpreter)
+    subprocess.check_call(["gcc", "-O1", "-shared", "-fPIC", "-o", str(tmp_path / "switch.so"), str(tmp_path / "switch.c")])
+    switch = ctypes.CDLL(str(tmp_path / "switch.so")).run
+    _, (qg, _, _), ((_, wg, sg, zg), (_, wu, su, zu), (_, wd, sd, zd)) = small
+    M, hidden, inter, k_int, n = 64, 512, 1024, 872, 1500
+    lib, vp = B.lib(), lambda t: ctypes.c_void_p(t.data_ptr())
+    xs = [dev_x(synth.draw_x(np.random.default_rng(600 + i), M, hidden, "bf16"), "bf16") for i in range(4)]
+    h = torch.zeros((M, k_int), device="cuda", dtype=torch.bfloat16)
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+
+    def call(x, y):                                        # (through ctypes: the other thread runs during the call)
+        assert lib.uniql_mlp_swiglu(vp(x), hidden, 1, vp(wg), vp(sg), vp(zg), vp(wu), vp(su), vp(zu), vp(wd), vp(sd), vp(zd), M, hidden,
+                                    inter, k_int, vp(h), k_int, vp(y), hidden, None, 0, stream) == 0
+
+    ref = torch.zeros((4, M, hidden), device="cuda", dtype=torch.bfloat16)
+    for i in range(4):
+        call(xs[i], ref[i])
+    y = torch.zeros((n, M, hidden), device="cuda", dtype=torch.bfloat16)
+    rows, stop = [y[i] for i in range(n)], ctypes.c_int(0)
+    t = threading.Thread(target=switch, args=(lib.uniql_set_option, lib.uniql_set_path, name, ctypes.byref(stop)))
+    t.start()
+    try:
+        for i in range(n):
+            call(xs[i % 4], rows[i])
+    finally:
+        stop.value = 1
+        t.join()
+        B.set_path(B.PATH_AUTO)
+        B.reset_options()
+    torch.cuda.synchronize()
+    err = (y.view(-1, 4, M, hidden).float() - ref.float()).abs().amax(dim=(2, 3)) / ref.float().abs().amax(dim=(1, 2))
+    assert float(err.max()) <= 1e-2, "%d of %d calls off by up to %.2g" % (int((err > 1e-2).sum()), n, float(err.max()))
+
+
 def test_repeated_calls_own_workspace_and_bitwise_repeatability(B, small):
     _, qs, ds = small
     x = synth.draw_x(np.random.default_rng(7), 2, 512, "f16")
