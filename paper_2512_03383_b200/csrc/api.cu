@@ -243,7 +243,8 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
         int rc = lib_workspace(&cfg.workspace, &cfg.ws_bytes, cfg.stream);
         if (rc != UNIQL_OK) return rc;
       }
-      const size_t own = dec ? decode_workspace_bytes(p.M, p.K + kGroup, n_total) : prefill_workspace_bytes(p.M, p.K);
+      const bool copy_x = p.dt == UNIQL_BF16 && !p.x_f16;
+      const size_t own = dec ? decode_workspace_bytes(p.M, p.K + kGroup, n_total) : batch_workspace_bytes(p.M, copy_x ? p.k_in : 0);
       if (cfg.ws_bytes >= at[p.n_jobs] + own + 256) {
         LaunchCfg dc = cfg;
         dc.ws_bytes = (cfg.ws_bytes - at[p.n_jobs]) & ~(size_t)255;
@@ -627,9 +628,12 @@ int mlp_tensor_core(const void* x, int ldx, int dt, const uint8_t* wg, const voi
 
 extern "C" size_t uniql_mlp_workspace_bytes(int M, int hidden, int inter) {
   if (M < 1 || hidden < 1 || inter < 1) return 0;
+  // (an odd number of groups: the down projection's copy of the scales and zero-points, see dispatch_as())
+  const int G = (inter + kGroup - 1) / kGroup;
+  const size_t pad = G % 2 != 0 && M <= 128 ? (size_t)hidden * ((G + 7) / 8 * 8) * 4 + 768 : 0;
   // tensor-core kernel, two launches (+ up to 128 rows the fp16 copies of both activations of bf16 at once)
   if (M > 16)
-    return prefill_workspace_bytes(M, hidden > inter ? hidden : inter) +
+    return prefill_workspace_bytes(M, hidden > inter ? hidden : inter) + pad +
            (M <= 128 ? (size_t)M * (((hidden < inter ? hidden : inter) + 63) / 64 * 64) * 2 + 512 : 0);
   // (16 rows or fewer in bf16 also run on the tensor-core kernel: room for its fp16 copy of the activations)
   const size_t a = mlp_decode_workspace_bytes(M, hidden, inter), b = prefill_workspace_bytes(M, hidden > inter ? hidden : inter);
@@ -637,6 +641,10 @@ extern "C" size_t uniql_mlp_workspace_bytes(int M, int hidden, int inter) {
   if (M <= 4) {
     const size_t c0 = gemv_workspace_bytes(M, hidden, 2 * inter), c1 = gemv_workspace_bytes(M, inter, hidden);
     c = c0 > c1 ? c0 : c1;
+  }
+  if (pad) {
+    const size_t down = decode_workspace_bytes(M, inter + kGroup, hidden) + pad;
+    c = c > down ? c : down;
   }
   return a > b ? (a > c ? a : c) : (b > c ? b : c);
 }

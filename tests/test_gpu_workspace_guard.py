@@ -121,3 +121,39 @@ def test_advertised_workspace_gives_the_bits_of_the_librarys_own(B, M, dtype):
             B.qlinear_ex(x, K, *dw[1:], None, M, K, N, None, K, None, N, out, N, workspace=w)
         assert band_intact(buf, nbytes) and B.workspace_status(ws) == 0
         assert torch.equal(y[0], y[1]), "M=%d %s %s" % (M, dtype, (N, K))
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("M", [3, 8, 16, 17, 40, 128])
+@pytest.mark.parametrize("hidden,inter,k_int", [(2048, 1152, 1152), (2048, 1152, 872), (512, 2176, 1160), (512, 3200, 8), (896, 4864, 4864), (512, 1024, 870)])
+def test_mlp_block_of_odd_widths_in_the_advertised_workspace(B, M, dtype, hidden, inter, k_int):
+    """Widths of an odd number of groups (the down projection on a copy of its scales at the end of the workspace) and the fp16
+    copy of h beside it: nothing is written behind the advertised workspace, and it has room for what the library's own buffer
+    gives, bit for bit.  What the block refuses, it refuses in both."""
+    rng = np.random.default_rng(M + inter + k_int)
+    qg, qu, qd = (synth.random_qweight_fast(rng, n, k) for n, k in ((inter, hidden), (inter, hidden), (hidden, inter)))
+    dg, du, dd = (dev_weight(q) for q in (qg, qu, qd))
+    x = synth.draw_x(rng, M, hidden, dtype)
+    xd = dev_x(x, dtype)
+    nbytes = B.mlp_workspace_bytes(M, hidden, inter)
+    buf, ws = guarded(B, nbytes)
+    ldh = k_int + (-k_int) % 8
+    outs = []
+    for w in (None, ws):
+        h, y = (torch.zeros((M, n), dtype=xd.dtype, device="cuda") for n in (ldh, hidden))
+        try:
+            B.mlp_swiglu(xd, hidden, *dg[1:], *du[1:], *dd[1:], M, hidden, inter, k_int, h, ldh, y, hidden, workspace=w)
+            outs.append((h, y))
+        except RuntimeError as e:
+            assert "unsupported" in str(e)
+            outs.append(None)
+    assert band_intact(buf, nbytes) and B.workspace_status(ws) == 0
+    if outs[0] is None:                                    # (fp16 at decode sizes: widths that are multiples of 256, k_int of 8)
+        assert outs[1] is None and dtype == "f16" and M <= 16 and (hidden % 256 or inter % 256 or k_int % 8)
+        return
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    rows = sorted(set(rng.integers(0, hidden, 32).tolist() + [0, hidden - 1]))
+    h_ref, y_ref = oracle.mlp_swiglu(x, dg[0], qg.scales, qg.zeros, du[0], qu.scales, qu.zeros, dd[0], qd.scales, qd.zeros, k_int,
+                                     out_rows=rows, h_dtype=dtype)
+    check_output(outs[0][0][:, :k_int], h_ref, dtype, 6e-4, "h")
+    check_output(outs[0][1][:, torch.as_tensor(rows, device="cuda")], y_ref, dtype, TOL_Y if dtype == "f16" else 2e-3, "y")
