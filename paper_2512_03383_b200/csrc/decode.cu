@@ -940,70 +940,76 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
       }
       // U units of eight activations per thread, 16 / U lanes per (row, group).  Lane l takes the units l, l + 16 / U, ... of
       // its group's sixteen (consecutive 16 bytes of x from lane to lane), the U groups of a half-warp beginning at different
-      // ones: their 8-byte stores, 128 bytes apart from group to group, then hit distinct banks.  UN: threads' worth in flight.
-      auto quantise = [&](auto units, auto in_flight) {
-        constexpr int U = decltype(units)::value, UN = decltype(in_flight)::value, LG = 16 / U;
+      // ones: their 8-byte stores, 128 bytes apart from group to group, then hit distinct banks.  halves: blocks on 4-channel
+      // boundaries, every unit loaded in two halves.
+      auto quantise = [&](auto units, auto halves) {
+        constexpr int U = decltype(units)::value, LG = 16 / U;
         const int l = lane & (LG - 1), rot = (lane / LG) & (U - 1);
         const int n = my_pairs * LG, n32 = (n + 31) & ~31;
-        for (int u0 = ctid; u0 < n32; u0 += CTH * UN) {
-          uint4 in[UN][U];
-          int lvs[UN], row[UN];
+        for (int u = ctid; u < n32; u += CTH) {                      // (whole warps stay in the shuffles)
+          uint4 in[U];
+          int lv = -1, m = 0;
 #pragma unroll
-          for (int j = 0; j < UN; ++j) {
-            const int u = u0 + j * CTH;
-            lvs[j] = -1; row[j] = 0;
+          for (int k = 0; k < U; ++k) in[k] = make_uint4(0, 0, 0, 0);
+          if (u < n) {
+            const int pair = ((u / LG) << csh) + crank, row = row_of(pair), group = needed_group(pair - row * Gn);
+            if (group < Gk) {
+              lv = group; m = row;
+              const T* xrow = x + (size_t)m * ldx;
 #pragma unroll
-            for (int k = 0; k < U; ++k) in[j][k] = make_uint4(0, 0, 0, 0);
-            if (u < n) {
-              const int pair = ((u / LG) << csh) + crank, m = row_of(pair), lv = needed_group(pair - m * Gn);
-              if (lv < Gk) {
-                lvs[j] = lv; row[j] = m;
-                const T* xrow = x + (size_t)m * ldx;
-#pragma unroll
-                for (int k = 0; k < U; ++k) {
-                  const int ch = (sg_lo + lv) * kGroup + 8 * (l + LG * ((k + rot) & (U - 1)));
-                  if (NPH == 1 && NT != 2 && P.x4) {
-                    in[j][k] = load_halves(xrow, ch, compact_of);
-                  } else {
-                    const int t0 = compact_of(ch);
-                    if (t0 >= 0) in[j][k] = load16(xrow + t0);
-                  }
+              for (int k = 0; k < U; ++k) {
+                const int ch = (sg_lo + lv) * kGroup + 8 * (l + LG * ((k + rot) & (U - 1)));
+                if constexpr (decltype(halves)::value) {
+                  in[k] = load_halves(xrow, ch, compact_of);
+                } else {
+                  const int t0 = compact_of(ch);
+                  if (t0 >= 0) in[k] = load16(xrow + t0);
                 }
               }
             }
           }
+          uint2 hi[U], lo[U];
+          int isum;
+          float inv_scale;
+          quantise_units<T, U>(in, hi, lo, isum, inv_scale);
+          if (lv >= 0) {
+            // unit c'*4 + i (word i of lane quarter c'): 8 bytes at c'*32 + i*8 of the group's 128 bytes
+            const int at = (2 * m) * c.xrow + lv * 128 + l * 8;
 #pragma unroll
-          for (int j = 0; j < UN; ++j) {
-            if (u0 + j * CTH >= n32) break;                          // warp-uniform
-            uint2 hi[U], lo[U];
-            int isum;
-            float inv_scale;
-            quantise_units<T, U>(in[j], hi, lo, isum, inv_scale);
-            if (lvs[j] >= 0) {
-              // unit c'*4 + i (word i of lane quarter c'): 8 bytes at c'*32 + i*8 of the group's 128 bytes
-              const int m = row[j], at = (2 * m) * c.xrow + lvs[j] * 128 + l * 8;
-#pragma unroll
-              for (int k = 0; k < U; ++k) {
-                const int o = at + ((k + rot) & (U - 1)) * (LG * 8);
-                *reinterpret_cast<uint2*>(xb + o) = hi[k];
-                *reinterpret_cast<uint2*>(xb + o + c.xrow) = lo[k];
-                if (xc) {
-                  st_peer_v2(px + (uint32_t)o, hi[k].x, hi[k].y);
-                  st_peer_v2(px + (uint32_t)(o + c.xrow), lo[k].x, lo[k].y);
-                }
+            for (int k = 0; k < U; ++k) {
+              const int o = at + ((k + rot) & (U - 1)) * (LG * 8);
+              *reinterpret_cast<uint2*>(xb + o) = hi[k];
+              *reinterpret_cast<uint2*>(xb + o + c.xrow) = lo[k];
+              if (xc) {
+                st_peer_v2(px + (uint32_t)o, hi[k].x, hi[k].y);
+                st_peer_v2(px + (uint32_t)(o + c.xrow), lo[k].x, lo[k].y);
               }
-              if (l == 0) {
-                xg[lvs[j] * 8 * MT + m] = make_float2((float)isum, inv_scale);
-                if (xc) st_peer_v2(pxg + (uint32_t)((lvs[j] * 8 * MT + m) * 8), (uint32_t)__float_as_int((float)isum), (uint32_t)__float_as_int(inv_scale));
-              }
+            }
+            if (l == 0) {
+              xg[lv * 8 * MT + m] = make_float2((float)isum, inv_scale);
+              if (xc) st_peer_v2(pxg + (uint32_t)((lv * 8 * MT + m) * 8), (uint32_t)__float_as_int((float)isum), (uint32_t)__float_as_int(inv_scale));
             }
           }
         }
       };
+      // The fewest units per lane with which the block's threads take every pair at once: a lane's chain is the longer the more
+      // it has (2560 x 4096 at two rows, 64 pairs, one / two / four units: 5.35 / 4.91 / 5.43 us; 2560 x 2560 at one row, 20 pairs,
+      // one / two 4.27 / 4.60 us), and beyond two the issue slots count.  The loads in halves are forms of their own, which need few
+      // pairs: as a branch inside the one with four units they cost every launch of the instance (with two threads' worth in
+      // flight there: Mamba2-2.7B mixer at one row 12.14 -> 11.81 us, Qwen2.5-7B layer in bf16 at two rows, keep 0.85, 47.3 -> 44.6 us).
       using std::integral_constant;
-      if (my_pairs * 16 <= CTH) quantise(integral_constant<int, 1>(), integral_constant<int, 1>());
-      else if (my_pairs * 32 <= 3 * CTH) quantise(integral_constant<int, 2>(), integral_constant<int, 1>());
-      else quantise(integral_constant<int, 4>(), integral_constant<int, 2>());
+      using std::true_type;
+      using std::false_type;
+      if (NPH == 1 && NT != 2 && P.x4) {
+        if (my_pairs * 16 <= CTH) quantise(integral_constant<int, 1>(), true_type());
+        else quantise(integral_constant<int, 2>(), true_type());
+      } else if (my_pairs * 16 <= CTH) {
+        quantise(integral_constant<int, 1>(), false_type());
+      } else if (my_pairs * 8 <= CTH) {
+        quantise(integral_constant<int, 2>(), false_type());
+      } else {
+        quantise(integral_constant<int, 4>(), false_type());
+      }
       if (xc) {
         // both halves are in place once the sixteen consumer warps of each block have arrived at this block's
         // barrier (bounded wait; the other block cannot leave before it has seen this block's arrivals, and this

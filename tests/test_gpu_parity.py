@@ -576,3 +576,25 @@ def test_odd_number_of_groups(B, M, N, K, k_in, k_out, dtype):
     y2, _ = run_ex(B, qw, dw, x, dtype, None, k_in, None, k_out, bias=bias, ldx_pad=-k_in % 8, ldy_pad=1, workspace=big)
     assert torch.equal(y, y2)
     assert B.workspace_status(big) == 0 and B.workspace_status() == 0
+
+
+# Llama-size rows: every block stages all (row, group) pairs, 32 / 33 .. 64 / 65 and more of them (one, two or four units of eight
+# channels per lane, several passes of the block's threads), on 8- and on 4-channel boundaries.
+@pytest.mark.parametrize("M,K", [(1, 4096), (1, 4352), (1, 8192), (1, 8448), (2, 2048), (2, 2304), (2, 4096), (2, 4352), (3, 2560), (3, 2816),
+                                 (4, 1024), (4, 1280), (4, 2048), (4, 4352), (5, 768), (7, 1280), (8, 512), (8, 1024), (8, 2304)])
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+def test_staging_of_every_number_of_pairs(B, M, K, dtype):
+    N = 64 * 150
+    rng = np.random.default_rng(10 * K + M)
+    qw = synth.random_qweight_fast(rng, N, K)
+    packed, wp, ws, wz = dev_weight(qw)
+    rows = sorted(set(rng.integers(0, N, 40).tolist() + [0, 63, N - 1]))
+    B.set_path(B.PATH_DECODE)
+    for in_map in (None, synth.map_per_head(K // 128, 128, 108), synth.map_per_head(K // 64, 64, 52)):
+        k_in = synth.map_size(in_map) if in_map else K
+        x = synth.draw_x(rng, M, k_in, dtype)
+        y = torch.zeros((M, N), dtype=torch.float16 if dtype == "f16" else torch.bfloat16, device="cuda")
+        B.qlinear_ex(dev_x(x, dtype), k_in, wp, ws, wz, None, M, K, N, in_map, k_in if in_map is None else 0, None, N, y, N)
+        ref = oracle.qlinear(x, packed, qw.scales, qw.zeros, rows, oracle.expand_map(in_map) if in_map else oracle.leading(K))
+        check_output(y[:, torch.as_tensor(rows, device="cuda")], ref, dtype, TIGHT, "M=%d K=%d %s" % (M, K, in_map and in_map[0]))
+    assert B.workspace_status() == 0
