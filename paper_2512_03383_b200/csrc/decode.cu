@@ -455,11 +455,11 @@ __device__ inline void store_tile(const Params& p, const TileFam& f, const TileP
 // units into n_rp equal ranges (stream-K) balances the bytes but every tile then ends with a hand-over
 // between blocks (park, arrival count, reduction by the last block: about the time of three chunks);
 // when that costs more than it saves, the left-over tiles are given whole to R blocks instead.
+__host__ __device__ inline bool tail_split(int n_rp, int R, int Cq) { return R * Cq / n_rp + 3 < Cq; }
 __host__ __device__ inline int tail_blocks(int n_rp, int R, int Cq) {
   const int Ut = R * Cq;
   if (Ut == 0) return 1;
-  const bool split = Ut / n_rp + 3 < Cq;
-  const int Bt = split ? n_rp : R;
+  const int Bt = tail_split(n_rp, R, Cq) ? n_rp : R;
   return Bt < Ut ? Bt : Ut;
 }
 
@@ -941,53 +941,62 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
       // U units of eight activations per thread, 16 / U lanes per (row, group).  Lane l takes the units l, l + 16 / U, ... of
       // its group's sixteen (consecutive 16 bytes of x from lane to lane), the U groups of a half-warp beginning at different
       // ones: their 8-byte stores, 128 bytes apart from group to group, then hit distinct banks.  halves: blocks on 4-channel
-      // boundaries, every unit loaded in two halves.
-      auto quantise = [&](auto units, auto halves) {
-        constexpr int U = decltype(units)::value, LG = 16 / U;
+      // boundaries, every unit loaded in two halves.  in_flight: threads' worth of loads before the first is used.
+      auto quantise = [&](auto units, auto in_flight, auto halves) {
+        constexpr int U = decltype(units)::value, UN = decltype(in_flight)::value, LG = 16 / U;
         const int l = lane & (LG - 1), rot = (lane / LG) & (U - 1);
         const int n = my_pairs * LG, n32 = (n + 31) & ~31;
-        for (int u = ctid; u < n32; u += CTH) {                      // (whole warps stay in the shuffles)
-          uint4 in[U];
-          int lv = -1, m = 0;
+        for (int u0 = ctid; u0 < n32; u0 += CTH * UN) {              // (whole warps stay in the shuffles)
+          uint4 in[UN][U];
+          int lvs[UN], row[UN];
 #pragma unroll
-          for (int k = 0; k < U; ++k) in[k] = make_uint4(0, 0, 0, 0);
-          if (u < n) {
-            const int pair = ((u / LG) << csh) + crank, row = row_of(pair), group = needed_group(pair - row * Gn);
-            if (group < Gk) {
-              lv = group; m = row;
-              const T* xrow = x + (size_t)m * ldx;
+          for (int j = 0; j < UN; ++j) {
+            const int u = u0 + j * CTH;
+            lvs[j] = -1; row[j] = 0;
 #pragma unroll
-              for (int k = 0; k < U; ++k) {
-                const int ch = (sg_lo + lv) * kGroup + 8 * (l + LG * ((k + rot) & (U - 1)));
-                if constexpr (decltype(halves)::value) {
-                  in[k] = load_halves(xrow, ch, compact_of);
-                } else {
-                  const int t0 = compact_of(ch);
-                  if (t0 >= 0) in[k] = load16(xrow + t0);
+            for (int k = 0; k < U; ++k) in[j][k] = make_uint4(0, 0, 0, 0);
+            if (u < n) {
+              const int pair = ((u / LG) << csh) + crank, m = row_of(pair), lv = needed_group(pair - m * Gn);
+              if (lv < Gk) {
+                lvs[j] = lv; row[j] = m;
+                const T* xrow = x + (size_t)m * ldx;
+#pragma unroll
+                for (int k = 0; k < U; ++k) {
+                  const int ch = (sg_lo + lv) * kGroup + 8 * (l + LG * ((k + rot) & (U - 1)));
+                  if constexpr (decltype(halves)::value) {
+                    in[j][k] = load_halves(xrow, ch, compact_of);
+                  } else {
+                    const int t0 = compact_of(ch);
+                    if (t0 >= 0) in[j][k] = load16(xrow + t0);
+                  }
                 }
               }
             }
           }
-          uint2 hi[U], lo[U];
-          int isum;
-          float inv_scale;
-          quantise_units<T, U>(in, hi, lo, isum, inv_scale);
-          if (lv >= 0) {
-            // unit c'*4 + i (word i of lane quarter c'): 8 bytes at c'*32 + i*8 of the group's 128 bytes
-            const int at = (2 * m) * c.xrow + lv * 128 + l * 8;
 #pragma unroll
-            for (int k = 0; k < U; ++k) {
-              const int o = at + ((k + rot) & (U - 1)) * (LG * 8);
-              *reinterpret_cast<uint2*>(xb + o) = hi[k];
-              *reinterpret_cast<uint2*>(xb + o + c.xrow) = lo[k];
-              if (xc) {
-                st_peer_v2(px + (uint32_t)o, hi[k].x, hi[k].y);
-                st_peer_v2(px + (uint32_t)(o + c.xrow), lo[k].x, lo[k].y);
+          for (int j = 0; j < UN; ++j) {
+            if (UN > 1 && u0 + j * CTH >= n32) break;                // warp-uniform
+            uint2 hi[U], lo[U];
+            int isum;
+            float inv_scale;
+            quantise_units<T, U>(in[j], hi, lo, isum, inv_scale);
+            if (lvs[j] >= 0) {
+              // unit c'*4 + i (word i of lane quarter c'): 8 bytes at c'*32 + i*8 of the group's 128 bytes
+              const int m = row[j], at = (2 * m) * c.xrow + lvs[j] * 128 + l * 8;
+#pragma unroll
+              for (int k = 0; k < U; ++k) {
+                const int o = at + ((k + rot) & (U - 1)) * (LG * 8);
+                *reinterpret_cast<uint2*>(xb + o) = hi[k];
+                *reinterpret_cast<uint2*>(xb + o + c.xrow) = lo[k];
+                if (xc) {
+                  st_peer_v2(px + (uint32_t)o, hi[k].x, hi[k].y);
+                  st_peer_v2(px + (uint32_t)(o + c.xrow), lo[k].x, lo[k].y);
+                }
               }
-            }
-            if (l == 0) {
-              xg[lv * 8 * MT + m] = make_float2((float)isum, inv_scale);
-              if (xc) st_peer_v2(pxg + (uint32_t)((lv * 8 * MT + m) * 8), (uint32_t)__float_as_int((float)isum), (uint32_t)__float_as_int(inv_scale));
+              if (l == 0) {
+                xg[lvs[j] * 8 * MT + m] = make_float2((float)isum, inv_scale);
+                if (xc) st_peer_v2(pxg + (uint32_t)((lvs[j] * 8 * MT + m) * 8), (uint32_t)__float_as_int((float)isum), (uint32_t)__float_as_int(inv_scale));
+              }
             }
           }
         }
@@ -1001,14 +1010,14 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
       using std::true_type;
       using std::false_type;
       if (NPH == 1 && NT != 2 && P.x4) {
-        if (my_pairs * 16 <= CTH) quantise(integral_constant<int, 1>(), true_type());
-        else quantise(integral_constant<int, 2>(), true_type());
+        if (my_pairs * 16 <= CTH) quantise(integral_constant<int, 1>(), integral_constant<int, 1>(), true_type());
+        else quantise(integral_constant<int, 2>(), integral_constant<int, 1>(), true_type());
       } else if (my_pairs * 16 <= CTH) {
-        quantise(integral_constant<int, 1>(), false_type());
+        quantise(integral_constant<int, 1>(), integral_constant<int, 1>(), false_type());
       } else if (my_pairs * 8 <= CTH) {
-        quantise(integral_constant<int, 2>(), false_type());
+        quantise(integral_constant<int, 2>(), integral_constant<int, 1>(), false_type());
       } else {
-        quantise(integral_constant<int, 4>(), false_type());
+        quantise(integral_constant<int, 4>(), integral_constant<int, NT == 2 ? 2 : 1>(), false_type());
       }
       if (xc) {
         // both halves are in place once the sixteen consumer warps of each block have arrived at this block's
@@ -1665,9 +1674,17 @@ void visited_range(const ChanMap& m, int gran, int* first, int* total) {
 
 // Split of the visited groups into k-parts and the shared-memory plan: as few k-parts as let the staged
 // activations fit beside a deep enough ring of stages.  Returns 0 when nothing fits.
-// A fourth stage before the second buffer of parked sums (one_buf): the bytes in flight are what a launch streams with, while
-// the epilogue warps drain a buffer in a fraction of a tile's time.
-size_t plan_split(DecodeCfg* c, int M, int g_total, int gran, bool i8, bool one_buf = true) {
+// Up to eight rows the parked sums have two buffers.  One of them is given up
+//  - for a fourth stage: the bytes in flight are what a launch streams with, while the epilogue warps drain a buffer in a fraction
+//    of a tile's time (lm_head at eight rows 69.8 -> 66.9 us, 1 - 3 % at 60 sizes from 148 to 2004 tiles).  Not from six rows on
+//    where blocks have two or more whole tiles and the left-over ones are split (`tiles` 64-row tiles): what the one buffer holds
+//    up then stands in front of the hand-over (7 x 4608 and 8 x 4096, 300, 448 and 596 tiles: 2.1 us, 5 - 15 %, at every split size).
+//    (Where every block ends on a whole tile the last drain stands behind the one before it: 8 x 4096, 148 tiles, launched alone
+//    11.5 -> 11.8 us.  Two buffers there, and wherever more than half of the blocks end so, cost a Bamba-v2-9B mixer at eight rows 33.5 ->
+//    34.8 us.)
+//  - fewer: also for three stages where two buffers would take a k-part more (4 x 13312, 64 tiles 14.8 -> 13.3 us; SwiGLU block of
+//    6144 x 16384 at eight rows 76.8 -> 58.9 us).
+size_t plan_split(DecodeCfg* c, int M, int g_total, int gran, bool i8, int tiles, bool fewer) {
   const int MT = M <= 8 ? 1 : 2;
   const int part_bufs = M <= 8 ? 2 : 1;
   int n_kp = opt(kOptDecodeKp);
@@ -1675,6 +1692,10 @@ size_t plan_split(DecodeCfg* c, int M, int g_total, int gran, bool i8, bool one_
   const int want = (stages >= 2 && stages <= MAX_STAGES) ? stages : 4;
   size_t smem = 0;
   bool fits = false;
+  auto blocks_per_part = [](int parts) {
+    const int n_rp = opt(kOptDecodeRp) < 1 ? sm_count() / parts : opt(kOptDecodeRp);
+    return n_rp < 1 ? 1 : n_rp;
+  };
   if (n_kp >= 1) {
     if (n_kp > kMaxKParts) n_kp = kMaxKParts;
     const int gp = round_up((g_total + n_kp - 1) / n_kp, gran);
@@ -1684,23 +1705,26 @@ size_t plan_split(DecodeCfg* c, int M, int g_total, int gran, bool i8, bool one_
     }
     c->gp = gp;
   } else {
-    for (n_kp = 1; n_kp <= kMaxKParts && !fits; ++n_kp)
+    for (n_kp = 1; n_kp <= kMaxKParts && !fits; ++n_kp) {
+      const int gp = round_up((g_total + n_kp - 1) / n_kp, gran), n_rp = blocks_per_part(n_kp);
+      const int whole = tiles / n_rp, left = tiles % n_rp;
+      const bool held_up = M >= 6 && whole >= 2 && left != 0 && tail_split(n_rp, left, (gp + CG - 1) / CG);
+      const bool deeper = tiles > 0 && !held_up;
       for (int s = want; s >= 3 && !fits; --s) {
-        const int gp = round_up((g_total + n_kp - 1) / n_kp, gran);
-        for (int bufs = part_bufs; bufs >= (one_buf ? 1 : part_bufs) && !fits; --bufs) {
+        const int least = (s > 3 ? deeper : fewer) ? 1 : part_bufs;
+        for (int bufs = part_bufs; bufs >= least && !fits; --bufs) {
           smem = plan_smem(c, M, MT, gp, s, bufs, i8);
           fits = smem <= (size_t)kSmemMax;
         }
-        c->gp = gp;
       }
+      c->gp = gp;
+    }
   }
   if (!fits) return 0;
   c->g_total = g_total;
   c->gran = gran;
   c->n_kp = (g_total + c->gp - 1) / c->gp;
-  int n_rp = opt(kOptDecodeRp);
-  if (n_rp < 1) n_rp = sm_count() / c->n_kp;
-  if (n_rp < 1) n_rp = 1;
+  const int n_rp = blocks_per_part(c->n_kp);
   c->n_rp = n_rp;
   // the kernel cuts the left-over units with 32-bit products of at most n_rp * n_rp * (chunks per tile)
   if ((long long)n_rp * n_rp * ((c->gp + CG - 1) / CG) >= (1ll << 31)) return 0;
@@ -1827,7 +1851,7 @@ size_t decode_workspace_bytes(int M, int K, int N_total) {
   DecodeCfg c;
   memset(&c, 0, sizeof(c));
   const int G = (K + kGroup - 1) / kGroup;
-  if (!plan_split(&c, M, G, 2, false, false)) return (size_t)kWsHeader;
+  if (!plan_split(&c, M, G, 2, false, 0, false)) return (size_t)kWsHeader;
   const size_t chunks = (size_t)(G + CG - 1) / CG;
   const size_t tiles = (size_t)(N_total + RB - 1) / RB + (size_t)N_total / 32 + 2 * kMaxJobs;
   const size_t slots = tiles * 2 * c.n_kp + (size_t)c.n_rp * c.n_kp * (chunks + 2 * c.n_kp);
@@ -1862,6 +1886,37 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
   // streamed: their staged copy never fits beside a ring of more than two positions (Llama-3-8B MLP at M = 16:
   // 55 us in one pass, 82 us as two launches of eight rows, 145 us with the input channels split over two groups
   // of blocks).
+  // (From five rows on a plan that stages whole only with a single buffer of parked sums is taken for narrow tiles, which
+  //  streamed launches do not have, and for few tiles: 6 x 8192, 64 tiles streamed 16.7, staged 11.0 us, 16 tiles 9.3 and 8.6; 96 to
+  //  224 tiles 12.8 - 22.9 and 15.0 - 24.7.)
+  bool all_plain = true;
+  long t64 = 0, t32 = 0;
+  for (int j = 0; j < p.n_jobs; ++j) {
+    const JobDev& jb = p.job[j];
+    if (jb.rope.enabled) {
+      all_plain = false;
+      t64 += (long)((jb.rope.head_keep / 2 + RB / 2 - 1) / (RB / 2)) * jb.rope.n_heads;
+      continue;
+    }
+    for (int k = 0; k < jb.omap.n_fam; ++k) {
+      const Fam& a = jb.omap.fam[k];
+      t64 += (long)((a.keep + RB - 1) / RB) * a.count;
+      t32 += (long)((a.keep + RB / 2 - 1) / (RB / 2)) * a.count;
+    }
+  }
+  // Narrow tiles (32 rows x 16 groups) when the schedule they give is shorter: matrices with fewer 64-row tiles than blocks then
+  // run without a hand-over between blocks (UNIQL_DECODE_NARROW=0/1 forces).  Only where there are fewer wide tiles than blocks
+  // and the input channels are not split: measured, the smaller boxes of the narrow tiles cost more than a better balance of
+  // many tiles gains.
+  auto narrow_pays = [&](const DecodeCfg& a) {
+    if (!all_plain || a.x_stream) return false;
+    const int force = opt(kOptDecodeNarrow);
+    if (force == 0 || force == 1) return force == 1;
+    const int Gk0 = g_total < a.gp ? g_total : a.gp;
+    return a.n_kp == 1 && t64 < a.n_rp &&
+           schedule_cost(t32, (Gk0 + 2 * CG - 1) / (2 * CG), a.n_rp) < schedule_cost(t64, (Gk0 + CG - 1) / CG, a.n_rp);
+  };
+  const int n_tiles = t64 < (1 << 24) ? (int)t64 : (1 << 24);
   size_t smem = 0;
   c.stage_bytes = STAGE_BYTES;
   {
@@ -1873,44 +1928,20 @@ int launch_decode(const Params& p, const LaunchCfg& cfg) {
         if (!smem) c.stage_bytes = STAGE_BYTES;
       }
     } else if (i8 && force != 0) {
-      DecodeCfg t = c;
-      const size_t s0 = plan_split(&t, p.M, g_total, gran, true);
-      if (force == 1 || !s0 || (t.n_kp > 1 && p.M >= 5)) {
+      DecodeCfg t = c, b = c;
+      bool staged = plan_split(&t, p.M, g_total, gran, true, n_tiles, true) != 0;
+      if (staged && p.M >= 5)
+        staged = t.n_kp == 1 && ((plan_split(&b, p.M, g_total, gran, true, n_tiles, false) != 0 && b.n_kp == 1) || 2 * t64 <= t.n_rp || narrow_pays(t));
+      if (force == 1 || !staged) {
         smem = plan_stream(&c, p.M, g_total, gran);
         c.x_stream = smem != 0;
         if (!smem) c.stage_bytes = STAGE_BYTES;
       }
     }
   }
-  if (!c.x_stream) smem = plan_split(&c, p.M, g_total, gran, i8);
+  if (!c.x_stream) smem = plan_split(&c, p.M, g_total, gran, i8, n_tiles, true);
   if (!smem) return UNIQL_ERR_UNSUPPORTED;
-
-  // ---- narrow tiles (32 rows x 16 groups) when the schedule they give is shorter: matrices with fewer
-  //      64-row tiles than blocks then run without a hand-over between blocks (UNIQL_DECODE_NARROW=0/1 forces)
-  bool narrow = false;
-  {
-    bool all_plain = true;
-    long t64 = 0, t32 = 0;
-    for (int j = 0; j < p.n_jobs; ++j) {
-      const JobDev& jb = p.job[j];
-      if (jb.rope.enabled) { all_plain = false; continue; }
-      for (int k = 0; k < jb.omap.n_fam; ++k) {
-        const Fam& a = jb.omap.fam[k];
-        t64 += (long)((a.keep + RB - 1) / RB) * a.count;
-        t32 += (long)((a.keep + RB / 2 - 1) / (RB / 2)) * a.count;
-      }
-    }
-    if (all_plain && !c.x_stream) {
-      const int Gk0 = g_total < c.gp ? g_total : c.gp;
-      // (only where there are fewer wide tiles than blocks and the input channels are not split: measured,
-      //  the smaller boxes of the narrow tiles cost more than a better balance of many tiles gains)
-      narrow = c.n_kp == 1 && t64 < c.n_rp &&
-               schedule_cost(t32, (Gk0 + 2 * CG - 1) / (2 * CG), c.n_rp) < schedule_cost(t64, (Gk0 + CG - 1) / CG, c.n_rp);
-      const int force = opt(kOptDecodeNarrow);
-      if (force == 0) narrow = false;
-      if (force == 1) narrow = true;
-    }
-  }
+  const bool narrow = narrow_pays(c);
   c.cgz = narrow ? 2 * CG : CG;
 
   // ---- tile families and their tensor maps
@@ -2079,7 +2110,7 @@ int launch_mlp_phases(const MlpDecode& d, int first, int count, const LaunchCfg&
   c.x_stream = smem != 0;
   if (!smem) {
     c.stage_bytes = STAGE_BYTES;
-    smem = plan_split(&c, d.M, g_max, gran, true);
+    smem = plan_split(&c, d.M, g_max, gran, true, first == 0 ? (d.k_int + RB / 2 - 1) / (RB / 2) : (d.hidden + RB - 1) / RB, true);
   }
   if (!smem) return UNIQL_ERR_UNSUPPORTED;
   if (count > 1 && (c.n_kp != 1 || d.M > 8)) return UNIQL_ERR_UNSUPPORTED;

@@ -598,3 +598,23 @@ def test_staging_of_every_number_of_pairs(B, M, K, dtype):
         ref = oracle.qlinear(x, packed, qw.scales, qw.zeros, rows, oracle.expand_map(in_map) if in_map else oracle.leading(K))
         check_output(y[:, torch.as_tensor(rows, device="cuda")], ref, dtype, TIGHT, "M=%d K=%d %s" % (M, K, in_map and in_map[0]))
     assert B.workspace_status() == 0
+
+
+# Rows that change over between two buffers of parked sums and one, between staged and streamed activations, and between one and two
+# parts of the input channels; tiles: fewer than blocks, whole rounds, and left-over ones that are split or not.
+@pytest.mark.parametrize("M,K", [(2, 19456), (3, 11520), (3, 17920), (4, 8448), (4, 12544), (5, 6400), (5, 10240), (6, 5376), (6, 8192), (7, 4608),
+                                 (7, 5120), (7, 7168), (8, 4096), (8, 4352), (8, 6144)])
+def test_plans_at_their_borders(B, M, K):
+    rng = np.random.default_rng(K + M)
+    qw = synth.random_qweight_fast(rng, 64 * 300 + 8, K)
+    packed, wp, ws, wz = dev_weight(qw)
+    x = synth.draw_x(rng, M, K, "f16")
+    xd = dev_x(x, "f16")
+    B.set_path(B.PATH_DECODE)
+    for N in (200, 64 * 96, 64 * 148, 64 * 300 + 8):
+        rows = sorted(set(rng.integers(0, N, 24).tolist() + [0, N - 1]))
+        y = torch.zeros((M, N), dtype=torch.float16, device="cuda")
+        B.qlinear_ex(xd, K, wp, ws, wz, None, M, K, N, None, K, None, N, y, N)
+        ref = oracle.qlinear(x, packed, qw.scales, qw.zeros, rows, oracle.leading(K))
+        check_output(y[:, torch.as_tensor(rows, device="cuda")], ref, "f16", TIGHT, "M=%d K=%d N=%d" % (M, K, N))
+    assert B.workspace_status() == 0
