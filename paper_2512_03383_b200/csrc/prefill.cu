@@ -60,14 +60,18 @@ struct SegIter {
 
 // bf16 activations -> fp16 copy in the workspace, once per call (every weight tile re-reads the tile of
 // activations, so converting there would repeat the work once per 128 weight rows).
+// Few blocks of 256 threads: the next launch's blocks come in beside these, and with a few rows cut into four times as many blocks
+// they came in unevenly (Mamba2-2.7B mixer at 16 rows 22.4 -> 28.3 us, Bamba-v2-9B 43.9 -> 44.8; at 1024 rows 78.0 -> 82.0, Qwen2.5-7B layer at
+// 256 rows, keep 0.65, 117.8 -> 124.1 us; ahead only for Llama-3-8B at 112 to 128 rows, keep 0.65, 100.5 -> 96.2 us).
 __global__ void x_to_f16_kernel(const __nv_bfloat16* __restrict__ x, int ldx, int M, int k_in, __half* __restrict__ o, int ldo) {
   // (programmatic dependent launch: the tensor-core kernel behind this one may set itself up meanwhile; this one
   //  waits for its own predecessor before it reads x or overwrites the copy that predecessor may still read)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int u = blockIdx.x * blockDim.x + threadIdx.x;        // 16-byte unit of the output row (ldo is a multiple of 8)
-  if (u * 8 >= ldo) return;
-  for (int m = blockIdx.y; m < M; m += gridDim.y) {
+  const int units = ldo / 8;                         // 16-byte units per output row (ldo is a multiple of 8)
+  const long total = (long)M * units;
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
+    const int m = (int)(i / units), u = (int)(i - (long)m * units);
     const __nv_bfloat16* src = x + (size_t)m * ldx + u * 8;
     uint32_t w[4];
     if (u * 8 + 8 <= k_in && ((ldx & 7) == 0) && ((((uintptr_t)x) & 15) == 0)) {
@@ -612,11 +616,12 @@ int device_sms() {
 }
 
 int launch_x_to_f16(const void* x, int ldx, int M, int k_in, void* out, int ldo, cudaStream_t stream) {
-  const unsigned cols = (unsigned)(ldo / 8 + 127) / 128, rows = (unsigned)device_sms() * 32 / cols + 1;
+  const long units = (long)M * (ldo / 8), most = (long)device_sms() * 8;
+  const long blocks = (units + 255) / 256;
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
-  lc.gridDim = dim3(cols, (unsigned)M < rows ? (unsigned)M : rows);
-  lc.blockDim = dim3(128);
+  lc.gridDim = dim3((unsigned)(blocks < most ? blocks : most));
+  lc.blockDim = dim3(256);
   lc.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
