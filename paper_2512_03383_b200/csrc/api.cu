@@ -211,8 +211,9 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
   }
   if (gv_else && !relaid) gv = true;
   // An odd number of groups: the decode kernel or, above sixteen rows, the batch kernel on a copy of the scales and zero-points
-  // with padded rows, a sixteenth of the weight's bytes (on single blocks of the tensor-core kernel, which took them before,
-  // 10192 x 10624 at two rows was 41 us where its bytes take 7).  Not under options that run a batch as two halves.
+  // with rows padded to eight groups, a sixteenth of the codes' bytes (short rows more: all of a half for one group).  On single
+  // blocks of the tensor-core kernel, which takes what stays here, 10192 x 10624 at two rows is 52 us where its bytes take 8 (here
+  // 18).  Not under options that run a batch as two halves.
   if (path == UNIQL_PATH_AUTO && !gv && !dec_ok && p.M <= 128 && !halves && (p.K / kGroup) % 2 != 0) {
     Params q = p;
     const int G = p.K / kGroup;
@@ -230,14 +231,20 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
       at[j + 1] = at[j] + (((size_t)rows[j] * q.sz_pitch * 4 + 255) & ~(size_t)255);
       q.job[j].scales = q.job[j].zeros = nullptr;            // (aligned as the copies will be)
     }
-    // (nine to sixteen rows have a second kernel in front, which quantises the activations: worth it from ten million codes on --
-    //  9 million 11.5 -> 11.6 us, half a million 9.2 -> 10.2 us, 17 million 18.5 -> 14.9 us)
-    const bool dec = p.M <= 16 && (p.M <= 8 || codes >= 10000000) && decodes(q) && on_integers(q);
-    // (above 64 rows the exchange of shared tiles takes its share: single blocks -> batch kernel at 128 rows 0.5 million codes 9.7 ->
-    //  13.2 us, 9 million 12.3 -> 10.5, 17 million 23.2 -> 16.9, 78 million 43.3 -> 45.3; at 48 rows 9.4 -> 7.5, 11.7 -> 8.6, 18.7 ->
-    //  13.7, 41.3 -> 26.5)
-    const bool bat = p.M > 16 && (p.M <= 64 || (codes >= 5000000 && codes <= 40000000)) && (p.dt != UNIQL_BF16 || opt(kOptPrefillConvert) != 1) &&
-                     batch_supported(q);
+    // A single block walks its tile's groups one by one and the copy is a launch of its own (2 us), so few groups stay unless there
+    // are tiles for several rounds.  Single blocks -> decode kernel at one / eight rows: 512 x 384 5.9 -> 6.9 / 5.9 -> 6.8 us, 2048 x 384
+    // 6.2 -> 7.0 / 7.1, 9216 x 384 6.7 -> 5.9 / 8.5, 14336 x 384 7.8 -> 6.3 / 9.1, 32768 x 384 11.2 -> 8.3 / 11.3, 128 x 640 7.7 -> 5.9 / 8.0 -> 7.0.
+    // Nine to sixteen rows have a second kernel in front, which quantises the activations: at nine rows half a million codes
+    // 9.2 -> 10.2 us, 9 million 11.5 -> 11.6, 6144 x 1664 13.3 -> 10.4, 17 million 18.4 -> 14.5; with nine groups 9216 / 16384 / 28672 rows
+    // 11.7 -> 11.5 / 13.5 -> 14.3 / 33.0 -> 19.6; 32768 x 384 11.5 -> 15.5, x 640 14.9 -> 16.7.
+    const int groups = (p.k_in + kGroup - 1) / kGroup;
+    const bool pays = p.M <= 8 ? groups >= 5 || (groups >= 3 && codes >= (p.M <= 4 ? 3500000 : 10000000)) : groups >= 9 && codes >= 10000000;
+    const bool dec = p.M <= 16 && pays && decodes(q) && on_integers(q);
+    // Batch kernel at 17 / 64 rows: 2048 x 384 6.3 -> 7.0 / 6.5 -> 7.3, 14336 x 384 8.0 -> 7.4 / 8.2 -> 7.8, 4096 x 640 7.9 -> 7.8 / 8.0 -> 8.2, 896 x 896
+    // 8.7 -> 8.3 / 9.0 -> 8.6, 65536 x 128 12.6 -> 10.6 / 12.7 -> 11.5.  Above 64 rows the exchange of shared tiles takes its share: at 128 rows 0.5
+    // million codes 9.7 -> 13.2 us, 9 million 12.3 -> 10.5, 17 million 23.2 -> 15.8, 78 million 43.3 -> 45.3.
+    const bool bat = p.M > 16 && (codes >= 5000000 ? p.M <= 64 || codes <= 40000000 : p.M <= 64 && groups >= 7) &&
+                     (p.dt != UNIQL_BF16 || opt(kOptPrefillConvert) != 1) && batch_supported(q);
     if (small && (dec || bat)) {
       if (!cfg.workspace) {
         int rc = lib_workspace(&cfg.workspace, &cfg.ws_bytes, cfg.stream);
