@@ -578,6 +578,58 @@ def test_odd_number_of_groups(B, M, N, K, k_in, k_out, dtype):
     assert B.workspace_status(big) == 0 and B.workspace_status() == 0
 
 
+def odd_call(B, qws, dws, x, dtype, in_map, k_in, outs, workspace=None):
+    """One call of several matrices with their own output maps; returns the outputs."""
+    xd = dev_x(x, dtype)
+    ys = [torch.full((x.shape[0], n + 1), -77.0, dtype=xd.dtype, device="cuda") for _, n in outs]
+    jobs = [dict(packed_w=d[1], scales=d[2], zeros=d[3], N=q.N, out_map=m, k_out=0 if m else n, y=y, ldy=n + 1)
+            for q, d, (m, n), y in zip(qws, dws, outs, ys)]
+    B.qlinear_multi(xd, x.shape[1], x.shape[0], qws[0].K, in_map, k_in, jobs, workspace=workspace)
+    torch.cuda.synchronize()
+    assert all((y[:, -1] == -77.0).all() for y in ys)
+    return [y[:, :-1] for y in ys]
+
+
+@pytest.mark.parametrize("M", [1, 4, 6, 8, 12, 17, 64, 128])
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("K,in_map,k_in", [(1152, None, 1152), (1152, None, 1146), (1152, None, 1148), (1152, synth.map_per_head(9, 128, 108), 0),
+                                           (1152, synth.map_per_head(9, 128, 88), 0), (896, synth.map_per_head(14, 64, 52), 0),
+                                           (1664, [(256, 128, 120, 11)], 0)])
+def test_odd_number_of_groups_of_several_matrices(B, M, dtype, K, in_map, k_in):
+    """The padded copies of several matrices behind one another, rows up to the last kept one of each output map, activations on
+    every boundary (re-laid above sixteen rows and in bf16; fp16 at decode sizes takes the general path), in the library's buffer
+    and in one of the advertised size under a band of canaries, with the same bits; without room for the copies another path
+    answers, and nothing is written behind the room there is.  Tolerance: weights rounded to fp16."""
+    rng = np.random.default_rng(K + M + k_in)
+    Ns = (640, 200, 96)
+    qws = [synth.draw_qweight(rng, n, K) for n in Ns]
+    dws = [dev_weight(q) for q in qws]
+    outs = [(synth.map_per_head(5, 128, 100), 500), (None, 180), ([(8, 16, 4, 5)], 20)]
+    n_in = synth.map_size(in_map) if in_map else k_in
+    x = synth.draw_x(rng, M, n_in, dtype)
+    I = oracle.expand_map(in_map) if in_map else oracle.leading(k_in)
+    ys = odd_call(B, qws, dws, x, dtype, in_map, k_in, outs)
+    for y, q, d, (m, n) in zip(ys, qws, dws, outs):
+        ref = oracle.qlinear(x, d[0], q.scales, q.zeros, oracle.expand_map(m) if m else oracle.leading(n), I)
+        check_output(y, ref, dtype, 5e-4, "M=%d K=%d N=%d %s" % (M, K, q.N, dtype))
+    full = B.workspace_bytes(M, K, sum(Ns))
+    for nbytes in (full, (1 << 18) + 256 + M * (K + 64) * 2 + 1024):
+        buf = torch.full((nbytes + (1 << 20),), 0xA5, dtype=torch.uint8, device="cuda")
+        ws = buf[:nbytes]
+        B.workspace_init(ws)
+        try:
+            y2 = odd_call(B, qws, dws, x, dtype, in_map, k_in, outs, workspace=ws)
+        except RuntimeError as e:                          # (decode sizes whose kernel wants its own scratch)
+            assert nbytes < full and "workspace too small" in str(e)
+            y2 = None
+        assert bool((buf[nbytes:] == 0xA5).all()) and B.workspace_status(ws) == 0
+        for y, z, q, d, (m, n) in zip(ys, y2 or [], qws, dws, outs):
+            if nbytes == full:
+                assert torch.equal(y, z)
+            ref = oracle.qlinear(x, d[0], q.scales, q.zeros, oracle.expand_map(m) if m else oracle.leading(n), I)
+            check_output(z, ref, dtype, 5e-4, "M=%d K=%d N=%d %s in %d bytes" % (M, K, q.N, dtype, nbytes))
+
+
 # Llama-size rows: every block stages all (row, group) pairs, 32 / 33 .. 64 / 65 and more of them (one, two or four units of eight
 # channels per lane, several passes of the block's threads), on 8- and on 4-channel boundaries.
 @pytest.mark.parametrize("M,K", [(1, 4096), (1, 4352), (1, 8192), (1, 8448), (2, 2048), (2, 2304), (2, 4096), (2, 4352), (3, 2560), (3, 2816),
