@@ -169,3 +169,19 @@ def test_heads_that_keep_4_mod_8_channels(B, M, heads, dim, keep):
         check_output(y, ref, "f16", TOL, "M=%d %d heads of %d keep %d" % (M, heads, dim, keep))
     assert B.workspace_status() == 0
     B.reset_options()
+
+
+@pytest.mark.parametrize("M", [17, 64, 128])
+@pytest.mark.parametrize("fam", [(256, 128, 108, 6), (512, 128, 84, 3), (256, 64, 52, 9), (256, 64, 60, 12)])
+def test_heads_that_keep_4_mod_8_channels_behind_channel_0(B, M, fam):
+    """The same with the first head on a later 256-channel boundary, the only one where they are read in place."""
+    rng = np.random.default_rng(37 * M + fam[2])
+    qw = synth.draw_qweight(rng, 200, 1024)
+    dw = dev_weight(qw)
+    x = synth.draw_x(rng, M, fam[2] * fam[3], "f16")
+    for split in (0, -1):
+        B.set_option("prefill_streamk", split)
+        y, ref = run_ex(B, qw, dw, x, "f16", [fam], 0, None, 200, ldx_pad=8 + (-x.shape[1]) % 8, ldy_pad=1)
+        check_output(y, ref, "f16", TOL, "M=%d %s" % (M, fam))
+    assert B.workspace_status() == 0
+    B.reset_options()

@@ -502,6 +502,17 @@ def test_qkv_one_launch(B, path, M, keep, v_keep):
             check_output(g, ref, dtype, tol, "qkv keep %d/%d M=%d %s" % (keep, v_keep, M, dtype))
 
 
+@pytest.mark.parametrize("M", [1, 6, 17, 64])
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("K,keep,v_keep", [(896, 128, 128), (896, 84, 108), (1664, 108, 100)])
+def test_qkv_of_an_odd_number_of_groups(B, M, dtype, K, keep, v_keep):
+    """Three padded copies of scales: rotated pairs, whose last kept row lies inside the last half head, beside plain rows."""
+    rng = np.random.default_rng(180 + keep + M)
+    for (g, ref) in run_rope(B, rng, M, K, 6, 2, 128, keep, 500000.0, dtype, bias=True, v_keep=v_keep):
+        check_output(g, ref, dtype, TIGHT if M < 17 else 5e-4, "qkv K=%d keep %d/%d M=%d %s" % (K, keep, v_keep, M, dtype))
+    assert B.workspace_status() == 0
+
+
 def test_qk_rope_bf16_table_and_split(B):
     rng = np.random.default_rng(71)
     invf = (1e6 ** (-np.arange(64) / 64.0)) * 0.5          # a caller table (scaled-RoPE variants)
@@ -562,8 +573,9 @@ def test_llama_mlp_full_size(B, M):
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
 def test_odd_number_of_groups(B, M, N, K, k_in, k_out, dtype):
     """Rows of scales on 2-byte boundaries: the decode kernel on a copy with padded rows (its own tolerance; from ten million codes
-    on also at nine to sixteen rows), above sixteen rows the batch kernel (weights rounded once to fp16), also in a caller
-    workspace of the advertised size, with the same bits; a workspace without room for the copy takes the general path."""
+    on also at nine to sixteen rows), above sixteen rows the batch kernel (weights rounded once to fp16), few groups on single
+    blocks, also in a caller workspace of the advertised size, with the same bits; a workspace without room for the copy (the
+    header and the fp16 copy of bf16 activations alone) takes the general path."""
     rng = np.random.default_rng(M + N + K)
     qw = synth.draw_qweight(rng, N, K)
     dw = dev_weight(qw)
@@ -576,6 +588,11 @@ def test_odd_number_of_groups(B, M, N, K, k_in, k_out, dtype):
     y2, _ = run_ex(B, qw, dw, x, dtype, None, k_in, None, k_out, bias=bias, ldx_pad=-k_in % 8, ldy_pad=1, workspace=big)
     assert torch.equal(y, y2)
     assert B.workspace_status(big) == 0 and B.workspace_status() == 0
+    small = torch.empty((1 << 18) + 512 + (M * (K + 64) * 2 if dtype == "bf16" else 0), dtype=torch.uint8, device="cuda")
+    B.workspace_init(small)
+    y3, _ = run_ex(B, qw, dw, x, dtype, None, k_in, None, k_out, bias=bias, ldx_pad=-k_in % 8, ldy_pad=1, workspace=small)
+    check_output(y3, ref, dtype, 5e-4, "small workspace M=%d %dx%d" % (M, N, K))
+    assert B.workspace_status(small) == 0
 
 
 def odd_call(B, qws, dws, x, dtype, in_map, k_in, outs, workspace=None):

@@ -157,3 +157,24 @@ def test_mlp_block_of_odd_widths_in_the_advertised_workspace(B, M, dtype, hidden
                                      out_rows=rows, h_dtype=dtype)
     check_output(outs[0][0][:, :k_int], h_ref, dtype, 6e-4, "h")
     check_output(outs[0][1][:, torch.as_tensor(rows, device="cuda")], y_ref, dtype, TOL_Y if dtype == "f16" else 2e-3, "y")
+
+
+@pytest.mark.parametrize("M", [17, 33, 128])
+@pytest.mark.parametrize("k_int", [8, 200, 870])
+def test_copy_of_h_from_the_gated_launch_or_from_a_pass_of_its_own(B, M, k_int):
+    """bf16: one byte less than the room for the copy that the gated launch makes, and a small kernel in between makes it; same
+    bits, and nothing is written behind either workspace."""
+    hidden, inter = 512, 1024
+    _, _, ds = draw_mlp(78, hidden, inter)
+    xd = dev_x(synth.draw_x(np.random.default_rng(1600 + M), M, hidden, "bf16"), "bf16")
+    relay = (M * (hidden + 8) * 2 + 255) // 256 * 256 + 512                      # what the size query of a linear adds for re-laying
+    tight = (M * ((k_int + 63) // 64 * 64) * 2 + 255) // 256 * 256 + (B.workspace_bytes(M, hidden, 1) - relay) + 256
+    outs = []
+    for nbytes in (B.mlp_workspace_bytes(M, hidden, inter), tight, tight - 1):
+        buf, ws = guarded(B, nbytes)
+        h, y = (torch.zeros((M, n), dtype=xd.dtype, device="cuda") for n in (872, hidden))
+        B.mlp_swiglu(xd, hidden, *ds[0][1:], *ds[1][1:], *ds[2][1:], M, hidden, inter, k_int, h, 872, y, hidden, workspace=ws)
+        assert band_intact(buf, nbytes) and B.workspace_status(ws) == 0
+        outs.append((h, y))
+    for h, y in outs[1:]:
+        assert torch.equal(h, outs[0][0]) and torch.equal(y, outs[0][1])
