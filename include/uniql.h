@@ -21,13 +21,16 @@
  *    host before anything is launched; nothing aborts or throws.
  *  - There is no CPU fallback: without a usable CUDA device calls return
  *    UNIQL_ERR_CUDA.
- *  - Decode launches (M <= 16) and the launches of the tensor-core kernel (M > 16) carry the
+ *  - Decode launches (M <= 16), the launches of the tensor-core kernels (M > 16), the small kernels in front of
+ *    either (which copy activations or scales) and uniql_embed_rows carry the
  *    programmatic-stream-serialization attribute: back-to-back calls on one stream overlap their launch
  *    set-up and first weight stages with the tail of the preceding one (1.6 us per decode launch, 2 - 4 us
  *    per tensor-core launch), while everything that can depend on the preceding kernel (activations,
  *    outputs, workspace, bias, positions, indices) is touched only after it has completed.  Packed weights,
  *    scales and zero-points must not be written by a call's immediate predecessor on the stream
- *    unless that predecessor is a plain kernel (which completes before its successor starts).
+ *    unless that predecessor is a plain kernel (which completes before its successor starts; of the kernels of this
+ *    library those of uniql_pack_u4, uniql_unpack_u4 and uniql_dequant and the generic one).  uniql_embed_rows reads its
+ *    table, like its ids, after its predecessor has completed, and lets its successor in from then on.
  *    uniql_set_option("pdl", 0) (or UNIQL_PDL=0 in the environment at load time) turns the attribute off.
  *
  * Weight format (the interchange format; benchmark configuration 1)
@@ -87,10 +90,18 @@ typedef enum { UNIQL_F16 = 0, UNIQL_BF16 = 1 } uniql_dtype;
  *    8-byte aligned);
  *  - fp16 at twelve to sixteen rows and bf16 at nine to sixteen go to the batch kernel instead where its rules hold, unless an
  *    option of the decode kernel ("decode_*") is off its default (fp16);
+ *  - K / 128 odd (rows of scales on 2-byte boundaries): the decode kernel, or at 17 to 128 rows the batch kernel, on a copy of the
+ *    scales and zero-points with padded rows, which a small kernel per matrix writes to the end of the workspace, where the
+ *    matrix is large enough by the size rules of the dispatch and the workspace has room; else single blocks as below;
  *  - everything else goes to the tensor cores (UNIQL_PATH_PREFILL: the batch kernel up to 128 rows, block pairs above,
  *    single blocks for what neither takes) when their alignment rules hold (activations 16-byte aligned, or re-laid, with
  *    a row pitch that is a multiple of 8, input map a leading block or one family of per-head blocks on 64-channel
- *    boundaries with keep % 8 == 0), otherwise to the generic kernel. */
+ *    boundaries with keep % 8 == 0; fp16 heads of 64 or 128 channels from a 256-channel boundary on that keep 4 (mod 8) are
+ *    read in place at 17 to 128 rows, others re-laid), otherwise to the generic kernel.
+ * The decode kernel's integer path holds codes exactly and activations in 16-bit fixed point per row and group of 128 against the
+ * group's largest (what is more than a factor 2^15 below it is lost; a group with an Inf or a NaN makes the outputs that use
+ * it NaN); the tensor-core kernels hold weights rounded to fp16 and activations in fp16 (bf16: converted, see the workspace
+ * below).  Matrices with an odd number of groups are on either by the rules above. */
 typedef enum { UNIQL_PATH_AUTO = 0, UNIQL_PATH_GENERIC = 1, UNIQL_PATH_DECODE = 2,
                UNIQL_PATH_PREFILL = 3, UNIQL_PATH_GEMV = 4 } uniql_path;
 
@@ -196,7 +207,11 @@ int uniql_embed_rows(const uint8_t* packed, const void* scales, const void* zero
  * than two blocks on a tile the last bit of an fp32 sum, and rarely of the rounded output, can differ
  * between two runs on the same input; uniql_set_option("prefill_streamk", 0) switches the splitting off.  Activations below fp16's range are affected too: bf16 values under 2^-24 become zero
  * and those under 2^-14 lose significand bits in the fp16 copy.  Without room for the
- * sums every tile is computed by one block (reproducible, slower for shapes that fill few SMs). */
+ * sums every tile is computed by one block (reproducible, slower for shapes that fill few SMs).
+ * At the end of the workspace lie, where a call needs them: the re-laid copy of the activations, up to 128 rows the copy of the
+ * scales and zero-points of matrices with an odd number of groups (4 bytes x N x K / 128 rounded up to a multiple of 8), and,
+ * SwiGLU block in bf16 at 17 to 128 rows, h once more in fp16.  The size queries have room for all of them (N_total: stored
+ * rows of all matrices); without room the call takes another kernel or another pass, same results within the tolerance. */
 size_t uniql_workspace_bytes(int M, int K, int N_total);
 int uniql_workspace_init(void* workspace, size_t bytes, void* stream);
 /* Every wait inside the kernels is bounded.  When one expires the kernel stops early and writes

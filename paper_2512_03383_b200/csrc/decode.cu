@@ -754,8 +754,8 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
     auto give_up = [&]() { if (lane == 0) atomicExch(c.status, UNIQL_ERR_TIMEOUT); };
     int tiles_done = 0;
     // ... and this kernel may have been started before its predecessor finished: outputs, workspace, bias,
-    // positions and indices are touched only after the predecessor is complete (the producer warp does not
-    // wait: weights, scales and zero-points are not produced by a preceding decode launch)
+    // positions and indices are touched only after the predecessor is complete (the producer warp waits only where the
+    // scales and zero-points are a copy that the kernel in front makes: sz_wait)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int ph = 0; ph < NPH; ++ph) {
       const PhaseCtx pc = (NPH == 1 || ph == 0) ? pc0 : phase_ctx(c, ph, kp, rp);
@@ -1677,8 +1677,8 @@ void visited_range(const ChanMap& m, int gran, int* first, int* total) {
 // Up to eight rows the parked sums have two buffers.  One of them is given up
 //  - for a fourth stage: the bytes in flight are what a launch streams with, while the epilogue warps drain a buffer in a fraction
 //    of a tile's time (lm_head at eight rows 69.8 -> 66.9 us, 1 - 3 % at 60 sizes from 148 to 2004 tiles).  Not from six rows on
-//    where blocks have two or more whole tiles and the left-over ones are split (`tiles` 64-row tiles): what the one buffer holds
-//    up then stands in front of the hand-over (7 x 4608 and 8 x 4096, 300, 448 and 596 tiles: 2.1 us, 5 - 15 %, at every split size).
+//    where blocks have two or more whole tiles and the left-over ones are split (`tiles` 64-row tiles): the hand-over of a split tile,
+//    which comes first, then holds the one buffer (7 x 4608 and 8 x 4096, 300, 448 and 596 tiles: 2.1 us, 5 - 15 %, at every split size).
 //    (Where every block ends on a whole tile the last drain stands behind the one before it: 8 x 4096, 148 tiles, launched alone
 //    11.5 -> 11.8 us.  Two buffers there, and wherever more than half of the blocks end so, cost a Bamba-v2-9B mixer at eight rows 33.5 ->
 //    34.8 us.)

@@ -15,8 +15,8 @@ namespace uniql {
 // Every block of a decode launch quantises the whole activation matrix between its predecessor's end and its own first MMA.
 // Long matrices are bound by issue slots there: one unit per lane is about 110 instructions per unit, of which the
 // reductions over the lanes and the exponent come once per lane; four units per lane about 50 (Llama-3-8B layer at four rows
-// and keep 0.65 41.9 -> 37.0 us).  Short ones are bound by the chain of one lane (2048 activations: 4.1 us a call with one
-// unit per lane, 4.8 with four).
+// and keep 0.65 42.0 -> 37.1 us).  Short ones are bound by the chain of one lane (2048 activations: 4.1 us a call with one
+// unit per lane, 4.8 with four).  The rule stands where the decode kernel stages its activations.
 template <typename T, int U>
 __device__ inline void quantise_units(const uint4 (&in)[U], uint2 (&hi)[U], uint2 (&lo)[U], int& isum_out, float& inv_scale_out) {
   using T2 = typename DT<T>::T2;
