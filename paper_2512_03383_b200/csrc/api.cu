@@ -238,12 +238,14 @@ int dispatch_as(const Params& p_in, int path, void* workspace, size_t ws_bytes, 
     // 9.2 -> 10.2 us, 9 million 11.5 -> 11.6, 6144 x 1664 13.3 -> 10.4, 17 million 18.4 -> 14.5; with nine groups 9216 / 16384 / 28672 rows
     // 11.7 -> 11.5 / 13.5 -> 14.3 / 33.0 -> 19.6; 32768 x 384 11.5 -> 15.5, x 640 14.9 -> 16.7.
     const int groups = (p.k_in + kGroup - 1) / kGroup;
-    const bool pays = p.M <= 8 ? groups >= 5 || (groups >= 3 && codes >= (p.M <= 4 ? 3500000 : 10000000)) : groups >= 9 && codes >= 10000000;
+    // (a copy per matrix: q|k|v of 640 channels at eight rows 7.2 -> 8.2 us, of 896 9.3 -> 8.3)
+    const bool pays = p.M <= 8 ? groups >= (p.M > 4 && p.n_jobs > 2 ? 7 : 5) || (groups >= 3 && codes >= (p.M <= 4 ? 3500000 : 10000000)) : groups >= 9 && codes >= 10000000;
     const bool dec = p.M <= 16 && pays && decodes(q) && on_integers(q);
     // Batch kernel at 17 / 64 rows: 2048 x 384 6.3 -> 7.0 / 6.5 -> 7.3, 14336 x 384 8.0 -> 7.4 / 8.2 -> 7.8, 4096 x 640 7.9 -> 7.8 / 8.0 -> 8.2, 896 x 896
     // 8.7 -> 8.3 / 9.0 -> 8.6, 65536 x 128 12.6 -> 10.6 / 12.7 -> 11.5.  Above 64 rows the exchange of shared tiles takes its share: at 128 rows 0.5
     // million codes 9.7 -> 13.2 us, 9 million 12.3 -> 10.5, 17 million 23.2 -> 15.8, 78 million 43.3 -> 45.3.
-    const bool bat = p.M > 16 && (codes >= 5000000 ? p.M <= 64 || codes <= 40000000 : p.M <= 64 && groups >= 7) &&
+    // Several matrices at 17 / 64 rows: q|k|v of 896 channels 10.1 -> 10.5 / 11.1 -> 11.4, of 1152 11.9 -> 11.0 / 13.1 -> 11.5 us.
+    const bool bat = p.M > 16 && (codes >= 5000000 ? p.M <= 64 || codes <= 40000000 : p.M <= 64 && groups >= (p.n_jobs > 1 ? 9 : 7)) &&
                      (p.dt != UNIQL_BF16 || opt(kOptPrefillConvert) != 1) && batch_supported(q);
     if (small && (dec || bat)) {
       if (!cfg.workspace) {
