@@ -316,8 +316,7 @@ __global__ void __launch_bounds__(NTHB, 2) batch_kernel(const __grid_constant__ 
       asm volatile("fence.acq_rel.cluster;" ::: "memory");
       pmbar_arrive_peer(ppeer_addr(xb, (uint32_t)lane));
     }
-    const bool ok = __all_sync(0xffffffffu, pmbar_wait_cluster(xb, (count >> 1) & 1, abort_flag));
-    if (!ok) { failed = true; return; }
+    if (!pmbar_wait_cluster_warp(xb, (count >> 1) & 1, abort_flag)) { failed = true; return; }
     for (int own = half; rank + own * c.p < n_ch; own += 2) {
       const int ch = rank + own * c.p;
       uint32_t v[8];

@@ -182,10 +182,13 @@ __global__ void __launch_bounds__(PTH, 1) pair_kernel(const __grid_constant__ Pa
       // last_seg: a de-quantiser warp on the block's last segment.  It waits here and not before the call: the row's loads above -- map,
       // bias, rotation index, one behind the other, 1 us -- then run beside the last MMAs (layers back to back: Llama-3-8B at 512 rows, keep
       // 0.75, 168.6 -> 166.9 us, Qwen2.5-7B at 677 rows 226.6 -> 225.2).
-      if (last_seg && !pmbar_wait(last_full, 0, abort_flag, true)) failed = true;
-      for (int h = h_lo; h < h_hi && !failed && !last_seg; ++h)
-        if (!pmbar_wait(acc_full + 8 * (acc0 + h), au & 1, abort_flag)) failed = true;
-      if (failed) return;
+      // (left at once where a wait expires: with one test of `failed` behind both the instances for whole tiles spill)
+      if (last_seg) {
+        if (!pmbar_poll_warp(last_full, 0, abort_flag, true)) { failed = true; return; }
+      } else {
+        for (int h = h_lo; h < h_hi; ++h)
+          if (!pmbar_poll_warp(acc_full + 8 * (acc0 + h), au & 1, abort_flag)) { failed = true; return; }
+      }
       tc_fence_after();
       // (the two accumulators are neighbours in tensor memory: a tile of two boxes is 512 consecutive columns)
       const uint32_t t_acc = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc0 * MAXBN);
@@ -221,7 +224,7 @@ __global__ void __launch_bounds__(PTH, 1) pair_kernel(const __grid_constant__ Pa
           asm volatile("fence.acq_rel.cluster;" ::: "memory");
           pmbar_arrive_peer(ppeer_addr(xq + 8 * q, (uint32_t)(2 * lane) + crank));
         }
-        if (!__all_sync(0xffffffffu, pmbar_wait_cluster(xq + 8 * q, 0, abort_flag))) { failed = true; return; }
+        if (!pmbar_wait_cluster_warp(xq + 8 * q, 0, abort_flag)) { failed = true; return; }
         for (int own = ch0; part + own * n_share < N_CH; own += chs) {
           const int tk = (part + own * n_share) * CH;
           if (tt * ntok + tk >= p.M) break;
@@ -447,7 +450,7 @@ __global__ void __launch_bounds__(PTH, 1) pair_kernel(const __grid_constant__ Pa
           q1[m] = make_uint4(0, 0, 0, 0); s1[m] = s0[m]; z1[m] = z0[m];
           if (live[m] && more) fetch(m, st1, q1[m], s1[m], z1[m]);
         }
-        if (it >= NA && !pmbar_wait(empty_a + 8 * s, (use - 1) & 1, abort_flag)) { failed = true; break; }
+        if (it >= NA && !pmbar_wait_warp(empty_a + 8 * s, (use - 1) & 1, abort_flag)) { failed = true; break; }
 #pragma unroll
         for (int m = 0; m < 2; ++m) {
           if (m >= n_items) break;

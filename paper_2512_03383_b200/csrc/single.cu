@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant
   auto epi_sync = [&]() -> bool {
     __syncwarp();
     if (lane == 0) pmbar_arrive(epi_bar);
-    const bool ok = pmbar_wait(epi_bar, epar, abort_flag);
+    const bool ok = pmbar_poll_warp(epi_bar, epar, abort_flag);
     epar ^= 1;
     return ok;
   };
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant
   auto help_sync = [&]() -> bool {
     __syncwarp();
     if (lane == 0) pmbar_arrive(help_bar);
-    const bool ok = pmbar_wait(help_bar, hpar, abort_flag);
+    const bool ok = pmbar_poll_warp(help_bar, hpar, abort_flag);
     hpar ^= 1;
     return ok;
   };
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant
         }
       };
       for (int h = h_lo; h < h_hi && !failed && !acc_known_full; ++h)
-        if (!pmbar_wait(acc_full + 8 * (acc0 + h), au & 1, abort_flag)) failed = true;
+        if (!pmbar_poll_warp(acc_full + 8 * (acc0 + h), au & 1, abort_flag)) failed = true;
       if (failed) return;
       tc_fence_after();
       // (the two accumulators are neighbours in tensor memory: a tile of two boxes is 512 consecutive columns)
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant
           //      barrier; the first block adds them to its own sums (always own + other: the same bits every run)
           //      and finishes the tile.  No traffic through L2, no counter, nothing to clear.
           {
-            if (!pmbar_wait_cluster(px_done, 0, abort_flag)) { failed = true; return; }
+            if (!pmbar_wait_cluster_warp(px_done, 0, abort_flag)) { failed = true; return; }
             // (16 tokens at a time, as the read-back of the slots: what the registers of a thread hold)
             for (int tk = 16 * ch0; tk < ntok; tk += 16 * chs) {
               uint32_t v[16];
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant
         float* mine = c.partials + ((size_t)(t - T0) + (c.sk_atomic ? 0 : blockIdx.x)) * slot_f;
         if (pair_send) {
           // (the second block of a pair: its "slot" is the first block's rings, once they are idle)
-          if (!pmbar_wait_cluster(px_ready, 0, abort_flag)) { failed = true; return; }
+          if (!pmbar_wait_cluster_warp(px_ready, 0, abort_flag)) { failed = true; return; }
           mine = ppeer_generic(smem, 0u);
         }
         for (int ch = ch0; ch < ntok / EPI_TOK; ch += chs) {
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant
           if (HEADS) kw.step(c, 1);
           const int h_lo = sg.half < 0 ? 0 : sg.half, h_hi = sg.half < 0 ? c.nh : sg.half + 1;
           for (int h = h_lo; h < h_hi; ++h, ++jb) {
-            if (jb >= BSLOTS && !pmbar_wait(empty_b + 8 * s, par, abort_flag, true)) { failed = true; break; }
+            if (jb >= BSLOTS && !pmbar_wait_lane(empty_b + 8 * s, par, abort_flag, true)) { failed = true; break; }
             const uint32_t fb = full_b + 8 * s;
             pmbar_expect_tx(fb, (uint32_t)(c.bn * BK * 2));
             // (a box that starts at or beyond the last token is all zeros: the tensor map ends at M)
@@ -609,7 +609,7 @@ __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant
           q1[m] = make_uint4(0, 0, 0, 0); s1[m] = s0[m]; z1[m] = z0[m];
           if (live[m] && more) fetch(m, st1, q1[m], s1[m], z1[m]);
         }
-        if (it >= PSTAGES && !pmbar_wait(empty_a + 8 * s, (use - 1) & 1, abort_flag)) { failed = true; break; }
+        if (it >= PSTAGES && !pmbar_wait_warp(empty_a + 8 * s, (use - 1) & 1, abort_flag)) { failed = true; break; }
 #pragma unroll
         for (int m = 0; m < 2; ++m) {
           if (m >= n_items) break;
@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant
           for (int h = 0; h < c.nh && !failed; ++h) {
             const int jb2 = it * c.nh + h;                 // the k-block's boxes in the order the producer issued them
             const int sb = jb2 % BSLOTS;
-            if (!pmbar_wait(full_b + 8 * sb, (uint32_t)(jb2 / BSLOTS) & 1, abort_flag)) { failed = true; break; }
+            if (!pmbar_wait_warp(full_b + 8 * sb, (uint32_t)(jb2 / BSLOTS) & 1, abort_flag)) { failed = true; break; }
             const uint32_t b_st = sbase + B_RING + sb * B_BYTES;
             for (int ci = dt; ci < c.bn * 8; ci += TEAM_TH) {
               uint32_t v0, v1, v2, v3;
@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(PTH, 1) one_block_kernel(const __grid_constant
     // quadrant (warps 8 + q, 12 + q, 16 + q, 20 + q: chunks 1, 2, 3, 4 of every five)
     if (c.helpers && !failed && n_seg > 0) {
       asm volatile("griddepcontrol.wait;" ::: "memory");   // outputs and workspace: after the preceding kernel
-      if (!pmbar_wait(last_full, 0, abort_flag, true)) failed = true;
+      if (!pmbar_poll_warp(last_full, 0, abort_flag, true)) failed = true;
       if (!failed) epilogue_segment(last_sg, n_seg - 1, 1 + (warp - DQ_WARP0) / 4, 5, true);
     }
   } else if (warp >= EPI_WARP0) {

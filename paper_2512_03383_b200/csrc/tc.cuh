@@ -30,8 +30,11 @@ __device__ inline bool pmbar_try(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
+// A bounded wait has one answer per warp: a warp whose lanes disagreed about an expired wait -- the phase may complete between two
+// lanes' last polls -- would part, and its next warp-wide instruction would wait for the missing lanes.  The vote also brings the lanes
+// together in front of that instruction.  Only a thread that waits on its own takes the form without it.
 // `relaxed`: sleep between polls (roles that run several stages ahead and must not steal issue slots)
-__device__ inline bool pmbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, bool relaxed = false) {
+__device__ inline bool pmbar_wait_lane(uint32_t bar, uint32_t parity, volatile int* abort_flag, bool relaxed = false) {
   for (int i = 0; i < kPWait; ++i) {
     if (pmbar_try(bar, parity)) return true;
     if (relaxed) __nanosleep(200);
@@ -39,6 +42,9 @@ __device__ inline bool pmbar_wait(uint32_t bar, uint32_t parity, volatile int* a
   }
   *abort_flag = 1;
   return false;
+}
+__device__ inline bool pmbar_poll_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, bool relaxed = false) {
+  return __all_sync(0xffffffffu, pmbar_wait_lane(bar, parity, abort_flag, relaxed));
 }
 // As pmbar_try, but the hardware may suspend the thread for up to a microsecond until the phase completes.
 __device__ inline bool pmbar_try_suspend(uint32_t bar, uint32_t parity) {
@@ -50,8 +56,7 @@ __device__ inline bool pmbar_try_suspend(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity), "r"(1000u) : "memory");
   return ok != 0;
 }
-// The same for a whole warp: one answer for all lanes (a warp whose lanes disagreed about an expired wait would part, and
-// its next warp-wide instruction would wait for the missing lanes).
+// pmbar_poll_warp with these polls, for the roles whose next step hangs on the phase.
 __device__ inline bool pmbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   if (__all_sync(0xffffffffu, pmbar_try(bar, parity))) return true;
   bool ok = false;
@@ -98,20 +103,26 @@ __device__ inline void pmbar_signal_peer(uint32_t addr) {
 __device__ inline void pmbar_arrive_peer(uint32_t addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
-__device__ inline bool pmbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+__device__ inline bool pmbar_try_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
+__device__ inline bool pmbar_wait_cluster_lane(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   for (int i = 0; i < kPWait; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    if (ok) return true;
+    if (pmbar_try_cluster(bar, parity)) return true;
     __nanosleep(20);
     if ((i & 63) == 63 && *abort_flag) return false;
   }
   *abort_flag = 1;
   return false;
+}
+__device__ inline bool pmbar_wait_cluster_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, pmbar_wait_cluster_lane(bar, parity, abort_flag));
 }
 __device__ inline void tma_box2(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t bar) {
   asm volatile(
