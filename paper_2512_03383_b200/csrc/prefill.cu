@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(PTH, 1) pair_kernel(const __grid_constant__ Pa
   //      also hands the accumulators back).
   const int q = warp & 3;                          // TMEM lanes 32q .. 32q+31
   const int etid = 32 * q + lane;                  // tile row handled in the store phase
-  auto epilogue_segment = [&](const Seg& sg, int tcount, int ch0, int chs, bool last_seg) {
+  auto epilogue_segment = [&](const Seg& sg, int tcount, int ch0, int chs, bool helper) {
       const int acc0 = c.nh == 2 ? 0 : (tcount & 1);     // as in the MMA warp
       const int au = c.nh == 2 ? tcount : (tcount >> 1);
       const int ntok = c.bn * c.nh;                      // tokens of the tile
@@ -179,11 +179,12 @@ __global__ void __launch_bounds__(PTH, 1) pair_kernel(const __grid_constant__ Pa
       // this thread owns tile row etid (= its TMEM lane); a rope pair sits in lanes 2i, 2i + 1
       const RowStore<T> rs(p, jn, tile_row(p.job[jn], tl, etid), (etid & 1) != 0);
       auto store_chunk = [&](int tok0, const auto& val) { rs.store(p, tt * ntok + tok0, val); };
-      // last_seg: a de-quantiser warp on the block's last segment.  It waits here and not before the call: the row's loads above -- map,
-      // bias, rotation index, one behind the other, 1 us -- then run beside the last MMAs (layers back to back: Llama-3-8B at 512 rows, keep
-      // 0.75, 168.6 -> 166.9 us, Qwen2.5-7B at 677 rows 226.6 -> 225.2).
-      // (left at once where a wait expires: with one test of `failed` behind both the instances for whole tiles spill)
-      if (last_seg) {
+      // helper: a de-quantiser warp on the block's last segment, which follows the barrier of that segment alone.  It waits here and not in
+      // front of the call: the row's index arithmetic above, and what loads a bias and a rotation need, run beside the last MMAs
+      // (passes back to back, in turn with the wait in front: Llama-3-8B layer at 512 rows, keep 0.75, 194.1 -> 192.8 us, Mamba2-2.7B
+      // mixer at 1024 rows, keep 0.75, 76.7 -> 76.1, Qwen2.5-7B layer at 677 rows, keep 0.65, 254.6 -> 253.6, where the runs of one
+      // side differ by 0.1 - 0.6 %).  Left at once where a wait expires: with one test of `failed` behind both waits whole tiles spill.
+      if (helper) {
         if (!pmbar_poll_warp(last_full, 0, abort_flag, true)) { failed = true; return; }
       } else {
         for (int h = h_lo; h < h_hi; ++h)
