@@ -204,32 +204,14 @@ __device__ inline bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
-// Bounded waits: false when the limit expired or another warp of the block already gave up.  The phase may complete between two
-// lanes' last polls, so what a warp does together behind a wait needs one answer for its lanes: mbar_wait_warp.  The lanes of the
-// hot loops keep their own answers, since a vote in front of every stage cost 1 - 3 % of a launch (Qwen2.5-7B layer in bf16 at two rows
-// 44.7 -> 45.5 us, Mamba2-2.7B mixer at one row 11.75 -> 12.1): a consumer lane stays with its warp (`expired`), and what the producer's
-// lanes do they do each on its own.
-__device__ inline bool mbar_wait_lane(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+// Bounded wait: false when the limit expired or another warp of the block already gave up.
+__device__ inline bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   for (int i = 0; i < kWaitLimit; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
     if ((i & 63) == 63 && *abort_flag) return false;
   }
   *abort_flag = 1;
   return false;
-}
-__device__ inline bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  return __all_sync(0xffffffffu, mbar_wait_lane(bar, parity, abort_flag));
-}
-__device__ inline bool mbar_wait_cluster_lane(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  for (int i = 0; i < kWaitLimit; ++i) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    if ((i & 63) == 63 && *abort_flag) return false;
-  }
-  *abort_flag = 1;
-  return false;
-}
-__device__ inline bool mbar_wait_cluster_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  return __all_sync(0xffffffffu, mbar_wait_cluster_lane(bar, parity, abort_flag));
 }
 // One box of a 3-D tensor map into shared memory (no multicast), completion counted on `bar`.
 __device__ inline void tma_box3(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
@@ -652,9 +634,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
       const __half* srow[2] = {nullptr, nullptr};
       const __half* zrow[2] = {nullptr, nullptr};
       for (int iu = 0; iu < wk.n_units; ++iu, ++it) {
-        // (a lane whose wait expired leaves on its own: the others' copies do not need it, the stage never fills without it,
-        //  and a __syncwarp does not wait for a lane that is gone)
-        if (it >= S) ok = mbar_wait_lane(bar_empty + 8 * s, ring_parity, abort_flag);
+        if (it >= S) ok = mbar_wait(bar_empty + 8 * s, ring_parity, abort_flag);
         if (!ok) break;
         const bool new_tile = ui.tile != tile_prev;
         if (new_tile) {
@@ -757,7 +737,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
         const uint32_t full = bar_full + 8 * (j % S);
         for (int i = 0; i < kWaitLimit && !mbar_try_wait(full, (j / S) & 1); ++i) {}
       }
-      atomicExch(c.status, UNIQL_ERR_TIMEOUT);
+      if (lane == 0) atomicExch(c.status, UNIQL_ERR_TIMEOUT);
     }
     return;
   }
@@ -792,7 +772,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
         if (tile_end) {
           const int buf = c.part_bufs > 1 ? (tiles_done & 1) : 0;
           const int use = c.part_bufs > 1 ? (tiles_done >> 1) : tiles_done;
-          if (!mbar_wait_warp(bar_pfull + 8 * buf, use & 1, abort_flag)) { give_up(); return; }
+          if (!mbar_wait(bar_pfull + 8 * buf, use & 1, abort_flag)) { give_up(); return; }
           const float* pr = part + buf * part_stride;
           auto local_sum = [&](int slot, int m) -> float {
             float v = 0.f;
@@ -892,14 +872,10 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
   const int g_first = c.cgz > CG ? rg * CG + kpw : kpw;
   uint32_t cons_parity = 0;
   auto give_up = [&]() { if (lane == 0) atomicExch(c.status, UNIQL_ERR_TIMEOUT); };
-  // A lane whose wait for a stage or for a buffer of parked sums expired goes on beside the others to the end of its loop (the MMAs and
-  // shuffles are of whole warps; the launch has failed, and its later waits see the abort flag) and signals nothing from then on.
-  bool tell = lane == 0;                   // this lane arrives for its warp
-  auto expired = [&]() { tell = false; atomicExch(c.status, UNIQL_ERR_TIMEOUT); };
   auto consumer_sync = [&]() -> bool {
     __syncwarp();
     if (lane == 0) mbar_arrive(bar_cons);
-    const bool ok = mbar_wait_warp(bar_cons, cons_parity, abort_flag);
+    const bool ok = mbar_wait(bar_cons, cons_parity, abort_flag);
     cons_parity ^= 1;
     if (!ok) give_up();
     return ok;
@@ -1053,7 +1029,12 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
           mbar_arrive(bar_epi);
           mbar_arrive_peer(peer_addr(bar_epi, (uint32_t)(crank ^ 1)));
         }
-        if (!mbar_wait_cluster_warp(bar_epi, 0, abort_flag)) { give_up(); return false; }
+        bool ok = false;
+        for (int i = 0; i < kWaitLimit && !ok; ++i) {
+          ok = mbar_try_wait_cluster(bar_epi, 0);
+          if (!ok && (i & 63) == 63 && *abort_flag) break;
+        }
+        if (!ok) { *abort_flag = 1; give_up(); return false; }
         return true;
       }
     } else {
@@ -1198,14 +1179,17 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
           atomicExch(c.status, UNIQL_ERR_TIMEOUT);
         }
       }
-      if (!consumer_sync() || __any_sync(0xffffffffu, *abort_flag != 0)) return;
+      if (!consumer_sync() || *abort_flag) return;
     }
     if (wk.n_units == 0) continue;
     if (!xstream && !stage_x(ph, pc)) return;
     UnitIter ui;
     ui.start(wk);
     for (int i = 0; i < wk.n_units; ++i) {
-      if (!mbar_try_wait(bar_full + 8 * s, ring_parity) && !mbar_wait_lane(bar_full + 8 * s, ring_parity, abort_flag)) expired();
+      if (!mbar_try_wait(bar_full + 8 * s, ring_parity) && !mbar_wait(bar_full + 8 * s, ring_parity, abort_flag)) {
+        give_up();
+        return;
+      }
       const int gi = ui.chunk * c.cgz + g_first;
       if (gi < Gk) {
         const uint32_t st = sbase + (uint32_t)s * (xs_on ? (uint32_t)c.stage_bytes : (uint32_t)STAGE_BYTES);
@@ -1313,12 +1297,12 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
         }
       }
       __syncwarp();
-      if (tell) mbar_arrive(bar_empty + 8 * s);
+      if (lane == 0) mbar_arrive(bar_empty + 8 * s);
       if (++s == S) { s = 0; ring_parity ^= 1; }
       if (ui.tile_end(wk, i)) {
         const int buf = c.part_bufs > 1 ? (tiles_done & 1) : 0;
         const int use = c.part_bufs > 1 ? (tiles_done >> 1) : tiles_done;
-        if (use > 0 && !mbar_wait_lane(bar_pfree + 8 * buf, (use - 1) & 1, abort_flag)) expired();
+        if (use > 0 && !mbar_wait(bar_pfree + 8 * buf, (use - 1) & 1, abort_flag)) { give_up(); return; }
         float* pb = part + buf * part_stride + kpw * RM;
 #pragma unroll
         for (int sub = 0; sub < 2; ++sub)
@@ -1332,7 +1316,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
             out8[sub][nt][0] = out8[sub][nt][1] = 0.f;
           }
         __syncwarp();
-        if (tell) mbar_arrive(bar_pfull + 8 * buf);
+        if (lane == 0) mbar_arrive(bar_pfull + 8 * buf);
         ++tiles_done;
       }
       if (i + 1 < wk.n_units) ui.advance(wk, i + 1);
@@ -1378,7 +1362,10 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
 #pragma unroll
     for (int j = 0; j < 4; ++j) xr[mt][j] = make_uint4(0, 0, 0, 0);
   for (int i = 0; i < wk.n_units; ++i) {
-    if (!mbar_try_wait(bar_full + 8 * s, ring_parity) && !mbar_wait_lane(bar_full + 8 * s, ring_parity, abort_flag)) expired();
+    if (!mbar_try_wait(bar_full + 8 * s, ring_parity) && !mbar_wait(bar_full + 8 * s, ring_parity, abort_flag)) {
+      give_up();
+      return;
+    }
     const int gi = ui.chunk * c.cgz + g_first;
     if (gi < Gk) {
       const uint32_t st = sbase + (uint32_t)s * (uint32_t)STAGE_BYTES;
@@ -1449,7 +1436,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
         }
     }
     __syncwarp();
-    if (tell) mbar_arrive(bar_empty + 8 * s);
+    if (lane == 0) mbar_arrive(bar_empty + 8 * s);
     if (++s == S) { s = 0; ring_parity ^= 1; }
 
     const bool tile_end = ui.tile_end(wk, i);
@@ -1457,7 +1444,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
       // ---- park this warp's partial sums for the epilogue warps: part[buf][group slot kpw][m][row slot]
       const int buf = c.part_bufs > 1 ? (tiles_done & 1) : 0;
       const int use = c.part_bufs > 1 ? (tiles_done >> 1) : tiles_done;
-      if (use > 0 && !mbar_wait_lane(bar_pfree + 8 * buf, (use - 1) & 1, abort_flag)) expired();
+      if (use > 0 && !mbar_wait(bar_pfree + 8 * buf, (use - 1) & 1, abort_flag)) { give_up(); return; }
       float* pb = part + buf * part_stride + kpw * RM;
 #pragma unroll
       for (int sub = 0; sub < 2; ++sub)
@@ -1478,7 +1465,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
 #pragma unroll
           for (int i2 = 0; i2 < 4; ++i2) out[sub][mt][i2] = 0.f;
       __syncwarp();
-      if (tell) mbar_arrive(bar_pfull + 8 * buf);
+      if (lane == 0) mbar_arrive(bar_pfull + 8 * buf);
       ++tiles_done;
     }
     if (i + 1 < wk.n_units) ui.advance(wk, i + 1);

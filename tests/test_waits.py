@@ -10,7 +10,7 @@ import subprocess
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2512_03383_b200", "csrc")
-USERS = {"tc.cuh": ["prefill.cu", "single.cu", "batch.cu"], "decode.cu": ["decode.cu"]}
+USERS = {"tc.cuh": ["prefill.cu", "single.cu", "batch.cu"]}
 
 HOST = r"""
 #include <barrier>
@@ -116,14 +116,7 @@ def test_waits_of_one_lane_stand_in_code_of_one_lane(user):
     where = next(w for w, u in USERS.items() if user in u)
     for name, at, text in calls(source(user), functions(source(where))):
         line = text[text.rfind("\n", 0, at) + 1:text.find("\n", at)]
-        if line.rstrip().endswith(") expired();"):
-            # a lane of a whole warp that stays with its warp: it says so, signals nothing any more, and does not leave
-            body = re.search(r"auto expired = \[&\]\(\) \{(.*?)\};", text).group(1)
-            assert "tell = false" in body and "atomicExch(c.status" in body and "return" not in body
-        elif "ok = mbar_wait_lane(" in line:    # the decode kernel's producer: its lanes work and leave on their own, each with the status
-            after = text[text.index("if (!ok) {", at):]
-            assert "lane == 0" not in after[:after.index("return;")]
-        elif name.endswith("_lane"):
+        if name.endswith("_lane"):
             assert any("lane == 0" in b for b in blocks_around(text, at)), line
         elif "_try" in name:                   # a poll of a lane decides nothing but how long the lane polls
             assert line.strip().startswith("for (") and line.rstrip().endswith("{}"), line
