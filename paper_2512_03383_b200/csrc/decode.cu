@@ -204,7 +204,12 @@ __device__ inline bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
-// Bounded wait: false when the limit expired or another warp of the block already gave up.
+// Bounded wait: false when the limit expired or another warp of the block already gave up.  Every lane has its own answer, and a lane
+// that is told no leaves the kernel and writes the status itself: had the phase completed between two lanes' last polls, the others would
+// work on with a lane less and the sums would be wrong, so no lane may leave without a word.  (Nothing waits for a lane that has left the
+// kernel.  One answer per warp instead costs launches: a vote in front of every stage 1 - 3 %, at one to four rows above all, lanes that
+// stay to the end of their loop or a vote behind every stage 1 - 2 % at five to sixteen rows, Llama-3-8B layer at ten rows 72.6 -> 73.2
+// to 74.1 us.)
 __device__ inline bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   for (int i = 0; i < kWaitLimit; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
@@ -737,7 +742,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
         const uint32_t full = bar_full + 8 * (j % S);
         for (int i = 0; i < kWaitLimit && !mbar_try_wait(full, (j / S) & 1); ++i) {}
       }
-      if (lane == 0) atomicExch(c.status, UNIQL_ERR_TIMEOUT);
+      atomicExch(c.status, UNIQL_ERR_TIMEOUT);
     }
     return;
   }
@@ -751,7 +756,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
   // every (row slot, batch row), then stores the tile, or parks the sum for the block that finishes it.
   if (warp > CW) {
     const int etid = tid - (CW + 1) * 32;
-    auto give_up = [&]() { if (lane == 0) atomicExch(c.status, UNIQL_ERR_TIMEOUT); };
+    auto give_up = [&]() { atomicExch(c.status, UNIQL_ERR_TIMEOUT); };
     int tiles_done = 0;
     // ... and this kernel may have been started before its predecessor finished: outputs, workspace, bias,
     // positions and indices are touched only after the predecessor is complete (the producer warp waits only where the
@@ -871,7 +876,7 @@ __global__ void __launch_bounds__(NTH, 1) decode_kernel(const __grid_constant__ 
   // group of the chunk this warp works on: narrow tiles put eight more groups of the same rows in slots 32..63
   const int g_first = c.cgz > CG ? rg * CG + kpw : kpw;
   uint32_t cons_parity = 0;
-  auto give_up = [&]() { if (lane == 0) atomicExch(c.status, UNIQL_ERR_TIMEOUT); };
+  auto give_up = [&]() { atomicExch(c.status, UNIQL_ERR_TIMEOUT); };
   auto consumer_sync = [&]() -> bool {
     __syncwarp();
     if (lane == 0) mbar_arrive(bar_cons);

@@ -120,3 +120,21 @@ def test_waits_of_one_lane_stand_in_code_of_one_lane(user):
             assert any("lane == 0" in b for b in blocks_around(text, at)), line
         elif "_try" in name:                   # a poll of a lane decides nothing but how long the lane polls
             assert line.strip().startswith("for (") and line.rstrip().endswith("{}"), line
+
+
+def test_lanes_of_the_decode_kernel_leave_with_the_status():
+    """Its lanes keep their own answers and leave the kernel on their own: each that does writes the status (were it lane 0 alone,
+    another lane could leave, the sums be wrong and the launch report none)."""
+    text = source("decode.cu")
+    assert not re.search(r"lane == 0\)\s*atomicExch\(c\.status", text)
+    assert len(re.findall(r"auto give_up = \[&\]\(\) \{ atomicExch\(c\.status, UNIQL_ERR_TIMEOUT\); \};", text)) == 2
+    waits = calls(text, ["mbar_wait"])
+    assert len(waits) >= 7
+    for _, at, rest in waits:
+        behind = rest[at:at + 400]
+        if re.search(r"\bok = $", rest[:at]):      # the producer, and the barrier of the consumers
+            assert re.search(r"if \(!ok\) (break|give_up\(\))", behind), behind
+        else:
+            assert re.search(r"^[^;{]*\{\s*give_up\(\);\s*return;", behind), behind
+    producer = text[text.index("if (!ok) {\n"):]
+    assert re.search(r"\n\s*atomicExch\(c\.status, UNIQL_ERR_TIMEOUT\);\n\s*\}\n\s*return;", producer)
