@@ -33,7 +33,7 @@ __device__ inline bool pmbar_try(uint32_t bar, uint32_t parity) {
 // A bounded wait has one answer per warp: a warp whose lanes disagreed about an expired wait -- the phase may complete between two
 // lanes' last polls -- would part, and its next warp-wide instruction would wait for the missing lanes.  The vote also brings the lanes
 // together in front of that instruction.  Only a thread that waits on its own takes the form without it.  (What the vote costs where it is
-// asked for every k-block, the de-quantisers of the block pairs: 0.1 - 0.5 % of a pass; Llama-3-8B layer at 512 rows 193.0 -> 193.8 us.)
+// asked for every k-block, the de-quantisers of the block pairs: 0.1 - 0.7 % of a pass; Llama-3-8B layer at 512 rows 193.0 -> 193.8 us.)
 // `relaxed`: sleep between polls (roles that run several stages ahead and must not steal issue slots)
 __device__ inline bool pmbar_wait_lane(uint32_t bar, uint32_t parity, volatile int* abort_flag, bool relaxed = false) {
   for (int i = 0; i < kPWait; ++i) {
